@@ -402,7 +402,11 @@ int pt_checkpoint(pt_handle *h, void *buf, size_t *len);
  * ladder.  PT_ERR_ARG on a size or shape mismatch. */
 int pt_restore(pt_handle *h, const void *buf, size_t len);
 
-/* Launch schedule (results are identical for every valid choice):
+/* Launch schedule (results are identical for every valid choice).  A new handle
+ * plans its launches itself, from the sizes and the device (replica-lane mapping:
+ * a lane per replica); pt_set_schedule and pt_set_mapping replace the plan by the
+ * given mapping, and pt_get_schedule / pt_get_mapping return the values they start
+ * from:
  * slot_parallel = temperature slots one CTA processes concurrently per run
  * (threads per run = slot_parallel * L^2, a multiple of 32, <= 1024),
  * runs_per_cta = runs sharing one CTA, sweeps_per_launch = sweeps per kernel
@@ -445,10 +449,10 @@ int pt_get_mapping(const pt_handle *h, int32_t *team);
 int pt_set_walk_stats(pt_handle *h, int32_t on);
 int pt_get_walk_stats(pt_handle *h, uint64_t *hot, uint64_t *trips, uint64_t *n_passes);
 
-/* Autotuner: times every feasible (slot_parallel, runs_per_cta in {1,2,4})
- * of both mappings (slot-major teams of 2..32 lanes, 1/8 .. all slots per
- * team) for `trial_sweeps` sweeps of a batch of n_inst (1..16) copies of this
- * instance, the shape of engineer_run's speculative batches, and keeps the
+/* Autotuner: times the planned launch and every feasible (slot_parallel,
+ * runs_per_cta in {1,2,4}) of both set mappings (slot-major teams of 2..32 lanes,
+ * 1/8 .. all slots per team) for `trial_sweeps` sweeps of a batch of n_inst (1..16)
+ * copies of this instance, the shape of engineer_run's speculative batches, and keeps the
  * fastest.  The main runs are untouched; results never depend on the choice. */
 int pt_autotune(pt_handle *h, int32_t n_inst, int32_t trial_sweeps);
 

@@ -236,11 +236,11 @@ int build_group(pt_batch* b, int k)
     int cap = 0;
     BK(sweep_smem_capacity(&cap), "shared memory capacity");
     if (smem > cap) return bfail(b, PT_ERR_ARG, "a bundle needs more shared memory than a CTA can have");
-    BK(set_sweep_smem_limit(cap), "cudaFuncSetAttribute");
+    BK(set_sweep_smem_limit(cap, s.team, false, g.L), "cudaFuncSetAttribute");
     int dev = 0, sms = 0, per_sm = 0;
     BK(cudaGetDevice(&dev), "cudaGetDevice");
     BK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
-    BK(sweep_occupancy(block, (int)smem, &per_sm, sm), "occupancy");
+    BK(sweep_occupancy(block, (int)smem, &per_sm, s.team, false, g.L), "occupancy");
     if (per_sm < 1) return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " fits no CTA on an SM");
     Bundle* d = nullptr;
     BK(balloc(&d, bundles.size()), "cudaMalloc bundles");
@@ -287,7 +287,7 @@ int run_graph(pt_batch* b, int nsweeps, int xevery)
             e = cudaStreamWaitEvent(g.st, b->ev_fork, 0);
             if (e == cudaSuccess)
                 e = launch_sweeps(b->d_desc, g.d_bundles, (int)g.bundles.size(), g.grid, g.block, g.smem,
-                                  (uint32_t)b->sweep, nsweeps, xevery, 0, b->d_queue + k, g.st, g.s.team > 0, false,
+                                  (uint32_t)b->sweep, nsweeps, xevery, 0, b->d_queue + k, g.st, g.s.team, false,
                                   g.L);
             if (e == cudaSuccess) e = cudaEventRecord(g.ev, g.st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, g.ev, 0);
@@ -757,7 +757,7 @@ int pt_batch_autotune(pt_batch* b, int32_t trial_sweeps, int32_t* block_out)
                 if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue + k, 0, sizeof(int), b->stream);
                 if (e == cudaSuccess)
                     e = launch_sweeps(b->d_desc, g.d_bundles, (int)g.bundles.size(), g.grid, g.block, g.smem, 0u,
-                                      trial_sweeps, 1, 0, b->d_queue + k, b->stream, g.s.team > 0, false, g.L);
+                                      trial_sweeps, 1, 0, b->d_queue + k, b->stream, g.s.team, false, g.L);
                 if (e == cudaSuccess) e = cudaEventRecord(b->e1, b->stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(b->e1);
                 float t = 0.f;

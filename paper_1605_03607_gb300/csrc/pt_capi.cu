@@ -48,7 +48,7 @@ struct Group {
     int* d_queue = nullptr;
     std::vector<InstDesc> desc;
     std::vector<Bundle> bundles;
-    int block = 0, smem = 0;
+    int block = 0, smem = 0, team = 0;
     uint64_t sweep = 0;
     // temperature random walk (main group only, when tracked)
     bool walk = false;
@@ -77,6 +77,7 @@ struct pt_handle {
     Group main, cand;
     int sp = 0, ipc = 0, spl = 4096;
     int team = 0;              // 0: cell-major mapping; > 0: slot-major with teams of this size
+    bool planned = true;       // until a schedule is set: the replica-lane mapping, shaped by lane_plan
     uint64_t launches = 0;
     // timing of sweep launches
     bool timing = false;
@@ -266,18 +267,28 @@ int group_schedule(pt_handle* h, Group& g)
 {
     std::vector<Bundle> bundles;
     const int L2 = g.L * g.L;
+    int cap = 0, team = h->team, sp = h->sp, ipc = h->ipc;
+    LaneShape shape;
+    CK(sweep_smem_capacity(&cap), "shared memory capacity");
+    if (h->planned) {
+        int dev = 0, sms = 0;
+        CK(cudaGetDevice(&dev), "cudaGetDevice");
+        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
+        shape = lane_plan(g.L, g.NT, h->kt, g.R, g.n_inst, g.walk, sms, cap);
+        team = -shape.gr;
+        sp = shape.W;
+        ipc = shape.gr * shape.G;
+    }
     for (int i = 0; i < g.n_inst; ++i)
-        for (int r = 0; r < g.R; r += h->ipc) {
+        for (int r = 0; r < g.R; r += ipc) {
             Bundle b;
-            b.inst = i; b.run0 = r; b.nitems = std::min(h->ipc, g.R - r); b.sp = h->sp; b.team = h->team;
+            b.inst = i; b.run0 = r; b.nitems = std::min(ipc, g.R - r); b.sp = sp; b.team = team;
             bundles.push_back(b);
         }
-    const int block = (h->team > 0 ? h->sp * h->team : h->sp * L2) * h->ipc;
-    const int smem = (int)bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, g.walk, h->kt);
-    int cap = 0;
-    CK(sweep_smem_capacity(&cap), "shared memory capacity");
+    const int block = team < 0 ? lane_threads(g.NT, shape) : (team > 0 ? sp * team : sp * L2) * ipc;
+    const int smem = (int)bundle_smem_bytes(g.L, g.NT, ipc, team, g.walk, h->kt);
     if (smem > cap) return fail(h, PT_ERR_ARG, "bundle needs more shared memory than a CTA can have");
-    CK(set_sweep_smem_limit(cap), "cudaFuncSetAttribute");
+    CK(set_sweep_smem_limit(cap, team, g.walk, g.L), "cudaFuncSetAttribute");
     Bundle* d = nullptr;
     Bundle* dsub = nullptr;
     CK(dalloc(&d, bundles.size()), "cudaMalloc bundles");
@@ -296,6 +307,7 @@ int group_schedule(pt_handle* h, Group& g)
     g.bundles.swap(bundles);
     g.block = block;
     g.smem = smem;
+    g.team = team;
     return PT_OK;
 }
 
@@ -365,7 +377,7 @@ int group_sweeps(pt_handle* h, Group& g, int64_t n, int xevery, const Bundle* ds
         const int chunk = (int)std::min<int64_t>(h->spl, n - done);
         if (h->timing) CK(cudaEventRecord(h->ev[2 * li], h->stream), "event");
         CK(launch_sweeps(g.d_desc, db, nb, nb, g.block, g.smem, (uint32_t)g.sweep, chunk, xevery, 0, nullptr,
-                         h->stream, h->team > 0, g.walk, g.L),
+                         h->stream, g.team, g.walk, g.L),
            "sweep kernel");
         if (g.walk && g.NT > 1 && xevery > 0)
             g.walk_passes += (g.sweep + chunk) / (uint64_t)xevery - g.sweep / (uint64_t)xevery;
@@ -730,24 +742,27 @@ int32_t loops_gs(const int32_t* loops, int n)
     return e;
 }
 
-// Mapping (team, slot_parallel, runs_per_cta) of every group of the handle.
+// Mapping (team, slot_parallel, runs_per_cta; or the planned replica-lane one) of
+// every group of the handle.
 // On failure the handle keeps its previous mapping: a group whose new bundle
 // list could not be built keeps its old one (group_schedule), and the groups
 // already switched are switched back.
-int apply_schedule(pt_handle* h, int team, int sp, int ipc)
+int apply_schedule(pt_handle* h, bool planned, int team, int sp, int ipc)
 {
     const int ot = h->team, osp = h->sp, oipc = h->ipc;
+    const bool opl = h->planned;
+    h->planned = planned;
     h->team = team;
     h->sp = sp;
     h->ipc = std::min(ipc, h->R);
     int rc = group_schedule(h, h->main);
     if (!rc && h->cand.n_inst > 0 && (rc = group_schedule(h, h->cand))) {
         const std::string why = h->err;
-        h->team = ot; h->sp = osp; h->ipc = oipc;
+        h->team = ot; h->sp = osp; h->ipc = oipc; h->planned = opl;
         group_schedule(h, h->main);
         h->err = why;
     }
-    if (rc) { h->team = ot; h->sp = osp; h->ipc = oipc; }
+    if (rc) { h->team = ot; h->sp = osp; h->ipc = oipc; h->planned = opl; }
     return rc;
 }
 
@@ -983,7 +998,7 @@ int pt_exchange(pt_handle* h)
     if (!h) return PT_ERR_ARG;
     Group& g = h->main;
     CK(launch_sweeps(g.d_desc, g.d_bundles, (int)g.bundles.size(), (int)g.bundles.size(), g.block,
-                     g.smem, (uint32_t)g.sweep, 0, 0, 1, nullptr, h->stream, h->team > 0, g.walk, g.L),
+                     g.smem, (uint32_t)g.sweep, 0, 0, 1, nullptr, h->stream, g.team, g.walk, g.L),
        "exchange kernel");
     ++h->launches;
     if (g.walk && g.NT > 1) g.walk_passes += 1;
@@ -1715,7 +1730,8 @@ int pt_set_schedule(pt_handle* h, int32_t sp, int32_t ipc, int32_t spl)
     if (spl < 0) return fail(h, PT_ERR_ARG, "sweeps_per_launch must be >= 0");
     int rc = check_schedule(h, h->L, h->NT, nsp, nipc, h->team);
     if (rc) return rc;
-    if ((rc = apply_schedule(h, h->team, nsp, nipc))) return rc;
+    const bool keep = h->planned && sp <= 0 && ipc <= 0;       // only the launch length changes
+    if (!keep && (rc = apply_schedule(h, false, h->team, nsp, nipc))) return rc;
     if (spl > 0) h->spl = spl;
     CK(cudaStreamSynchronize(h->stream), "sync schedule");
     return PT_OK;
@@ -1727,7 +1743,7 @@ int pt_set_mapping(pt_handle* h, int32_t team, int32_t slot_parallel, int32_t ru
     const int nsp = slot_parallel > 0 ? slot_parallel : h->sp, nipc = runs_per_cta > 0 ? runs_per_cta : h->ipc;
     int rc = check_schedule(h, h->L, h->NT, nsp, nipc, team);
     if (rc) return rc;
-    if ((rc = apply_schedule(h, team, nsp, nipc))) return rc;
+    if ((rc = apply_schedule(h, false, team, nsp, nipc))) return rc;
     CK(cudaStreamSynchronize(h->stream), "sync mapping");
     return PT_OK;
 }
@@ -1748,7 +1764,7 @@ int pt_set_walk_stats(pt_handle* h, int32_t on)
         // the walk arrays enlarge each run's shared-memory block: check first
         int cap = 0;
         CK(sweep_smem_capacity(&cap), "shared memory capacity");
-        if (bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, true, h->kt) > cap)
+        if (!h->planned && bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, true, h->kt) > cap)
             return fail(h, PT_ERR_ARG, "the current schedule leaves no shared memory for the walk counters");
         unsigned long long *whot = nullptr, *wtrips = nullptr;
         uint8_t* wstate = nullptr;
@@ -1811,10 +1827,11 @@ int pt_get_walk_stats(pt_handle* h, uint64_t* hot, uint64_t* trips, uint64_t* n_
 }
 
 // Times candidate schedules on a batch of `n_inst` copies of this instance
-// (the speculative engineering batch) and keeps the fastest.  Candidates: every
-// slot_parallel with slot_parallel * L^2 a multiple of 32 and at most 1024
-// threads, with runs per CTA 1, 2 or 4 (shared memory permitting).  The
-// candidate batch is left in an unspecified state; the main runs are untouched.
+// (the speculative engineering batch) and keeps the fastest.  Candidates: the
+// planned replica-lane shape, then every slot_parallel with slot_parallel * L^2
+// a multiple of 32 and at most 1024 threads and the slot-major teams, with runs
+// per CTA 1, 2 or 4 (shared memory permitting).  The candidate batch is left in
+// an unspecified state; the main runs are untouched.
 int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
 {
     if (!h || n_inst < 1 || n_inst > 16 || trial_sweeps < 1) return fail(h, PT_ERR_ARG, "need 1 <= n_inst <= 16, trial_sweeps >= 1");
@@ -1832,48 +1849,48 @@ int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
     int cap = 0;
     CK(sweep_smem_capacity(&cap), "shared memory capacity");
     const int old_sp = h->sp, old_ipc = h->ipc, old_team = h->team;
-    const bool old_timing = h->timing;
-    h->timing = true;
-    double best_rate = 0.0;
-    int best_sp = old_sp, best_ipc = old_ipc, best_team = old_team;
-    // candidate (team, slot_parallel) pairs: cell-major (team 0) and slot-major
-    std::vector<std::pair<int, int>> cands;
+    const bool old_timing = h->timing, old_planned = h->planned;
+    struct Cand { bool planned; int team, sp, ipc; };
+    std::vector<Cand> cands = {{true, old_team, old_sp, old_ipc}};
     for (int sp = 1; sp <= h->NT && sp * L2 <= MAX_THREADS; ++sp)
-        if ((sp * L2) % 32 == 0) cands.push_back({0, sp});
+        if ((sp * L2) % 32 == 0)
+            for (int ipc : {1, 2, 4})
+                if (sp * L2 * ipc <= MAX_THREADS) cands.push_back({false, 0, sp, ipc});
     for (int team : {2, 4, 8, 16, 32}) {
         if (team > L2) break;
         for (int nt : {h->NT, (h->NT + 1) / 2, (h->NT + 3) / 4, (h->NT + 7) / 8})
-            if (nt >= 1 && nt * team >= 32 && nt * team <= MAX_THREADS_SM) cands.push_back({team, nt});
+            for (int ipc : {1, 2, 4})
+                if (nt >= 1 && nt * team >= 32 && nt * team * ipc <= MAX_THREADS_SM) cands.push_back({false, team, nt, ipc});
     }
-    for (const auto& c : cands) {
-        const int team = c.first, sp = c.second;
-        const int tpr = team > 0 ? sp * team : sp * L2;
-        for (int ipc : {1, 2, 4}) {
-            if (tpr * ipc > (team > 0 ? MAX_THREADS_SM : MAX_THREADS) || ipc > h->R) break;
-            if (bundle_smem_bytes(h->L, h->NT, ipc, team, false, h->kt) > cap) break;
-            h->team = team;
-            h->sp = sp;
-            h->ipc = ipc;
-            if (!(rc = group_schedule(h, g))) rc = group_sweeps(h, g, trial_sweeps, 1);
-            if (rc) {
-                h->timing = old_timing;
-                h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
-                return rc;
-            }
-            CK(cudaStreamSynchronize(h->stream), "sync autotune");
-            double ms = 0.0;
-            for (int i = 0; i < h->ev_used; ++i) {
-                float t = 0.f;
-                CK(cudaEventElapsedTime(&t, h->ev[2 * i], h->ev[2 * i + 1]), "event time");
-                ms += t;
-            }
-            const double rate = (double)g.n_inst * h->R * h->NT * h->N * trial_sweeps / (ms * 1e-3);
-            if (rate > best_rate) { best_rate = rate; best_sp = sp; best_ipc = ipc; best_team = team; }
+    h->timing = true;
+    double best_ms = 1e300;
+    Cand best = cands[0];
+    for (const Cand& c : cands) {
+        if (!c.planned && (c.ipc > h->R || bundle_smem_bytes(h->L, h->NT, c.ipc, c.team, false, h->kt) > cap)) continue;
+        h->planned = c.planned;
+        h->team = c.team;
+        h->sp = c.sp;
+        h->ipc = c.ipc;
+        if (!(rc = group_schedule(h, g))) rc = group_sweeps(h, g, trial_sweeps, 1);
+        cudaError_t e = rc ? cudaSuccess : cudaStreamSynchronize(h->stream);
+        double ms = 0.0;
+        for (int i = 0; i < h->ev_used && !rc && e == cudaSuccess; ++i) {
+            float t = 0.f;
+            e = cudaEventElapsedTime(&t, h->ev[2 * i], h->ev[2 * i + 1]);
+            ms += t;
         }
+        if (rc || e != cudaSuccess) {
+            h->timing = old_timing;
+            h->planned = old_planned;
+            h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
+            return rc ? rc : cuda_fail(h, e, "sync autotune");
+        }
+        if (ms < best_ms) { best_ms = ms; best = c; }
     }
     h->timing = old_timing;
+    h->planned = old_planned;
     h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
-    if ((rc = apply_schedule(h, best_team, best_sp, best_ipc))) return rc;
+    if ((rc = apply_schedule(h, best.planned, best.team, best.sp, best.ipc))) return rc;
     CK(cudaStreamSynchronize(h->stream), "sync autotune");
     return PT_OK;
 }

@@ -22,6 +22,10 @@ constexpr int MAX_THREADS = 1024;
 // CTA size limit of the slot-major sweep kernel: its register budget (up to
 // 80 per thread) fits 768 threads per CTA.
 constexpr int MAX_THREADS_SM = 768;
+// CTA size limit of the replica-lane kernel, and its groups: one hardware barrier
+// each besides the CTA's.
+constexpr int LANE_THREADS = 1024;
+constexpr int LANE_GROUPS = 15;
 
 // Per instance.  All pointers are device pointers.
 //
@@ -63,14 +67,11 @@ struct InstDesc {
 //              and every sp-th temperature slot.
 //   team  > 0 (slot-major): sp teams of `team` lanes (a power of two <= 32)
 //              per run; a team owns every sp-th slot, its lanes split the cells.
+//   team  < 0 (replica-lane): groups of -team runs whose replicas fill the lanes
+//              of warps ("columns" of 32); sp warps per column split the cells.
 struct Bundle {
     int32_t inst, run0, nitems, sp, team;
 };
-
-__host__ __device__ inline int threads_per_run(int L, const Bundle& b)
-{
-    return b.team > 0 ? b.sp * b.team : b.sp * L * L;
-}
 
 // Shared-memory layout of one bundle: the Metropolis table of the instance,
 // then per item (run): spins [NT][N] (colour-major words per buffer, plus
@@ -134,8 +135,51 @@ void set_global_error(const char* msg);
 constexpr int CELL_REC = 12;
 __host__ __device__ inline int64_t cell_table_bytes(int L) { return 4LL * CELL_REC * 2 * L * L; }
 
+// Replica-lane mapping.  A lane owns one replica (configuration buffer), its
+// spins held as one byte per (colour, cell): four times the 4-bit mask of the
+// cell's negative spins of that colour, so a byte is the offset of its entry in a
+// 16-word table.  A group of `gr` runs fills columns of 32 replicas, `W` warps per
+// column split the cells, and groups never wait for each other.  Shared memory:
+//   lut    [2][L^2][3][16] words: for every (colour, cell), the summed fields
+//          of its 4 spins from the opposite group of the cell and from the
+//          minus- and plus-neighbour groups, packed one byte per spin
+//          (the sum of the three entries is 128 - h_i, byte by byte)
+//   thr    [ceil(NT/32)][kt][32] acceptance thresholds, a column per slot; an
+//          entry of a field k <= 0 is read from the bytes below it and not used,
+//          so the table starts at least kt - 1 rows above the bundle's start
+//   xtab   exchange offsets [NT], search hints [NT]
+//   per group: pre [2][L^2] the sweep's Philox terms of the cell's spins; then per
+//          column spins [2][L + L^2 + L][32] bytes (L cells of zeros at either end
+//          stand for the missing neighbours of the border: their fields are 0);
+//          then per run E, criteria, counters, slot maps, walk, record (ItemLayout)
+struct LaneLayout {
+    int32_t ncols;                           // columns of a group
+    int32_t lut, thr, xtab, groups;          // byte offsets
+    int32_t spins, col_bytes, runs, run_bytes, group_bytes, bytes;   // spins, runs: inside a group
+};
+
+__host__ __device__ inline LaneLayout lane_layout(int L, int NT, int kt, int gr, int ngroups, bool walk)
+{
+    const int L2 = L * L;
+    LaneLayout o;
+    o.ncols = (gr * NT + 31) / 32;
+    o.lut = 0;
+    const int lut_end = 384 * L2, below = 128 * (kt - 1);
+    o.thr = (lut_end > below ? lut_end : below);
+    o.xtab = o.thr + (NT + 31) / 32 * kt * 128;
+    o.groups = (int32_t)pad16(o.xtab + 8 * NT);
+    o.spins = 32 * L2;
+    o.col_bytes = 64 * (L2 + 2 * L);
+    o.runs = o.spins + o.ncols * o.col_bytes;
+    o.run_bytes = (int32_t)(item_layout(0, NT, 0, walk).bytes + 64 * ((NT + 6) / 8 + 1));   // + exchange scratch
+    o.group_bytes = o.runs + gr * o.run_bytes;
+    o.bytes = o.groups + ngroups * o.group_bytes;
+    return o;
+}
+
 inline int64_t bundle_smem_bytes(int L, int NT, int nitems, int team = 0, bool walk = false, int kt = KT_DEFAULT)
 {
+    if (team < 0) return lane_layout(L, NT, kt, -team, (nitems - team - 1) / -team, walk).bytes;
     if (team > 0)
         return table_bytes(NT, kt) + cell_table_bytes(L) +
                (int64_t)nitems * item_layout(L, NT, sm_pad(L, team), walk).bytes;

@@ -4,7 +4,11 @@
 // (Appendix A), parallel tempering of Sec. II (independent Metropolis updates,
 // neighbour swaps with detailed-balance acceptance), sweeps as in Sec. III.B.
 //
-// Design (GB300):
+// Three mappings of the work to threads: replica-lane (pt_lane.cuh; the one used
+// unless a schedule is set), cell-major and slot-major (below; set_mapping and
+// set_schedule).  Results never depend on the mapping.
+//
+// Design of cell-major and slot-major:
 //   * One CTA "bundle" = a few PT runs of one instance.  Every replica of those
 //     runs lives in shared memory for the whole launch as int8 spins, one
 //     32-bit word per group of 4 same-colour spins of a cell, colour-major.
@@ -97,18 +101,18 @@ __device__ __forceinline__ int half_gap_search(const uint32_t* tab, int H, uint3
 // point gives the exact result; keeping the first estimate live through the
 // search measured 1 % slower).  Debug builds also search on the closed-form
 // path and record code 8 if the two ever differ.
-__device__ __forceinline__ int critical_half_gap(const InstDesc& in, const int32_t* xoff_sm,
+__device__ __forceinline__ int critical_half_gap(const uint32_t* xthr, int NT, const int32_t* xoff_sm,
                                                  const float* xhint_sm, int p, uint32_t u)
 {
     const int o = xoff_sm[p];
 #ifdef PT_DEBUG
-    const int total = xoff_sm[in.NT - 1];
+    const int total = xoff_sm[NT - 1];
     const int H = (o < 0 || xoff_sm[p + 1] < o || xoff_sm[p + 1] > total)
                       ? (atomicCAS(&g_pt_debug_code, 0u, 3u), 0) : xoff_sm[p + 1] - o;
 #else
     const int H = xoff_sm[p + 1] - o;
 #endif
-    const uint32_t* tab = in.xthr + o - 1;       // tab[h], h = 1..H
+    const uint32_t* tab = xthr + o - 1;       // tab[h], h = 1..H
     if (u == 0u) return H;                       // every entry is >= 1
     const float hint = xhint_sm[p];
     const float x = u < (1u << 24) ? (float)(u + 1u) : (float)u;
@@ -236,19 +240,17 @@ __device__ __forceinline__ void colour_phase(const CellRegs& cr, uint32_t* sw, i
 // (called by one group of 32 threads; lane l handles pairs l and l + 32, the
 // four lanes of pairs 4c..4c+3 each forming the Philox call c and taking its
 // own word).  Table offsets and search hints come from shared memory.
-__device__ __forceinline__ void exchange_prepare(const InstDesc& in, const uint32_t* thr_sm, int lane,
+__device__ __forceinline__ void exchange_prepare(const uint32_t* xthr, const int32_t* xoff_sm, int lane,
                                                  uint32_t s, uint32_t runbits, uint32_t k0, uint32_t k1,
                                                  int NT, int32_t* cc)
 {
-    // bundle tables: thr [NT][kt], then exchange offsets [NT] and search hints [NT]
-    const int32_t* xoff_sm = reinterpret_cast<const int32_t*>(thr_sm + NT * in.kt);
-    const float* xhint_sm = reinterpret_cast<const float*>(thr_sm + NT * in.kt + NT);
+    const float* xhint_sm = reinterpret_cast<const float*>(xoff_sm + NT);   // offsets [NT], then search hints [NT]
     const int npairs = NT - 1;
     for (int p = lane; p < npairs; p += 32) {
         const uint4 w = philox10(s, runbits, (uint32_t)(p >> 2), 1u, k0, k1);
         const int e = p & 3;
         const uint32_t u = e == 0 ? w.x : e == 1 ? w.y : e == 2 ? w.z : w.w;
-        cc[p] = critical_half_gap(in, xoff_sm, xhint_sm, p, u);
+        cc[p] = critical_half_gap(xthr, NT, xoff_sm, xhint_sm, p, u);
     }
 }
 
@@ -467,6 +469,7 @@ __device__ void process_bundle(const InstDesc* __restrict__ insts, const Bundle 
     // bundle tables: thr [NT][kt], then exchange offsets [NT] and search hints [NT]
     const int KTI = in.kt;
     uint32_t* thr_sm = reinterpret_cast<uint32_t*>(smem);
+    const int32_t* xoff_sm = reinterpret_cast<const int32_t*>(thr_sm + NT * KTI);
     unsigned char* ib = smem + table_bytes(NT, KTI) + (active ? item : 0) * lay.bytes;
     uint32_t* sw = reinterpret_cast<uint32_t*>(ib + lay.spins);
     int32_t* Es = reinterpret_cast<int32_t*>(ib + lay.E);
@@ -540,7 +543,7 @@ __device__ void process_bundle(const InstDesc* __restrict__ insts, const Bundle 
     const uint32_t s_first = (mode == 0) ? sweep0 + 1u : sweep0;
     __syncthreads();                            // tables staged before the first exchange preparation
     if (n_iter > 0 && exch(s_first) && active && j >= prep_warp_j0)
-        exchange_prepare(in, thr_sm, j - prep_warp_j0, s_first, runbits, k0, k1, NT, ccrit + (s_first & 1u) * NT);
+        exchange_prepare(in.xthr, xoff_sm, j - prep_warp_j0, s_first, runbits, k0, k1, NT, ccrit + (s_first & 1u) * NT);
     __syncthreads();
 
     for (int it = 0; it < n_iter; ++it) {
@@ -581,7 +584,7 @@ __device__ void process_bundle(const InstDesc* __restrict__ insts, const Bundle 
         }
         // meanwhile the last warp prepares the next sweep's exchange criteria
         if (it + 1 < n_iter && exch(s + 1u) && active && j >= prep_warp_j0)
-            exchange_prepare(in, thr_sm, j - prep_warp_j0, s + 1u, runbits, k0, k1, NT, ccrit + ((s + 1u) & 1u) * NT);
+            exchange_prepare(in.xthr, xoff_sm, j - prep_warp_j0, s + 1u, runbits, k0, k1, NT, ccrit + ((s + 1u) & 1u) * NT);
         __syncthreads();
     }
 
@@ -688,6 +691,7 @@ __device__ void process_bundle_sm(const InstDesc* __restrict__ insts, const Bund
 
     const int KTI = in.kt;
     uint32_t* thr_sm = reinterpret_cast<uint32_t*>(smem);
+    const int32_t* xoff_sm = reinterpret_cast<const int32_t*>(thr_sm + NT * KTI);
     uint32_t* rec_sm = reinterpret_cast<uint32_t*>(smem + table_bytes(NT, KTI));   // [2][L2][CELL_REC]
     unsigned char* ib = smem + table_bytes(NT, KTI) + cell_table_bytes(L) + (active ? item : 0) * lay.bytes;
     uint32_t* sw = reinterpret_cast<uint32_t*>(ib + lay.spins);
@@ -764,7 +768,7 @@ __device__ void process_bundle_sm(const InstDesc* __restrict__ insts, const Bund
     const uint32_t s_first = (mode == 0) ? sweep0 + 1u : sweep0;
     __syncthreads();                            // tables staged before the first exchange preparation
     if (n_iter > 0 && exch(s_first) && active && j >= prep_warp_j0)
-        exchange_prepare(in, thr_sm, j - prep_warp_j0, s_first, runbits, k0, k1, NT, ccrit + (s_first & 1u) * NT);
+        exchange_prepare(in.xthr, xoff_sm, j - prep_warp_j0, s_first, runbits, k0, k1, NT, ccrit + (s_first & 1u) * NT);
     __syncthreads();
 
     for (int it = 0; it < n_iter; ++it) {
@@ -820,7 +824,7 @@ __device__ void process_bundle_sm(const InstDesc* __restrict__ insts, const Bund
             }
         }
         if (it + 1 < n_iter && exch(s + 1u) && active && j >= prep_warp_j0)
-            exchange_prepare(in, thr_sm, j - prep_warp_j0, s + 1u, runbits, k0, k1, NT,
+            exchange_prepare(in.xthr, xoff_sm, j - prep_warp_j0, s + 1u, runbits, k0, k1, NT,
                              ccrit + ((s + 1u) & 1u) * NT);
         __syncthreads();
     }
@@ -850,6 +854,39 @@ __device__ void process_bundle_sm(const InstDesc* __restrict__ insts, const Bund
         }
     }
     __syncthreads();
+}
+
+}  // namespace
+}  // namespace ptg
+
+#include "pt_lane.cuh"
+
+namespace ptg {
+namespace {
+
+// Bundles of the replica-lane mapping, one after the other (queue: pulled from
+// the launch's work counter).
+template <int LT>
+__global__ void __launch_bounds__(LANE_THREADS, 1)
+pt_lane_kernel(const InstDesc* __restrict__ insts, const Bundle* __restrict__ bundles, int nbundles, uint32_t sweep0,
+               int nsweeps, int xevery, int mode, int* __restrict__ queue)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_next;
+    int b = blockIdx.x;
+    if (queue) {
+        if (threadIdx.x == 0) s_next = atomicAdd(queue, 1);
+        __syncthreads();
+        b = s_next;
+    }
+    while (b < nbundles) {
+        process_bundle_lane<LT>(insts, bundles[b], sweep0, nsweeps, xevery, mode, smem);
+        if (!queue) break;
+        if (threadIdx.x == 0) s_next = atomicAdd(queue, 1);
+        __syncthreads();
+        b = s_next;
+        __syncthreads();
+    }
 }
 
 // SLOT_MAJOR selects the mapping of every bundle of the launch, WALK whether
@@ -1061,6 +1098,33 @@ unsigned debug_take() { return 0u; }
 #define DBG(e, st, what) (e)
 #endif
 
+namespace {
+// The sweep kernel of a mapping (by the sign of `team`) for lattice side L.
+const void* sweep_kernel(int team, bool walk, int L)
+{
+    if (team < 0) {
+        switch (L) {
+        case 4: return (const void*)pt_lane_kernel<4>;
+        case 6: return (const void*)pt_lane_kernel<6>;
+        case 8: return (const void*)pt_lane_kernel<8>;
+        case 10: return (const void*)pt_lane_kernel<10>;
+        case 12: return (const void*)pt_lane_kernel<12>;
+        case 14: return (const void*)pt_lane_kernel<14>;
+        case 16: return (const void*)pt_lane_kernel<16>;
+        default: return (const void*)pt_lane_kernel<0>;
+        }
+    }
+    if (team == 0) return walk ? (const void*)pt_sweep_kernel<false, true> : (const void*)pt_sweep_kernel<false, false>;
+    switch (L) {
+    case 4: return walk ? (const void*)pt_sweep_kernel<true, true, 4> : (const void*)pt_sweep_kernel<true, false, 4>;
+    case 8: return walk ? (const void*)pt_sweep_kernel<true, true, 8> : (const void*)pt_sweep_kernel<true, false, 8>;
+    case 12: return walk ? (const void*)pt_sweep_kernel<true, true, 12> : (const void*)pt_sweep_kernel<true, false, 12>;
+    case 16: return walk ? (const void*)pt_sweep_kernel<true, true, 16> : (const void*)pt_sweep_kernel<true, false, 16>;
+    default: return walk ? (const void*)pt_sweep_kernel<true, true> : (const void*)pt_sweep_kernel<true, false>;
+    }
+}
+}  // namespace
+
 cudaError_t sweep_smem_capacity(int* bytes)
 {
     int dev = 0, optin = 0;
@@ -1068,43 +1132,18 @@ cudaError_t sweep_smem_capacity(int* bytes)
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
-    size_t stat = 0;
-    const void* ks[12] = {(const void*)pt_sweep_kernel<false, false>, (const void*)pt_sweep_kernel<true, false>,
-                          (const void*)pt_sweep_kernel<false, true>, (const void*)pt_sweep_kernel<true, true>,
-                          (const void*)pt_sweep_kernel<true, false, 4>, (const void*)pt_sweep_kernel<true, false, 8>,
-                          (const void*)pt_sweep_kernel<true, false, 12>, (const void*)pt_sweep_kernel<true, false, 16>,
-                          (const void*)pt_sweep_kernel<true, true, 4>, (const void*)pt_sweep_kernel<true, true, 8>,
-                          (const void*)pt_sweep_kernel<true, true, 12>, (const void*)pt_sweep_kernel<true, true, 16>};
-    for (const void* k : ks) {
-        cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, k);
-        if (e != cudaSuccess) return e;
-        stat = fa.sharedSizeBytes > stat ? fa.sharedSizeBytes : stat;
-    }
-    *bytes = optin - (int)stat;
+    *bytes = optin - 16;                     // the kernels' own shared memory: the next bundle's index
     return cudaSuccess;
 }
 
-cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, bool slot_major, bool walk)
+cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, int team, bool walk, int L)
 {
-    const void* k = slot_major ? (walk ? (const void*)pt_sweep_kernel<true, true> : (const void*)pt_sweep_kernel<true, false>)
-                               : (walk ? (const void*)pt_sweep_kernel<false, true> : (const void*)pt_sweep_kernel<false, false>);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, block, smem_bytes);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_kernel(team, walk, L), block, smem_bytes);
 }
 
-cudaError_t set_sweep_smem_limit(int bytes)
+cudaError_t set_sweep_smem_limit(int bytes, int team, bool walk, int L)
 {
-    const void* ks[12] = {(const void*)pt_sweep_kernel<false, false>, (const void*)pt_sweep_kernel<true, false>,
-                          (const void*)pt_sweep_kernel<false, true>, (const void*)pt_sweep_kernel<true, true>,
-                          (const void*)pt_sweep_kernel<true, false, 4>, (const void*)pt_sweep_kernel<true, false, 8>,
-                          (const void*)pt_sweep_kernel<true, false, 12>, (const void*)pt_sweep_kernel<true, false, 16>,
-                          (const void*)pt_sweep_kernel<true, true, 4>, (const void*)pt_sweep_kernel<true, true, 8>,
-                          (const void*)pt_sweep_kernel<true, true, 12>, (const void*)pt_sweep_kernel<true, true, 16>};
-    for (const void* k : ks) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return cudaFuncSetAttribute(sweep_kernel(team, walk, L), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 cudaError_t launch_init(const InstDesc* insts, const int2* items, int nitems, bool draw,
@@ -1125,32 +1164,11 @@ cudaError_t launch_energy(const InstDesc* insts, const int2* items, int nitems, 
 
 cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nbundles, int grid,
                           int block, int smem_bytes, uint32_t sweep0, int nsweeps, int xevery,
-                          int mode, int* queue, cudaStream_t st, bool slot_major, bool walk, int L)
+                          int mode, int* queue, cudaStream_t st, int team, bool walk, int L)
 {
     if (nbundles <= 0) return cudaSuccess;
-#define PT_SM_LAUNCH(W, LT)                                                                                   \
-    pt_sweep_kernel<true, W, LT><<<grid, block, smem_bytes, st>>>(insts, bundles, nbundles, sweep0, nsweeps, \
-                                                                  xevery, mode, queue)
-#define PT_SM_LAUNCH_L(W)                                                                                     \
-    do {                                                                                                      \
-        if (L == 4) PT_SM_LAUNCH(W, 4);                                                                       \
-        else if (L == 8) PT_SM_LAUNCH(W, 8);                                                                  \
-        else if (L == 12) PT_SM_LAUNCH(W, 12);                                                                \
-        else if (L == 16) PT_SM_LAUNCH(W, 16);                                                                \
-        else PT_SM_LAUNCH(W, 0);                                                                              \
-    } while (0)
-    if (slot_major && walk)
-        PT_SM_LAUNCH_L(true);
-    else if (slot_major)
-        PT_SM_LAUNCH_L(false);
-#undef PT_SM_LAUNCH_L
-#undef PT_SM_LAUNCH
-    else if (walk)
-        pt_sweep_kernel<false, true><<<grid, block, smem_bytes, st>>>(insts, bundles, nbundles, sweep0, nsweeps,
-                                                                      xevery, mode, queue);
-    else
-        pt_sweep_kernel<false, false><<<grid, block, smem_bytes, st>>>(insts, bundles, nbundles, sweep0, nsweeps,
-                                                                       xevery, mode, queue);
+    void* args[] = {&insts, &bundles, &nbundles, &sweep0, &nsweeps, &xevery, &mode, &queue};
+    cudaLaunchKernel(sweep_kernel(team, walk, L), dim3(grid), dim3(block), args, smem_bytes, st);
     return DBG(cudaGetLastError(), st, "sweep kernel");
 }
 

@@ -6,26 +6,28 @@
 
 namespace ptg {
 
-// Largest dynamic shared memory a sweep-kernel CTA may request on the current device.
+// Largest dynamic shared memory a sweep-kernel CTA may request on the current
+// device, and the limit set for the kernel that launch_sweeps picks for
+// (team, walk, L).
 cudaError_t sweep_smem_capacity(int* bytes);
-cudaError_t set_sweep_smem_limit(int bytes);
+cudaError_t set_sweep_smem_limit(int bytes, int team = 0, bool walk = false, int L = 0);
 // Resident sweep-kernel CTAs per SM for a block size and dynamic shared memory.
-cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, bool slot_major = false,
-                            bool walk = false);
+cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, int team = 0, bool walk = false,
+                            int L = 0);
 cudaError_t launch_init(const InstDesc* insts, const int2* items, int nitems, bool draw,
                         cudaStream_t st);
 cudaError_t launch_energy(const InstDesc* insts, const int2* items, int nitems, int32_t first_value,
                           cudaStream_t st);
 // mode 0: nsweeps sweeps s = sweep0+1..; mode 1: one exchange sweep with counter sweep0.
-// slot_major: every bundle uses the slot-major mapping (Bundle::team > 0),
-// otherwise the cell-major one (Bundle::team == 0).  walk: the instances carry
+// team: the mapping of every bundle by its sign (Bundle::team).  walk: the instances carry
 // walk arrays (InstDesc::whot, wtrips, wstate) and the launch updates them.
 // L: the lattice side of every instance in the launch (0 if unknown or mixed);
-// both slot-major kernels (walk tracked or not) have instantiations for
-// L = 4, 8, 12 and 16 with the side as a compile-time constant.
+// the replica-lane kernel (even L >= 4) and both slot-major kernels (walk tracked
+// or not; L = 4, 8, 12, 16) have instantiations with the side as a compile-time
+// constant.
 cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nbundles, int grid,
                           int block, int smem_bytes, uint32_t sweep0, int nsweeps, int xevery,
-                          int mode, int* queue, cudaStream_t st, bool slot_major = false,
+                          int mode, int* queue, cudaStream_t st, int team = 0,
                           bool walk = false, int L = 0);
 // dist [n][n]: spins differing between sampled configurations of instance 0
 // (sample k: run run[k], slot slot[k]; device arrays).

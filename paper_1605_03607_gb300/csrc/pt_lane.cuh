@@ -1,0 +1,518 @@
+// pt_lane.cuh -- the replica-lane sweep kernel (included by pt_kernels.cu).
+//
+// One lane = one replica (configuration buffer) of a run, at the temperature of
+// the slot that holds it.  A warp updates one cell's 4 spins of a colour in 32
+// replicas at once (a "warp word"), so everything that belongs to the cell is
+// warp-uniform: its coupler tables, its neighbours' addresses, and the products
+// of the Philox call that do not depend on the replica.  What that buys over a
+// lane per cell (pt_sweep_kernel), per 4-spin word:
+//   * the local fields come from three 16-entry tables (16 entries lie in 16
+//     banks: no conflicts) and one add, instead of 8 dp4a on couplers loaded
+//     per word;
+//   * the threshold's shared address is one dp4a (byte extraction, row pitch and
+//     the slot's column in one instruction), and a slot's thresholds lie in its
+//     own bank; a field k <= 0 accepts through the sign of its byte;
+//   * 16 wide multiplies per Philox call instead of 17, the round keys in uniform
+//     registers;
+//   * 2 x 2 cells a step: half of the neighbours are loaded once for two cells, and
+//     loop and address instructions are shared.
+// Bound: warp instruction issue.  A wide multiply holds the dispatch of its
+// sub-partition for two cycles (4 on its pipe); 82 instructions and 16 wide
+// multiplies a word leave 115 clocks at the 85 % issue rate that this mix reaches,
+// against 110 instructions and 199 clocks before.  Measured, C_8 x 32 slots,
+// 1024 runs: 14.4 us per sweep (1.17e12 attempts/s; slot-major 4/32/1: 20.7 us,
+// 8.1e11); one C_8 instance of 64 runs: 3.1 us per sweep (cell-major default: 11.7).
+// Measured and left: 1 or 2 cells a step instead of 4 (1 % slower), keys as immediates
+// (recomputed per round, 7 more uniform instructions a word), accept flags by LOP3
+// instead of adds (1 % slower), by selects (2 % slower).
+#pragma once
+
+namespace ptg {
+namespace {
+
+// The terms of a group's Philox call that depend on (sweep, group) only.
+__device__ __forceinline__ uint4 lane_pre(uint32_t s, int col, int q, int L, uint32_t k0, uint32_t k1)
+{
+    const int r = q / L, c = q - r * L, u = (r + c + col) & 1;
+    const PhiloxPre p = philox_pre(s, (uint32_t)(2 * q + u), k0, k1);
+    return make_uint4(p.x0b, p.z2x, p.z3, 0u);
+}
+
+// One entry of the field tables: `which` 0 the cell's opposite group (with the
+// bias of 128 per byte), 1 / 2 the minus / plus neighbour, for the mask `nib` of
+// that group's negative spins.  jw holds the negated couplers (InstDesc), so the
+// three entries of an update add up to 128 - h_i in byte i.
+__device__ __forceinline__ uint32_t lane_field(const uint32_t* jw, int which, int nib)
+{
+    uint32_t w = 0u, sg = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sg |= ((nib >> k) & 1 ? 0xFFu : 0x01u) << (8 * k);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int v;
+        if (which == 0) {
+            v = 128 + __dp4a((int)jw[k], (int)sg, 0);
+        } else {
+            const int j = (int)(int8_t)(jw[4 + k] >> (16 * (k & 1) + 8 * (which - 1)));
+            v = (nib >> k) & 1 ? -j : j;
+        }
+        w += (uint32_t)v << (8 * k);
+    }
+    return w;
+}
+
+// 0xFF in every byte of x whose sign bit is set, 0 in the others.
+__device__ __forceinline__ uint32_t byte_signs(uint32_t x)
+{
+    uint32_t m;
+    asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(m) : "r"(x));
+    return m;
+}
+
+struct LaneConst {
+    uint32_t c1, y2x, y1k;           // Philox: run and slot word, terms of the sweep
+    uint32_t ka[7], kb[7];           // round keys of rounds 3..9
+    uint32_t tcol;                   // shared address of this slot's threshold column, row k = -127
+    int kt;
+};
+
+// U cells of one colour, their 4 spins each: `o` their bytes (replaced), `hb` the packed
+// 128 - h_i, `pr` the cells' Philox terms.  Step by step over the cells, so that their
+// chains of dependent instructions overlap.
+template <int U>
+__device__ __forceinline__ void lane_words(uint32_t (&o)[U], const uint32_t (&hb)[U], const uint4 (&pr)[U],
+                                           const LaneConst& lc, uint32_t& dk, uint32_t& pc)
+{
+    uint32_t kb[U], a0[U], a1[U], a2[U], a3[U], th[U][4];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        // byte j of m: 0xFF where spin j is -1 (its mask bit moved to the byte's sign, which is replicated)
+        const uint32_t m = byte_signs(o[i] * 0x04081020u);
+        kb[i] = (hb[i] ^ m) - (~m & 0x01010101u);                 // 127 + k, k = -s h: dE = 2 k
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            // shared address of row k of the slot's column: byte j of kb times 128 plus the column
+            uint32_t a = __dp4a(kb[i], 0x80u << (8 * j), lc.tcol);
+#ifdef PT_DEBUG
+            const int k = (int)((kb[i] >> (8 * j)) & 255u) - 127;
+            if (k >= lc.kt || k <= -lc.kt) { atomicCAS(&g_pt_debug_code, 0u, 1u); a = lc.tcol + 127u * 128u; }
+#endif
+            asm("ld.shared.u32 %0, [%1];" : "=r"(th[i][j]) : "r"(a));
+        }
+    }
+    // the Philox call (philox_slot) from the cell's and the sweep's terms
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        const uint64_t C = (uint64_t)PHILOX_M0 * (pr[i].x ^ lc.c1);
+        const uint64_t F = (uint64_t)PHILOX_M1 * ((uint32_t)(C >> 32) ^ lc.y2x);
+        a0[i] = (uint32_t)(F >> 32) ^ lc.y1k;
+        a1[i] = (uint32_t)F;
+        a2[i] = pr[i].y ^ (uint32_t)C;
+        a3[i] = pr[i].z;
+    }
+#pragma unroll
+    for (int r = 0; r < 7; ++r)
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const uint64_t p0 = (uint64_t)PHILOX_M0 * a0[i], p1 = (uint64_t)PHILOX_M1 * a2[i];
+            a0[i] = (uint32_t)(p1 >> 32) ^ a1[i] ^ lc.ka[r];
+            a2[i] = (uint32_t)(p0 >> 32) ^ a3[i] ^ lc.kb[r];
+            a1[i] = (uint32_t)p1;
+            a3[i] = (uint32_t)p0;
+        }
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        uint32_t f = 0u;
+        if (a0[i] < th[i][0]) f += 0x00000080u;
+        if (a1[i] < th[i][1]) f += 0x00008000u;
+        if (a2[i] < th[i][2]) f += 0x00800000u;
+        if (a3[i] < th[i][3]) f += 0x80000000u;
+        f = (f | ~kb[i]) & 0x80808080u;                           // k <= 0: accepted
+        dk = __dp4a(kb[i], f, dk);                                // += 128 (k + 127) per accepted flip
+        pc = __dp4a(f, 0x01010101u, pc);                          // += 128 per accepted flip
+        o[i] ^= (f * 0x00204081u) >> 26;                          // the four flags to bits 2..5
+    }
+}
+
+__device__ __forceinline__ uint32_t lane_fields(const unsigned char* lut, uint32_t in, uint32_t mn, uint32_t pl)
+{
+    return *reinterpret_cast<const uint32_t*>(lut + in) + *reinterpret_cast<const uint32_t*>(lut + 64 + mn) +
+           *reinterpret_cast<const uint32_t*>(lut + 128 + pl);
+}
+
+// The pair of cells q, q + 1 (U = 2; q alone for U = 1) of one colour, odd L.  V = 0:
+// cell q has its neighbours above and below (`up` bytes away), cell q + 1 to its left
+// and right; V = 1: the other way round.  Pointers are to cell q.
+template <int U, int V>
+__device__ __forceinline__ void lane_pair(const unsigned char* lut, unsigned char* own, const unsigned char* opp, int up,
+                                          const uint4* pre, const LaneConst& lc, uint32_t& dk, uint32_t& pc)
+{
+    uint32_t o[U], hb[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        const int d = (i ^ V) & 1 ? 32 : up;
+        o[i] = own[i * 32];
+        hb[i] = lane_fields(lut + i * 192, opp[i * 32], opp[i * 32 - d], opp[i * 32 + d]);
+    }
+    uint4 pr[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i) pr[i] = pre[i];
+    lane_words<U>(o, hb, pr, lc, dk, pc);
+#pragma unroll
+    for (int i = 0; i < U; ++i) own[i * 32] = (unsigned char)o[i];
+}
+
+// A block of 2 x 2 cells, even row and column first: cells q, q + 1, q + L, q + L + 1.
+// Two of them have their neighbours above and below, two to the left and right, and
+// half of these neighbours lie in the block.
+template <int COL>
+__device__ __forceinline__ void lane_block(const unsigned char* lut, unsigned char* own, const unsigned char* opp, int L,
+                                           const uint4* pre, const LaneConst& lc, uint32_t& dk, uint32_t& pc)
+{
+    const int at[4] = {0, 1, L, L + 1};
+    // neighbours outside the block: of the first, second, third and fourth cell
+    const int ext[4] = {COL ? -1 : -L, COL ? 1 - L : 2, COL ? 2 * L : L - 1, COL ? L + 2 : 2 * L + 1};
+    uint32_t o[4], b[4], x[4], hb[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o[i] = own[at[i] * 32];
+        b[i] = opp[at[i] * 32];
+        x[i] = opp[ext[i] * 32];
+    }
+    hb[0] = lane_fields(lut, b[0], x[0], COL ? b[1] : b[2]);
+    hb[1] = COL ? lane_fields(lut + 192, b[1], x[1], b[3]) : lane_fields(lut + 192, b[1], b[0], x[1]);
+    hb[2] = COL ? lane_fields(lut + 192 * L, b[2], b[0], x[2]) : lane_fields(lut + 192 * L, b[2], x[2], b[3]);
+    hb[3] = lane_fields(lut + 192 * (L + 1), b[3], COL ? b[2] : b[1], x[3]);
+    uint4 pr[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) pr[i] = pre[at[i]];
+    lane_words<4>(o, hb, pr, lc, dk, pc);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) own[at[i] * 32] = (unsigned char)o[i];
+}
+
+// One colour of a column: this warp's share of the cells.
+template <int LT, int COL>
+__device__ __forceinline__ void lane_phase(const unsigned char* lut, unsigned char* own, const unsigned char* opp,
+                                           const uint4* pre, int w, int W, int Lr, const LaneConst& lc, uint32_t& dk,
+                                           uint32_t& pc)
+{
+    const int L = LT ? LT : Lr;
+    if (L & 1) {                                // cells alternate in orientation over all rows
+        const int n = L * L / 2;
+        int j = w;
+        for (; j < n; j += W)
+            lane_pair<2, COL>(lut + j * 384, own + j * 64, opp + j * 64, 32 * L, pre + 2 * j, lc, dk, pc);
+        if (j == n) lane_pair<1, COL>(lut + j * 384, own + j * 64, opp + j * 64, 32 * L, pre + 2 * j, lc, dk, pc);
+        return;
+    }
+    const unsigned hl = (unsigned)L / 2u;
+    for (unsigned j = w; j < hl * hl; j += W) {
+        const unsigned r = j / hl, q = 2u * (j + r * hl);    // block (r, j - r hl): cell (2 r, 2 (j - r hl))
+        lane_block<COL>(lut + q * 192, own + q * 32, opp + q * 32, L, pre + q, lc, dk, pc);
+    }
+}
+
+// The ascending exchange sweep of one run by all 32 lanes of a warp (TWO: 32 < NT <= 64,
+// lane l holds slots l and l + 32).  Going up from slot 0 a configuration of energy x is
+// carried along; pair p is rejected, and the configuration of slot p + 1 carried on
+// instead, when its bound b_p = E_{p+1} - 2 c_p exceeds x.  The recurrence runs on all
+// lanes alike from (b_p, E_{p+1}) pairs broadcast out of shared memory, a compare and a
+// select per pair; what each slot then holds follows from the rejected pairs in parallel:
+// slot s takes the old content of slot s + 1 when pair s was accepted, and otherwise the
+// configuration carried into it, which came from the lowest slot of the run of accepted
+// pairs that ends at pair s - 1.  xp: scratch, padded to a multiple of 8 with pairs that
+// are never rejected.  Returns the lowest slot energy.
+template <bool TWO>
+__device__ __forceinline__ int lane_exchange(int32_t* Es, uint8_t* perm, uint8_t* inv, uint32_t* xacc, const int32_t* cc,
+                                             int2* xp, int NT, int lane)
+{
+    constexpr int H = TWO ? 2 : 1;
+    const int np = NT - 1, npad = (np + 7) & ~7;
+    int m = INT_MAX;
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const int s = lane + 32 * h;
+        if (s < NT) m = min(m, Es[s]);
+        if (s < npad) {
+            const int e = s < np ? Es[s + 1] : 0;
+            xp[s] = make_int2(s < np ? e - 2 * cc[s] : INT_MIN, e);
+        }
+    }
+    __syncwarp();
+    int x = Es[0];
+    uint32_t rej[H];
+    const int4* x4 = reinterpret_cast<const int4*>(xp);
+    int4 v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = x4[i];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        rej[h] = 0u;
+        for (int p0 = 0; p0 < 32 && 32 * h + p0 < np; p0 += 8) {
+            int4 nx[4];                            // the next eight pairs (the scratch is followed by room for them)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) nx[i] = x4[16 * h + p0 / 2 + 4 + i];
+            uint32_t r8 = 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (x < v[i].x) { x = v[i].y; r8 |= 1u << (2 * i); }
+                if (x < v[i].z) { x = v[i].w; r8 |= 2u << (2 * i); }
+            }
+            rej[h] |= r8 << p0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = nx[i];
+        }
+    }
+    // accepted pairs (pairs np and above: none)
+    uint32_t acc[H];
+    acc[0] = ~rej[0] & (np >= 32 ? 0xFFFFFFFFu : (1u << np) - 1u);
+    if (TWO) acc[H - 1] = ~rej[H - 1] & ((1u << (np - 32)) - 1u);
+    int e_new[H], b_new[H], src[H];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const int s = lane + 32 * h;
+        uint32_t below = ~acc[h] & ((1u << lane) - 1u);           // rejected pairs under s, this word
+        src[h] = 32 * h + 32 - __clz((int)below);
+        if (TWO && h == 1 && below == 0u) src[h] = 32 - __clz((int)~acc[0]);
+        if ((acc[h] >> lane) & 1u) src[h] = s + 1;
+        e_new[h] = b_new[h] = 0;
+        if (s < NT) {
+            e_new[h] = Es[src[h]];
+            b_new[h] = perm[src[h]];
+        }
+    }
+    m = __reduce_min_sync(FULL, m);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+        const int s = lane + 32 * h;
+        if (s < NT) {
+            Es[s] = e_new[h];
+            perm[s] = (uint8_t)b_new[h];
+            inv[b_new[h]] = (uint8_t)s;
+            if (s < np) xacc[s] += (acc[h] >> lane) & 1u;
+        }
+    }
+    __syncwarp();
+    return m;
+}
+
+// walk_update by all lanes of a warp: the hot half's copies are distinct.
+__device__ __forceinline__ void walk_update_warp(const uint8_t* perm, uint32_t* whot, uint32_t* wtr, uint8_t* wst, int NT,
+                                                 int lane)
+{
+    for (int t = NT - NT / 2 + lane; t < NT; t += 32) whot[perm[t]] += 1u;
+    if (lane == 0) {
+        const int c = perm[0];
+        if (wst[c] == 2) wtr[c] += 1u;
+        wst[c] = 1;
+        const int h = perm[NT - 1];
+        if (wst[h] == 1) wst[h] = 2;
+    }
+    __syncwarp();
+}
+
+template <int LT>
+__device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bundle bd, uint32_t sweep0, int nsweeps,
+                                    int xevery, int mode, unsigned char* smem)
+{
+    const InstDesc& in = insts[bd.inst];
+#ifdef PT_DEBUG
+    if (LT && in.L != LT) {                     // uniform per CTA: the whole CTA skips the bundle
+        if (threadIdx.x == 0) atomicCAS(&g_pt_debug_code, 0u, 9u);
+        return;
+    }
+#endif
+    const int L = LT ? LT : in.L, NT = in.NT, L2 = L * L, N = 8 * L2, NW = 2 * L2, W = bd.sp, gr = -bd.team;
+    const int ngroups = (bd.nitems + gr - 1) / gr;
+    const bool walk = in.wstate != nullptr;
+    const LaneLayout lay = lane_layout(L, NT, in.kt, gr, ngroups, walk);
+    const ItemLayout rl = item_layout(0, NT, 0, walk);
+    const int tid = threadIdx.x, lane = tid & 31;
+    // read through a warp reduction: warp-uniform for the compiler too
+    const int wid = (int)__reduce_or_sync(FULL, (unsigned)(tid >> 5));
+    const uint32_t k0 = __reduce_or_sync(FULL, in.seed), k1 = __reduce_or_sync(FULL, in.uid);
+    // this warp's group, its place in it, its column and its share of the cells
+    const int gw = W * lay.ncols, grp = wid / gw, gwid = wid - grp * gw, col = gwid / W, w = gwid - col * W;
+    const bool active = grp < ngroups;
+    const int nit = active ? min(gr, bd.nitems - grp * gr) : 0;      // runs of the group
+    const int rep = col * 32 + lane;
+    const bool valid = rep < nit * NT;
+    const int item = valid ? rep / NT : 0, buf = valid ? rep - item * NT : 0;
+
+    auto group_base = [&](int g) { return smem + lay.groups + g * lay.group_bytes; };
+    auto run_base = [&](int g, int i) { return group_base(g) + lay.runs + i * lay.run_bytes; };
+    unsigned char* const gb = group_base(active ? grp : 0);
+    const int grun = bd.run0 + grp * gr;                             // the group's first run
+    int32_t* xoff_sm = reinterpret_cast<int32_t*>(smem + lay.xtab);
+    uint4* pre = reinterpret_cast<uint4*>(gb);
+    auto gsync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gw * 32) : "memory"); };
+    const int n_iter = (mode == 0) ? nsweeps : 1;
+    const uint32_t s_first = (mode == 0) ? sweep0 + 1u : sweep0;
+    const uint32_t* const xthr = in.xthr;
+    // sweeps to the next exchange, counted down from sweep s_first on (0: exchange after that sweep)
+    const bool xon = NT > 1 && (mode == 1 || xevery > 0);
+    const uint32_t xper = mode == 1 || xevery < 1 ? 1u : (uint32_t)xevery;
+    uint32_t xwait = (xper - s_first % xper) % xper;
+    if (mode == 1) xwait = 0u;
+
+    // ---- tables, then this bundle's runs
+    {
+        uint32_t* lut = reinterpret_cast<uint32_t*>(smem + lay.lut);
+        for (int i = tid; i < 2 * L2 * 48; i += blockDim.x) {
+            const int cq = i / 48, e = i - cq * 48, c = cq / L2, q = cq - c * L2;
+            lut[i] = lane_field(in.jw + (q * 2 + c) * 8, e >> 4, e & 15);
+        }
+        uint32_t* thr = reinterpret_cast<uint32_t*>(smem + lay.thr);
+        for (int i = tid; i < (NT + 31) / 32 * 32 * in.kt; i += blockDim.x) {
+            const int b = i / (32 * in.kt), k = (i >> 5) - b * in.kt, t = b * 32 + (i & 31);
+            thr[i] = t < NT ? in.thr[t * in.kt + k] : 0u;
+        }
+        for (int p = tid; p < NT; p += blockDim.x) {
+            xoff_sm[p] = in.xoff[p];
+            reinterpret_cast<float*>(xoff_sm + NT)[p] = p < NT - 1 ? in.xhint[p] : 0.0f;
+        }
+        for (int g = 0; g < ngroups; ++g) {
+            uint32_t* sp = reinterpret_cast<uint32_t*>(group_base(g) + lay.spins);
+            for (int i = tid; i < lay.ncols * lay.col_bytes / 4; i += blockDim.x) sp[i] = 0u;
+            uint4* pg = reinterpret_cast<uint4*>(group_base(g));
+            for (int i = tid; i < 2 * L2; i += blockDim.x)
+                pg[i] = lane_pre(s_first, i >= L2, i >= L2 ? i - L2 : i, L, k0, k1);
+        }
+    }
+    for (int i = tid; i < bd.nitems * NT; i += blockDim.x) {
+        const int r = i / NT, t = i - r * NT;
+        unsigned char* rb = run_base(r / gr, r % gr);
+        const size_t g = (size_t)(bd.run0 + r) * NT + t;
+        const int b = PT_IDX((int)in.perm[g], NT, 2u);
+        reinterpret_cast<int32_t*>(rb + rl.E)[t] = in.E[g];
+        (rb + rl.perm)[t] = (uint8_t)b;
+        (rb + rl.inv)[b] = (uint8_t)t;
+        reinterpret_cast<uint32_t*>(rb + rl.macc)[t] = 0u;
+        reinterpret_cast<uint32_t*>(rb + rl.xacc)[t] = 0u;
+        if (walk) {
+            reinterpret_cast<uint32_t*>(rb + rl.whot)[t] = 0u;
+            reinterpret_cast<uint32_t*>(rb + rl.wtrips)[t] = 0u;
+            (rb + rl.wstate)[t] = in.wstate[g];
+        }
+        if (t == 0) {
+            reinterpret_cast<int32_t*>(rb + rl.misc)[0] = in.best[bd.run0 + r];
+            reinterpret_cast<int32_t*>(rb + rl.misc)[1] = in.first[bd.run0 + r];
+        }
+    }
+    __syncthreads();
+    // spin word i of run r (buffer b, group g = 2 cell + u) and its byte in shared memory
+    uint32_t* gsp = reinterpret_cast<uint32_t*>(in.spins + (size_t)bd.run0 * NT * N);
+    auto spin_byte = [&](int r, int i) {
+        const int b = i / NW, g = i - b * NW, q = g >> 1, y = q / L, x = q - y * L, cl = (y + x + (g & 1)) & 1;
+        const int p = (r % gr) * NT + b;
+        return group_base(r / gr) + lay.spins + (p >> 5) * lay.col_bytes + cl * (lay.col_bytes / 2) + (q + L) * 32 + (p & 31);
+    };
+    for (int r = 0; r < bd.nitems; ++r)
+        for (int i = tid; i < NT * NW; i += blockDim.x)
+            *spin_byte(r, i) = (unsigned char)(((gsp[(size_t)r * NT * NW + i] & 0x80808080u) * 0x00204081u) >> 26);
+    if (n_iter > 0 && xon && xwait == 0u)
+        for (int r = gw - 1 - gwid; r < nit; r += gw)
+            exchange_prepare(xthr, xoff_sm, lane, s_first, (uint32_t)(grun + r) << 16, k0, k1, NT,
+                             reinterpret_cast<int32_t*>(run_base(grp, r) + rl.ccrit) + (s_first & 1u) * NT);
+    __syncthreads();
+
+    if (active) {
+        unsigned char* rb = run_base(grp, item);
+        unsigned char* s0 = gb + lay.spins + col * lay.col_bytes + L * 32 + lane;     // colour 0, cell 0
+        unsigned char* s1 = s0 + lay.col_bytes / 2;
+        const unsigned char* lut0 = smem + lay.lut;
+        const uint32_t thr_at = (uint32_t)__cvta_generic_to_shared(smem + lay.thr);
+        LaneConst lc;
+        lc.kt = in.kt;
+#pragma unroll
+        for (int r = 0; r < 7; ++r) {           // through a warp reduction each, so that they are kept, not recomputed
+            lc.ka[r] = __reduce_or_sync(FULL, k0 + (3u + r) * PHILOX_W0);
+            lc.kb[r] = __reduce_or_sync(FULL, k1 + (3u + r) * PHILOX_W1);
+        }
+        const int nchain = nit < gw ? nit : gw;
+        for (int it = 0; it < n_iter; ++it) {
+            const uint32_t s = s_first + (uint32_t)it;
+            const bool do_x = xon && xwait == 0u;
+            xwait = xwait == 0u ? xper - 1u : xwait - 1u;          // from here on: of sweep s + 1
+            if (mode == 0) {
+                uint32_t dk = 0u, pc = 0u;
+                const int t = PT_IDX((int)(rb + rl.inv)[buf], NT, 2u);
+                const PhiloxPre ps = philox_pre(s, 0u, k0, k1);
+                lc.y2x = ps.y2x;
+                lc.y1k = ps.y1k;
+                lc.c1 = ((uint32_t)(grun + item) << 16) | (uint32_t)t;
+                lc.tcol = thr_at + (uint32_t)((t >> 5) * lc.kt * 128 + (t & 31) * 4) - 127u * 128u;
+                lane_phase<LT, 0>(lut0, s0, s1, pre, w, W, L, lc, dk, pc);
+                if (W > 1) gsync();
+                lane_phase<LT, 1>(lut0 + L2 * 192, s1, s0, pre + L2, w, W, L, lc, dk, pc);
+                const int n = (int)(pc >> 7), sk = (int)(dk >> 7) - 127 * n;   // accepted flips, sum of their k
+                if (valid) {
+                    if (sk) atomicAdd(reinterpret_cast<int32_t*>(rb + rl.E) + t, 2 * sk);
+                    if (n) atomicAdd(reinterpret_cast<uint32_t*>(rb + rl.macc) + t, (uint32_t)n);
+                }
+            }
+            gsync();
+            for (int r = gwid; r < nit; r += gw) {
+                unsigned char* xb = run_base(grp, r);
+                int32_t* Es = reinterpret_cast<int32_t*>(xb + rl.E);
+                int32_t* misc = reinterpret_cast<int32_t*>(xb + rl.misc);
+                int m;
+                if (do_x) {
+                    uint32_t* xacc = reinterpret_cast<uint32_t*>(xb + rl.xacc);
+                    const int32_t* cc = reinterpret_cast<const int32_t*>(xb + rl.ccrit) + (s & 1u) * NT;
+                    int2* xp = reinterpret_cast<int2*>(xb + rl.bytes);
+                    m = NT > 32 ? lane_exchange<true>(Es, xb + rl.perm, xb + rl.inv, xacc, cc, xp, NT, lane)
+                                : lane_exchange<false>(Es, xb + rl.perm, xb + rl.inv, xacc, cc, xp, NT, lane);
+                    if (walk)
+                        walk_update_warp(xb + rl.perm, reinterpret_cast<uint32_t*>(xb + rl.whot),
+                                         reinterpret_cast<uint32_t*>(xb + rl.wtrips), xb + rl.wstate, NT, lane);
+                } else {
+                    m = slot_min_warp(Es, NT, lane);
+                }
+                if (lane == 0 && mode == 0 && m < misc[0]) {
+                    misc[0] = m;
+                    misc[1] = (int32_t)s;
+                }
+            }
+            if (it + 1 < n_iter) {              // meanwhile the group's other warps prepare its next sweep
+                if (xon && xwait == 0u)
+                    for (int r = gw - 1 - gwid; r < nit; r += gw)
+                        exchange_prepare(xthr, xoff_sm, lane, s + 1u, (uint32_t)(grun + r) << 16, k0, k1, NT,
+                                         reinterpret_cast<int32_t*>(run_base(grp, r) + rl.ccrit) + ((s + 1u) & 1u) * NT);
+                const int f0 = gw > nchain ? nchain : 0;
+                for (int i = gwid >= f0 ? (gwid - f0) * 32 + lane : 2 * L2; i < 2 * L2; i += 32 * (gw - f0))
+                    pre[i] = lane_pre(s + 1u, i >= L2, i >= L2 ? i - L2 : i, L, k0, k1);
+            }
+            gsync();
+        }
+    }
+
+    // ---- write the state back
+    __syncthreads();
+    for (int r = 0; r < bd.nitems; ++r)
+        for (int i = tid; i < NT * NW; i += blockDim.x)
+            gsp[(size_t)r * NT * NW + i] = byte_signs(*spin_byte(r, i) * 0x04081020u) | 0x01010101u;   // 0xFF or 1
+    for (int i = tid; i < bd.nitems * NT; i += blockDim.x) {
+        const int r = i / NT, t = i - r * NT, run = bd.run0 + r;
+        const unsigned char* xb = run_base(r / gr, r % gr);
+        const size_t g = (size_t)run * NT + t;
+        in.E[g] = reinterpret_cast<const int32_t*>(xb + rl.E)[t];
+        in.perm[g] = (xb + rl.perm)[t];
+        in.macc[g] += reinterpret_cast<const uint32_t*>(xb + rl.macc)[t];
+        if (t < NT - 1) in.xacc[(size_t)run * (NT > 1 ? NT - 1 : 1) + t] += reinterpret_cast<const uint32_t*>(xb + rl.xacc)[t];
+        if (walk) {
+            in.whot[g] += reinterpret_cast<const uint32_t*>(xb + rl.whot)[t];
+            in.wtrips[g] += reinterpret_cast<const uint32_t*>(xb + rl.wtrips)[t];
+            in.wstate[g] = (xb + rl.wstate)[t];
+        }
+        if (t == 0) {
+            in.best[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[0];
+            in.first[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[1];
+        }
+    }
+    __syncthreads();
+}
+
+}  // namespace
+}  // namespace ptg
