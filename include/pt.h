@@ -548,7 +548,9 @@ int pt_batch_tts(pt_batch *b, int32_t horizon, int32_t *tts, int32_t *n_hit, int
 int pt_batch_get_state(pt_batch *b, int32_t inst, int8_t *spins, int32_t *E, int32_t *best,
                        int32_t *first, uint64_t *macc, uint64_t *xacc);
 
-/* Schedule of the instances of size chimera_L: slot_parallel slots
+/* Schedule of the instances of size chimera_L (a new batch plans each size itself,
+ * with the replica-lane mapping; a set schedule or mapping replaces that plan):
+ * slot_parallel slots
  * (cell-major: slot_parallel * L^2 threads per run) or teams (slot-major:
  * slot_parallel * team threads per run, at the size's largest temperature
  * count; an instance with fewer temperatures gets proportionally fewer
@@ -574,7 +576,7 @@ int pt_batch_set_mapping(pt_batch *b, int32_t chimera_L, int32_t team, int32_t s
                          int32_t runs_per_cta);
 int pt_batch_get_mapping(const pt_batch *b, int32_t chimera_L, int32_t *team);
 
-/* Autotuner: size by size, times every feasible cell-major (slot_parallel,
+/* Autotuner: size by size, times the planned shape and every feasible cell-major (slot_parallel,
  * runs_per_cta) and slot-major (team, slot_parallel, runs_per_cta) on all
  * instances of that size over `trial_sweeps` sweeps, with the CTA size the
  * bundle needs, keeps the fastest, then resets the runs.  *block (may be

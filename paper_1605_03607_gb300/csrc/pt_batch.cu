@@ -33,9 +33,11 @@ namespace {
 // Schedule of one size: runs per CTA and, per run, either slot_parallel slots
 // of L^2 threads (cell-major, team 0) or slot_parallel teams of `team` lanes
 // (slot-major, at the size's largest temperature count).  block 0: the CTA
-// size is the bundle's thread count rounded up to a warp.
+// size is the bundle's thread count rounded up to a warp.  planned: until a
+// schedule is set, the replica-lane mapping (lane_plan_batch) instead.
 struct ShapeSched {
     int sp = 0, ipc = 0, team = 0, block = 0;
+    bool planned = false;
 };
 
 struct SizeGroup {
@@ -44,7 +46,7 @@ struct SizeGroup {
     ShapeSched s;
     std::vector<Bundle> bundles;
     Bundle* d_bundles = nullptr;
-    int block = 0, smem = 0, grid = 0;
+    int block = 0, smem = 0, grid = 0, team = 0;
     cudaStream_t st = nullptr;        // capture branch
     cudaEvent_t ev = nullptr;
     cudaGraphNode_t knode = nullptr;
@@ -139,6 +141,7 @@ void default_shape_sched(int L, int NT, int R, bool slot_major, ShapeSched& s, i
 {
     const int L2 = L * L;
     s.block = 0;
+    s.planned = false;
     if (slot_major) {
         // teams of about L^2/16 lanes (2..32), one buffer each, widened until a
         // run has at least a warp; up to about 384 threads per CTA
@@ -195,52 +198,74 @@ int build_group(pt_batch* b, int k)
     SizeGroup& g = b->groups[k];
     const ShapeSched& s = g.s;
     const bool sm = s.team > 0;
-    if (s.sp < 1 || s.ipc < 1 || (sm && (s.team > 32 || (s.team & (s.team - 1)) != 0)))
-        return bfail(b, PT_ERR_ARG, "bad schedule values");
-    if ((sm ? s.sp * s.team : s.sp * g.L * g.L) < 32)
-        return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit (threads per run >= 32)");
     std::vector<Bundle> bundles;
-    int threads = 0;
+    int block = 0, cap = 0, dev = 0, sms = 0;
     int64_t smem = 0;
-    for (int i = 0; i < b->n_inst; ++i) {
-        if (b->L[i] != g.L) continue;
-        int spi = 0, ipci = 0;
-        instance_shape(b, g, b->NT[i], &spi, &ipci);
-        const int tpr = sm ? spi * s.team : spi * g.L * g.L;
-        if (tpr < 32)
-            return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit (threads per run >= 32)");
-        for (int r = 0; r < b->R; r += ipci) {
-            Bundle bd;
-            bd.inst = i; bd.run0 = r; bd.nitems = std::min(ipci, b->R - r); bd.sp = spi; bd.team = s.team;
-            bundles.push_back(bd);
+    BK(sweep_smem_capacity(&cap), "shared memory capacity");
+    BK(cudaGetDevice(&dev), "cudaGetDevice");
+    BK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
+    if (s.planned) {
+        std::vector<int> nts;
+        for (int i = 0; i < b->n_inst; ++i)
+            if (b->L[i] == g.L) nts.push_back(b->NT[i]);
+        int W = 1, ct = 1;
+        if (!lane_plan_batch(g.L, nts, b->kt, b->R, sms, cap, &W, &ct))
+            return bfail(b, PT_ERR_ARG, "L=" + std::to_string(g.L) + " fits no CTA");
+        for (int i = 0; i < b->n_inst; ++i) {
+            if (b->L[i] != g.L) continue;
+            LaneShape ls;
+            lane_fill(g.L, b->NT[i], b->kt, b->R, W, ct, cap, &ls);
+            for (int r = 0; r < b->R; r += ls.gr * ls.G) {
+                Bundle bd;
+                bd.inst = i; bd.run0 = r; bd.nitems = std::min(ls.gr * ls.G, b->R - r); bd.sp = W; bd.team = -ls.gr;
+                bundles.push_back(bd);
+            }
+            block = std::max(block, lane_threads(b->NT[i], ls));
+            smem = std::max<int64_t>(smem, bundle_smem_bytes(g.L, b->NT[i], ls.gr * ls.G, -ls.gr, false, b->kt));
         }
-        threads = std::max(threads, tpr * ipci);
-        smem = std::max<int64_t>(smem, bundle_smem_bytes(g.L, b->NT[i], ipci, s.team, false, b->kt));
+    } else {
+        if (s.sp < 1 || s.ipc < 1 || (sm && (s.team > 32 || (s.team & (s.team - 1)) != 0)))
+            return bfail(b, PT_ERR_ARG, "bad schedule values");
+        if ((sm ? s.sp * s.team : s.sp * g.L * g.L) < 32)
+            return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit (threads per run >= 32)");
+        int threads = 0;
+        for (int i = 0; i < b->n_inst; ++i) {
+            if (b->L[i] != g.L) continue;
+            int spi = 0, ipci = 0;
+            instance_shape(b, g, b->NT[i], &spi, &ipci);
+            const int tpr = sm ? spi * s.team : spi * g.L * g.L;
+            if (tpr < 32)
+                return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit (threads per run >= 32)");
+            for (int r = 0; r < b->R; r += ipci) {
+                Bundle bd;
+                bd.inst = i; bd.run0 = r; bd.nitems = std::min(ipci, b->R - r); bd.sp = spi; bd.team = s.team;
+                bundles.push_back(bd);
+            }
+            threads = std::max(threads, tpr * ipci);
+            smem = std::max<int64_t>(smem, bundle_smem_bytes(g.L, b->NT[i], ipci, s.team, false, b->kt));
+        }
+        block = (threads + 31) / 32 * 32;
+        if (s.block > 0) {
+            if (s.block < block || s.block % 32 != 0)
+                return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit the block");
+            block = s.block;
+        }
+        if (block > (sm ? MAX_THREADS_SM : MAX_THREADS))
+            return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit: " +
+                                            std::to_string(block) + " threads per CTA (limit " +
+                                            std::to_string(sm ? MAX_THREADS_SM : MAX_THREADS) + ")");
     }
-    int block = (threads + 31) / 32 * 32;
-    if (s.block > 0) {
-        if (s.block < block || s.block % 32 != 0)
-            return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit the block");
-        block = s.block;
-    }
-    if (block > (sm ? MAX_THREADS_SM : MAX_THREADS))
-        return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " does not fit: " +
-                                        std::to_string(block) + " threads per CTA (limit " +
-                                        std::to_string(sm ? MAX_THREADS_SM : MAX_THREADS) + ")");
+    const int team = s.planned ? -1 : s.team;      // the mapping of the group's launches, by its sign
     // longest bundles first (work per sweep = runs x slots x spins)
     std::stable_sort(bundles.begin(), bundles.end(), [&](const Bundle& x, const Bundle& y) {
         const int64_t cx = (int64_t)x.nitems * b->NT[x.inst] * b->N[x.inst];
         const int64_t cy = (int64_t)y.nitems * b->NT[y.inst] * b->N[y.inst];
         return cx > cy;
     });
-    int cap = 0;
-    BK(sweep_smem_capacity(&cap), "shared memory capacity");
     if (smem > cap) return bfail(b, PT_ERR_ARG, "a bundle needs more shared memory than a CTA can have");
-    BK(set_sweep_smem_limit(cap, s.team, false, g.L), "cudaFuncSetAttribute");
-    int dev = 0, sms = 0, per_sm = 0;
-    BK(cudaGetDevice(&dev), "cudaGetDevice");
-    BK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
-    BK(sweep_occupancy(block, (int)smem, &per_sm, s.team, false, g.L), "occupancy");
+    BK(set_sweep_smem_limit(cap, team, false, g.L), "cudaFuncSetAttribute");
+    int per_sm = 0;
+    BK(sweep_occupancy(block, (int)smem, &per_sm, team, false, g.L), "occupancy");
     if (per_sm < 1) return bfail(b, PT_ERR_ARG, "schedule of L=" + std::to_string(g.L) + " fits no CTA on an SM");
     Bundle* d = nullptr;
     BK(balloc(&d, bundles.size()), "cudaMalloc bundles");
@@ -253,6 +278,7 @@ int build_group(pt_batch* b, int k)
     g.bundles.swap(bundles);
     g.block = block;
     g.smem = (int)smem;
+    g.team = team;
     g.grid = std::max(1, std::min<int>((int)g.bundles.size(), sms * per_sm));
     // the captured graph holds the old bundle lists
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
@@ -287,7 +313,7 @@ int run_graph(pt_batch* b, int nsweeps, int xevery)
             e = cudaStreamWaitEvent(g.st, b->ev_fork, 0);
             if (e == cudaSuccess)
                 e = launch_sweeps(b->d_desc, g.d_bundles, (int)g.bundles.size(), g.grid, g.block, g.smem,
-                                  (uint32_t)b->sweep, nsweeps, xevery, 0, b->d_queue + k, g.st, g.s.team, false,
+                                  (uint32_t)b->sweep, nsweeps, xevery, 0, b->d_queue + k, g.st, g.team, false,
                                   g.L);
             if (e == cudaSuccess) e = cudaEventRecord(g.ev, g.st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, g.ev, 0);
@@ -493,6 +519,7 @@ int pt_batch_create(pt_batch** out, int32_t n_inst, const pt_instance_desc* d, i
         for (int i = 0; i < n_inst; ++i)
             if (b->L[i] == g.L) g.work += (int64_t)n_runs * b->NT[i] * b->N[i];
         default_shape_sched(g.L, g.ntmax, n_runs, false, g.s, b->kt);
+        g.s.planned = true;
         b->groups.push_back(g);
     }
     std::stable_sort(b->groups.begin(), b->groups.end(),
@@ -628,6 +655,7 @@ int pt_batch_set_schedule(pt_batch* b, int32_t block, int32_t chimera_L, int32_t
         for (size_t k = 0; k < b->groups.size(); ++k) {
             ShapeSched s = b->groups[k].s;
             s.block = block;
+            s.planned = false;
             const int rc = set_group(b, (int)k, s);
             if (rc) {
                 for (size_t m = 0; m < k; ++m) set_group(b, (int)m, old[m]);
@@ -642,6 +670,7 @@ int pt_batch_set_schedule(pt_batch* b, int32_t block, int32_t chimera_L, int32_t
         s.sp = slot_parallel;
         s.ipc = std::min<int>(runs_per_cta, b->R);
         s.block = block;
+        s.planned = false;
         const int rc = set_group(b, k, s);
         if (rc) return rc;
     }
@@ -677,6 +706,7 @@ int pt_batch_set_mapping(pt_batch* b, int32_t chimera_L, int32_t team, int32_t s
         if (slot_parallel > 0) s.sp = slot_parallel;
         if (runs_per_cta > 0) s.ipc = std::min<int>(runs_per_cta, b->R);
         s.block = 0;
+        s.planned = false;
         const int rc = set_group(b, k, s);
         if (rc) return rc;
     }
@@ -706,8 +736,8 @@ int pt_batch_get_mapping(const pt_batch* b, int32_t chimera_L, int32_t* team)
     return PT_OK;
 }
 
-// Times candidate schedules and keeps the fastest, size by size: every
-// cell-major (slot_parallel, runs_per_cta) and slot-major (team,
+// Times candidate schedules and keeps the fastest, size by size: the planned
+// replica-lane shape, every cell-major (slot_parallel, runs_per_cta) and slot-major (team,
 // slot_parallel, runs_per_cta) that fits runs all instances of that size
 // alone for `trial_sweeps` sweeps (the faster of two launches), with the CTA
 // size the bundle needs.  The state is reset afterwards.
@@ -720,6 +750,9 @@ int pt_batch_autotune(pt_batch* b, int32_t trial_sweeps, int32_t* block_out)
         SizeGroup& g = b->groups[k];
         const int L2 = g.L * g.L, NT = g.ntmax;
         std::vector<ShapeSched> cands;
+        ShapeSched planned = g.s;                  // the replica-lane shape first
+        planned.planned = true;
+        cands.push_back(planned);
         for (int sp : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64}) {
             const int tpr = sp * L2;
             if (sp > NT || tpr > MAX_THREADS) break;
@@ -757,7 +790,7 @@ int pt_batch_autotune(pt_batch* b, int32_t trial_sweeps, int32_t* block_out)
                 if (e == cudaSuccess) e = cudaMemsetAsync(b->d_queue + k, 0, sizeof(int), b->stream);
                 if (e == cudaSuccess)
                     e = launch_sweeps(b->d_desc, g.d_bundles, (int)g.bundles.size(), g.grid, g.block, g.smem, 0u,
-                                      trial_sweeps, 1, 0, b->d_queue + k, b->stream, g.s.team, false, g.L);
+                                      trial_sweeps, 1, 0, b->d_queue + k, b->stream, g.team, false, g.L);
                 if (e == cudaSuccess) e = cudaEventRecord(b->e1, b->stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(b->e1);
                 float t = 0.f;

@@ -225,16 +225,17 @@ inline int lane_threads(int NT, const LaneShape& s) { return 32 * s.W * lane_col
 
 // Estimated SM clocks per sweep of an SM that holds `k` CTAs of the shape: a warp word (one
 // cell and colour of a column) takes 117 + 130 / w clocks of a sub-partition that runs w
-// warps, exchange and barriers 1300 + 26 NT, shared by the groups that run side by side; no
-// group is faster than alone.  Fitted to 900 measured (shape, size) pairs from C_2 to C_16:
-// the lowest estimate's time is 1 % above the best shape's on average, 10 % at most.
+// warps (a CTA's warps go round the four of them: a count that is no multiple of four loads
+// one more than the others), exchange and barriers 910, which the groups of the SM overlap;
+// no group is faster than alone.  Fitted to 900 measured (shape, size) pairs from C_2 to
+// C_16: the lowest estimate's time is 0.5 % above the best shape's on average, 3 % at most.
 inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);      // what the warps of a column share out
-    const int c = lane_columns(NT, s.gr), per = (units + s.W - 1) / s.W;
-    const double words = 2.0 * L * L * c * per * s.W / units, n = (double)k * s.G;
-    const double w1 = 0.25 * c * s.W, x = 1300.0 + 26.0 * NT;
-    const double together = 0.25 * words * n * (117.0 + 130.0 / (w1 * n)) + x / n;
+    const int c = lane_columns(NT, s.gr), per = (units + s.W - 1) / s.W, nw = s.G * c * s.W;
+    const double words = 2.0 * L * L * c * per * s.W / units * ((nw + 3) / 4 * 4) / nw, n = (double)k * s.G;
+    const double w1 = 0.25 * c * s.W, x = 910.0;
+    const double together = 0.25 * words * n * (117.0 + 130.0 / (w1 * n)) + x / std::pow(n, 0.7);
     return std::max(together, 0.25 * words * (117.0 + 130.0 / w1) + x);
 }
 
@@ -263,6 +264,63 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
                 if (t < best_t * 0.999) { best_t = t; best = s; }
             }
     return best;
+}
+
+// Shape of a batch's instances of one lattice side (their temperature counts `NTs`), whose
+// CTAs of 32 W Ct threads pull bundles from a queue: for an instance the (gr, G) with the
+// fewest bundles that fills at most Ct columns, and the (W, Ct) with the lowest estimated
+// total.  False if no shape fits.
+inline bool lane_fill(int L, int NT, int kt, int R, int W, int Ct, int cap, LaneShape* best)
+{
+    int fewest = 0;
+    for (int gr = 1; gr <= 8 && gr <= R; ++gr) {
+        const int c = lane_columns(NT, gr);
+        int G = std::min(std::min(Ct / c, LANE_GROUPS), (R + gr - 1) / gr);
+        while (G > 0 && lane_layout(L, NT, kt, gr, G, false).bytes > cap) --G;
+        if (G < 1) continue;
+        const int n = (R + gr * G - 1) / (gr * G);
+        if (fewest == 0 || n < fewest) {
+            fewest = n;
+            best->W = W;
+            best->gr = gr;
+            best->G = G;
+        }
+    }
+    return fewest > 0;
+}
+
+inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, int sms, int cap, int* W, int* Ct)
+{
+    const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
+    double best = 1e300;
+    for (int ct = 1; ct <= 32; ++ct)
+        for (int w : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
+            const int threads = 32 * w * ct;
+            if (threads > LANE_THREADS || (w > units && w > 1)) break;
+            int64_t smem = 0, ctas = 0;
+            bool ok = true;
+            std::vector<LaneShape> s(NTs.size());
+            for (size_t i = 0; ok && i < NTs.size(); ++i) {
+                ok = lane_fill(L, NTs[i], kt, R, w, ct, cap, &s[i]);
+                if (!ok) break;
+                smem = std::max<int64_t>(smem, lane_layout(L, NTs[i], kt, s[i].gr, s[i].G, false).bytes);
+                ctas += (R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G);
+            }
+            if (!ok) continue;
+            const int fit = std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
+            const int k = (int)std::min<int64_t>(fit, (ctas + sms - 1) / sms);      // CTAs an SM holds at a time
+            double t = 0.0, longest = 0.0;
+            for (size_t i = 0; i < NTs.size(); ++i) {
+                const double one = lane_clocks(L, NTs[i], s[i], k);
+                t += one / k * ((R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G));
+                longest = std::max(longest, one);
+            }
+            t = std::max(t / sms, longest);
+            // the launch's tail: whole rounds of CTAs, which other sizes of the batch may fill
+            t = 0.5 * (t + std::max(t, longest * (double)((ctas + (int64_t)k * sms - 1) / ((int64_t)k * sms))));
+            if (t < best * 0.999) { best = t; *W = w; *Ct = ct; }
+        }
+    return best < 1e300;
 }
 
 }  // namespace ptg

@@ -337,7 +337,7 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
     const bool active = grp < ngroups;
     const int nit = active ? min(gr, bd.nitems - grp * gr) : 0;      // runs of the group
     const int rep = col * 32 + lane;
-    const bool valid = rep < nit * NT;
+    const bool valid = rep < nit * NT, busy = col * 32 < nit * NT;   // busy: the column holds a replica
     const int item = valid ? rep / NT : 0, buf = valid ? rep - item * NT : 0;
 
     auto group_base = [&](int g) { return smem + lay.groups + g * lay.group_bytes; };
@@ -443,9 +443,9 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
                 lc.y1k = ps.y1k;
                 lc.c1 = ((uint32_t)(grun + item) << 16) | (uint32_t)t;
                 lc.tcol = thr_at + (uint32_t)((t >> 5) * lc.kt * 128 + (t & 31) * 4) - 127u * 128u;
-                lane_phase<LT, 0>(lut0, s0, s1, pre, w, W, L, lc, dk, pc);
+                if (busy) lane_phase<LT, 0>(lut0, s0, s1, pre, w, W, L, lc, dk, pc);
                 if (W > 1) gsync();
-                lane_phase<LT, 1>(lut0 + L2 * 192, s1, s0, pre + L2, w, W, L, lc, dk, pc);
+                if (busy) lane_phase<LT, 1>(lut0 + L2 * 192, s1, s0, pre + L2, w, W, L, lc, dk, pc);
                 const int n = (int)(pc >> 7), sk = (int)(dk >> 7) - 127 * n;   // accepted flips, sum of their k
                 if (valid) {
                     if (sk) atomicAdd(reinterpret_cast<int32_t*>(rb + rl.E) + t, 2 * sk);

@@ -95,3 +95,21 @@ def test_planned_longest_tables(P, L, kmax):
         st = h.state()
     for k in ("spins", "E", "best", "first", "macc", "xacc"):
         assert np.array_equal(st[k], getattr(ref, k)), k
+
+
+def test_planned_batch_of_uneven_instances(P):
+    """One CTA size for instances of 24 to 48 temperatures: groups of different column counts,
+    CTAs with idle warps, last groups short of runs."""
+    R, seed = 9, 77
+    inst = [dict(L=L, J=W.random_couplers(L, seed, i), betas=W.beta_ladder(NT, 0.1, 3.0), uid=i)
+            for i, (L, NT) in enumerate([(4, 24), (4, 33), (4, 48), (3, 30), (3, 40), (6, 36), (4, 1)])]
+    with P.PTBatch(inst, R, seed) as b:
+        b.run(7, 1)
+        b.run(12, 2)
+        for i, x in enumerate(inst):
+            st = b.state(i)
+            ref = oracle.PTState(x["L"], x["J"], x["betas"], R, seed, i)
+            ref.sweeps(7, 1)
+            ref.sweeps(12, 2)
+            for k in ("spins", "E", "best", "first", "macc") + (("xacc",) if len(x["betas"]) > 1 else ()):
+                assert np.array_equal(st[k], getattr(ref, k)), (i, k)
