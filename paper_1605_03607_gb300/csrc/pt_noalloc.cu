@@ -27,7 +27,7 @@
 //
 // Set-up: the first call on a device (with that device current) resolves the
 // array's device address with cudaGetSymbolAddress and raises the sweep
-// kernel's shared-memory limit; make that first call outside any stream
+// kernels' shared-memory limit; make that first call outside any stream
 // capture.
 #include <cmath>
 #include <cstdint>
@@ -69,7 +69,7 @@ int32_t h_out[3];
 
 std::mutex g_mu;
 unsigned char* g_base[MAX_DEVICES];   // device address of g_scratch per device (set up once)
-int g_smem_cap[MAX_DEVICES];
+int g_smem_cap[MAX_DEVICES], g_sms[MAX_DEVICES];
 
 // Failures are reported through pt_last_error(NULL).
 int noalloc_fail(int code, const char* msg)
@@ -136,7 +136,8 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
         if (e != cudaSuccess || !p) return noalloc_cuda_fail("cudaGetSymbolAddress of the scratch array", e, nullptr, false);
         int cap = 0;
         cudaError_t e2 = sweep_smem_capacity(&cap);
-        if (e2 == cudaSuccess) e2 = set_sweep_smem_limit(cap);
+        for (int l = 1; l <= MAX_L && e2 == cudaSuccess; ++l) e2 = set_sweep_smem_limit(cap, -1, false, l);
+        if (e2 == cudaSuccess) e2 = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e2 != cudaSuccess) return noalloc_cuda_fail("setting the sweep kernel's shared-memory limit", e2, nullptr, false);
         g_smem_cap[dev] = cap;
         g_base[dev] = static_cast<unsigned char*>(p);
@@ -151,20 +152,20 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
     pack_couplers(L, J, h_jw);
     build_neighbours(L, h_nbr);
 
-    // schedule: about 256 threads per run, a multiple of 32, one run per CTA
+    // the shape a handle of this size plans for itself
     const int L2 = L * L;
-    int sp = 256 / L2 > 1 ? 256 / L2 : 1;
-    if (sp > n_temps) sp = n_temps;
-    while ((sp * L2) % 32 != 0) ++sp;
-    const int block = sp * L2;
-    const int smem = (int)bundle_smem_bytes(L, n_temps, 1, 0, false, kt);
-    if (block > MAX_THREADS || smem > g_smem_cap[dev])
-        return noalloc_fail(PT_ERR_ARG, "one run needs more shared memory than a CTA can have");
+    const LaneShape shape = lane_plan(L, n_temps, kt, n_runs, 1, false, g_sms[dev], g_smem_cap[dev]);
+    const int ipc = shape.gr * shape.G, block = lane_threads(n_temps, shape);
+    const int smem = (int)bundle_smem_bytes(L, n_temps, ipc, -shape.gr, false, kt);
+    int n_bundles = 0;
     for (int r = 0; r < n_runs; ++r) {
         h_items[r] = make_int2(0, r);
-        h_bundles[r].inst = 0; h_bundles[r].run0 = r; h_bundles[r].nitems = 1; h_bundles[r].sp = sp;
-        h_bundles[r].team = 0;
+        if (r % ipc != 0) continue;
+        Bundle& b = h_bundles[n_bundles++];
+        b.inst = 0; b.run0 = r; b.nitems = n_runs - r < ipc ? n_runs - r : ipc; b.sp = shape.W; b.team = -shape.gr;
     }
+    if (smem > g_smem_cap[dev])
+        return noalloc_fail(PT_ERR_ARG, "one run needs more shared memory than a CTA can have");
 
     // carve the scratch
     size_t off = 0;
@@ -184,7 +185,7 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
     const size_t o_xthr = carve(off, 4 * (size_t)(nx > 0 ? nx : 1));
     const size_t o_desc = carve(off, sizeof(InstDesc));
     const size_t o_items = carve(off, sizeof(int2) * (size_t)n_runs);
-    const size_t o_bund = carve(off, sizeof(Bundle) * (size_t)n_runs);
+    const size_t o_bund = carve(off, sizeof(Bundle) * (size_t)n_bundles);
     const size_t o_out = carve(off, 16);
     if (off > PT_NOALLOC_BYTES) return noalloc_fail(PT_ERR_ARG, "problem exceeds the 4 MiB no-alloc scratch");
 
@@ -221,7 +222,7 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
         return noalloc_cuda_fail("cudaMemcpyAsync (staging upload)", ce, st, true);
     if ((ce = up(o_desc, &h_desc, sizeof(InstDesc))) != cudaSuccess) return noalloc_cuda_fail("cudaMemcpyAsync (staging upload)", ce, st, true);
     if ((ce = up(o_items, h_items, sizeof(int2) * (size_t)n_runs)) != cudaSuccess) return noalloc_cuda_fail("cudaMemcpyAsync (staging upload)", ce, st, true);
-    if ((ce = up(o_bund, h_bundles, sizeof(Bundle) * (size_t)n_runs)) != cudaSuccess) return noalloc_cuda_fail("cudaMemcpyAsync (staging upload)", ce, st, true);
+    if ((ce = up(o_bund, h_bundles, sizeof(Bundle) * (size_t)n_bundles)) != cudaSuccess) return noalloc_cuda_fail("cudaMemcpyAsync (staging upload)", ce, st, true);
 
     const InstDesc* dd = reinterpret_cast<const InstDesc*>(base + o_desc);
     const int2* di = reinterpret_cast<const int2*>(base + o_items);
@@ -234,8 +235,8 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
     const int64_t total = (int64_t)S * pass_mult;
     for (int64_t done = 0; done < total;) {
         const int chunk = (int)(total - done < 4096 ? total - done : 4096);
-        if ((ce = launch_sweeps(dd, db, n_runs, n_runs, block, smem, (uint32_t)done, chunk, exchange_every, 0,
-                                nullptr, st)) != cudaSuccess)
+        if ((ce = launch_sweeps(dd, db, n_bundles, n_bundles, block, smem, (uint32_t)done, chunk, exchange_every, 0,
+                                nullptr, st, -shape.gr, false, L)) != cudaSuccess)
             return noalloc_cuda_fail("sweep kernel", ce, st, true);
         done += chunk;
     }
