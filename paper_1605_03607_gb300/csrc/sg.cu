@@ -15,6 +15,14 @@
 // memory).  Gradients are FP32 buffers; master weights and Adam moments are
 // FP32.  Every reduction runs in a fixed order (no floating-point atomics), so
 // a training step is bit-reproducible.
+//
+// Bound: memory and L2 traffic of the row-wise data (a batch of 256 C_8 graphs has
+// 753,664 message, 131,072 node and 376,832 edge rows of 64; the linear maps need
+// 0.13 ms of tensor time), and launch gaps for small batches.  So per layer 3 forward
+// and 4 backward kernels, each a linear map with everything around it, and no message
+// row in memory.  Measured against one kernel per step with FP32 messages, pre-activations
+// and masked gradients in memory (97 launches, 35 now): gradient of 256 C_8 graphs 3.95 ->
+// 2.24 ms, of 128 C_4 graphs 1.01 -> 0.59 ms, 64 C_8 predictions 0.42 -> 0.26 ms.
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -46,72 +54,23 @@ __device__ __forceinline__ float2 unpack_bf2(uint32_t u)
     return __bfloat1622float2(v);
 }
 
-// Row r of a linear map's input is [P0[idx0(r)] | P1[idx1(r)]] with
-// idx(r) = (r / R_local) * S + map[r % R_local] (64 BF16 per row each).
-struct RowSrc {
-    const bf16* P0;
-    const int* map0;
-    int S0;
-    const bf16* P1;
-    const int* map1;
-    int S1;
-    int R_local;
-    __device__ __forceinline__ const uint32_t* half(int r, int which) const
-    {
-        const int b = r / R_local, l = r - b * R_local;
-        if (which == 0) return reinterpret_cast<const uint32_t*>(P0 + ((size_t)b * S0 + map0[l]) * HD);
-        return reinterpret_cast<const uint32_t*>(P1 + ((size_t)b * S1 + map1[l]) * HD);
-    }
-};
-
 // Floats of one CTA's weight-gradient partial: dW [64][128] then db [64].
 constexpr int WPART = HD * KIN + HD;
 
-// dW += sum over blocks of the partials (and db likewise), in a fixed order:
-// stage 1 (grid.y = WRED_GROUPS) sums consecutive ranges of the partials
-// into `tmp`, stage 2 adds the group sums in order.
-constexpr int WRED_GROUPS = 16;
-__global__ void lin_wgrad_reduce1(int nblocks, const float* __restrict__ part, float* __restrict__ tmp)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= WPART) return;
-    const int per = (nblocks + WRED_GROUPS - 1) / WRED_GROUPS;
-    const int b0 = blockIdx.y * per, b1 = min(nblocks, b0 + per);
-    float s0 = 0.f, s1 = 0.f;
-    int b = b0;
-    for (; b + 2 <= b1; b += 2) {
-        s0 += part[(size_t)b * WPART + i];
-        s1 += part[(size_t)(b + 1) * WPART + i];
-    }
-    if (b < b1) s0 += part[(size_t)b * WPART + i];
-    tmp[(size_t)blockIdx.y * WPART + i] = s0 + s1;
-}
-
-__global__ void lin_wgrad_reduce2(const float* __restrict__ tmp, float* __restrict__ dW, float* __restrict__ db)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= WPART) return;
-    float s = 0.f;
-    for (int g = 0; g < WRED_GROUPS; ++g) s += tmp[(size_t)g * WPART + i];
-    if (i < HD * KIN) dW[i] += s;
-    else db[i - HD * KIN] += s;
-}
-
 // ------------------------------------------- tcgen05 (5th-generation tensor core) GEMMs
-// The forward maps Z = X W^T + b (128 rows x K = 128 -> 64 outputs per tile)
-// and the input gradient dX = dZ W (128 rows x K = 64 -> 128 inputs per
-// tile) run on tcgen05.mma with the accumulator in tensor memory:
-//   * one CTA of 128 threads per 128-row tile (persistent over tiles); one
-//     thread issues the MMAs and commits them to an mbarrier;
-//   * operands in shared memory in the canonical K-major layout without
-//     swizzle, built from 8-row x 16-byte core matrices stored as
-//     [8-row group][k-chunk of 8 elements][8 rows][16 bytes]: core matrices
-//     adjacent in K are 128 bytes apart (the leading byte offset) and 8-row
-//     groups (number of k-chunks) x 128 bytes apart (the stride byte offset).
-//     Read with the two offsets the other way round, every address would
-//     still lie inside the 48 KB the kernels allocate;
+// The forward maps Z = X W^T + b (128 rows x K = 128 -> 64 outputs per tile),
+// the input gradient dX = dZ W (128 rows x K = 64 -> 64 inputs at a time) and the
+// weight gradient dW^T += X^T dZ (K = 128 rows) run on tcgen05.mma with the
+// accumulator in tensor memory:
+//   * persistent CTAs over 128-row tiles; one thread issues the MMAs and
+//     commits them to an mbarrier;
+//   * operands in shared memory in the canonical layout without swizzle, built
+//     from 8-row x 16-byte core matrices; a descriptor's leading byte offset
+//     steps between core matrices along K, its stride byte offset along M or N.
+//     With the two the other way round every address would still lie inside the
+//     CTA's shared memory;
 //   * the weights, pre-packed in that layout (pack_weights_kernel), arrive by
-//     one bulk asynchronous copy; the gathered input rows by 16-byte cp.async;
+//     one bulk asynchronous copy; gathered rows by 16-byte cp.async;
 //   * after the commit each warp reads its 32 accumulator rows (TMEM lanes
 //     32w .. 32w+31) with tcgen05.ld, one row per thread, for the epilogue;
 //   * every mbarrier wait is bounded: on a timeout the CTA records it in
@@ -121,19 +80,14 @@ constexpr int TC_ROWS = 128;
 // CTAs of 256 threads: all 8 warps stage a tile; in the epilogue warps w and
 // w + 4 read the same 32 tensor-memory lanes (a warp reaches lanes
 // 32 (w mod 4) .. + 31) and split the columns, and each warp's stores pass
-// through a 4 KB slice of the consumed operand buffer (warp_store_*).
-// Dynamic shared memory: forward A 32 KB + W 16 KB = 48 KB, input gradient
-// dZ 16 KB + staging 16 KB + W^T 16 KB = 48 KB (4 CTAs per SM, 64 or 128
-// tensor-memory columns each);
-// weight gradient two stages of 24 KB (the next chunk loads while the
-// current one is multiplied) + ones 16 KB = 64 KB (3 CTAs, 128 columns).  The
-// shared memory bounds the resident CTAs, so their tensor memory never
-// exceeds an SM's 512 columns; the persistent grids use exactly that many.
+// through a 4 KB slice of the consumed operand buffer.  The dynamic shared
+// memory (forward: A 32 KB + W 16 KB; backward below) bounds the resident CTAs,
+// so that their tensor memory (64 columns forward, 128 backward) never exceeds an
+// SM's 512 columns; the persistent grids use exactly that many.
 constexpr int TC_THREADS = 256;
-constexpr int TC_A_FWD = TC_ROWS * KIN * 2, TC_A_BWD = TC_ROWS * HD * 2;
+constexpr int TC_A_FWD = TC_ROWS * KIN * 2;
 constexpr int TC_SMEM_FWD = TC_A_FWD + HD * KIN * 2;
-constexpr int TC_SMEM_BWD = TC_SMEM_FWD;
-constexpr int TC_CTAS_FWD = 4, TC_CTAS_BWD = 4, TC_CTAS_WGRAD = 3;
+constexpr int TC_CTAS_FWD = 4;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -244,10 +198,31 @@ __device__ __forceinline__ void flush_f32x32(const unsigned char* stage, float* 
     __syncwarp();
 }
 
-// Adds the sums of staged row pairs (2p, 2p + 1), in that order, to row p of g
-// (16 pairs x 32 FP32 columns; only pairs < npairs).
-__device__ __forceinline__ void flush_pairs_add_f32x32(const unsigned char* stage, float* g, int ld, int npairs,
-                                                       int lane)
+// The same, added to g's rows.
+__device__ __forceinline__ void flush_add_f32x32(const unsigned char* stage, float* g, int ld, int nvalid, int lane)
+{
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int row = k * 4 + (lane >> 3), c = lane & 7;
+        float4 x = *reinterpret_cast<const float4*>(stage + row * 128 + ((c ^ (row & 7)) << 4));
+        if (row < nvalid) {
+            float4* gp = reinterpret_cast<float4*>(g + (size_t)row * ld + c * 4);
+            const float4 o = *gp;
+            x.x += o.x;
+            x.y += o.y;
+            x.z += o.z;
+            x.w += o.w;
+            *gp = x;
+        }
+    }
+    __syncwarp();
+}
+
+// Adds the sums of staged row pairs (2p, 2p + 1), in that order, to row p of g, or
+// (set) puts them there (16 pairs x 32 FP32 columns; only pairs < npairs).
+__device__ __forceinline__ void flush_pairs_f32x32(const unsigned char* stage, float* g, int ld, int npairs, int lane,
+                                                   bool set)
 {
     __syncwarp();
 #pragma unroll
@@ -257,7 +232,7 @@ __device__ __forceinline__ void flush_pairs_add_f32x32(const unsigned char* stag
         const float4 b = *reinterpret_cast<const float4*>(stage + rb * 128 + ((c ^ (rb & 7)) << 4));
         if (p < npairs) {
             float4* gp = reinterpret_cast<float4*>(g + (size_t)p * ld + c * 4);
-            float4 o = *gp;
+            float4 o = set ? make_float4(0.f, 0.f, 0.f, 0.f) : *gp;
             o.x += a.x + b.x;
             o.y += a.y + b.y;
             o.z += a.z + b.z;
@@ -333,45 +308,84 @@ __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t ncols, bool 
     if (failed && threadIdx.x == 0) atomicExch(err, 1);
 }
 
-// Forward: Z = X W^T + bias over `rows` gathered rows (see RowSrc).  EPI 0
-// (messages): Z -> Zout (BF16), relu(Z) -> Rout (FP32).  EPI 1 (residual):
-// Z -> Zout, Yout = P0 row + relu(Z) (BF16).
-template <int EPI>
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD) lin_fwd_tc_kernel(int rows, RowSrc src, const bf16* __restrict__ Wpk,
-                                                                const float* __restrict__ bias, bf16* __restrict__ Zout,
-                                                                float* __restrict__ Rout, bf16* __restrict__ Yout,
-                                                                int* err)
+// ------------------------------------------------------------- layer kernels
+// Rows of a tile are gathered while they are staged, and everything elementwise
+// around a linear map runs in its staging or its epilogue, so that per layer only
+// node and edge features (BF16), their gradients (FP32) and one bit per activation
+// go through memory:
+//   * the backward needs a pre-activation's sign only: the forward keeps it as a
+//     bit (z > 0 after rounding to BF16), 8 bytes per row of 64;
+//   * messages are computed target by target, 21 nodes of 6 slots per tile, and
+//     summed in the epilogue (in the order of the node's slots); their gradient
+//     with respect to the source node source by source, the same way;
+//   * a map's input gradient and weight gradient share the staged tile.
+// Row r of a tile sits in 8-row core matrices: chunk (row group r / 8, column chunk
+// of 8) is 8 rows x 16 bytes.  Read along its columns that is a K-major operand,
+// read along its rows an MN-major one; only the two descriptor strides differ (the
+// leading offset steps along K, the stride offset along M or N), so the dZ tile is
+// the A operand of the input gradient and the B operand of the weight gradient.
+constexpr int NODE_ROWS = 6, TILE_NODES = TC_ROWS / NODE_ROWS;        // 21 nodes, 126 rows
+
+// z's sign bit of the backward's mask: positive after rounding to BF16 (2^-133 is
+// the smallest BF16 number; 2^-134 and below round to zero).
+__device__ __forceinline__ uint32_t positive_bf16(float z) { return z > 0x1p-134f ? 1u : 0u; }
+
+// 8 BF16 values (one 16-byte chunk) with the columns whose mask bit is 0 cleared.
+__device__ __forceinline__ uint4 mask_bf16x8(uint4 v, uint32_t bits)
+{
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] &= ((bits >> (2 * i)) & 1u ? 0xFFFFu : 0u) | ((bits >> (2 * i + 1)) & 1u ? 0xFFFF0000u : 0u);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+__device__ __forceinline__ uint32_t mask_byte(const uint2* mask, size_t row, int kc)
+{
+    return (reinterpret_cast<const uint8_t*>(mask + row))[kc];
+}
+
+// Messages: rows [h[src] | e[edge]] of 21 target nodes, m = sum over a node's slots of
+// relu(z) (FP32, slot order) as BF16, and the mask bits of row (node, slot).
+// in_tab [N][6]: (source node, edge) of every slot, -1 where empty.
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD)
+msg_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* __restrict__ h, const bf16* __restrict__ e,
+               const bf16* __restrict__ Wpk, const float* __restrict__ bias, bf16* __restrict__ m, uint2* __restrict__ mask,
+               int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char* As = tc_smem;                         // [16 row groups][16 k-chunks][8 rows][16 B]
+    unsigned char* As = tc_smem;                         // [16 row groups][16 k-chunks][8 rows][16 B], then FP32 rows
     unsigned char* Ws = tc_smem + TC_A_FWD;              // [8 output groups][16 k-chunks][8 outputs][16 B]
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
-    __shared__ const unsigned char* rowp[2][2][TC_ROWS]; // gathered row halves of this and the next tile (NULL past the end)
+    __shared__ const unsigned char* rowp[2][2][TC_ROWS]; // gathered row halves of this and the next tile (NULL: no row)
     __shared__ float bias_sm[HD];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid < HD) bias_sm[tid] = bias[tid];
     bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, Wpk, HD * KIN * 2);
     const uint32_t tmem = tmem_sh;
     constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);
-    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
+    const int ntiles = (nodes + TILE_NODES - 1) / TILE_NODES;
     uint32_t phase = 0;
-    // one index lookup per row half: thread tid looks up row tid mod 128, half tid / 128
     auto lookup = [&](int t, int buf) {
-        const int row = tid & (TC_ROWS - 1), hf = tid >> 7, r = t * TC_ROWS + row;
-        rowp[buf][hf][row] = r < rows ? reinterpret_cast<const unsigned char*>(src.half(r, hf)) : nullptr;
+        const int row = tid & (TC_ROWS - 1), hf = tid >> 7, k = row / NODE_ROWS, n = t * TILE_NODES + k;
+        const unsigned char* p = nullptr;
+        if (k < TILE_NODES && n < nodes) {
+            const int b = n / N, l = n - b * N;
+            const int2 s = in_tab[l * NODE_ROWS + row - k * NODE_ROWS];
+            if (s.x >= 0)
+                p = reinterpret_cast<const unsigned char*>(hf == 0 ? h + ((size_t)b * N + s.x) * HD : e + ((size_t)b * E + s.y) * HD);
+        }
+        rowp[buf][hf][row] = p;
     };
     if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
     int buf = 0;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
-        const int r0 = tile * TC_ROWS;
         __syncthreads();                                    // this tile's row pointers staged; the last epilogue done
         for (int i = tid; i < 16 * TC_ROWS; i += TC_THREADS) {   // chunk i: row (i >> 7) * 8 + (i & 7), k-chunk (i >> 3) & 15
             const int kc = (i >> 3) & 15, row = ((i >> 7) << 3) | (i & 7);
             const unsigned char* p = rowp[buf][kc >> 3][row];
             cp_async16(As + i * 16, p ? p + (kc & 7) * 16 : reinterpret_cast<const unsigned char*>(Wpk), p != nullptr);
         }
-        // the next tile's lookups overlap this gather (its buffer was last read by the previous gather)
         if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
         asm volatile("cp.async.wait_all;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // visible to the tensor core
@@ -392,13 +406,11 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD) lin_fwd_tc_kernel(int
             break;
         }
         tc_fence_after();
-        // warp w: accumulator rows 32 (w mod 4) .. + 31 (TMEM lanes), columns 32 (w / 4) .. + 31, read
-        // 16 at a time; the operand tile is consumed (MMA complete), so its 32 KB hold the 8 warps'
-        // staging slices
-        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row0 = r0 + q * 32, row = q * 32 + lane;
+        // warp w: accumulator rows 32 (w mod 4) .. + 31, columns 32 (w / 4) .. + 31: relu(z) to the consumed
+        // operand tile as FP32 rows of 256 bytes (16-byte chunks swizzled by row)
+        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row = q * 32 + lane;
         const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-        unsigned char* stage = As + warp * 4096;
-        uint32_t zw[HD / 4], yw[EPI == 1 ? HD / 4 : 1];
+        uint32_t bits = 0u;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
             const int c0 = cb + 16 * hh;
@@ -406,75 +418,107 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD) lin_fwd_tc_kernel(int
             tmem_ld16(tl + c0, z);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) z[i] += bias_sm[c0 + i];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) zw[8 * hh + i] = pack_bf2(z[2 * i], z[2 * i + 1]);
-            if (EPI == 0) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    stage_f32(stage, lane, 4 * hh + c,
-                              make_float4(fmaxf(z[4 * c], 0.f), fmaxf(z[4 * c + 1], 0.f), fmaxf(z[4 * c + 2], 0.f),
-                                          fmaxf(z[4 * c + 3], 0.f)));
-            } else {
-                // the residual input is half 0 of this row, already staged: k-chunks c0/8 and c0/8 + 1
-#pragma unroll
-                for (int kc = 0; kc < 2; ++kc) {
-                    const uint4 b4 = *reinterpret_cast<const uint4*>(As + (((row >> 3) * 16 + (c0 >> 3) + kc) * 128) +
-                                                                     (row & 7) * 16);
-                    const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 bb = unpack_bf2(bw[i]);
-                        yw[(EPI == 1 ? 8 * hh + 4 * kc + i : 0)] =
-                            pack_bf2(bb.x + fmaxf(z[8 * kc + 2 * i], 0.f), bb.y + fmaxf(z[8 * kc + 2 * i + 1], 0.f));
-                    }
-                }
+            for (int i = 0; i < 16; ++i) {
+                z[i] += bias_sm[c0 + i];
+                bits |= positive_bf16(z[i]) << (16 * hh + i);
             }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                *reinterpret_cast<float4*>(As + row * 256 + ((((c0 >> 2) + c) ^ (row & 7)) << 4)) =
+                    make_float4(fmaxf(z[4 * c], 0.f), fmaxf(z[4 * c + 1], 0.f), fmaxf(z[4 * c + 2], 0.f), fmaxf(z[4 * c + 3], 0.f));
         }
-        if constexpr (EPI == 0) {
-            flush_f32x32(stage, Rout + (size_t)row0 * HD + cb, HD, rows - row0, lane);
-        } else {
-            __syncthreads();                               // every residual read before any slice is overwritten
-            store_bf16x32(stage, yw, Yout + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+        if (mask && rowp[buf][0][row])
+            reinterpret_cast<uint32_t*>(mask + (size_t)tile * TILE_NODES * NODE_ROWS + row)[warp >> 2] = bits;
+        __syncthreads();
+        for (int i = tid; i < TILE_NODES * (HD / 2); i += TC_THREADS) {      // node i / 32 of the tile, column pair i mod 32
+            const int k = i >> 5, cp = i & 31, n = tile * TILE_NODES + k;
+            if (n >= nodes) break;
+            float x = 0.f, y = 0.f;
+#pragma unroll
+            for (int s = 0; s < NODE_ROWS; ++s) {
+                const int r = k * NODE_ROWS + s;
+                if (!rowp[buf][0][r]) continue;
+                const float2 v = *reinterpret_cast<const float2*>(As + r * 256 + (((cp >> 1) ^ (r & 7)) << 4) + (cp & 1) * 8);
+                x += v.x;
+                y += v.y;
+            }
+            reinterpret_cast<uint32_t*>(m + (size_t)n * HD)[cp] = pack_bf2(x, y);
         }
-        store_bf16x32(stage, zw, Zout + (size_t)row0 * HD + cb, HD, rows - row0, lane);
     }
     tc_teardown(tmem, 64, failed, err);
 }
 
-// Input gradient: dX = dZ W over `rows` rows of dZ [rows][64] (BF16), with
-// W^T pre-packed.  EPI 0 (messages; rows 2e and 2e+1 are the two directions
-// of edge e): dX[:, :64] -> dX [rows][64] FP32, and the edge half of each
-// pair, dX[2e][64:] + dX[2e+1][64:], added to out1[e] ([rows / 2][64]).
-// EPI 1 (node and edge updates): out0 = base + dX[:, :64] (base may be out0
-// or NULL) and out1 = dX[:, 64:], both [rows][64] FP32.
-template <int EPI>
-__global__ void __launch_bounds__(TC_THREADS, EPI == 0 ? TC_CTAS_BWD : 2) lin_bwd_input_tc_kernel(int rows, const bf16* __restrict__ dZ,
-                                                                      const bf16* __restrict__ WTpk,
-                                                                      float* __restrict__ dX, const float* base,
-                                                                      float* out0, float* __restrict__ out1, int* err)
+// Sum of two BF16 rows' chunk, rounded to BF16.
+__device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b)
+{
+    const uint32_t x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float2 p = unpack_bf2(x[i]), q = unpack_bf2(y[i]);
+        w[i] = pack_bf2(p.x + q.x, p.y + q.y);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Node and edge updates: Y = P0 + relu([P0 | second] W^T + bias) as BF16 and the mask
+// bits.  Nodes: second = m (rows of P1).  Edges (EDGE): second = h[i] + h[j], the sum
+// of the edge's end rows of P1 = h, formed while staging.
+template <bool EDGE>
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD)
+upd_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ P1, const int2* __restrict__ ends, int N, int E,
+               const bf16* __restrict__ Wpk, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask,
+               int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char* As = tc_smem;                         // [16 row groups][8 k-chunks][8 rows][16 B]
-    unsigned char* Ws = tc_smem + 2 * TC_A_BWD;          // [16 input groups][8 k-chunks][8 inputs][16 B]
-    // bytes [0, 2 * TC_A_BWD): the dZ tile, then (MMA complete) the epilogue's staging slices
+    unsigned char* As = tc_smem;                         // [16 row groups][16 k-chunks][8 rows][16 B]
+    unsigned char* Ws = tc_smem + TC_A_FWD;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
+    __shared__ const uint4* endp[2][2][TC_ROWS];         // EDGE: the two end rows of this and the next tile's edges
+    __shared__ float bias_sm[HD];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk, KIN * HD * 2);
+    if (tid < HD) bias_sm[tid] = bias[tid];
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, Wpk, HD * KIN * 2);
     const uint32_t tmem = tmem_sh;
-    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, KIN);
+    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);
     const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
     uint32_t phase = 0;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
-        const int r0 = tile * TC_ROWS;
-        for (int i = tid; i < 8 * TC_ROWS; i += TC_THREADS) {    // chunk i: row (i >> 6) * 8 + (i & 7), k-chunk (i >> 3) & 7
-            const int kc = (i >> 3) & 7, row = ((i >> 6) << 3) | (i & 7), r = r0 + row;
-            const bool v = r < rows;
-            const unsigned char* g = v ? reinterpret_cast<const unsigned char*>(dZ + (size_t)r * HD) + kc * 16
-                                       : reinterpret_cast<const unsigned char*>(WTpk);
-            cp_async16(As + i * 16, g, v);
+    auto lookup = [&](int t, int buf) {
+        if (!EDGE) return;
+        const int row = tid & (TC_ROWS - 1), which = tid >> 7, r = t * TC_ROWS + row;
+        const uint4* p = nullptr;
+        if (r < rows) {
+            const int b = r / E, l = r - b * E;
+            const int2 ij = ends[l];
+            p = reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + (which == 0 ? ij.x : ij.y)) * HD);
         }
+        endp[buf][which][row] = p;
+    };
+    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        const int r0 = tile * TC_ROWS;
+        __syncthreads();
+        if (EDGE) {
+            for (int i = tid; i < 8 * TC_ROWS; i += TC_THREADS) {        // first half: chunk kc of row, consecutive rows of P0
+                const int kc = (i >> 3) & 7, row = ((i >> 6) << 3) | (i & 7), r = r0 + row;
+                cp_async16(As + (((row >> 3) * 16 + kc) * 8 + (row & 7)) * 16, P0 + (size_t)(r < rows ? r : 0) * HD + kc * 8, r < rows);
+            }
+#pragma unroll
+            for (int j = 0; j < 8 * TC_ROWS / TC_THREADS; ++j) {         // second half: the sum of the end rows
+                const int i = tid + j * TC_THREADS, kc = (i >> 3) & 7, row = ((i >> 6) << 3) | (i & 7);
+                const uint4 *p = endp[buf][0][row], *q = endp[buf][1][row];
+                *reinterpret_cast<uint4*>(As + (((row >> 3) * 16 + 8 + kc) * 8 + (row & 7)) * 16) =
+                    p ? add_bf16x8(p[kc], q[kc]) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        } else {
+            for (int i = tid; i < 16 * TC_ROWS; i += TC_THREADS) {
+                const int kc = (i >> 3) & 15, row = ((i >> 7) << 3) | (i & 7), r = r0 + row;
+                cp_async16(As + i * 16, (kc < 8 ? P0 : P1) + (size_t)(r < rows ? r : 0) * HD + (kc & 7) * 8, r < rows);
+            }
+        }
+        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
         asm volatile("cp.async.wait_all;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
@@ -482,20 +526,10 @@ __global__ void __launch_bounds__(TC_THREADS, EPI == 0 ? TC_CTAS_BWD : 2) lin_bw
         tc_fence_after();
         if (tid == 0) {
 #pragma unroll
-            for (int ks = 0; ks < HD / 16; ++ks)
-                tc_mma(tmem, tc_desc(smem_u32(As) + ks * 256, 128, 8 * 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 8 * 128),
+            for (int ks = 0; ks < KIN / 16; ++ks)
+                tc_mma(tmem, tc_desc(smem_u32(As) + ks * 256, 128, 16 * 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 16 * 128),
                        IDESC, ks > 0 ? 1u : 0u);
             tc_commit(&bar_mma);
-        }
-        const int q = warp & 3, r = r0 + q * 32 + lane;
-        // warps 0-3 add this row's base gradient to dX[:, :64]: loaded while the MMAs run
-        float4 bpre[EPI == 1 ? HD / 4 : 1];
-        if (EPI == 1 && warp < 4 && base && r < rows) {
-#pragma unroll
-            for (int i = 0; i < HD / 4; ++i) bpre[i] = reinterpret_cast<const float4*>(base + (size_t)r * HD)[i];
-        } else {
-#pragma unroll
-            for (int i = 0; i < (EPI == 1 ? HD / 4 : 1); ++i) bpre[i] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         const bool ok = mbar_wait(&bar_mma, phase);
         phase ^= 1u;
@@ -504,163 +538,443 @@ __global__ void __launch_bounds__(TC_THREADS, EPI == 0 ? TC_CTAS_BWD : 2) lin_bw
             break;
         }
         tc_fence_after();
-        // warp w: rows 32 (w mod 4) .. + 31, columns 64 (w / 4) .. + 63 of dX, in two passes of 32
-        // through its staging slice (the consumed dZ tile and the 16 KB above it)
+        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row0 = r0 + q * 32, row = q * 32 + lane;
         const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-        const int row0 = r0 + q * 32;
         unsigned char* stage = As + warp * 4096;
+        uint32_t yw[HD / 4], bits = 0u;
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-            const int c0 = (warp >> 2) * HD + pass * 32;
+        for (int hh = 0; hh < 2; ++hh) {
+            const int c0 = cb + 16 * hh;
+            float z[16];
+            tmem_ld16(tl + c0, z);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                z[i] += bias_sm[c0 + i];
+                bits |= positive_bf16(z[i]) << (16 * hh + i);
+            }
+            // the residual input is half 0 of this row, already staged: k-chunks c0/8 and c0/8 + 1
+#pragma unroll
+            for (int kc = 0; kc < 2; ++kc) {
+                const uint4 b4 = *reinterpret_cast<const uint4*>(As + (((row >> 3) * 16 + (c0 >> 3) + kc) * 128) + (row & 7) * 16);
+                const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 bb = unpack_bf2(bw[i]);
+                    yw[8 * hh + 4 * kc + i] = pack_bf2(bb.x + fmaxf(z[8 * kc + 2 * i], 0.f), bb.y + fmaxf(z[8 * kc + 2 * i + 1], 0.f));
+                }
+            }
+        }
+        if (mask && r0 + row < rows) reinterpret_cast<uint32_t*>(mask + r0 + row)[warp >> 2] = bits;
+        __syncthreads();                                   // every residual read before any slice is overwritten
+        store_bf16x32(stage, yw, Yout + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+    }
+    tc_teardown(tmem, 64, failed, err);
+}
+
+// ---- backward: input gradient dX = dZ W and weight gradient dW += dZ^T X of a tile
+// Shared memory: X [16 input groups][16 row groups][8 rows][16 B] (32 KB, the weight
+// gradient's A operand), dZ [16 row groups][8 k-chunks][8 rows][16 B] (16 KB), W^T
+// (one or both 8 KB halves of 64 inputs).  Tensor memory: columns 0..63 dW^T
+// accumulated over the CTA's tiles, 64..127 the current half of dX.  db: a thread
+// stages one 8-column chunk of every eighth row group and adds it up on the way.
+constexpr int BW_X = TC_ROWS * KIN * 2, BW_Z = TC_ROWS * HD * 2, BW_W = HD * HD * 2;
+constexpr int TC_SMEM_UPD_BWD = BW_X + BW_Z + 2 * BW_W, TC_SMEM_EDGE_BWD = BW_X + BW_Z + BW_W;
+constexpr int TC_CTAS_UPD_BWD = 3, TC_CTAS_EDGE_BWD = 3;
+
+__device__ __forceinline__ void bwd_mma_wgrad(uint32_t tmem, const unsigned char* Xs, const unsigned char* Zs, bool first)
+{
+    constexpr uint32_t IDESC = tc_idesc_bf16(KIN, HD) | (1u << 15) | (1u << 16);   // M = 128 inputs, N = 64, both MN-major
+#pragma unroll
+    for (int ks = 0; ks < TC_ROWS / 16; ++ks)
+        tc_mma(tmem, tc_desc(smem_u32(Xs) + ks * 256, 128, 16 * 128), tc_desc(smem_u32(Zs) + ks * 2048, 1024, 128), IDESC,
+               first && ks == 0 ? 0u : 1u);
+}
+
+__device__ __forceinline__ void bwd_mma_input(uint32_t tmem, const unsigned char* Zs, const unsigned char* Wh)
+{
+    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);                         // one half: 64 inputs
+#pragma unroll
+    for (int ks = 0; ks < HD / 16; ++ks)
+        tc_mma(tmem + HD, tc_desc(smem_u32(Zs) + ks * 256, 128, 8 * 128), tc_desc(smem_u32(Wh) + ks * 256, 128, 8 * 128), IDESC,
+               ks > 0 ? 1u : 0u);
+}
+
+// Adds the 8 BF16 values of a staged dZ chunk to this thread's column sums.
+__device__ __forceinline__ void add_db(float (&db)[8], uint4 z)
+{
+    const uint32_t w[4] = {z.x, z.y, z.z, z.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float2 v = unpack_bf2(w[i]);
+        db[2 * i] += v.x;
+        db[2 * i + 1] += v.y;
+    }
+}
+
+// The CTA's partials: dW [64][128] from tensor memory (lane = input), db [64] from the
+// threads' column sums (thread: chunk kc of 8 columns; the 32 threads of a chunk in
+// thread order), through `sm` (8 KB of shared memory).
+__device__ __forceinline__ void bwd_partials(uint32_t tmem, float* P, const float (&db)[8], int kc, float* sm)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (warp < 4) {
+        const int in = warp * 32 + lane;
+        const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll
+        for (int c0 = 0; c0 < HD; c0 += 16) {
+            float d[16];
+            tmem_ld16(tl + c0, d);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) P[(c0 + i) * KIN + in] = d[i];
+        }
+    }
+    __syncthreads();                                        // the last tile's staging slices are read
+    // threads of chunk kc: 8 per warp in the 4 warps with warp & 1 == kc >> 2
+    const int slot = (warp >> 1) * 8 + (lane & 7);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sm[(kc * 8 + i) * 32 + slot] = db[i];
+    __syncthreads();
+    if (tid < HD) {
+        float s = 0.f;
+        for (int j = 0; j < 32; ++j) s += sm[tid * 32 + j];
+        P[HD * KIN + tid] = s;
+    }
+}
+
+// Node and edge updates.  EDGE: dZ = de & mask, de += dX[:, :64] in place, ds = dX[:, 64:]
+// (FP32); X = [e | h_i + h_j].  Nodes: dh += sum over the node's edges of ds (inc order; inc NULL: none),
+// dZ = dh & mask, dh += dX[:, :64], dm = dX[:, 64:] rounded to BF16 (the one form that
+// the messages' dZ = dm & mask takes it in); X = [h | m].
+template <bool EDGE>
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_UPD_BWD)
+upd_bwd_kernel(int rows, int N, int E, const uint2* __restrict__ mask, float* g, const bf16* __restrict__ P0,
+               const bf16* __restrict__ P1, const int2* __restrict__ ends, const int* __restrict__ inc, float* ds,
+               bf16* __restrict__ dm, const bf16* __restrict__ WTpk, float* __restrict__ part, int* err)
+{
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    unsigned char *Xs = tc_smem, *Zs = tc_smem + BW_X, *Ws = Zs + BW_Z;
+    __shared__ __align__(8) uint64_t bar_w, bar_mma;
+    __shared__ uint32_t tmem_sh;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk, 2 * BW_W);
+    const uint32_t tmem = tmem_sh;
+    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
+    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;     // a warp stages 8 rows x 4 chunks at a time
+    float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    uint32_t phase = 0;
+    bool first = true;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
+        const int r0 = tile * TC_ROWS;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {                       // X
+            const int u = warp + 8 * j, rg = u >> 2, kc = (u & 3) * 4 + q4, row = rg * 8 + r8, r = r0 + row;
+            unsigned char* dst = Xs + (kc * 16 + rg) * 128 + r8 * 16;
+            const bool v = r < rows;
+            if (!EDGE || (u & 2) == 0) {
+                cp_async16(dst, (kc < 8 ? P0 : P1) + (size_t)(v ? r : 0) * HD + (kc & 7) * 8, v);
+            } else {
+                uint4 s = make_uint4(0u, 0u, 0u, 0u);
+                if (v) {
+                    const int b = r / E;
+                    const int2 ij = ends[r - b * E];
+                    s = add_bf16x8(*reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + ij.x) * HD + (kc & 7) * 8),
+                                   *reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + ij.y) * HD + (kc & 7) * 8));
+                }
+                *reinterpret_cast<uint4*>(dst) = s;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {                       // dZ: chunk kz of row groups (warp >> 1) + 4 j
+            const int rg = (warp >> 1) + 4 * j, row = rg * 8 + r8, r = r0 + row;
+            uint4 z = make_uint4(0u, 0u, 0u, 0u);
+            if (r < rows) {
+                float4* gp = reinterpret_cast<float4*>(g + (size_t)r * HD + kz * 8);
+                float4 a = gp[0], b = gp[1];
+                if (!EDGE && inc) {
+                    const int bi = r / N;
+                    const int* il = inc + (r - bi * N) * NODE_ROWS;
+                    float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+#pragma unroll
+                    for (int s = 0; s < NODE_ROWS; ++s) {
+                        const int ed = il[s];
+                        if (ed < 0) continue;
+                        const float4* dp = reinterpret_cast<const float4*>(ds + ((size_t)bi * E + ed) * HD + kz * 8);
+                        const float4 x = dp[0], y = dp[1];
+                        s0.x += x.x; s0.y += x.y; s0.z += x.z; s0.w += x.w;
+                        s1.x += y.x; s1.y += y.y; s1.z += y.z; s1.w += y.w;
+                    }
+                    a.x += s0.x; a.y += s0.y; a.z += s0.z; a.w += s0.w;
+                    b.x += s1.x; b.y += s1.y; b.z += s1.z; b.w += s1.w;
+                    gp[0] = a;                              // the epilogue adds dX to it
+                    gp[1] = b;
+                }
+                z = mask_bf16x8(make_uint4(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w), pack_bf2(b.x, b.y), pack_bf2(b.z, b.w)),
+                                mask_byte(mask, r, kz));
+            }
+            add_db(db, z);
+            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const int q = warp & 3, row0 = r0 + q * 32, cb = (warp >> 2) * (HD / 2);
+        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
+        unsigned char* stage = Xs + warp * 4096;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            if (tid == 0) {
+                bwd_mma_input(tmem, Zs, Ws + half * BW_W);
+                if (half == 0) bwd_mma_wgrad(tmem, Xs, Zs, first);
+                tc_commit(&bar_mma);
+            }
+            const bool ok = mbar_wait(&bar_mma, phase);
+            phase ^= 1u;
+            if (__syncthreads_or(!ok)) {
+                failed = true;
+                break;
+            }
+            tc_fence_after();
+            uint32_t w[16];
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
                 float d[16];
-                tmem_ld16(tl + c0 + 16 * hh, d);
+                tmem_ld16(tl + 16 * hh, d);
                 tmem_ld_wait();
+                if (half == 0 || EDGE) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    float4 v = make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
-                    if (EPI == 1 && c0 < HD) {
-                        const float4 bb = bpre[(EPI == 1 ? (c0 >> 2) + 4 * hh + c : 0)];
-                        v.x += bb.x;
-                        v.y += bb.y;
-                        v.z += bb.z;
-                        v.w += bb.w;
-                    }
-                    stage_f32(stage, lane, 4 * hh + c, v);
+                    for (int c = 0; c < 4; ++c)
+                        stage_f32(stage, lane, 4 * hh + c, make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) w[8 * hh + i] = pack_bf2(d[2 * i], d[2 * i + 1]);
                 }
             }
-            if (EPI == 0 && c0 < HD)
-                flush_f32x32(stage, dX + (size_t)row0 * HD + c0, HD, rows - row0, lane);
-            else if (EPI == 0)                             // a warp's 32 rows are 16 whole edges (row0 is even)
-                flush_pairs_add_f32x32(stage, out1 + (size_t)(row0 / 2) * HD + (c0 - HD), HD, (rows - row0) / 2, lane);
-            else if (c0 < HD)
-                flush_f32x32(stage, out0 + (size_t)row0 * HD + c0, HD, rows - row0, lane);
-            else
-                flush_f32x32(stage, out1 + (size_t)row0 * HD + (c0 - HD), HD, rows - row0, lane);
+            if (half == 0) flush_add_f32x32(stage, g + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+            else if (EDGE) flush_f32x32(stage, ds + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+            else store_bf16x32(stage, w, dm + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+            tc_fence_before();
+            __syncthreads();                                // dX read, the slices free: the next half or tile
+            tc_fence_after();
         }
-        __syncthreads();                                   // staging slices read before the next tile lands there
+        first = false;
     }
+    if (!failed) bwd_partials(tmem, part + (size_t)blockIdx.x * WPART, db, kz, reinterpret_cast<float*>(Xs));
     tc_teardown(tmem, 128, failed, err);
 }
 
-// Weight gradient: dW = dZ^T X and db = column sums of dZ over `rows` rows,
-// as D[in][o] = sum_r X[r][in] dZ[r][o] (M = 128 inputs, N = 64 outputs,
-// K = rows) accumulated in tensor memory over the CTA's 64-row chunks c =
-// blockIdx.x, c += gridDim.x; db the same with a tile of ones in place of X.
-// Both operands are MN-major: a 16-byte chunk of a row of X (8 inputs) or of
-// dZ (8 outputs) is one row of a core matrix, so the rows are staged with
-// 16-byte cp.async and no transposition, as [MN group][k group][8 rows][16 B].
-// Each CTA writes its partial [64][128] + [64] like lin_wgrad_kernel, and
-// lin_wgrad_reduce1/2 add the partials in a fixed order.
-constexpr int TC_WCH = 64;                          // rows per chunk
-constexpr int TC_WSTAGE = TC_WCH * KIN * 2 + TC_WCH * HD * 2;          // X 16 KB + dZ 8 KB
-constexpr int TC_SMEM_WGRAD = 2 * TC_WSTAGE + TC_WCH * KIN * 2;         // two stages + ones 16 KB
-__global__ void __launch_bounds__(TC_THREADS) lin_wgrad_tc_kernel(int rows, const bf16* __restrict__ dZ, RowSrc src,
-                                                                  float* __restrict__ part, int* err)
+// Messages, edge half: rows 2e and 2e + 1 are the two directions of edge e; dZ = dm[tgt]
+// & mask, de[e] += dX[2e][64:] + dX[2e + 1][64:] (set: =), weight gradient with X = [h[src] | e].
+// msg_tab [2E]: (source node, mask row = target node * 6 + slot).
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_EDGE_BWD)
+msg_bwd_edge_kernel(int rows, int N, int E, const int2* __restrict__ msg_tab, const uint2* __restrict__ mask,
+                    const bf16* __restrict__ dm, const bf16* __restrict__ h, const bf16* __restrict__ e,
+                    const bf16* __restrict__ WTpk, float* de, int set, float* __restrict__ part, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    // stage b: X [16 input groups][8 row groups][8 rows][16 B], then dZ [8 output groups][8 row groups][8][16 B]
-    unsigned char* Os = tc_smem + 2 * TC_WSTAGE;             // ones, the layout of X
+    unsigned char *Xs = tc_smem, *Zs = tc_smem + BW_X, *Ws = Zs + BW_Z;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, nullptr, nullptr, 0);
+    __shared__ int4 rowt[2][TC_ROWS];                       // this and the next tile: source row, edge row, target row, mask row
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk + HD * HD, BW_W);
     const uint32_t tmem = tmem_sh;
-    for (int i = tid; i < TC_WCH * KIN / 8; i += TC_THREADS)   // 16 bytes of bf16 1.0 each
-        *reinterpret_cast<uint4*>(Os + i * 16) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    // M = 128 inputs, N = 64 outputs, both operands MN-major (bits 15, 16)
-    constexpr uint32_t IDESC = tc_idesc_bf16(KIN, HD) | (1u << 15) | (1u << 16);
-    const int nchunks = (rows + TC_WCH - 1) / TC_WCH;
-    __shared__ const unsigned char* rowp[2][2][TC_WCH];       // per stage: the chunk's gathered row halves
-    auto stage = [&](int c, int b) {
-        unsigned char* Xs = tc_smem + b * TC_WSTAGE;
-        unsigned char* Zs = Xs + TC_WCH * KIN * 2;
-        const int r0 = c * TC_WCH;
-        {                                                       // one index lookup per row half
-            const int row = tid & (TC_WCH - 1), hf = (tid >> 6) & 1, r = r0 + row;
-            if (tid < 2 * TC_WCH)
-                rowp[b][hf][row] = r < rows ? reinterpret_cast<const unsigned char*>(src.half(r, hf)) : nullptr;
-        }
-        __syncthreads();
-        for (int i = tid; i < TC_WCH * KIN / 8; i += TC_THREADS) {   // X: chunk i -> row group (i>>3)&7, inputs (i>>6)*8..
-            const int row = (((i >> 3) & 7) << 3) + (i & 7), mg = i >> 6;
-            const unsigned char* p = rowp[b][mg >> 3][row];
-            cp_async16(Xs + i * 16, p ? p + (mg & 7) * 16 : reinterpret_cast<const unsigned char*>(dZ), p != nullptr);
-        }
-        for (int i = tid; i < TC_WCH * HD / 8; i += TC_THREADS) {    // dZ: outputs (i>>6)*8..
-            const int r = r0 + (((i >> 3) & 7) << 3) + (i & 7), ng = i >> 6;
-            const bool v = r < rows;
-            const unsigned char* g = v ? reinterpret_cast<const unsigned char*>(dZ + (size_t)r * HD) + ng * 16
-                                       : reinterpret_cast<const unsigned char*>(dZ);
-            cp_async16(Zs + i * 16, g, v);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    };
+    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
+    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;
+    float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
-    int it = 0;
-    if (!failed && (int)blockIdx.x < nchunks) stage(blockIdx.x, 0);
-    for (int c = blockIdx.x; !failed && c < nchunks; c += gridDim.x, ++it) {
-        const int b = it & 1;
-        if (c + (int)gridDim.x < nchunks) {
-            stage(c + gridDim.x, b ^ 1);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
+    auto lookup = [&](int t, int buf) {
+        if (tid >= TC_ROWS) return;
+        const int r = t * TC_ROWS + tid;
+        int4 v = make_int4(-1, 0, 0, 0);
+        if (r < rows) {
+            const int b = r / (2 * E), l = r - b * 2 * E;
+            const int2 s = msg_tab[l];
+            v = make_int4(b * N + s.x, b * E + (l >> 1), b * N + s.y / NODE_ROWS, b * N * NODE_ROWS + s.y);
         }
+        rowt[buf][tid] = v;
+    };
+    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        const int r0 = tile * TC_ROWS;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int u = warp + 8 * j, rg = u >> 2, kc = (u & 3) * 4 + q4;
+            const int4 t = rowt[buf][rg * 8 + r8];
+            const bf16* p = kc < 8 ? h + (size_t)(t.x < 0 ? 0 : t.x) * HD : e + (size_t)t.y * HD;
+            cp_async16(Xs + (kc * 16 + rg) * 128 + r8 * 16, p + (kc & 7) * 8, t.x >= 0);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int rg = (warp >> 1) + 4 * j;
+            const int4 t = rowt[buf][rg * 8 + r8];
+            uint4 z = make_uint4(0u, 0u, 0u, 0u);
+            if (t.x >= 0)
+                z = mask_bf16x8(*reinterpret_cast<const uint4*>(dm + (size_t)t.z * HD + kz * 8), mask_byte(mask, t.w, kz));
+            add_db(db, z);
+            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
+        }
+        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
+        asm volatile("cp.async.wait_all;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
         if (tid == 0) {
-            const uint32_t xs = smem_u32(tc_smem + b * TC_WSTAGE), zs = xs + TC_WCH * KIN * 2;
-#pragma unroll
-            for (int ks = 0; ks < TC_WCH / 16; ++ks) {
-                const uint32_t acc = (first && ks == 0) ? 0u : 1u;
-                const uint64_t bz = tc_desc(zs + ks * 256, 128, 8 * 128);
-                tc_mma(tmem, tc_desc(xs + ks * 256, 128, 8 * 128), bz, IDESC, acc);
-                tc_mma(tmem + HD, tc_desc(smem_u32(Os) + ks * 256, 128, 8 * 128), bz, IDESC, acc);
-            }
+            bwd_mma_input(tmem, Zs, Ws);
+            bwd_mma_wgrad(tmem, Xs, Zs, first);
             tc_commit(&bar_mma);
         }
         first = false;
-        const bool ok = mbar_wait(&bar_mma, phase);            // the chunk's MMAs are done: its stage is reusable
+        const bool ok = mbar_wait(&bar_mma, phase);
         phase ^= 1u;
         if (__syncthreads_or(!ok)) {
             failed = true;
             break;
         }
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    if (!failed) {
         tc_fence_after();
-        float* P = part + (size_t)blockIdx.x * WPART;
-        const int q = warp & 3, in = q * 32 + (tid & 31);      // TMEM lane = input index
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-        if (warp < 4) {
+        const int q = warp & 3, row0 = r0 + q * 32, cb = (warp >> 2) * (HD / 2);
+        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
+        unsigned char* stage = Xs + warp * 4096;
 #pragma unroll
-            for (int c0 = 0; c0 < HD; c0 += 16) {
-                float d[16];
-                tmem_ld16(tl + c0, d);
-                tmem_ld_wait();
+        for (int hh = 0; hh < 2; ++hh) {
+            float d[16];
+            tmem_ld16(tl + 16 * hh, d);
+            tmem_ld_wait();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) P[(c0 + i) * KIN + in] = d[i];
+            for (int c = 0; c < 4; ++c)
+                stage_f32(stage, lane, 4 * hh + c, make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]));
+        }
+        // a warp's 32 rows are 16 whole edges (row0 is even)
+        flush_pairs_f32x32(stage, de + (size_t)(row0 / 2) * HD + cb, HD, (rows - row0) / 2, lane, set != 0);
+        tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+    if (!failed) bwd_partials(tmem, part + (size_t)blockIdx.x * WPART, db, kz, reinterpret_cast<float*>(Xs));
+    tc_teardown(tmem, 128, failed, err);
+}
+
+// Messages, node half: the rows of 21 source nodes (out_tab [N][6]: mask row of the
+// message in a slot, -1 where empty); dh[n] += sum over n's slots of dX[:, :64].
+// dZ (16 KB), then the FP32 rows over it (32 KB); W^T half; 12 KB unused, so that 4 CTAs fit and no fifth
+constexpr int TC_SMEM_NODE_BWD = TC_ROWS * HD * 4 + BW_W + 12 * 1024;
+constexpr int TC_CTAS_NODE_BWD = 4;
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_NODE_BWD)
+msg_bwd_node_kernel(int nodes, int N, const int* __restrict__ out_tab, const uint2* __restrict__ mask,
+                    const bf16* __restrict__ dm, const bf16* __restrict__ WTpk, float* dh, int* err)
+{
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    unsigned char *Zs = tc_smem, *Ws = tc_smem + TC_ROWS * HD * 4;
+    __shared__ __align__(8) uint64_t bar_w, bar_mma;
+    __shared__ uint32_t tmem_sh;
+    __shared__ int rowm[2][TC_ROWS];                        // this and the next tile: mask row (-1: none)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk, BW_W);
+    const uint32_t tmem = tmem_sh;
+    const int ntiles = (nodes + TILE_NODES - 1) / TILE_NODES;
+    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;
+    uint32_t phase = 0;
+    auto lookup = [&](int t, int buf) {
+        if (tid >= TC_ROWS) return;
+        const int k = tid / NODE_ROWS, n = t * TILE_NODES + k;
+        int v = -1;
+        if (k < TILE_NODES && n < nodes) {
+            const int b = n / N, s = out_tab[(n - b * N) * NODE_ROWS + tid - k * NODE_ROWS];
+            if (s >= 0) v = b * N * NODE_ROWS + s;
+        }
+        rowm[buf][tid] = v;
+    };
+    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
+    int buf = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int rg = (warp >> 1) + 4 * j, t = rowm[buf][rg * 8 + r8];
+            uint4 z = make_uint4(0u, 0u, 0u, 0u);
+            if (t >= 0)
+                z = mask_bf16x8(*reinterpret_cast<const uint4*>(dm + (size_t)(t / NODE_ROWS) * HD + kz * 8), mask_byte(mask, t, kz));
+            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
+        }
+        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (tid == 0) {
+            bwd_mma_input(tmem, Zs, Ws);
+            tc_commit(&bar_mma);
+        }
+        const bool ok = mbar_wait(&bar_mma, phase);
+        phase ^= 1u;
+        if (__syncthreads_or(!ok)) {
+            failed = true;
+            break;
+        }
+        tc_fence_after();
+        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row = q * 32 + lane;
+        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+            float d[16];
+            tmem_ld16(tl + 16 * hh, d);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                *reinterpret_cast<float4*>(Zs + row * 256 + ((((cb + 16 * hh) >> 2) + c) ^ (row & 7)) * 16) =
+                    make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
+        }
+        tc_fence_before();
+        __syncthreads();
+        for (int i = tid; i < TILE_NODES * (HD / 2); i += TC_THREADS) {
+            const int k = i >> 5, cp = i & 31, n = tile * TILE_NODES + k;
+            if (n >= nodes) break;
+            float x = 0.f, y = 0.f;
+#pragma unroll
+            for (int s = 0; s < NODE_ROWS; ++s) {
+                const int r = k * NODE_ROWS + s;
+                if (rowm[buf][r] < 0) continue;
+                const float2 v = *reinterpret_cast<const float2*>(Zs + r * 256 + (((cp >> 1) ^ (r & 7)) << 4) + (cp & 1) * 8);
+                x += v.x;
+                y += v.y;
             }
-        } else {
-#pragma unroll
-            for (int c0 = 0; c0 < HD; c0 += 16) {               // every lane holds the column sums
-                float d[16];
-                tmem_ld16(tl + HD + c0, d);
-                tmem_ld_wait();
-                if (in == 0)
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) P[HD * KIN + c0 + i] = d[i];
-            }
+            float2* p = reinterpret_cast<float2*>(dh + (size_t)n * HD) + cp;
+            float2 o = *p;
+            o.x += x;
+            o.y += y;
+            *p = o;
         }
     }
     tc_teardown(tmem, 128, failed, err);
+}
+
+// dW += sum over a map's CTA partials, db likewise, for all maps at once (blockIdx.y):
+// four interleaved sums added in a fixed order.
+struct WMaps {
+    float *dW[24], *db[24];
+    int n[24];                       // partials of the map
+};
+__global__ void wgrad_reduce_kernel(WMaps maps, size_t stride, const float* __restrict__ part)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+    if (i >= WPART) return;
+    const float* p = part + k * stride + i;
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    int b = 0;
+    for (; b + 4 <= maps.n[k]; b += 4)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[j] += p[(size_t)(b + j) * WPART];
+    for (int j = 0; b < maps.n[k]; ++b, ++j) s[j] += p[(size_t)b * WPART];
+    const float t = (s[0] + s[1]) + (s[2] + s[3]);
+    if (i < HD * KIN) maps.dW[k][i] += t;
+    else maps.db[k][i - HD * KIN] += t;
 }
 
 // Packs the BF16 matrix W [64 outputs][128 inputs] of every layer map into the
@@ -688,113 +1002,77 @@ __global__ void pack_weights_kernel(int nmat, const bf16* const* __restrict__ Ws
 }
 
 // ------------------------------------------------------- elementwise kernels
-// h0[b][n] = X[u_n]; e0[b][e] = Jt[idx(J)]
+// h0[b][n] = X[u_n]; e0[b][e] = Jt[idx(J)]; a thread converts 8 columns of a row
 __global__ void embed_kernel(int B, int N, int E, const int* __restrict__ u, const int8_t* __restrict__ J,
                              const float* __restrict__ Xemb, const float* __restrict__ Jemb, bf16* h, bf16* e)
 {
-    const size_t total = (size_t)B * (N + E) * HD;
+    const size_t nN = (size_t)B * N, total = (nN + (size_t)B * E) * (HD / 8);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t row = i / HD;
-        const int c = (int)(i % HD);
-        if (row < (size_t)B * N) {
-            const int n = (int)(row % N);
-            h[i] = __float2bfloat16_rn(Xemb[u[n] * HD + c]);
+        const size_t row = i / (HD / 8);
+        const int c = (int)(i % (HD / 8));
+        const float* src;
+        bf16* dst;
+        if (row < nN) {
+            src = Xemb + u[row % N] * HD;
+            dst = h + row * HD;
         } else {
-            const size_t re = row - (size_t)B * N;
-            const int j = J[re];
-            const int idx = j < 0 ? j + 3 : j + 2;          // -3,-2,-1,1,2,3 -> 0..5
-            e[re * HD + c] = __float2bfloat16_rn(Jemb[idx * HD + c]);
+            const int j = J[row - nN];
+            src = Jemb + (j < 0 ? j + 3 : j + 2) * HD;      // -3,-2,-1,1,2,3 -> 0..5
+            dst = e + (row - nN) * HD;
         }
+        const float4 a = reinterpret_cast<const float4*>(src)[2 * c], b = reinterpret_cast<const float4*>(src)[2 * c + 1];
+        reinterpret_cast<uint4*>(dst)[c] = make_uint4(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w), pack_bf2(b.x, b.y), pack_bf2(b.z, b.w));
     }
 }
 
-// m[b][n] = sum over the message rows into n of R (FP32 sum, BF16 result)
-__global__ void aggregate_kernel(int B, int N, int E, const int* __restrict__ in_rows, const float* __restrict__ R, bf16* m)
-{
-    const size_t total = (size_t)B * N * (HD / 2);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t bn = i / (HD / 2);
-        const int cp = (int)(i % (HD / 2));
-        const int b = (int)(bn / N), n = (int)(bn % N);
-        float x = 0.f, y = 0.f;
-        for (int s = 0; s < MAXDEG; ++s) {
-            const int r = in_rows[n * MAXDEG + s];
-            if (r < 0) continue;
-            const float2 v = reinterpret_cast<const float2*>(R + ((size_t)b * 2 * E + r) * HD)[cp];
-            x += v.x;
-            y += v.y;
-        }
-        reinterpret_cast<uint32_t*>(m + bn * HD)[cp] = pack_bf2(x, y);
-    }
-}
-
-// s[b][e] = h[b][ei] + h[b][ej]
-__global__ void endpoint_sum_kernel(int B, int N, int E, const int* __restrict__ ei, const int* __restrict__ ej,
-                                    const bf16* __restrict__ h, bf16* s)
-{
-    const size_t total = (size_t)B * E * (HD / 2);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t be = i / (HD / 2);
-        const int cp = (int)(i % (HD / 2));
-        const int b = (int)(be / E), e = (int)(be % E);
-        const float2 x = unpack_bf2(reinterpret_cast<const uint32_t*>(h + ((size_t)b * N + ei[e]) * HD)[cp]);
-        const float2 y = unpack_bf2(reinterpret_cast<const uint32_t*>(h + ((size_t)b * N + ej[e]) * HD)[cp]);
-        reinterpret_cast<uint32_t*>(s + be * HD)[cp] = pack_bf2(x.x + y.x, x.y + y.y);
-    }
-}
-
-// dZ[r] = G[gidx(r)] * (Z[r] > 0) as BF16.  gmap (optional) sends row r to
-// gradient row (r / R_local) * S + gmap[r % R_local].
-__global__ void relu_mask_kernel(int rows, const float* __restrict__ G, const int* __restrict__ gmap, int R_local, int S,
-                                 const bf16* __restrict__ Z, bf16* dZ)
-{
-    const size_t total = (size_t)rows * (HD / 2);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int r = (int)(i / (HD / 2)), cp = (int)(i % (HD / 2));
-        size_t gr = r;
-        if (gmap) gr = (size_t)(r / R_local) * S + gmap[r % R_local];
-        const float2 gv = reinterpret_cast<const float2*>(G + gr * HD)[cp];
-        const float2 z = unpack_bf2(reinterpret_cast<const uint32_t*>(Z + (size_t)r * HD)[cp]);
-        reinterpret_cast<uint32_t*>(dZ + (size_t)r * HD)[cp] = pack_bf2(z.x > 0.f ? gv.x : 0.f, z.y > 0.f ? gv.y : 0.f);
-    }
-}
-
-// out[b][n] += sum over list[n][0..5] (>= 0) of src[b][list][off..off+63] (src rows of width `w`)
-__global__ void gather_add_kernel(int B, int N, int Rsrc, const int* __restrict__ list, const float* __restrict__ src,
-                                  int w, int off, float* out)
-{
-    const size_t total = (size_t)B * N * HD;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t bn = i / HD;
-        const int c = (int)(i % HD);
-        const int b = (int)(bn / N), n = (int)(bn % N);
-        float acc = 0.f;
-        for (int s = 0; s < MAXDEG; ++s) {
-            const int r = list[n * MAXDEG + s];
-            if (r >= 0) acc += src[((size_t)b * Rsrc + r) * w + off + c];
-        }
-        out[i] += acc;
-    }
-}
-
-// readout forward + loss gradient (one block per graph, HD threads)
-__global__ void readout_kernel(int N, const bf16* __restrict__ h, const float* __restrict__ W1, const float* __restrict__ b1,
+// readout forward + loss gradient (one block of 256 threads per graph).  The node mean is
+// summed node by node (64 threads, a column each) from rows that the block stages 64 at a
+// time, the next 64 on their way meanwhile.
+constexpr int RO_ROWS = 64, RO_THREADS = 256;
+__global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* __restrict__ h, const float* __restrict__ W1, const float* __restrict__ b1,
                                const float* __restrict__ w2, const float* __restrict__ b2, float* y, float* gbuf,
                                float* zbuf, const float* __restrict__ target, float inv_B, float* dybuf,
                                float* sqbuf, float* dh)
 {
-    __shared__ float gs[HD], as[HD], red[HD], dz[HD];
-    const int b = blockIdx.x, c = threadIdx.x;
+    __shared__ __align__(16) float gs[HD];
+    __shared__ float as[HD], red[HD], dz[HD];
+    __shared__ __align__(16) bf16 rows[RO_ROWS][HD];
+    const int b = blockIdx.x, tid = threadIdx.x, c = tid;
+    const uint4* src = reinterpret_cast<const uint4*>(h + (size_t)b * N * HD);
+    constexpr int PER = RO_ROWS * HD / 8 / RO_THREADS;      // 16-byte pieces per thread
+    uint4 v[PER];
+    auto fetch = [&](int n0) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int i = tid + j * RO_THREADS;
+            v[j] = n0 + i / (HD / 8) < N ? src[(size_t)n0 * (HD / 8) + i] : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    fetch(0);
     float acc = 0.f;
-    for (int n = 0; n < N; ++n) acc += __bfloat162float(h[((size_t)b * N + n) * HD + c]);
-    gs[c] = acc / (float)N;
+    for (int n0 = 0; n0 < N; n0 += RO_ROWS) {
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PER; ++j) reinterpret_cast<uint4*>(&rows[0][0])[tid + j * RO_THREADS] = v[j];
+        __syncthreads();
+        if (n0 + RO_ROWS < N) fetch(n0 + RO_ROWS);
+        if (c < HD) {
+            const int m = min(RO_ROWS, N - n0);
+#pragma unroll 8
+            for (int n = 0; n < m; ++n) acc += __bfloat162float(rows[n][c]);
+        }
+    }
+    if (c < HD) gs[c] = acc / (float)N;
     __syncthreads();
-    float z = b1[c];
-    for (int k = 0; k < HD; ++k) z += W1[c * HD + k] * gs[k];
-    as[c] = fmaxf(z, 0.f);
-    red[c] = as[c] * w2[c];
-    gbuf[b * HD + c] = gs[c];
-    zbuf[b * HD + c] = z;
+    float z = 0.f;
+    if (c < HD) {
+        z = b1[c];
+        for (int k = 0; k < HD; ++k) z += W1[c * HD + k] * gs[k];
+        as[c] = fmaxf(z, 0.f);
+        red[c] = as[c] * w2[c];
+        gbuf[b * HD + c] = gs[c];
+        zbuf[b * HD + c] = z;
+    }
     __syncthreads();
     for (int s = HD / 2; s > 0; s >>= 1) {
         if (c < s) red[c] += red[c + s];
@@ -808,12 +1086,18 @@ __global__ void readout_kernel(int N, const bf16* __restrict__ h, const float* _
         dybuf[b] = dy;                             // over graphs by readout_grad_kernel)
         sqbuf[b] = (yb - target[b]) * (yb - target[b]) * inv_B;
     }
-    dz[c] = z > 0.f ? dy * w2[c] : 0.f;
+    if (c < HD) dz[c] = z > 0.f ? dy * w2[c] : 0.f;
     __syncthreads();
-    float dg = 0.f;
-    for (int o = 0; o < HD; ++o) dg += dz[o] * W1[o * HD + c];
-    dg /= (float)N;
-    for (int n = 0; n < N; ++n) dh[((size_t)b * N + n) * HD + c] = dg;
+    if (c < HD) {
+        float dg = 0.f;
+        for (int o = 0; o < HD; ++o) dg += dz[o] * W1[o * HD + c];
+        dg /= (float)N;
+        gs[c] = dg;
+    }
+    __syncthreads();
+    const float4 d = reinterpret_cast<const float4*>(gs)[tid & (HD / 4 - 1)];
+    float4* out = reinterpret_cast<float4*>(dh + (size_t)b * N * HD);
+    for (int i = tid; i < N * (HD / 4); i += RO_THREADS) out[i] = d;
 }
 
 // Readout parameter gradients and the loss, summed over the B graphs in graph
@@ -946,18 +1230,18 @@ struct sg_model {
     std::vector<int64_t> oWm, obm, oWu, obu, oWe, obe;
     // graph + activation buffers for the current (L, Bcap)
     int L = 0, N = 0, E = 0, Bcap = 0;
-    int *d_u = nullptr, *d_ei = nullptr, *d_ej = nullptr, *d_in_rows = nullptr, *d_out_rows = nullptr,
-        *d_inc = nullptr, *d_src = nullptr, *d_tgt = nullptr, *d_eid = nullptr, *d_iden = nullptr, *d_msg_edge = nullptr;
+    int *d_u = nullptr, *d_inc = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
+    int2 *d_ends = nullptr, *d_in_tab = nullptr, *d_msg_tab = nullptr;
     int8_t* d_J = nullptr;
     float *d_t = nullptr, *d_y = nullptr, *d_g = nullptr, *d_z = nullptr;
     float *d_dy = nullptr, *d_sq = nullptr;   // per graph: output gradient, loss term (readout)
     float* d_epart = nullptr;                 // embedding-gradient block partials [4 x SMs][8][64]
-    std::vector<bf16*> h, e, m, s, zm, zu, ze;
-    float *R = nullptr, *dX = nullptr, *dh = nullptr, *dh2 = nullptr, *de = nullptr, *dm = nullptr, *ds = nullptr;
-    bf16* dZ = nullptr;
-    float* wpart = nullptr;       // weight-gradient partials, one WPART block per persistent CTA
-    float* wred = nullptr;        // [WRED_GROUPS][WPART] group sums of the partials
-    int wblocks = 0;              // persistent CTAs of the weight-gradient kernel
+    std::vector<bf16*> h, e, m;
+    std::vector<uint2*> mm, mu, me;   // per layer: sign bits of the message, node and edge pre-activations
+    float *dh = nullptr, *de = nullptr, *ds = nullptr;
+    bf16* dm = nullptr;
+    float* wpart = nullptr;       // weight-gradient partials: [3 layers maps][wcap CTAs][WPART]
+    int wcap = 0;
     uint64_t launches = 0;
     std::string err = "no error";
 };
@@ -987,21 +1271,30 @@ cudaError_t salloc(T** p, size_t n)
 
 void free_graph(sg_model* M)
 {
-    int** ints[] = {&M->d_u, &M->d_ei, &M->d_ej, &M->d_in_rows, &M->d_out_rows, &M->d_inc, &M->d_src, &M->d_tgt,
-                    &M->d_eid, &M->d_iden, &M->d_msg_edge};
-    for (int** p : ints) { cudaFree(*p); *p = nullptr; }
+    cudaFree(M->d_u); cudaFree(M->d_inc); cudaFree(M->d_out_tab);
+    cudaFree(M->d_ends); cudaFree(M->d_in_tab); cudaFree(M->d_msg_tab);
+    M->d_u = M->d_inc = M->d_out_tab = nullptr;
+    M->d_ends = M->d_in_tab = M->d_msg_tab = nullptr;
     cudaFree(M->d_J); M->d_J = nullptr;
-    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_epart, &M->R, &M->dX, &M->dh,
-                    &M->dh2, &M->de, &M->dm, &M->ds};
+    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_epart, &M->dh, &M->de, &M->ds, &M->wpart};
     for (float** p : fl) { cudaFree(*p); *p = nullptr; }
-    cudaFree(M->dZ); M->dZ = nullptr;
-    cudaFree(M->wpart); M->wpart = nullptr;
-    cudaFree(M->wred); M->wred = nullptr;
-    for (auto* v : {&M->h, &M->e, &M->m, &M->s, &M->zm, &M->zu, &M->ze}) {
+    cudaFree(M->dm); M->dm = nullptr;
+    for (auto* v : {&M->h, &M->e, &M->m}) {
         for (bf16* p : *v) cudaFree(p);
         v->clear();
     }
+    for (auto* v : {&M->mm, &M->mu, &M->me}) {
+        for (uint2* p : *v) cudaFree(p);
+        v->clear();
+    }
     M->L = M->Bcap = 0;
+}
+
+// Persistent CTAs for `rows` rows in tiles of `per` at ctas_per_sm residents.
+int tc_grid(const sg_model* M, int rows, int ctas_per_sm, int per = TC_ROWS)
+{
+    const int tiles = (rows + per - 1) / per, cap = ctas_per_sm * M->sms;
+    return tiles < cap ? (tiles > 0 ? tiles : 1) : cap;
 }
 
 // Builds the Chimera C_L topology in the coupler order of pt.h and sizes the
@@ -1023,40 +1316,36 @@ int prepare(sg_model* M, int L, int B)
     for (int r = 0; r < L; ++r)
         for (int c = 0; c + 1 < L; ++c)
             for (int k = 0; k < 4; ++k) { ei.push_back(idx(r, c, 1, k)); ej.push_back(idx(r, c + 1, 1, k)); }
-    // message row 2e: source ej -> target ei; row 2e+1: source ei -> target ej
-    std::vector<int> u(N), src(2 * E), tgt(2 * E), eid(2 * E), iden(std::max(N, 2 * E));
-    std::vector<int> in_rows(N * MAXDEG, -1), out_rows(N * MAXDEG, -1), inc(N * MAXDEG, -1);
+    // message row 2e: source ej -> target ei; row 2e+1: source ei -> target ej.  A node's incoming and
+    // outgoing rows and its edges fill its 6 slots in ascending order
+    std::vector<int> u(N), inc(N * MAXDEG, -1), out_tab(N * MAXDEG, -1);
+    std::vector<int2> ends(E), in_tab(N * MAXDEG, make_int2(-1, -1)), msg_tab(2 * E);
     std::vector<int> cin(N, 0), cout(N, 0), cinc(N, 0);
     for (int i = 0; i < N; ++i) u[i] = (i >> 2) & 1;
-    for (int q = 0; q < (int)iden.size(); ++q) iden[q] = q;
     for (int e2 = 0; e2 < E; ++e2) {
-        src[2 * e2] = ej[e2]; tgt[2 * e2] = ei[e2];
-        src[2 * e2 + 1] = ei[e2]; tgt[2 * e2 + 1] = ej[e2];
-        eid[2 * e2] = eid[2 * e2 + 1] = e2;
+        ends[e2] = make_int2(ei[e2], ej[e2]);
         for (int d = 0; d < 2; ++d) {
-            const int r = 2 * e2 + d;
-            in_rows[tgt[r] * MAXDEG + cin[tgt[r]]++] = r;
-            out_rows[src[r] * MAXDEG + cout[src[r]]++] = r;
+            const int src = d == 0 ? ej[e2] : ei[e2], tgt = d == 0 ? ei[e2] : ej[e2];
+            const int slot = tgt * MAXDEG + cin[tgt]++;
+            in_tab[slot] = make_int2(src, e2);
+            msg_tab[2 * e2 + d] = make_int2(src, slot);
+            out_tab[src * MAXDEG + cout[src]++] = slot;
         }
         inc[ei[e2] * MAXDEG + cinc[ei[e2]]++] = e2;
         inc[ej[e2] * MAXDEG + cinc[ej[e2]]++] = e2;
     }
-    auto up = [&](int** d, const std::vector<int>& v) -> cudaError_t {
+    auto up = [&](auto** d, const auto& v) -> cudaError_t {
         cudaError_t r = salloc(d, v.size());
         if (r != cudaSuccess) return r;
-        return cudaMemcpy(*d, v.data(), 4 * v.size(), cudaMemcpyHostToDevice);
+        return cudaMemcpy(*d, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
     };
     SK(up(&M->d_u, u), "upload topology");
-    SK(up(&M->d_ei, ei), "upload topology");
-    SK(up(&M->d_ej, ej), "upload topology");
-    SK(up(&M->d_in_rows, in_rows), "upload topology");
-    SK(up(&M->d_out_rows, out_rows), "upload topology");
     SK(up(&M->d_inc, inc), "upload topology");
-    SK(up(&M->d_src, src), "upload topology");
-    SK(up(&M->d_tgt, tgt), "upload topology");
-    SK(up(&M->d_eid, eid), "upload topology");
-    SK(up(&M->d_iden, iden), "upload topology");
-    const size_t nN = (size_t)B * N, nE = (size_t)B * E, nM = 2 * nE;
+    SK(up(&M->d_out_tab, out_tab), "upload topology");
+    SK(up(&M->d_ends, ends), "upload topology");
+    SK(up(&M->d_in_tab, in_tab), "upload topology");
+    SK(up(&M->d_msg_tab, msg_tab), "upload topology");
+    const size_t nN = (size_t)B * N, nE = (size_t)B * E;
     SK(salloc(&M->d_J, nE), "cudaMalloc J");
     SK(salloc(&M->d_t, (size_t)B), "cudaMalloc t");
     SK(salloc(&M->d_y, (size_t)B), "cudaMalloc y");
@@ -1066,48 +1355,24 @@ int prepare(sg_model* M, int L, int B)
     SK(salloc(&M->d_sq, (size_t)B), "cudaMalloc sq");
     SK(salloc(&M->d_epart, (size_t)4 * M->sms * 8 * HD), "cudaMalloc embedding partials");
     M->h.assign(M->layers + 1, nullptr);
-    M->e.assign(M->layers + 1, nullptr);
-    M->m.assign(M->layers, nullptr);
-    M->s.assign(M->layers, nullptr);
-    M->zm.assign(M->layers, nullptr);
-    M->zu.assign(M->layers, nullptr);
-    M->ze.assign(M->layers, nullptr);
-    for (int l = 0; l <= M->layers; ++l) {
-        SK(salloc(&M->h[l], nN * HD), "cudaMalloc h");
-        SK(salloc(&M->e[l], nE * HD), "cudaMalloc e");
-    }
+    for (auto* v : {&M->e, &M->m}) v->assign(M->layers, nullptr);
+    for (auto* v : {&M->mm, &M->mu, &M->me}) v->assign(M->layers, nullptr);
+    for (int l = 0; l <= M->layers; ++l) SK(salloc(&M->h[l], nN * HD), "cudaMalloc h");
     for (int l = 0; l < M->layers; ++l) {
+        SK(salloc(&M->e[l], nE * HD), "cudaMalloc e");
         SK(salloc(&M->m[l], nN * HD), "cudaMalloc m");
-        SK(salloc(&M->s[l], nE * HD), "cudaMalloc s");
-        SK(salloc(&M->zm[l], nM * HD), "cudaMalloc zm");
-        SK(salloc(&M->zu[l], nN * HD), "cudaMalloc zu");
-        SK(salloc(&M->ze[l], nE * HD), "cudaMalloc ze");
+        SK(salloc(&M->mm[l], nN * MAXDEG), "cudaMalloc message mask");
+        SK(salloc(&M->mu[l], nN), "cudaMalloc node mask");
+        if (l + 1 < M->layers) SK(salloc(&M->me[l], nE), "cudaMalloc edge mask");
     }
-    SK(salloc(&M->R, nM * HD), "cudaMalloc R");
-    SK(salloc(&M->dX, nM * HD), "cudaMalloc dX");           // message rows' node half of the input gradient
-    SK(salloc(&M->dZ, nM * HD), "cudaMalloc dZ");
-    {
-        int dev = 0, sms = 0;
-        SK(cudaGetDevice(&dev), "cudaGetDevice");
-        SK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
-        M->wblocks = TC_CTAS_WGRAD * sms;     // persistent weight-gradient CTAs
-        SK(salloc(&M->wpart, (size_t)M->wblocks * WPART), "cudaMalloc wpart");
-        SK(salloc(&M->wred, (size_t)WRED_GROUPS * WPART), "cudaMalloc wred");
-    }
+    M->wcap = tc_grid(M, B * 2 * E, TC_CTAS_UPD_BWD > TC_CTAS_EDGE_BWD ? TC_CTAS_UPD_BWD : TC_CTAS_EDGE_BWD);
+    SK(salloc(&M->wpart, (size_t)3 * M->layers * M->wcap * WPART), "cudaMalloc wpart");
     SK(salloc(&M->dh, nN * HD), "cudaMalloc dh");
-    SK(salloc(&M->dh2, nN * HD), "cudaMalloc dh2");
     SK(salloc(&M->dm, nN * HD), "cudaMalloc dm");
     SK(salloc(&M->de, nE * HD), "cudaMalloc de");
     SK(salloc(&M->ds, nE * HD), "cudaMalloc ds");
     M->L = L; M->N = N; M->E = E; M->Bcap = B;
     return PT_OK;
-}
-
-RowSrc rows_of(const bf16* P0, const int* map0, int S0, const bf16* P1, const int* map1, int S1, int R_local)
-{
-    RowSrc r;
-    r.P0 = P0; r.map0 = map0; r.S0 = S0; r.P1 = P1; r.map1 = map1; r.S1 = S1; r.R_local = R_local;
-    return r;
 }
 
 // The tcgen05 operand copies of every layer matrix follow the BF16 weights.
@@ -1122,48 +1387,28 @@ void pack_weights(sg_model* M)
 const bf16* wpk_fwd(const sg_model* M, int l, int which) { return M->wpk + ((size_t)(l * 3 + which) * 2) * HD * KIN; }
 const bf16* wpk_bwd(const sg_model* M, int l, int which) { return wpk_fwd(M, l, which) + HD * KIN; }
 
-int tc_grid(const sg_model* M, int rows, int ctas_per_sm)
-{
-    const int tiles = (rows + TC_ROWS - 1) / TC_ROWS, cap = ctas_per_sm * M->sms;
-    return tiles < cap ? (tiles > 0 ? tiles : 1) : cap;
-}
-
-
-// dW += dZ^T X, db += column sums of dZ over `rows` rows (two launches).
-void lin_wgrad(sg_model* M, int rows, const RowSrc& src, float* dW, float* db)
-{
-    const int nchunks = (rows + TC_WCH - 1) / TC_WCH;
-    const int grid = nchunks < M->wblocks ? (nchunks > 0 ? nchunks : 1) : M->wblocks;
-    lin_wgrad_tc_kernel<<<grid, TC_THREADS, TC_SMEM_WGRAD, M->stream>>>(rows, M->dZ, src, M->wpart, M->d_err);
-    lin_wgrad_reduce1<<<dim3((WPART + 255) / 256, WRED_GROUPS), 256, 0, M->stream>>>(grid, M->wpart, M->wred);
-    lin_wgrad_reduce2<<<(WPART + 255) / 256, 256, 0, M->stream>>>(M->wred, dW, db);
-}
-
-int forward(sg_model* M, int B, bool train)
+// The last layer updates no edges: nothing after it reads them.
+void forward(sg_model* M, int B, bool train)
 {
     const int N = M->N, E = M->E;
     cudaStream_t st = M->stream;
-    embed_kernel<<<grid_for((size_t)B * (N + E) * HD), 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->theta + M->oX,
-                                                                       M->theta + M->oJ, M->h[0], M->e[0]);
+    embed_kernel<<<grid_for((size_t)B * (N + E) * (HD / 8)), 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->theta + M->oX,
+                                                                             M->theta + M->oJ, M->h[0], M->e[0]);
     M->launches++;
     for (int l = 0; l < M->layers; ++l) {
-        // messages: row 2e / 2e+1 of every graph: [h[src] | e[edge]]
-        const RowSrc ms = rows_of(M->h[l], M->d_src, N, M->e[l], M->d_eid, E, 2 * E);
-        lin_fwd_tc_kernel<0><<<tc_grid(M, B * 2 * E, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(B * 2 * E, ms, wpk_fwd(M, l, 0),
-                                                                           M->theta + M->obm[l], M->zm[l], M->R,
-                                                                           nullptr, M->d_err);
-        aggregate_kernel<<<grid_for((size_t)B * N * HD / 2), 256, 0, st>>>(B, N, E, M->d_in_rows, M->R, M->m[l]);
-        const RowSrc ns = rows_of(M->h[l], M->d_iden, N, M->m[l], M->d_iden, N, N);
-        lin_fwd_tc_kernel<1><<<tc_grid(M, B * N, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(B * N, ns, wpk_fwd(M, l, 1), M->theta + M->obu[l],
-                                                                       M->zu[l], nullptr, M->h[l + 1], M->d_err);
-        endpoint_sum_kernel<<<grid_for((size_t)B * E * HD / 2), 256, 0, st>>>(B, N, E, M->d_ei, M->d_ej, M->h[l + 1], M->s[l]);
-        const RowSrc es = rows_of(M->e[l], M->d_iden, E, M->s[l], M->d_iden, E, E);
-        lin_fwd_tc_kernel<1><<<tc_grid(M, B * E, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(B * E, es, wpk_fwd(M, l, 2), M->theta + M->obe[l],
-                                                                       M->ze[l], nullptr, M->e[l + 1], M->d_err);
-        M->launches += 5;
+        msg_fwd_kernel<<<tc_grid(M, B * N, TC_CTAS_FWD, TILE_NODES), TC_THREADS, TC_SMEM_FWD, st>>>(
+            B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], M->m[l], train ? M->mm[l] : nullptr,
+            M->d_err);
+        upd_fwd_kernel<false><<<tc_grid(M, B * N, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(
+            B * N, M->h[l], M->m[l], nullptr, N, E, wpk_fwd(M, l, 1), M->theta + M->obu[l], M->h[l + 1], train ? M->mu[l] : nullptr,
+            M->d_err);
+        M->launches += 2;
+        if (l + 1 == M->layers) break;
+        upd_fwd_kernel<true><<<tc_grid(M, B * E, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(
+            B * E, M->e[l], M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
+            train ? M->me[l] : nullptr, M->d_err);
+        M->launches++;
     }
-    (void)train;
-    return PT_OK;
 }
 
 // Gradient of the mean squared error into M->grad (zeroed first); loss into M->dloss.
@@ -1174,44 +1419,46 @@ int backward_all(sg_model* M, int B)
     float* G = M->grad;
     SK(cudaMemsetAsync(G, 0, sizeof(float) * M->nparams, st), "zero grad");
     SK(cudaMemsetAsync(M->dloss, 0, sizeof(float), st), "zero loss");
-    SK(cudaMemsetAsync(M->de, 0, sizeof(float) * (size_t)B * E * HD, st), "zero de");
-    readout_kernel<<<B, HD, 0, st>>>(N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1, M->theta + M->ow2,
-                                     M->theta + M->ob2, M->d_y, M->d_g, M->d_z, M->d_t, 1.f / (float)B, M->d_dy,
-                                     M->d_sq, M->dh);
+    readout_kernel<<<B, RO_THREADS, 0, st>>>(N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1, M->theta + M->ow2,
+                                             M->theta + M->ob2, M->d_y, M->d_g, M->d_z, M->d_t, 1.f / (float)B, M->d_dy,
+                                             M->d_sq, M->dh);
     readout_grad_kernel<<<HD + 1, HD, 0, st>>>(B, M->d_g, M->d_z, M->d_dy, M->d_sq, M->theta + M->ow2, M->dloss,
                                                G + M->oW1, G + M->ob1, G + M->ow2, G + M->ob2);
     M->launches += 2;
-    const size_t nN = (size_t)B * N, nE = (size_t)B * E;
+    WMaps maps;
+    int nmaps = 0;
+    const size_t stride = (size_t)M->wcap * WPART;
+    auto map = [&](int64_t oW, int64_t ob, int n) {      // the next map's partials
+        maps.dW[nmaps] = G + oW;
+        maps.db[nmaps] = G + ob;
+        maps.n[nmaps] = n;
+        return M->wpart + stride * nmaps++;
+    };
     for (int l = M->layers - 1; l >= 0; --l) {
-        // edge update: e' = e + relu(ze), ze = We [e | s] + be
-        relu_mask_kernel<<<grid_for(nE * HD / 2), 256, 0, st>>>(B * E, M->de, nullptr, 1, 1, M->ze[l], M->dZ);
-        // de += dX[:, :64] (into e), ds = dX[:, 64:]
-        lin_bwd_input_tc_kernel<1><<<tc_grid(M, B * E, TC_CTAS_BWD), TC_THREADS, TC_SMEM_BWD, st>>>(B * E, M->dZ, wpk_bwd(M, l, 2), nullptr,
-                                                                             M->de, M->de, M->ds, M->d_err);
-        const RowSrc es = rows_of(M->e[l], M->d_iden, E, M->s[l], M->d_iden, E, E);
-        lin_wgrad(M, B * E, es, G + M->oWe[l], G + M->obe[l]);
-        SK(cudaMemcpyAsync(M->dh2, M->dh, sizeof(float) * nN * HD, cudaMemcpyDeviceToDevice, st), "copy dh");
-        gather_add_kernel<<<grid_for(nN * HD), 256, 0, st>>>(B, N, E, M->d_inc, M->ds, HD, 0, M->dh2);
-        // node update: h' = h + relu(zu), zu = Wu [h | m] + bu
-        relu_mask_kernel<<<grid_for(nN * HD / 2), 256, 0, st>>>(B * N, M->dh2, nullptr, 1, 1, M->zu[l], M->dZ);
-        // dh = dh2 + dX[:, :64] (into h), dm = dX[:, 64:]
-        lin_bwd_input_tc_kernel<1><<<tc_grid(M, B * N, TC_CTAS_BWD), TC_THREADS, TC_SMEM_BWD, st>>>(B * N, M->dZ, wpk_bwd(M, l, 1), nullptr,
-                                                                             M->dh2, M->dh, M->dm, M->d_err);
-        const RowSrc ns = rows_of(M->h[l], M->d_iden, N, M->m[l], M->d_iden, N, N);
-        lin_wgrad(M, B * N, ns, G + M->oWu[l], G + M->obu[l]);
-        // messages: m_i = sum relu(zm) over rows into i
-        relu_mask_kernel<<<grid_for(nE * 2 * HD / 2), 256, 0, st>>>(B * 2 * E, M->dm, M->d_tgt, 2 * E, N, M->zm[l], M->dZ);
-        lin_bwd_input_tc_kernel<0><<<tc_grid(M, B * 2 * E, TC_CTAS_BWD), TC_THREADS, TC_SMEM_BWD, st>>>(B * 2 * E, M->dZ, wpk_bwd(M, l, 0),
-                                                                                 M->dX, nullptr, nullptr, M->de,
-                                                                                 M->d_err);
-        const RowSrc ms = rows_of(M->h[l], M->d_src, N, M->e[l], M->d_eid, E, 2 * E);
-        lin_wgrad(M, B * 2 * E, ms, G + M->oWm[l], G + M->obm[l]);
-        gather_add_kernel<<<grid_for(nN * HD), 256, 0, st>>>(B, N, 2 * E, M->d_out_rows, M->dX, HD, 0, M->dh);
-        M->launches += 17;
+        const bool last = l + 1 == M->layers;             // its edge update has no gradient
+        if (!last) {
+            const int g = tc_grid(M, B * E, TC_CTAS_UPD_BWD);
+            upd_bwd_kernel<true><<<g, TC_THREADS, TC_SMEM_UPD_BWD, st>>>(B * E, N, E, M->me[l], M->de, M->e[l], M->h[l + 1],
+                                                                         M->d_ends, nullptr, M->ds, nullptr, wpk_bwd(M, l, 2),
+                                                                         map(M->oWe[l], M->obe[l], g), M->d_err);
+            M->launches++;
+        }
+        int g = tc_grid(M, B * N, TC_CTAS_UPD_BWD);
+        upd_bwd_kernel<false><<<g, TC_THREADS, TC_SMEM_UPD_BWD, st>>>(B * N, N, E, M->mu[l], M->dh, M->h[l], M->m[l], nullptr,
+                                                                      last ? nullptr : M->d_inc, M->ds, M->dm, wpk_bwd(M, l, 1),
+                                                                      map(M->oWu[l], M->obu[l], g), M->d_err);
+        g = tc_grid(M, B * 2 * E, TC_CTAS_EDGE_BWD);
+        msg_bwd_edge_kernel<<<g, TC_THREADS, TC_SMEM_EDGE_BWD, st>>>(B * 2 * E, N, E, M->d_msg_tab, M->mm[l], M->dm, M->h[l],
+                                                                     M->e[l], wpk_bwd(M, l, 0), M->de, last ? 1 : 0,
+                                                                     map(M->oWm[l], M->obm[l], g), M->d_err);
+        msg_bwd_node_kernel<<<tc_grid(M, B * N, TC_CTAS_NODE_BWD, TILE_NODES), TC_THREADS, TC_SMEM_NODE_BWD, st>>>(
+            B * N, N, M->d_out_tab, M->mm[l], M->dm, wpk_bwd(M, l, 0), M->dh, M->d_err);
+        M->launches += 3;
     }
+    wgrad_reduce_kernel<<<dim3((WPART + 255) / 256, nmaps), 256, 0, st>>>(maps, stride, M->wpart);
     embed_bwd_kernel<<<4 * M->sms, 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->dh, M->de, M->d_epart);
     embed_bwd_reduce<<<(8 * HD + 255) / 256, 256, 0, st>>>(4 * M->sms, M->d_epart, G + M->oX, G + M->oJ);
-    M->launches += 2;
+    M->launches += 3;
     return PT_OK;
 }
 
@@ -1230,8 +1477,9 @@ int load_batch(sg_model* M, int L, int B, const int8_t* J, const float* t)
 {
     if (L < 1 || L > ptg::MAX_L || B < 1 || B > 4096 || !J) return sfail(M, PT_ERR_ARG, "need 1 <= L <= 16, 1 <= B <= 4096");
     const int E = 16 * L * L + 8 * L * (L - 1);
-    for (size_t i = 0; i < (size_t)B * E; ++i)
-        if (J[i] == 0 || J[i] < -3 || J[i] > 3) return sfail(M, PT_ERR_ARG, "surrogate couplers must be in {+-1, +-2, +-3}");
+    unsigned bad = 0u;                                // no early exit: the compiler vectorises the scan
+    for (size_t i = 0; i < (size_t)B * E; ++i) bad |= (unsigned)(J[i] == 0) | (unsigned)(J[i] < -3) | (unsigned)(J[i] > 3);
+    if (bad) return sfail(M, PT_ERR_ARG, "surrogate couplers must be in {+-1, +-2, +-3}");
     int rc = prepare(M, L, B);
     if (rc) return rc;
     SK(cudaMemcpyAsync(M->d_J, J, (size_t)B * E, cudaMemcpyHostToDevice, M->stream), "upload J");
@@ -1305,12 +1553,16 @@ int sg_create(sg_model** out, int32_t hidden, int32_t layers, void* stream)
         if (e == cudaSuccess) e = cudaMemset(M->d_err, 0, sizeof(int));
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const void* tk[5] = {(const void*)lin_fwd_tc_kernel<0>, (const void*)lin_fwd_tc_kernel<1>,
-                             (const void*)lin_bwd_input_tc_kernel<0>, (const void*)lin_bwd_input_tc_kernel<1>,
-                             (const void*)lin_wgrad_tc_kernel};
-        const int sm_bytes[5] = {TC_SMEM_FWD, TC_SMEM_FWD, TC_SMEM_BWD, TC_SMEM_BWD, TC_SMEM_WGRAD};
-        for (int q = 0; q < 5; ++q)
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(tk[q], cudaFuncAttributeMaxDynamicSharedMemorySize, sm_bytes[q]);
+        const struct { const void* k; int smem; } tk[] = {
+            {(const void*)msg_fwd_kernel, TC_SMEM_FWD},
+            {(const void*)upd_fwd_kernel<false>, TC_SMEM_FWD},
+            {(const void*)upd_fwd_kernel<true>, TC_SMEM_FWD},
+            {(const void*)upd_bwd_kernel<false>, TC_SMEM_UPD_BWD},
+            {(const void*)upd_bwd_kernel<true>, TC_SMEM_UPD_BWD},
+            {(const void*)msg_bwd_edge_kernel, TC_SMEM_EDGE_BWD},
+            {(const void*)msg_bwd_node_kernel, TC_SMEM_NODE_BWD}};
+        for (const auto& t : tk)
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(t.k, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem);
         if (e != cudaSuccess) {
             M->err = std::string("tensor-core set-up: ") + cudaGetErrorString(e);
             return bail(PT_ERR_CUDA);
@@ -1361,8 +1613,8 @@ int sg_forward(sg_model* M, int32_t L, int32_t B, const int8_t* J, float* y)
     if (!M || !y) return sfail(M, PT_ERR_ARG, "NULL argument");
     int rc = load_batch(M, L, B, J, nullptr);
     if (rc) return rc;
-    if ((rc = forward(M, B, false))) return rc;
-    readout_kernel<<<B, HD, 0, M->stream>>>(M->N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1,
+    forward(M, B, false);
+    readout_kernel<<<B, RO_THREADS, 0, M->stream>>>(M->N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1,
                                             M->theta + M->ow2, M->theta + M->ob2, M->d_y, M->d_g, M->d_z, nullptr,
                                             0.f, nullptr, nullptr, nullptr);
     M->launches++;
@@ -1379,7 +1631,7 @@ int sg_grad(sg_model* M, int32_t L, int32_t B, const int8_t* J, const float* t, 
     if (!M || !t) return sfail(M, PT_ERR_ARG, "NULL argument");
     int rc = load_batch(M, L, B, J, t);
     if (rc) return rc;
-    if ((rc = forward(M, B, true))) return rc;
+    forward(M, B, true);
     if ((rc = backward_all(M, B))) return rc;
     SK(cudaGetLastError(), "gradient kernels");
     if (grad) SK(cudaMemcpyAsync(grad, M->grad, sizeof(float) * M->nparams, cudaMemcpyDeviceToHost, M->stream), "download grad");
