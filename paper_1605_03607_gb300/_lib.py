@@ -271,12 +271,12 @@ class PTHandle:
         _check(load().pt_exchange(self.h), self.h)
 
     def state(self):
-        spins = np.zeros((self.R, self.NT, self.N), np.int8)
-        E = np.zeros((self.R, self.NT), np.int32)
-        perm = np.zeros((self.R, self.NT), np.uint8)
-        best = np.zeros(self.R, np.int32)
-        first = np.zeros(self.R, np.int32)
-        macc = np.zeros((self.R, self.NT), np.uint64)
+        spins = np.empty((self.R, self.NT, self.N), np.int8)
+        E = np.empty((self.R, self.NT), np.int32)
+        perm = np.empty((self.R, self.NT), np.uint8)
+        best = np.empty(self.R, np.int32)
+        first = np.empty(self.R, np.int32)
+        macc = np.empty((self.R, self.NT), np.uint64)
         xacc = np.zeros((self.R, max(self.NT - 1, 1)), np.uint64)
         sweep = np.zeros(1, np.uint64)
         _check(load().pt_get_state(self.h, _ptr(spins), _ptr(E), _ptr(perm), _ptr(best), _ptr(first),

@@ -27,12 +27,17 @@ using namespace ptg;
 
 namespace {
 
+constexpr size_t STAGE_MAX = 256 * 1024;     // pinned bytes a handle keeps for state downloads
+
 std::mutex g_err_mu;
 std::string g_create_err = "no error";
 
 // A set of instances of one shape (L, NT, R) sharing one ladder.
 struct Group {
     int L = 0, NT = 0, R = 0, n_inst = 0;
+    // the runs' state is one allocation: spins first, the records from rec_off on
+    uint8_t* block = nullptr;
+    size_t rec_off = 0, block_bytes = 0;
     int8_t* spins = nullptr;
     int32_t* E = nullptr;
     uint8_t* perm = nullptr;
@@ -48,7 +53,7 @@ struct Group {
     int* d_queue = nullptr;
     std::vector<InstDesc> desc;
     std::vector<Bundle> bundles;
-    int block = 0, smem = 0, team = 0;
+    int threads = 0, smem = 0, team = 0;
     uint64_t sweep = 0;
     // temperature random walk (main group only, when tracked)
     bool walk = false;
@@ -75,6 +80,8 @@ struct pt_handle {
     float* d_xhint = nullptr;
     int16_t* d_nbr = nullptr;
     Group main, cand;
+    uint8_t* stage = nullptr;  // pinned staging of state downloads
+    size_t stage_bytes = 0;
     int sp = 0, ipc = 0, spl = 4096;
     int team = 0;              // 0: cell-major mapping; > 0: slot-major with teams of this size
     bool planned = true;       // until a schedule is set: the replica-lane mapping, shaped by lane_plan
@@ -171,8 +178,7 @@ cudaError_t dalloc(T** p, size_t n)
 
 void free_group(Group& g)
 {
-    cudaFree(g.spins); cudaFree(g.E); cudaFree(g.perm); cudaFree(g.best); cudaFree(g.first);
-    cudaFree(g.macc); cudaFree(g.xacc); cudaFree(g.jw); cudaFree(g.d_desc); cudaFree(g.d_items);
+    cudaFree(g.block); cudaFree(g.jw); cudaFree(g.d_desc); cudaFree(g.d_items);
     cudaFree(g.d_bundles); cudaFree(g.d_sub); cudaFree(g.d_tts); cudaFree(g.d_queue);
     cudaFree(g.whot); cudaFree(g.wtrips); cudaFree(g.wstate); cudaFree(g.d_targets);
     g = Group();
@@ -224,13 +230,20 @@ int group_alloc(pt_handle* h, Group& g, int n_inst)
     const size_t reps = (size_t)n_inst * h->R * h->NT;
     const size_t runs = (size_t)n_inst * h->R;
     const size_t npair = (size_t)(h->NT > 1 ? h->NT - 1 : 1);
-    CK(dalloc(&g.spins, reps * h->N), "cudaMalloc spins");
-    CK(dalloc(&g.E, reps), "cudaMalloc E");
-    CK(dalloc(&g.perm, reps), "cudaMalloc perm");
-    CK(dalloc(&g.best, runs), "cudaMalloc best");
-    CK(dalloc(&g.first, runs), "cudaMalloc first");
-    CK(dalloc(&g.macc, reps), "cudaMalloc macc");
-    CK(dalloc(&g.xacc, runs * npair), "cudaMalloc xacc");
+    size_t off = 0;
+    auto take = [&](size_t bytes) { const size_t at = off; off = (off + bytes + 255) & ~(size_t)255; return at; };
+    const size_t o_spins = take(reps * h->N), o_E = take(4 * reps), o_perm = take(reps), o_best = take(4 * runs),
+                 o_first = take(4 * runs), o_macc = take(8 * reps), o_xacc = take(8 * runs * npair);
+    CK(dalloc(&g.block, off), "cudaMalloc state");
+    g.rec_off = o_E;
+    g.block_bytes = off;
+    g.spins = reinterpret_cast<int8_t*>(g.block + o_spins);
+    g.E = reinterpret_cast<int32_t*>(g.block + o_E);
+    g.perm = g.block + o_perm;
+    g.best = reinterpret_cast<int32_t*>(g.block + o_best);
+    g.first = reinterpret_cast<int32_t*>(g.block + o_first);
+    g.macc = reinterpret_cast<unsigned long long*>(g.block + o_macc);
+    g.xacc = reinterpret_cast<unsigned long long*>(g.block + o_xacc);
     CK(dalloc(&g.jw, (size_t)n_inst * h->L * h->L * 16), "cudaMalloc jw");
     CK(dalloc(&g.d_desc, (size_t)n_inst), "cudaMalloc desc");
     CK(dalloc(&g.d_items, runs), "cudaMalloc items");
@@ -305,7 +318,7 @@ int group_schedule(pt_handle* h, Group& g)
     g.d_sub = dsub;               // room for any subset of the full list
     g.d_bundles = d;
     g.bundles.swap(bundles);
-    g.block = block;
+    g.threads = block;
     g.smem = smem;
     g.team = team;
     return PT_OK;
@@ -376,7 +389,7 @@ int group_sweeps(pt_handle* h, Group& g, int64_t n, int xevery, const Bundle* ds
     while (done < n) {
         const int chunk = (int)std::min<int64_t>(h->spl, n - done);
         if (h->timing) CK(cudaEventRecord(h->ev[2 * li], h->stream), "event");
-        CK(launch_sweeps(g.d_desc, db, nb, nb, g.block, g.smem, (uint32_t)g.sweep, chunk, xevery, 0, nullptr,
+        CK(launch_sweeps(g.d_desc, db, nb, nb, g.threads, g.smem, (uint32_t)g.sweep, chunk, xevery, 0, nullptr,
                          h->stream, g.team, g.walk, g.L),
            "sweep kernel");
         if (g.walk && g.NT > 1 && xevery > 0)
@@ -889,6 +902,12 @@ int pt_create(pt_handle** out, int32_t L, const int8_t* J, int32_t n_edges, cons
     CKC(cudaMemcpy(h->d_nbr, nbr.data(), 2 * nbr.size(), cudaMemcpyHostToDevice), "upload nbr");
     default_schedule(L, n_temps, n_runs, h->sp, h->ipc, h->kt);
     if ((rc = group_alloc(h, h->main, 1))) return bail(rc);
+    h->stage_bytes = std::min<size_t>(h->main.block_bytes, STAGE_MAX);
+    if (cudaMallocHost(reinterpret_cast<void**>(&h->stage), h->stage_bytes) != cudaSuccess) {
+        cudaGetLastError();                   // no pinned memory left: state downloads go to pageable memory
+        h->stage = nullptr;
+        h->stage_bytes = 0;
+    }
     if ((rc = group_schedule(h, h->main))) return bail(rc);
     if ((rc = upload_couplers(h, h->main, 0, h->J.data()))) return bail(rc);
     if ((rc = upload_desc(h, h->main))) return bail(rc);
@@ -945,6 +964,7 @@ void pt_destroy(pt_handle* h)
     if (h->stream) cudaStreamSynchronize(h->stream);
     free_group(h->main);
     free_group(h->cand);
+    cudaFreeHost(h->stage);
     cudaFree(h->d_thr); cudaFree(h->d_xoff); cudaFree(h->d_xthr); cudaFree(h->d_xhint); cudaFree(h->d_nbr);
     for (cudaEvent_t e : h->ev) cudaEventDestroy(e);
     if (h->eb0) cudaEventDestroy(h->eb0);
@@ -997,7 +1017,7 @@ int pt_exchange(pt_handle* h)
 {
     if (!h) return PT_ERR_ARG;
     Group& g = h->main;
-    CK(launch_sweeps(g.d_desc, g.d_bundles, (int)g.bundles.size(), (int)g.bundles.size(), g.block,
+    CK(launch_sweeps(g.d_desc, g.d_bundles, (int)g.bundles.size(), (int)g.bundles.size(), g.threads,
                      g.smem, (uint32_t)g.sweep, 0, 0, 1, nullptr, h->stream, g.team, g.walk, g.L),
        "exchange kernel");
     ++h->launches;
@@ -1012,26 +1032,38 @@ int pt_get_state(pt_handle* h, int8_t* spins, int32_t* E, uint8_t* perm, int32_t
     if (!h) return PT_ERR_ARG;
     Group& g = h->main;
     const size_t reps = (size_t)h->R * h->NT, N = h->N;
-    std::vector<uint8_t> pm(reps);
-    CK(cudaMemcpyAsync(pm.data(), g.perm, reps, cudaMemcpyDeviceToHost, h->stream), "download perm");
+    // one copy of the records, or of the whole state, into the pinned staging where it fits (a copy of
+    // each array into pageable memory costs about 8 us); larger spins go straight to the caller's side
+    const bool whole = spins && g.block_bytes <= h->stage_bytes;
+    const size_t from = whole ? 0 : g.rec_off, bytes = g.block_bytes - from;
+    std::vector<uint8_t> rec;
     std::vector<int8_t> sp;
-    if (spins) {
+    uint8_t* host = h->stage;
+    if (bytes > h->stage_bytes) {
+        rec.resize(bytes);
+        host = rec.data();
+    }
+    CK(cudaMemcpyAsync(host, g.block + from, bytes, cudaMemcpyDeviceToHost, h->stream), "download state");
+    if (spins && !whole) {
         sp.resize(reps * N);
         CK(cudaMemcpyAsync(sp.data(), g.spins, reps * N, cudaMemcpyDeviceToHost, h->stream), "download spins");
     }
-    if (E) CK(cudaMemcpyAsync(E, g.E, 4 * reps, cudaMemcpyDeviceToHost, h->stream), "download E");
-    if (best) CK(cudaMemcpyAsync(best, g.best, 4 * (size_t)h->R, cudaMemcpyDeviceToHost, h->stream), "download best");
-    if (first) CK(cudaMemcpyAsync(first, g.first, 4 * (size_t)h->R, cudaMemcpyDeviceToHost, h->stream), "download first");
-    if (macc) CK(cudaMemcpyAsync(macc, g.macc, 8 * reps, cudaMemcpyDeviceToHost, h->stream), "download macc");
-    if (xacc && h->NT > 1)
-        CK(cudaMemcpyAsync(xacc, g.xacc, 8 * (size_t)h->R * (h->NT - 1), cudaMemcpyDeviceToHost, h->stream), "download xacc");
     CK(cudaStreamSynchronize(h->stream), "sync get_state");
-    if (perm) std::memcpy(perm, pm.data(), reps);
-    if (spins)   // slot order: slot t holds buffer perm[t]
+    auto at = [&](const void* d) { return host + (static_cast<const uint8_t*>(d) - g.block) - from; };
+    const uint8_t* pm = at(g.perm);
+    if (E) std::memcpy(E, at(g.E), 4 * reps);
+    if (best) std::memcpy(best, at(g.best), 4 * (size_t)h->R);
+    if (first) std::memcpy(first, at(g.first), 4 * (size_t)h->R);
+    if (macc) std::memcpy(macc, at(g.macc), 8 * reps);
+    if (xacc && h->NT > 1) std::memcpy(xacc, at(g.xacc), 8 * (size_t)h->R * (h->NT - 1));
+    if (perm) std::memcpy(perm, pm, reps);
+    if (spins) {                              // slot order: slot t holds buffer perm[t]
+        const int8_t* src = whole ? reinterpret_cast<const int8_t*>(at(g.spins)) : sp.data();
         for (int r = 0; r < h->R; ++r)
             for (int t = 0; t < h->NT; ++t)
                 std::memcpy(spins + ((size_t)r * h->NT + t) * N,
-                            sp.data() + ((size_t)r * h->NT + pm[(size_t)r * h->NT + t]) * N, N);
+                            src + ((size_t)r * h->NT + pm[(size_t)r * h->NT + t]) * N, N);
+    }
     if (sweep) *sweep = g.sweep;
     return PT_OK;
 }
