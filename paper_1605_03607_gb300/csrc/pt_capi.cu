@@ -27,10 +27,17 @@ using namespace ptg;
 
 namespace {
 
+constexpr size_t MAX_PLANS = 64;
 constexpr size_t STAGE_MAX = 256 * 1024;     // pinned bytes a handle keeps for state downloads
 
 std::mutex g_err_mu;
 std::string g_create_err = "no error";
+
+// A sweep launch over a list of bundles.
+struct Launch {
+    const Bundle* d = nullptr;
+    int n = 0, threads = 0, smem = 0, team = 0;
+};
 
 // A set of instances of one shape (L, NT, R) sharing one ladder.
 struct Group {
@@ -47,13 +54,13 @@ struct Group {
     InstDesc* d_desc = nullptr;
     int2* d_items = nullptr;
     Bundle* d_bundles = nullptr;
-    Bundle* d_sub = nullptr;         // a subset of the bundles (doubling budget: undecided instances)
+    Bundle* d_sub = nullptr;         // the list of the last subset_launch
     int32_t* d_tts = nullptr;        // [n_inst][3]
     int32_t* d_targets = nullptr;    // [n_inst] per-instance TTS targets (LAO)
     int* d_queue = nullptr;
     std::vector<InstDesc> desc;
     std::vector<Bundle> bundles;
-    int threads = 0, smem = 0, team = 0;
+    Launch all;                      // every run of every instance
     uint64_t sweep = 0;
     // temperature random walk (main group only, when tracked)
     bool walk = false;
@@ -85,6 +92,8 @@ struct pt_handle {
     int sp = 0, ipc = 0, spl = 4096;
     int team = 0;              // 0: cell-major mapping; > 0: slot-major with teams of this size
     bool planned = true;       // until a schedule is set: the replica-lane mapping, shaped by lane_plan
+    struct Plan { int kt, n_inst, R; bool walk; LaneShape s; };
+    std::vector<Plan> plans;   // shapes made so far (at most MAX_PLANS)
     uint64_t launches = 0;
     // timing of sweep launches
     bool timing = false;
@@ -274,38 +283,59 @@ int group_alloc(pt_handle* h, Group& g, int n_inst)
     return PT_OK;
 }
 
+// The planned shape for n_inst instances of R runs of group g.
+int planned_shape(pt_handle* h, const Group& g, int n_inst, int R, LaneShape& s)
+{
+    for (const pt_handle::Plan& p : h->plans)
+        if (p.kt == h->kt && p.n_inst == n_inst && p.R == R && p.walk == g.walk) {
+            s = p.s;
+            return PT_OK;
+        }
+    int cap = 0, dev = 0, sms = 0;
+    CK(sweep_smem_capacity(&cap), "shared memory capacity");
+    CK(cudaGetDevice(&dev), "cudaGetDevice");
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
+    s = lane_plan(g.L, g.NT, h->kt, R, n_inst, g.walk, sms, cap);
+    if (h->plans.size() >= MAX_PLANS) h->plans.erase(h->plans.begin());
+    h->plans.push_back({h->kt, n_inst, R, g.walk, s});
+    return PT_OK;
+}
+
 // The new bundle list replaces the group's only when every step succeeded, so
 // a failure leaves the previous schedule in place and launchable.
 int group_schedule(pt_handle* h, Group& g)
 {
     std::vector<Bundle> bundles;
-    const int L2 = g.L * g.L;
-    int cap = 0, team = h->team, sp = h->sp, ipc = h->ipc;
-    LaneShape shape;
+    int cap = 0;
     CK(sweep_smem_capacity(&cap), "shared memory capacity");
+    Launch l;
     if (h->planned) {
-        int dev = 0, sms = 0;
-        CK(cudaGetDevice(&dev), "cudaGetDevice");
-        CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
-        shape = lane_plan(g.L, g.NT, h->kt, g.R, g.n_inst, g.walk, sms, cap);
-        team = -shape.gr;
-        sp = shape.W;
-        ipc = shape.gr * shape.G;
+        LaneShape shape;
+        if (int rc = planned_shape(h, g, g.n_inst, g.R, shape)) return rc;
+        std::vector<int> insts(g.n_inst);
+        for (int i = 0; i < g.n_inst; ++i) insts[i] = i;
+        lane_bundles(shape, insts, g.R, bundles);
+        l.team = -shape.gr;
+        l.threads = lane_threads(g.NT, shape);
+        l.smem = (int)lane_smem(g.L, g.NT, h->kt, shape, g.walk);
+    } else {
+        for (int i = 0; i < g.n_inst; ++i)
+            for (int r = 0; r < g.R; r += h->ipc) {
+                Bundle b;
+                b.inst = i; b.run0 = r; b.nitems = std::min(h->ipc, g.R - r); b.sp = h->sp; b.team = h->team;
+                bundles.push_back(b);
+            }
+        l.team = h->team;
+        l.threads = (h->team > 0 ? h->sp * h->team : h->sp * g.L * g.L) * h->ipc;
+        l.smem = (int)bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, g.walk, h->kt);
     }
-    for (int i = 0; i < g.n_inst; ++i)
-        for (int r = 0; r < g.R; r += ipc) {
-            Bundle b;
-            b.inst = i; b.run0 = r; b.nitems = std::min(ipc, g.R - r); b.sp = sp; b.team = team;
-            bundles.push_back(b);
-        }
-    const int block = team < 0 ? lane_threads(g.NT, shape) : (team > 0 ? sp * team : sp * L2) * ipc;
-    const int smem = (int)bundle_smem_bytes(g.L, g.NT, ipc, team, g.walk, h->kt);
-    if (smem > cap) return fail(h, PT_ERR_ARG, "bundle needs more shared memory than a CTA can have");
-    CK(set_sweep_smem_limit(cap, team, g.walk, g.L), "cudaFuncSetAttribute");
+    if (l.smem > cap) return fail(h, PT_ERR_ARG, "bundle needs more shared memory than a CTA can have");
+    CK(set_sweep_smem_limit(cap, l.team, g.walk, g.L), "cudaFuncSetAttribute");
     Bundle* d = nullptr;
     Bundle* dsub = nullptr;
     CK(dalloc(&d, bundles.size()), "cudaMalloc bundles");
-    cudaError_t e = dalloc(&dsub, bundles.size());
+    // room for any subset: of the list, or (planned) with a shape of its own, a run per CTA at most
+    cudaError_t e = dalloc(&dsub, h->planned ? (size_t)g.n_inst * g.R : bundles.size());
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d, bundles.data(), sizeof(Bundle) * bundles.size(), cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) {
@@ -315,12 +345,40 @@ int group_schedule(pt_handle* h, Group& g)
     }
     cudaFree(g.d_bundles);
     cudaFree(g.d_sub);
-    g.d_sub = dsub;               // room for any subset of the full list
+    g.d_sub = dsub;
     g.d_bundles = d;
     g.bundles.swap(bundles);
-    g.threads = block;
-    g.smem = smem;
-    g.team = team;
+    l.d = d;
+    l.n = (int)g.bundles.size();
+    g.all = l;
+    return PT_OK;
+}
+
+// The launch over the first R runs of the listed instances, in the group's list of subsets.
+int subset_launch(pt_handle* h, Group& g, const std::vector<int>& insts, int R, Launch& l)
+{
+    l = g.all;
+    std::vector<Bundle> sub;
+    if (h->planned) {
+        LaneShape shape;
+        if (int rc = planned_shape(h, g, (int)insts.size(), R, shape)) return rc;
+        lane_bundles(shape, insts, R, sub);
+        l.team = -shape.gr;
+        l.threads = lane_threads(g.NT, shape);
+        l.smem = (int)lane_smem(g.L, g.NT, h->kt, shape, g.walk);
+    } else {
+        std::vector<char> in((size_t)g.desc.size(), 0);
+        for (int i : insts) in[(size_t)i] = 1;
+        for (Bundle b : g.bundles) {
+            if (!in[(size_t)b.inst] || b.run0 >= R) continue;
+            b.nitems = std::min(b.nitems, R - b.run0);
+            sub.push_back(b);
+        }
+    }
+    l.d = g.d_sub;
+    l.n = (int)sub.size();
+    CK(cudaMemcpyAsync(g.d_sub, sub.data(), sizeof(Bundle) * sub.size(), cudaMemcpyHostToDevice, h->stream),
+       "upload bundle subset");
     return PT_OK;
 }
 
@@ -375,10 +433,8 @@ int ensure_events(pt_handle* h, int n)
     return PT_OK;
 }
 
-int group_sweeps(pt_handle* h, Group& g, int64_t n, int xevery, const Bundle* dsub = nullptr, int nsub = 0)
+int group_sweeps(pt_handle* h, Group& g, int64_t n, int xevery, const Launch& l)
 {
-    const Bundle* db = dsub ? dsub : g.d_bundles;
-    const int nb = dsub ? nsub : (int)g.bundles.size();
     const int nl = (int)((n + h->spl - 1) / h->spl);
     if (h->timing) {
         int rc = ensure_events(h, 2 * nl);
@@ -389,8 +445,8 @@ int group_sweeps(pt_handle* h, Group& g, int64_t n, int xevery, const Bundle* ds
     while (done < n) {
         const int chunk = (int)std::min<int64_t>(h->spl, n - done);
         if (h->timing) CK(cudaEventRecord(h->ev[2 * li], h->stream), "event");
-        CK(launch_sweeps(g.d_desc, db, nb, nb, g.threads, g.smem, (uint32_t)g.sweep, chunk, xevery, 0, nullptr,
-                         h->stream, g.team, g.walk, g.L),
+        CK(launch_sweeps(g.d_desc, l.d, l.n, l.n, l.threads, l.smem, (uint32_t)g.sweep, chunk, xevery, 0, nullptr,
+                         h->stream, l.team, g.walk, g.L),
            "sweep kernel");
         if (g.walk && g.NT > 1 && xevery > 0)
             g.walk_passes += (g.sweep + chunk) / (uint64_t)xevery - g.sweep / (uint64_t)xevery;
@@ -436,7 +492,7 @@ int group_tts(pt_handle* h, Group& g, int32_t target, int32_t horizon, std::vect
 // targets (host, one per instance, may be NULL): per-instance TTS targets.
 int group_eval(pt_handle* h, Group& g, int32_t S, int32_t pass_mult, int32_t xevery,
                std::vector<int32_t>& out, int32_t target = PT_TARGET_BEST, const int32_t* targets = nullptr,
-               const Bundle* dsub = nullptr, int nsub = 0)
+               const Launch* sub = nullptr)
 {
     int rc;
     if (!h->eb0) {
@@ -446,7 +502,7 @@ int group_eval(pt_handle* h, Group& g, int32_t S, int32_t pass_mult, int32_t xev
     if ((rc = upload_desc(h, g))) return rc;
     CK(cudaEventRecord(h->eb0, h->stream), "event");
     if ((rc = group_reset(h, g, true))) return rc;
-    if ((rc = group_sweeps(h, g, (int64_t)S * pass_mult, xevery, dsub, nsub))) return rc;
+    if ((rc = group_sweeps(h, g, (int64_t)S * pass_mult, xevery, sub ? *sub : g.all))) return rc;
     if (targets)
         CK(cudaMemcpyAsync(g.d_targets, targets, sizeof(int32_t) * g.n_inst, cudaMemcpyHostToDevice, h->stream),
            "upload targets");
@@ -474,7 +530,7 @@ int group_eval(pt_handle* h, Group& g, int32_t S, int32_t pass_mult, int32_t xev
 // bundles.  Unsolved after Smax: TTS = Smax + 1.  out = n_inst x {tts, hits,
 // target}; levels = the deciding level of each instance.
 int group_eval_doubling(pt_handle* h, Group& g, int32_t S0, int32_t Smax, int32_t xevery, std::vector<int32_t>& out,
-                        std::vector<int32_t>& levels)
+                        std::vector<int32_t>& levels, int runs)
 {
     int rc;
     if (!h->eb0) {
@@ -488,16 +544,16 @@ int group_eval_doubling(pt_handle* h, Group& g, int32_t S0, int32_t Smax, int32_
     std::vector<char> open((size_t)n, 1);
     out.assign((size_t)n * 3, 0);
     levels.assign((size_t)n, 0);
-    std::vector<Bundle> sub;
+    std::vector<int> insts;
     std::vector<int32_t> lv_out;
     double ms_total = 0.0;
     for (int64_t lv = S0;; lv *= 2) {
-        sub.clear();
-        for (const Bundle& b : g.bundles)
-            if (b.inst < n && open[(size_t)b.inst]) sub.push_back(b);
-        CK(cudaMemcpyAsync(g.d_sub, sub.data(), sizeof(Bundle) * sub.size(), cudaMemcpyHostToDevice, h->stream),
-           "upload bundle subset");
-        if ((rc = group_sweeps(h, g, lv - (int64_t)g.sweep, xevery, g.d_sub, (int)sub.size()))) return rc;
+        insts.clear();
+        for (int i = 0; i < n; ++i)
+            if (open[(size_t)i]) insts.push_back(i);
+        Launch l;
+        if ((rc = subset_launch(h, g, insts, runs, l))) return rc;
+        if ((rc = group_sweeps(h, g, lv - (int64_t)g.sweep, xevery, l))) return rc;
         if ((rc = group_tts(h, g, PT_TARGET_BEST, (int32_t)lv, lv_out))) return rc;   // synchronises
         if ((rc = collect_timing(h))) return rc;
         if (h->timing) ms_total += h->last_ms;
@@ -585,29 +641,20 @@ int eval_candidates(pt_handle* h, int k, const int8_t* Jc, const uint32_t* uids,
     // (all runs when n_eval is 0): shrink the group view temporarily
     const int nr = (n_eval > 0 && n_eval < h->R) ? n_eval : h->R;
     const int n_full = g.n_inst;
-    std::vector<Bundle> keep = g.bundles;
     g.n_inst = k;
-    std::vector<Bundle> sub;
-    for (Bundle b : keep) {
-        if (b.inst >= k || b.run0 >= nr) continue;
-        b.nitems = std::min(b.nitems, nr - b.run0);
-        sub.push_back(b);
-    }
-    g.bundles = sub;
     for (int j = 0; j < k; ++j) g.desc[j].R = nr;            // the TTS reduction's run count
     if (h->rule.max_sweeps > 0 && !targets && target == PT_TARGET_BEST) {
-        rc = group_eval_doubling(h, g, h->rule.S, h->rule.max_sweeps, h->rule.exchange_every, res, h->last_levels);
+        rc = group_eval_doubling(h, g, h->rule.S, h->rule.max_sweeps, h->rule.exchange_every, res, h->last_levels, nr);
     } else {
-        rc = cudaMemcpyAsync(g.d_sub, sub.data(), sizeof(Bundle) * sub.size(), cudaMemcpyHostToDevice, h->stream)
-                 == cudaSuccess ? PT_OK : fail(h, PT_ERR_CUDA, "upload bundle subset");
-        if (!rc)
-            rc = group_eval(h, g, h->rule.S, h->rule.pass_mult, h->rule.exchange_every, res, target, targets,
-                            g.d_sub, (int)sub.size());
+        std::vector<int> insts(k);
+        for (int j = 0; j < k; ++j) insts[j] = j;
+        Launch l;
+        rc = subset_launch(h, g, insts, nr, l);
+        if (!rc) rc = group_eval(h, g, h->rule.S, h->rule.pass_mult, h->rule.exchange_every, res, target, targets, &l);
         h->last_levels.assign((size_t)k, h->rule.S * h->rule.pass_mult);
     }
     for (int j = 0; j < k; ++j) g.desc[j].R = h->R;
     g.n_inst = n_full;
-    g.bundles = keep;
     return rc;
 }
 
@@ -1007,7 +1054,7 @@ int pt_sweep(pt_handle* h, int32_t n_sweeps, int32_t exchange_every)
     if (n_sweeps < 0 || n_sweeps > (1 << 24) || exchange_every < 0)
         return fail(h, PT_ERR_ARG, "n_sweeps must be in [0, 2^24], exchange_every >= 0");
     if (h->main.sweep + (uint64_t)n_sweeps > 0x7FFFFFFFull) return fail(h, PT_ERR_STATE, "sweep counter would exceed 2^31-1");
-    int rc = group_sweeps(h, h->main, n_sweeps, exchange_every);
+    int rc = group_sweeps(h, h->main, n_sweeps, exchange_every, h->main.all);
     if (rc) return rc;
     CK(cudaStreamSynchronize(h->stream), "sync sweep");
     return collect_timing(h);
@@ -1017,8 +1064,8 @@ int pt_exchange(pt_handle* h)
 {
     if (!h) return PT_ERR_ARG;
     Group& g = h->main;
-    CK(launch_sweeps(g.d_desc, g.d_bundles, (int)g.bundles.size(), (int)g.bundles.size(), g.threads,
-                     g.smem, (uint32_t)g.sweep, 0, 0, 1, nullptr, h->stream, g.team, g.walk, g.L),
+    CK(launch_sweeps(g.d_desc, g.all.d, g.all.n, g.all.n, g.all.threads, g.all.smem, (uint32_t)g.sweep, 0, 0, 1, nullptr,
+                     h->stream, g.all.team, g.walk, g.L),
        "exchange kernel");
     ++h->launches;
     if (g.walk && g.NT > 1) g.walk_passes += 1;
@@ -1107,7 +1154,7 @@ int pt_tts_eval_doubling(pt_handle* h, uint32_t uid, int32_t S0, int32_t Smax, i
     h->uid = uid;
     h->main.desc[0].uid = uid;
     std::vector<int32_t> out, levels;
-    int rc = group_eval_doubling(h, h->main, S0, Smax, xevery, out, levels);
+    int rc = group_eval_doubling(h, h->main, S0, Smax, xevery, out, levels, h->R);
     if (rc) return rc;
     *tts = out[0];
     if (n_hit) *n_hit = out[1];
@@ -1903,7 +1950,7 @@ int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
         h->team = c.team;
         h->sp = c.sp;
         h->ipc = c.ipc;
-        if (!(rc = group_schedule(h, g))) rc = group_sweeps(h, g, trial_sweeps, 1);
+        if (!(rc = group_schedule(h, g))) rc = group_sweeps(h, g, trial_sweeps, 1, g.all);
         cudaError_t e = rc ? cudaSuccess : cudaStreamSynchronize(h->stream);
         double ms = 0.0;
         for (int i = 0; i < h->ev_used && !rc && e == cudaSuccess; ++i) {

@@ -218,6 +218,7 @@ inline std::string build_tables(int NT, int kt, const double* betas, Tables& tb)
 // ------------------------------------------------------------------------
 struct LaneShape {
     int W = 1, gr = 1, G = 1;          // warps per column, runs per group, groups per CTA
+    bool span = false;                 // a CTA may hold runs of two instances (with the same tables)
 };
 
 inline int lane_columns(int NT, int gr) { return (gr * NT + 31) / 32; }
@@ -241,29 +242,66 @@ inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
 
 // The shape with the lowest estimate for n_inst instances of R runs on `sms` SMs: all CTAs
 // of a launch run at once if they fit, else in waves.  One run per CTA spreads best over
-// the SMs; more runs share the field tables (384 L^2 bytes), which decides at large L.
+// the SMs; more runs share the field tables (384 L^2 bytes an instance), which decides at
+// large L.  Runs that do not divide into whole CTAs fill them up with the next instance's
+// (span): 16 C_8 instances of 64 runs (32 temperatures) are 147 CTAs of 7, one for each SM,
+// where CTAs of one instance came in two waves: 2048 sweeps 29.9 -> 28.1 ms.
 inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, int sms, int cap)
 {
+    const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
     LaneShape best;
     double best_t = 1e300;
     for (int gr = 1; gr <= 8 && gr <= R; ++gr)
         for (int G = 1; G <= LANE_GROUPS && (G - 1) * gr < R; ++G)
-            for (int W : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
-                LaneShape s;
-                s.W = W;
-                s.gr = gr;
-                s.G = G;
-                const int threads = lane_threads(NT, s), units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
-                if (threads > LANE_THREADS || (W > units && W > 1)) break;
-                const int64_t smem = lane_layout(L, NT, kt, gr, G, walk).bytes;
+            for (int span = 0; span < 2; ++span) {
+                const int64_t per = (R + gr - 1) / gr;                  // groups of an instance
+                if (span && (n_inst == 1 || per % G == 0)) continue;    // (G - 1) * gr < R: at most two instances a CTA
+                const int64_t smem = lane_layout(L, NT, kt, gr, G, walk, span ? 2 : 1).bytes;
                 if (smem > cap) continue;
-                const int fit = std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
-                const int64_t ctas = (int64_t)n_inst * ((R + gr * G - 1) / (gr * G)), wave = (int64_t)fit * sms;
-                const int rest = (int)((ctas % wave + sms - 1) / sms);
-                const double t = (double)(ctas / wave) * lane_clocks(L, NT, s, fit) + (rest ? lane_clocks(L, NT, s, rest) : 0.0);
-                if (t < best_t * 0.999) { best_t = t; best = s; }
+                for (int W : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
+                    LaneShape s;
+                    s.W = W;
+                    s.gr = gr;
+                    s.G = G;
+                    s.span = span != 0;
+                    const int threads = lane_threads(NT, s);
+                    if (threads > LANE_THREADS || (W > units && W > 1)) break;
+                    const int fit = std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
+                    const int64_t ctas = span ? (n_inst * per + G - 1) / G : n_inst * ((per + G - 1) / G), wave = (int64_t)fit * sms;
+                    const int rest = (int)((ctas % wave + sms - 1) / sms);
+                    const double t = (double)(ctas / wave) * lane_clocks(L, NT, s, fit) + (rest ? lane_clocks(L, NT, s, rest) : 0.0);
+                    if (t < best_t * 0.999) { best_t = t; best = s; }
+                }
             }
     return best;
+}
+
+inline int64_t lane_smem(int L, int NT, int kt, const LaneShape& s, bool walk)
+{
+    return lane_layout(L, NT, kt, s.gr, s.G, walk, s.span ? 2 : 1).bytes;
+}
+
+// Bundles of the first R runs of the listed instances.
+inline void lane_bundles(const LaneShape& s, const std::vector<int>& insts, int R, std::vector<Bundle>& out)
+{
+    out.clear();
+    int r = 0;
+    for (size_t a = 0; a < insts.size();) {
+        Bundle b;
+        b.inst = insts[a]; b.run0 = r; b.nitems = std::min(s.gr * s.G, R - r); b.sp = s.W; b.team = -s.gr;
+        r += b.nitems;
+        if (r == R) {
+            r = 0;
+            const int left = s.G - (b.nitems + s.gr - 1) / s.gr;
+            if (++a < insts.size() && s.span && left > 0) {
+                b.inst2 = insts[a];
+                b.nitems2 = std::min(left * s.gr, R);
+                r = b.nitems2;
+                if (r == R) { r = 0; ++a; }
+            }
+        }
+        out.push_back(b);
+    }
 }
 
 // Shape of a batch's instances of one lattice side (their temperature counts `NTs`), whose

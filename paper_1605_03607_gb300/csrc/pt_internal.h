@@ -69,8 +69,11 @@ struct InstDesc {
 //              per run; a team owns every sp-th slot, its lanes split the cells.
 //   team  < 0 (replica-lane): groups of -team runs whose replicas fill the lanes
 //              of warps ("columns" of 32); sp warps per column split the cells.
+//              nitems2 > 0: the groups go on with runs 0 .. nitems2 - 1 of inst2,
+//              an instance with the same tables (thr, xthr), and couplers of its own.
 struct Bundle {
     int32_t inst, run0, nitems, sp, team;
+    int32_t inst2 = 0, nitems2 = 0;
 };
 
 // Shared-memory layout of one bundle: the Metropolis table of the instance,
@@ -140,7 +143,7 @@ __host__ __device__ inline int64_t cell_table_bytes(int L) { return 4LL * CELL_R
 // cell's negative spins of that colour, so a byte is the offset of its entry in a
 // 16-word table.  A group of `gr` runs fills columns of 32 replicas, `W` warps per
 // column split the cells, and groups never wait for each other.  Shared memory:
-//   lut    [2][L^2][3][16] words: for every (colour, cell), the summed fields
+//   lut    per instance [2][L^2][3][16] words: for every (colour, cell), the summed fields
 //          of its 4 spins from the opposite group of the cell and from the
 //          minus- and plus-neighbour groups, packed one byte per spin
 //          (the sum of the three entries is 128 - h_i, byte by byte)
@@ -158,13 +161,13 @@ struct LaneLayout {
     int32_t spins, col_bytes, runs, run_bytes, group_bytes, bytes;   // spins, runs: inside a group
 };
 
-__host__ __device__ inline LaneLayout lane_layout(int L, int NT, int kt, int gr, int ngroups, bool walk)
+__host__ __device__ inline LaneLayout lane_layout(int L, int NT, int kt, int gr, int ngroups, bool walk, int ninst = 1)
 {
     const int L2 = L * L;
     LaneLayout o;
     o.ncols = (gr * NT + 31) / 32;
     o.lut = 0;
-    const int lut_end = 384 * L2, below = 128 * (kt - 1);
+    const int lut_end = 384 * L2 * ninst, below = 128 * (kt - 1);
     o.thr = (lut_end > below ? lut_end : below);
     o.xtab = o.thr + (NT + 31) / 32 * kt * 128;
     o.groups = (int32_t)pad16(o.xtab + 8 * NT);

@@ -316,26 +316,29 @@ template <int LT>
 __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bundle bd, uint32_t sweep0, int nsweeps,
                                     int xevery, int mode, unsigned char* smem)
 {
-    const InstDesc& in = insts[bd.inst];
+    const InstDesc& in0 = insts[bd.inst];
 #ifdef PT_DEBUG
-    if (LT && in.L != LT) {                     // uniform per CTA: the whole CTA skips the bundle
+    if (LT && in0.L != LT) {                    // uniform per CTA: the whole CTA skips the bundle
         if (threadIdx.x == 0) atomicCAS(&g_pt_debug_code, 0u, 9u);
         return;
     }
 #endif
-    const int L = LT ? LT : in.L, NT = in.NT, L2 = L * L, N = 8 * L2, NW = 2 * L2, W = bd.sp, gr = -bd.team;
-    const int ngroups = (bd.nitems + gr - 1) / gr;
-    const bool walk = in.wstate != nullptr;
-    const LaneLayout lay = lane_layout(L, NT, in.kt, gr, ngroups, walk);
+    const int L = LT ? LT : in0.L, NT = in0.NT, L2 = L * L, N = 8 * L2, NW = 2 * L2, W = bd.sp, gr = -bd.team;
+    const int ng1 = (bd.nitems + gr - 1) / gr, ngroups = ng1 + (bd.nitems2 + gr - 1) / gr, nruns = bd.nitems + bd.nitems2;
+    const bool walk = in0.wstate != nullptr;
+    const int kt = in0.kt;
+    const LaneLayout lay = lane_layout(L, NT, kt, gr, ngroups, walk, bd.nitems2 > 0 ? 2 : 1);
     const ItemLayout rl = item_layout(0, NT, 0, walk);
     const int tid = threadIdx.x, lane = tid & 31;
     // read through a warp reduction: warp-uniform for the compiler too
     const int wid = (int)__reduce_or_sync(FULL, (unsigned)(tid >> 5));
-    const uint32_t k0 = __reduce_or_sync(FULL, in.seed), k1 = __reduce_or_sync(FULL, in.uid);
     // this warp's group, its place in it, its column and its share of the cells
     const int gw = W * lay.ncols, grp = wid / gw, gwid = wid - grp * gw, col = gwid / W, w = gwid - col * W;
-    const bool active = grp < ngroups;
-    const int nit = active ? min(gr, bd.nitems - grp * gr) : 0;      // runs of the group
+    const bool active = grp < ngroups, second = grp >= ng1 && active;
+    const InstDesc& in = second ? insts[bd.inst2] : in0;
+    const uint32_t k0 = __reduce_or_sync(FULL, in.seed), k1 = __reduce_or_sync(FULL, in.uid);
+    const int done = (second ? grp - ng1 : grp) * gr;                // its instance's runs before the group's
+    const int nit = active ? min(gr, (second ? bd.nitems2 : bd.nitems) - done) : 0;      // runs of the group
     const int rep = col * 32 + lane;
     const bool valid = rep < nit * NT, busy = col * 32 < nit * NT;   // busy: the column holds a replica
     const int item = valid ? rep / NT : 0, buf = valid ? rep - item * NT : 0;
@@ -343,49 +346,59 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
     auto group_base = [&](int g) { return smem + lay.groups + g * lay.group_bytes; };
     auto run_base = [&](int g, int i) { return group_base(g) + lay.runs + i * lay.run_bytes; };
     unsigned char* const gb = group_base(active ? grp : 0);
-    const int grun = bd.run0 + grp * gr;                             // the group's first run
+    const int grun = (second ? 0 : bd.run0) + done;                  // the group's first run
     int32_t* xoff_sm = reinterpret_cast<int32_t*>(smem + lay.xtab);
     uint4* pre = reinterpret_cast<uint4*>(gb);
     auto gsync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gw * 32) : "memory"); };
     const int n_iter = (mode == 0) ? nsweeps : 1;
     const uint32_t s_first = (mode == 0) ? sweep0 + 1u : sweep0;
-    const uint32_t* const xthr = in.xthr;
+    const uint32_t* const xthr = in0.xthr;
     // sweeps to the next exchange, counted down from sweep s_first on (0: exchange after that sweep)
     const bool xon = NT > 1 && (mode == 1 || xevery > 0);
     const uint32_t xper = mode == 1 || xevery < 1 ? 1u : (uint32_t)xevery;
     uint32_t xwait = (xper - s_first % xper) % xper;
     if (mode == 1) xwait = 0u;
 
+    // run r of the bundle: its instance, its run there, and its place in shared memory
+    auto inst_of = [&](int r) -> const InstDesc& { return r < bd.nitems ? in0 : insts[bd.inst2]; };
+    auto run_of = [&](int r) { return r < bd.nitems ? bd.run0 + r : r - bd.nitems; };
+    auto slot_of = [&](int r) { return r < bd.nitems ? r : ng1 * gr + r - bd.nitems; };      // group * gr + place
+
     // ---- tables, then this bundle's runs
     {
         uint32_t* lut = reinterpret_cast<uint32_t*>(smem + lay.lut);
-        for (int i = tid; i < 2 * L2 * 48; i += blockDim.x) {
-            const int cq = i / 48, e = i - cq * 48, c = cq / L2, q = cq - c * L2;
-            lut[i] = lane_field(in.jw + (q * 2 + c) * 8, e >> 4, e & 15);
+        for (int s = 0; s < (bd.nitems2 > 0 ? 2 : 1); ++s, lut += 96 * L2) {
+            const uint32_t* jw = insts[s == 0 ? bd.inst : bd.inst2].jw;
+            for (int i = tid; i < 2 * L2 * 48; i += blockDim.x) {
+                const int cq = i / 48, e = i - cq * 48, c = cq / L2, q = cq - c * L2;
+                lut[i] = lane_field(jw + (q * 2 + c) * 8, e >> 4, e & 15);
+            }
         }
         uint32_t* thr = reinterpret_cast<uint32_t*>(smem + lay.thr);
-        for (int i = tid; i < (NT + 31) / 32 * 32 * in.kt; i += blockDim.x) {
-            const int b = i / (32 * in.kt), k = (i >> 5) - b * in.kt, t = b * 32 + (i & 31);
-            thr[i] = t < NT ? in.thr[t * in.kt + k] : 0u;
+        for (int i = tid; i < (NT + 31) / 32 * 32 * kt; i += blockDim.x) {
+            const int b = i / (32 * kt), k = (i >> 5) - b * kt, t = b * 32 + (i & 31);
+            thr[i] = t < NT ? in0.thr[t * kt + k] : 0u;
         }
         for (int p = tid; p < NT; p += blockDim.x) {
-            xoff_sm[p] = in.xoff[p];
-            reinterpret_cast<float*>(xoff_sm + NT)[p] = p < NT - 1 ? in.xhint[p] : 0.0f;
+            xoff_sm[p] = in0.xoff[p];
+            reinterpret_cast<float*>(xoff_sm + NT)[p] = p < NT - 1 ? in0.xhint[p] : 0.0f;
         }
         for (int g = 0; g < ngroups; ++g) {
             uint32_t* sp = reinterpret_cast<uint32_t*>(group_base(g) + lay.spins);
             for (int i = tid; i < lay.ncols * lay.col_bytes / 4; i += blockDim.x) sp[i] = 0u;
             uint4* pg = reinterpret_cast<uint4*>(group_base(g));
+            const InstDesc& ig = g < ng1 ? in0 : insts[bd.inst2];
             for (int i = tid; i < 2 * L2; i += blockDim.x)
-                pg[i] = lane_pre(s_first, i >= L2, i >= L2 ? i - L2 : i, L, k0, k1);
+                pg[i] = lane_pre(s_first, i >= L2, i >= L2 ? i - L2 : i, L, ig.seed, ig.uid);
         }
     }
-    for (int i = tid; i < bd.nitems * NT; i += blockDim.x) {
-        const int r = i / NT, t = i - r * NT;
-        unsigned char* rb = run_base(r / gr, r % gr);
-        const size_t g = (size_t)(bd.run0 + r) * NT + t;
-        const int b = PT_IDX((int)in.perm[g], NT, 2u);
-        reinterpret_cast<int32_t*>(rb + rl.E)[t] = in.E[g];
+    for (int i = tid; i < nruns * NT; i += blockDim.x) {
+        const int r = i / NT, t = i - r * NT, run = run_of(r), at = slot_of(r);
+        const InstDesc& ir = inst_of(r);
+        unsigned char* rb = run_base(at / gr, at % gr);
+        const size_t g = (size_t)run * NT + t;
+        const int b = PT_IDX((int)ir.perm[g], NT, 2u);
+        reinterpret_cast<int32_t*>(rb + rl.E)[t] = ir.E[g];
         (rb + rl.perm)[t] = (uint8_t)b;
         (rb + rl.inv)[b] = (uint8_t)t;
         reinterpret_cast<uint32_t*>(rb + rl.macc)[t] = 0u;
@@ -393,24 +406,27 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
         if (walk) {
             reinterpret_cast<uint32_t*>(rb + rl.whot)[t] = 0u;
             reinterpret_cast<uint32_t*>(rb + rl.wtrips)[t] = 0u;
-            (rb + rl.wstate)[t] = in.wstate[g];
+            (rb + rl.wstate)[t] = ir.wstate[g];
         }
         if (t == 0) {
-            reinterpret_cast<int32_t*>(rb + rl.misc)[0] = in.best[bd.run0 + r];
-            reinterpret_cast<int32_t*>(rb + rl.misc)[1] = in.first[bd.run0 + r];
+            reinterpret_cast<int32_t*>(rb + rl.misc)[0] = ir.best[run];
+            reinterpret_cast<int32_t*>(rb + rl.misc)[1] = ir.first[run];
         }
     }
     __syncthreads();
-    // spin word i of run r (buffer b, group g = 2 cell + u) and its byte in shared memory
-    uint32_t* gsp = reinterpret_cast<uint32_t*>(in.spins + (size_t)bd.run0 * NT * N);
-    auto spin_byte = [&](int r, int i) {
+    // spin word i of run r (buffer b, group g = 2 cell + u) in memory and its byte in shared memory
+    auto spin_words = [&](int r) { return reinterpret_cast<uint32_t*>(inst_of(r).spins + (size_t)run_of(r) * NT * N); };
+    auto spin_byte = [&](int at, int i) {
         const int b = i / NW, g = i - b * NW, q = g >> 1, y = q / L, x = q - y * L, cl = (y + x + (g & 1)) & 1;
-        const int p = (r % gr) * NT + b;
-        return group_base(r / gr) + lay.spins + (p >> 5) * lay.col_bytes + cl * (lay.col_bytes / 2) + (q + L) * 32 + (p & 31);
+        const int p = (at % gr) * NT + b;
+        return group_base(at / gr) + lay.spins + (p >> 5) * lay.col_bytes + cl * (lay.col_bytes / 2) + (q + L) * 32 + (p & 31);
     };
-    for (int r = 0; r < bd.nitems; ++r)
+    for (int r = 0; r < nruns; ++r) {
+        const uint32_t* gsp = spin_words(r);
+        const int at = slot_of(r);
         for (int i = tid; i < NT * NW; i += blockDim.x)
-            *spin_byte(r, i) = (unsigned char)(((gsp[(size_t)r * NT * NW + i] & 0x80808080u) * 0x00204081u) >> 26);
+            *spin_byte(at, i) = (unsigned char)(((gsp[i] & 0x80808080u) * 0x00204081u) >> 26);
+    }
     if (n_iter > 0 && xon && xwait == 0u)
         for (int r = gw - 1 - gwid; r < nit; r += gw)
             exchange_prepare(xthr, xoff_sm, lane, s_first, (uint32_t)(grun + r) << 16, k0, k1, NT,
@@ -421,10 +437,10 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
         unsigned char* rb = run_base(grp, item);
         unsigned char* s0 = gb + lay.spins + col * lay.col_bytes + L * 32 + lane;     // colour 0, cell 0
         unsigned char* s1 = s0 + lay.col_bytes / 2;
-        const unsigned char* lut0 = smem + lay.lut;
+        const unsigned char* lut0 = smem + lay.lut + (second ? 384 * L2 : 0);
         const uint32_t thr_at = (uint32_t)__cvta_generic_to_shared(smem + lay.thr);
         LaneConst lc;
-        lc.kt = in.kt;
+        lc.kt = kt;
 #pragma unroll
         for (int r = 0; r < 7; ++r) {           // through a warp reduction each, so that they are kept, not recomputed
             lc.ka[r] = __reduce_or_sync(FULL, k0 + (3u + r) * PHILOX_W0);
@@ -490,25 +506,29 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
 
     // ---- write the state back
     __syncthreads();
-    for (int r = 0; r < bd.nitems; ++r)
+    for (int r = 0; r < nruns; ++r) {
+        uint32_t* gsp = spin_words(r);
+        const int at = slot_of(r);
         for (int i = tid; i < NT * NW; i += blockDim.x)
-            gsp[(size_t)r * NT * NW + i] = byte_signs(*spin_byte(r, i) * 0x04081020u) | 0x01010101u;   // 0xFF or 1
-    for (int i = tid; i < bd.nitems * NT; i += blockDim.x) {
-        const int r = i / NT, t = i - r * NT, run = bd.run0 + r;
-        const unsigned char* xb = run_base(r / gr, r % gr);
+            gsp[i] = byte_signs(*spin_byte(at, i) * 0x04081020u) | 0x01010101u;   // 0xFF or 1
+    }
+    for (int i = tid; i < nruns * NT; i += blockDim.x) {
+        const int r = i / NT, t = i - r * NT, run = run_of(r), at = slot_of(r);
+        const InstDesc& ir = inst_of(r);
+        const unsigned char* xb = run_base(at / gr, at % gr);
         const size_t g = (size_t)run * NT + t;
-        in.E[g] = reinterpret_cast<const int32_t*>(xb + rl.E)[t];
-        in.perm[g] = (xb + rl.perm)[t];
-        in.macc[g] += reinterpret_cast<const uint32_t*>(xb + rl.macc)[t];
-        if (t < NT - 1) in.xacc[(size_t)run * (NT > 1 ? NT - 1 : 1) + t] += reinterpret_cast<const uint32_t*>(xb + rl.xacc)[t];
+        ir.E[g] = reinterpret_cast<const int32_t*>(xb + rl.E)[t];
+        ir.perm[g] = (xb + rl.perm)[t];
+        ir.macc[g] += reinterpret_cast<const uint32_t*>(xb + rl.macc)[t];
+        if (t < NT - 1) ir.xacc[(size_t)run * (NT > 1 ? NT - 1 : 1) + t] += reinterpret_cast<const uint32_t*>(xb + rl.xacc)[t];
         if (walk) {
-            in.whot[g] += reinterpret_cast<const uint32_t*>(xb + rl.whot)[t];
-            in.wtrips[g] += reinterpret_cast<const uint32_t*>(xb + rl.wtrips)[t];
-            in.wstate[g] = (xb + rl.wstate)[t];
+            ir.whot[g] += reinterpret_cast<const uint32_t*>(xb + rl.whot)[t];
+            ir.wtrips[g] += reinterpret_cast<const uint32_t*>(xb + rl.wtrips)[t];
+            ir.wstate[g] = (xb + rl.wstate)[t];
         }
         if (t == 0) {
-            in.best[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[0];
-            in.first[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[1];
+            ir.best[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[0];
+            ir.first[run] = reinterpret_cast<const int32_t*>(xb + rl.misc)[1];
         }
     }
     __syncthreads();

@@ -72,6 +72,26 @@ def test_planned_groups_of_candidates(P, L, NT, R, k):
         assert (out["tts"][j], out["n_hit"][j], out["target"][j]) == want, j
 
 
+@pytest.mark.parametrize("L,NT,R,k", [(2, 17, 25, 24), (3, 7, 100, 24), (6, 17, 25, 24), (8, 7, 256, 16)])
+@pytest.mark.parametrize("adaptive", [False, True])
+def test_planned_ctas_of_two_instances(P, L, NT, R, k, adaptive):
+    """Run counts that do not divide into whole CTAs: the last runs of one candidate share a CTA
+    with the first of the next.  With a doubling budget the candidates of a launch are no
+    longer consecutive and the shape changes from level to level."""
+    betas = W.beta_ladder(NT, 0.1, 3.0)
+    Js = np.stack([W.random_couplers(L, 5, j) for j in range(k)])
+    uids = np.arange(k) + 3
+    with P.PTHandle(L, Js[0], betas, R, 5, 0) as h:
+        out = h.tts_eval_many(Js, uids, 1 if adaptive else 4, 1, max_sweeps=8 if adaptive else 0)
+    for j in range(k):
+        if adaptive:
+            want = oracle.tts_eval_doubling(L, Js[j], betas, R, 5, j + 3, 1, 8, 1)
+            assert (out["tts"][j], out["n_hit"][j], out["target"][j]) == tuple(want[:3]), j
+        else:
+            want = oracle.tts_eval(L, Js[j], betas, R, 5, j + 3, 4, 1, 1)
+            assert (out["tts"][j], out["n_hit"][j], out["target"][j]) == want, j
+
+
 @pytest.mark.parametrize("L,kmax", [(1, 127), (2, 127), (3, 64)])
 def test_planned_longest_tables(P, L, kmax):
     """Local fields up to the largest allowed: the byte 127 + k of a field spans 0..254."""
