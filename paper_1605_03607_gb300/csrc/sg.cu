@@ -18,11 +18,14 @@
 //
 // Bound: memory and L2 traffic of the row-wise data (a batch of 256 C_8 graphs has
 // 753,664 message, 131,072 node and 376,832 edge rows of 64; the linear maps need
-// 0.13 ms of tensor time), and launch gaps for small batches.  So per layer 3 forward
-// and 4 backward kernels, each a linear map with everything around it, and no message
-// row in memory.  Measured against one kernel per step with FP32 messages, pre-activations
-// and masked gradients in memory (97 launches, 35 now): gradient of 256 C_8 graphs 3.95 ->
-// 2.24 ms, of 128 C_4 graphs 1.01 -> 0.59 ms, 64 C_8 predictions 0.42 -> 0.26 ms.
+// 0.13 ms of tensor time), above all its gathers into the SMs, and launch gaps for small
+// batches.  So per layer 2 forward and 2 backward kernels, each with every linear map of
+// its rows and everything around them, no message row in memory, and rows that a tile
+// gathers several times taken from L1.  Measured against one kernel per step with FP32
+// messages, pre-activations and masked gradients in memory (97 launches, 22 now):
+// gradient of 256 C_8 graphs 3.95 -> 1.53 ms, of 128 C_4 graphs 1.01 -> 0.44 ms, 64 C_8
+// predictions 0.42 -> 0.20 ms.  (With a kernel per map and message rows of 21 nodes
+// summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -62,32 +65,36 @@ constexpr int WPART = HD * KIN + HD;
 // the input gradient dX = dZ W (128 rows x K = 64 -> 64 inputs at a time) and the
 // weight gradient dW^T += X^T dZ (K = 128 rows) run on tcgen05.mma with the
 // accumulator in tensor memory:
-//   * persistent CTAs over 128-row tiles; one thread issues the MMAs and
-//     commits them to an mbarrier;
+//   * persistent CTAs over tiles of 128 rows (nodes or edges); one thread issues the
+//     MMAs and commits them to an mbarrier;
 //   * operands in shared memory in the canonical layout without swizzle, built
 //     from 8-row x 16-byte core matrices; a descriptor's leading byte offset
 //     steps between core matrices along K, its stride byte offset along M or N.
 //     With the two the other way round every address would still lie inside the
 //     CTA's shared memory;
 //   * the weights, pre-packed in that layout (pack_weights_kernel), arrive by
-//     one bulk asynchronous copy; gathered rows by 16-byte cp.async;
+//     bulk asynchronous copies; gathered rows by 16-byte cp.async;
 //   * after the commit each warp reads its 32 accumulator rows (TMEM lanes
 //     32w .. 32w+31) with tcgen05.ld, one row per thread, for the epilogue;
 //   * every mbarrier wait is bounded: on a timeout the CTA records it in
 //     *err, stops taking tiles, frees its tensor memory and returns.
 constexpr uint32_t TC_WAIT_LIMIT = 1u << 22;
 constexpr int TC_ROWS = 128;
-// CTAs of 256 threads: all 8 warps stage a tile; in the epilogue warps w and
-// w + 4 read the same 32 tensor-memory lanes (a warp reaches lanes
-// 32 (w mod 4) .. + 31) and split the columns, and each warp's stores pass
-// through a 4 KB slice of the consumed operand buffer.  The dynamic shared
-// memory (forward: A 32 KB + W 16 KB; backward below) bounds the resident CTAs,
-// so that their tensor memory (64 columns forward, 128 backward) never exceeds an
-// SM's 512 columns; the persistent grids use exactly that many.
+// CTAs of 256 threads.  In the epilogue warps w and w + 4 read the same 32 tensor-memory
+// lanes (a warp reaches lanes 32 (w mod 4) .. + 31) and split the columns.
 constexpr int TC_THREADS = 256;
-constexpr int TC_A_FWD = TC_ROWS * KIN * 2;
-constexpr int TC_SMEM_FWD = TC_A_FWD + HD * KIN * 2;
-constexpr int TC_CTAS_FWD = 4;
+
+// A staged operand: columns ("chunks") of 8 BF16 x 128 rows, 16 bytes a row, CH bytes
+// apart.  A warp's load or copy takes 4 whole rows of 128 bytes (8 lanes x 16 bytes a
+// row): half the L1 wavefronts of 8 half rows, which had the L1 data pipe 45-80 % busy.
+// The 16 bytes beyond 128 rows put the 8 chunks of a row into different banks.  Read
+// along its columns a tile is a K-major operand, along its rows an MN-major one: the dZ
+// tile is the A operand of the input gradient and the B operand of the weight gradient.
+constexpr int CH = TC_ROWS * 16 + 16;
+constexpr int OP64 = 8 * CH;                  // operand of 64 columns; one of 128 is two, adjacent
+constexpr int W64 = HD * HD * 2;              // 64 x 64 weights
+
+__device__ __forceinline__ unsigned char* op_at(unsigned char* t, int kc, int row) { return t + kc * CH + row * 16; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -129,19 +136,31 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
     return false;
 }
 
-// One bulk asynchronous copy global -> shared of `bytes` (a multiple of 16,
-// both addresses 16-byte aligned), completing on `bar`.
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
+// Bulk asynchronous copies global -> shared of n0 and n1 bytes (multiples of 16, 0: none;
+// addresses 16-byte aligned) to adjacent places, completing on `bar`.
+__device__ __forceinline__ void bulk_g2s(unsigned char* dst, const void* src0, uint32_t n0, const void* src1, uint32_t n1, uint64_t* bar)
 {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar))
-                 : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(n0 + n1) : "memory");
+    if (n0)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(dst)), "l"(src0), "r"(n0), "r"(smem_u32(bar))
+                     : "memory");
+    if (n1)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(smem_u32(dst + n0)), "l"(src1), "r"(n1), "r"(smem_u32(bar))
+                     : "memory");
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+
+// The same through L1: rows that several rows of a tile gather.
+__device__ __forceinline__ void cp_async16_l1(void* dst, const void* src, bool valid)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
                  : "memory");
 }
 
@@ -172,108 +191,59 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Epilogue stores of one warp's 32 accumulator rows (lane l holds row l),
-// staged through a 4 KB slice of shared memory so that each global store
-// instruction writes whole rows: 4 rows x 128 bytes (32 FP32 columns) or 8
-// rows x 64 bytes (32 BF16 columns) instead of one 16-byte piece of each of
-// 32 rows.  Row l's 16-byte chunk c sits at slot c ^ (l & 7) (FP32) or
-// c ^ ((l >> 1) & 3) (BF16) of its row, so neither the row-wise writes nor
-// the chunk-wise reads of a warp meet a bank conflict.  flush_* writes the
-// staged block: g points at the warp's first row and first column, ld is the
-// row pitch in elements, and only rows < nvalid are written.
-__device__ __forceinline__ void stage_f32(unsigned char* stage, int lane, int c, float4 v)
+// A warp's 32 accumulator rows (lane l holds row l), 32 BF16 columns packed in 16 words
+// each, through a 2 KB slice of shared memory so that each global store instruction
+// writes whole pieces of rows: 8 rows x 64 bytes.  Row l's 16-byte chunk c sits at slot
+// c ^ ((l >> 1) & 3) of its row, so neither the row-wise writes nor the chunk-wise reads
+// meet a bank conflict.  g points at the warp's first row and first column; only rows
+// < nvalid are written.
+__device__ __forceinline__ void store_bf16x32(unsigned char* stage, const uint32_t (&w)[16], bf16* g, int nvalid, int lane)
 {
-    *reinterpret_cast<float4*>(stage + lane * 128 + ((c ^ (lane & 7)) << 4)) = v;
-}
-
-__device__ __forceinline__ void flush_f32x32(const unsigned char* stage, float* g, int ld, int nvalid, int lane)
-{
-    __syncwarp();
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int row = k * 4 + (lane >> 3), c = lane & 7;
-        const float4 x = *reinterpret_cast<const float4*>(stage + row * 128 + ((c ^ (row & 7)) << 4));
-        if (row < nvalid) *reinterpret_cast<float4*>(g + (size_t)row * ld + c * 4) = x;
-    }
-    __syncwarp();
-}
-
-// The same, added to g's rows.
-__device__ __forceinline__ void flush_add_f32x32(const unsigned char* stage, float* g, int ld, int nvalid, int lane)
-{
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int row = k * 4 + (lane >> 3), c = lane & 7;
-        float4 x = *reinterpret_cast<const float4*>(stage + row * 128 + ((c ^ (row & 7)) << 4));
-        if (row < nvalid) {
-            float4* gp = reinterpret_cast<float4*>(g + (size_t)row * ld + c * 4);
-            const float4 o = *gp;
-            x.x += o.x;
-            x.y += o.y;
-            x.z += o.z;
-            x.w += o.w;
-            *gp = x;
-        }
-    }
-    __syncwarp();
-}
-
-// Adds the sums of staged row pairs (2p, 2p + 1), in that order, to row p of g, or
-// (set) puts them there (16 pairs x 32 FP32 columns; only pairs < npairs).
-__device__ __forceinline__ void flush_pairs_f32x32(const unsigned char* stage, float* g, int ld, int npairs, int lane,
-                                                   bool set)
-{
-    __syncwarp();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int p = k * 4 + (lane >> 3), c = lane & 7, ra = 2 * p, rb = ra + 1;
-        const float4 a = *reinterpret_cast<const float4*>(stage + ra * 128 + ((c ^ (ra & 7)) << 4));
-        const float4 b = *reinterpret_cast<const float4*>(stage + rb * 128 + ((c ^ (rb & 7)) << 4));
-        if (p < npairs) {
-            float4* gp = reinterpret_cast<float4*>(g + (size_t)p * ld + c * 4);
-            float4 o = set ? make_float4(0.f, 0.f, 0.f, 0.f) : *gp;
-            o.x += a.x + b.x;
-            o.y += a.y + b.y;
-            o.z += a.z + b.z;
-            o.w += a.w + b.w;
-            *gp = o;
-        }
-    }
-    __syncwarp();
-}
-
-__device__ __forceinline__ void stage_bf16(unsigned char* stage, int lane, int c, uint4 v)
-{
-    *reinterpret_cast<uint4*>(stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) = v;
-}
-
-__device__ __forceinline__ void flush_bf16x32(const unsigned char* stage, bf16* g, int ld, int nvalid, int lane)
-{
+    for (int c = 0; c < 4; ++c)
+        *reinterpret_cast<uint4*>(stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4)) =
+            make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
     __syncwarp();
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int row = k * 8 + (lane >> 2), c = lane & 3;
         const uint4 x = *reinterpret_cast<const uint4*>(stage + row * 64 + ((c ^ ((row >> 1) & 3)) << 4));
-        if (row < nvalid) *reinterpret_cast<uint4*>(g + (size_t)row * ld + c * 8) = x;
+        if (row < nvalid) *reinterpret_cast<uint4*>(g + (size_t)row * HD + c * 8) = x;
     }
     __syncwarp();
 }
 
-// A 32-column BF16 block packed in 16 words (2 per column pair) through the staging slice.
-__device__ __forceinline__ void store_bf16x32(unsigned char* stage, const uint32_t (&w)[16], bf16* g, int ld,
-                                              int nvalid, int lane)
+// FP32 tile of 128 rows x 64 columns over consumed operands (32 KB): 16-byte chunk c of
+// row r at slot c ^ (r & 7), so that neither a warp that writes chunk c of 32 rows nor one
+// that reads 8 chunks of 4 rows meets a bank conflict.
+__device__ __forceinline__ float4* tile_f32(unsigned char* t, int row, int c)
 {
-#pragma unroll
-    for (int c = 0; c < 4; ++c) stage_bf16(stage, lane, c, make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]));
-    flush_bf16x32(stage, g, ld, nvalid, lane);
+    return reinterpret_cast<float4*>(t + row * 256 + ((c ^ (row & 7)) << 4));
 }
 
-// Common prologue: tensor memory (ncols columns, warp 0), the two mbarriers,
-// and the packed weights (bytes) by one bulk copy.  Returns false (for every
-// thread) if the weights did not arrive within the wait limit.
-__device__ __forceinline__ bool tc_setup(uint32_t* tmem_sh, uint64_t* bar_w, uint64_t* bar_mma, uint32_t ncols,
-                                         void* Ws, const void* Wpk, uint32_t bytes)
+// 64 accumulator columns from tensor memory to an FP32 tile.
+__device__ __forceinline__ void tmem_to_tile(unsigned char* t, uint32_t tcol, int warp, int lane)
+{
+    const int q = warp & 3, cb = (warp >> 2) * (HD / 2);
+    const uint32_t tl = tcol + ((uint32_t)(q * 32) << 16) + cb;
+    float d[2][16];
+    tmem_ld16(tl, d[0]);
+    tmem_ld16(tl + 16, d[1]);
+    tmem_ld_wait();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float* v = &d[c >> 2][4 * (c & 3)];
+        *tile_f32(t, q * 32 + lane, (cb >> 2) + c) = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// Common prologue: tensor memory (ncols columns, warp 0), the two mbarriers, and the
+// packed weights by bulk copies.  Returns false (for every thread) if the weights did not
+// arrive within the wait limit.
+__device__ __forceinline__ bool tc_setup(uint32_t* tmem_sh, uint64_t* bar_w, uint64_t* bar_mma, uint32_t ncols, unsigned char* Ws,
+                                         const void* W0, uint32_t n0, const void* W1, uint32_t n1)
 {
     const int tid = threadIdx.x;
     if ((tid >> 5) == 0) {
@@ -290,11 +260,52 @@ __device__ __forceinline__ bool tc_setup(uint32_t* tmem_sh, uint64_t* bar_w, uin
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (bytes == 0) return true;
-    if (tid == 0) bulk_g2s(Ws, Wpk, bytes, bar_w);
+    if (tid == 0) bulk_g2s(Ws, W0, n0, W1, n1, bar_w);
     bool ok = mbar_wait(bar_w, 0);
-    if (!ok) ok = mbar_wait(bar_w, 0);         // second bounded wait for the copy still in flight
+    if (!ok) ok = mbar_wait(bar_w, 0);         // second bounded wait for the copies still in flight
     return !__syncthreads_or(!ok);
+}
+
+// The staged operands are complete: this thread's copies have landed and its stores are
+// visible to the tensor core; tensor-memory reads before it are ordered before the MMAs
+// after it.  True (for every thread) if any thread's last wait failed.
+__device__ __forceinline__ bool tc_ready(bool failed)
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    const bool f = __syncthreads_or(failed);
+    tc_fence_after();
+    return f;
+}
+
+// Z = A W^T: A 128 columns, W [8 output groups][16 k-chunks][8 outputs][16 B]
+__device__ __forceinline__ void mma_forward(uint32_t tmem, const unsigned char* As, const unsigned char* Ws)
+{
+#pragma unroll
+    for (int ks = 0; ks < KIN / 16; ++ks)
+        tc_mma(tmem, tc_desc(smem_u32(As) + ks * 2 * CH, CH, 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 16 * 128),
+               tc_idesc_bf16(TC_ROWS, HD), ks > 0 ? 1u : 0u);
+}
+
+// dX (+)= dZ W over nin (64 or 128) inputs: W^T [nin / 8 input groups][8 k-chunks][8][16 B]
+template <int NIN>
+__device__ __forceinline__ void mma_input(uint32_t tmem, const unsigned char* Zs, const unsigned char* Ws, bool add)
+{
+#pragma unroll
+    for (int ks = 0; ks < HD / 16; ++ks)
+        tc_mma(tmem, tc_desc(smem_u32(Zs) + ks * 2 * CH, CH, 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 8 * 128),
+               tc_idesc_bf16(TC_ROWS, NIN), add || ks > 0 ? 1u : 0u);
+}
+
+// dW^T (+)= X^T dZ: X 128 columns (M), dZ 64 (N), K = 128 rows; both MN-major
+__device__ __forceinline__ void mma_wgrad(uint32_t tmem, const unsigned char* Xs, const unsigned char* Zs, bool add)
+{
+    constexpr uint32_t IDESC = tc_idesc_bf16(KIN, HD) | (1u << 15) | (1u << 16);
+#pragma unroll
+    for (int ks = 0; ks < TC_ROWS / 16; ++ks)
+        tc_mma(tmem, tc_desc(smem_u32(Xs) + ks * 256, 128, CH), tc_desc(smem_u32(Zs) + ks * 256, 128, CH), IDESC,
+               add || ks > 0 ? 1u : 0u);
 }
 
 __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t ncols, bool failed, int* err)
@@ -309,22 +320,24 @@ __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t ncols, bool 
 }
 
 // ------------------------------------------------------------- layer kernels
-// Rows of a tile are gathered while they are staged, and everything elementwise
-// around a linear map runs in its staging or its epilogue, so that per layer only
-// node and edge features (BF16), their gradients (FP32) and one bit per activation
+// Rows are gathered while they are staged, everything elementwise around a linear map
+// runs in its staging or its epilogue, and maps that work on the same rows share a
+// kernel: forward, a layer's messages with its node update, then its edge update;
+// backward, a layer's messages with the updates of the layer below, edges then nodes.
+// Only node and edge features (BF16), their gradients (FP32) and one bit per activation
 // go through memory:
 //   * the backward needs a pre-activation's sign only: the forward keeps it as a
-//     bit (z > 0 after rounding to BF16), 8 bytes per row of 64;
-//   * messages are computed target by target, 21 nodes of 6 slots per tile, and
-//     summed in the epilogue (in the order of the node's slots); their gradient
-//     with respect to the source node source by source, the same way;
-//   * a map's input gradient and weight gradient share the staged tile.
-// Row r of a tile sits in 8-row core matrices: chunk (row group r / 8, column chunk
-// of 8) is 8 rows x 16 bytes.  Read along its columns that is a K-major operand,
-// read along its rows an MN-major one; only the two descriptor strides differ (the
-// leading offset steps along K, the stride offset along M or N), so the dZ tile is
-// the A operand of the input gradient and the B operand of the weight gradient.
-constexpr int NODE_ROWS = 6, TILE_NODES = TC_ROWS / NODE_ROWS;        // 21 nodes, 126 rows
+//     bit (z > 0 after rounding to BF16), 8 bytes per row of 64; messages' bits are kept
+//     slot by slot [6][nodes];
+//   * a tile is 128 nodes, whose messages are computed slot by slot, or 128 edges, whose
+//     messages are computed direction by direction.  So a thread sums relu(z) of its node
+//     in registers, and the input gradients of a node's (edge's) messages add up in
+//     tensor memory;
+//   * a map's input gradient and weight gradient share the staged tile, and an edge's two
+//     source rows of the messages are the end rows of the edge update below.
+// Thread mapping of staged rows: q8 = lane mod 8 is the 16-byte chunk, the row is
+// 4 warp + lane / 8 + 32 j, j = 0 .. 3.
+constexpr int SLOTS = MAXDEG;
 
 // z's sign bit of the backward's mask: positive after rounding to BF16 (2^-133 is
 // the smallest BF16 number; 2^-134 and below round to zero).
@@ -339,113 +352,18 @@ __device__ __forceinline__ uint4 mask_bf16x8(uint4 v, uint32_t bits)
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// 4 FP32 values rounded to BF16, the columns whose mask bit is 0 cleared.
+__device__ __forceinline__ uint2 mask_f32x4(float4 v, uint32_t bits)
+{
+    uint32_t a = pack_bf2(v.x, v.y), b = pack_bf2(v.z, v.w);
+    a &= (bits & 1u ? 0xFFFFu : 0u) | (bits & 2u ? 0xFFFF0000u : 0u);
+    b &= (bits & 4u ? 0xFFFFu : 0u) | (bits & 8u ? 0xFFFF0000u : 0u);
+    return make_uint2(a, b);
+}
+
 __device__ __forceinline__ uint32_t mask_byte(const uint2* mask, size_t row, int kc)
 {
     return (reinterpret_cast<const uint8_t*>(mask + row))[kc];
-}
-
-// Messages: rows [h[src] | e[edge]] of 21 target nodes, m = sum over a node's slots of
-// relu(z) (FP32, slot order) as BF16, and the mask bits of row (node, slot).
-// in_tab [N][6]: (source node, edge) of every slot, -1 where empty.
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD)
-msg_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* __restrict__ h, const bf16* __restrict__ e,
-               const bf16* __restrict__ Wpk, const float* __restrict__ bias, bf16* __restrict__ m, uint2* __restrict__ mask,
-               int* err)
-{
-    extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char* As = tc_smem;                         // [16 row groups][16 k-chunks][8 rows][16 B], then FP32 rows
-    unsigned char* Ws = tc_smem + TC_A_FWD;              // [8 output groups][16 k-chunks][8 outputs][16 B]
-    __shared__ __align__(8) uint64_t bar_w, bar_mma;
-    __shared__ uint32_t tmem_sh;
-    __shared__ const unsigned char* rowp[2][2][TC_ROWS]; // gathered row halves of this and the next tile (NULL: no row)
-    __shared__ float bias_sm[HD];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid < HD) bias_sm[tid] = bias[tid];
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, Wpk, HD * KIN * 2);
-    const uint32_t tmem = tmem_sh;
-    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);
-    const int ntiles = (nodes + TILE_NODES - 1) / TILE_NODES;
-    uint32_t phase = 0;
-    auto lookup = [&](int t, int buf) {
-        const int row = tid & (TC_ROWS - 1), hf = tid >> 7, k = row / NODE_ROWS, n = t * TILE_NODES + k;
-        const unsigned char* p = nullptr;
-        if (k < TILE_NODES && n < nodes) {
-            const int b = n / N, l = n - b * N;
-            const int2 s = in_tab[l * NODE_ROWS + row - k * NODE_ROWS];
-            if (s.x >= 0)
-                p = reinterpret_cast<const unsigned char*>(hf == 0 ? h + ((size_t)b * N + s.x) * HD : e + ((size_t)b * E + s.y) * HD);
-        }
-        rowp[buf][hf][row] = p;
-    };
-    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
-    int buf = 0;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
-        __syncthreads();                                    // this tile's row pointers staged; the last epilogue done
-        for (int i = tid; i < 16 * TC_ROWS; i += TC_THREADS) {   // chunk i: row (i >> 7) * 8 + (i & 7), k-chunk (i >> 3) & 15
-            const int kc = (i >> 3) & 15, row = ((i >> 7) << 3) | (i & 7);
-            const unsigned char* p = rowp[buf][kc >> 3][row];
-            cp_async16(As + i * 16, p ? p + (kc & 7) * 16 : reinterpret_cast<const unsigned char*>(Wpk), p != nullptr);
-        }
-        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // visible to the tensor core
-        tc_fence_before();
-        __syncthreads();                                    // also: the previous tile's TMEM reads are done
-        tc_fence_after();
-        if (tid == 0) {
-#pragma unroll
-            for (int ks = 0; ks < KIN / 16; ++ks)
-                tc_mma(tmem, tc_desc(smem_u32(As) + ks * 256, 128, 16 * 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 16 * 128),
-                       IDESC, ks > 0 ? 1u : 0u);
-            tc_commit(&bar_mma);
-        }
-        const bool ok = mbar_wait(&bar_mma, phase);
-        phase ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        tc_fence_after();
-        // warp w: accumulator rows 32 (w mod 4) .. + 31, columns 32 (w / 4) .. + 31: relu(z) to the consumed
-        // operand tile as FP32 rows of 256 bytes (16-byte chunks swizzled by row)
-        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row = q * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-        uint32_t bits = 0u;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            const int c0 = cb + 16 * hh;
-            float z[16];
-            tmem_ld16(tl + c0, z);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                z[i] += bias_sm[c0 + i];
-                bits |= positive_bf16(z[i]) << (16 * hh + i);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<float4*>(As + row * 256 + ((((c0 >> 2) + c) ^ (row & 7)) << 4)) =
-                    make_float4(fmaxf(z[4 * c], 0.f), fmaxf(z[4 * c + 1], 0.f), fmaxf(z[4 * c + 2], 0.f), fmaxf(z[4 * c + 3], 0.f));
-        }
-        if (mask && rowp[buf][0][row])
-            reinterpret_cast<uint32_t*>(mask + (size_t)tile * TILE_NODES * NODE_ROWS + row)[warp >> 2] = bits;
-        __syncthreads();
-        for (int i = tid; i < TILE_NODES * (HD / 2); i += TC_THREADS) {      // node i / 32 of the tile, column pair i mod 32
-            const int k = i >> 5, cp = i & 31, n = tile * TILE_NODES + k;
-            if (n >= nodes) break;
-            float x = 0.f, y = 0.f;
-#pragma unroll
-            for (int s = 0; s < NODE_ROWS; ++s) {
-                const int r = k * NODE_ROWS + s;
-                if (!rowp[buf][0][r]) continue;
-                const float2 v = *reinterpret_cast<const float2*>(As + r * 256 + (((cp >> 1) ^ (r & 7)) << 4) + (cp & 1) * 8);
-                x += v.x;
-                y += v.y;
-            }
-            reinterpret_cast<uint32_t*>(m + (size_t)n * HD)[cp] = pack_bf2(x, y);
-        }
-    }
-    tc_teardown(tmem, 64, failed, err);
 }
 
 // Sum of two BF16 rows' chunk, rounded to BF16.
@@ -461,102 +379,232 @@ __device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b)
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Node and edge updates: Y = P0 + relu([P0 | second] W^T + bias) as BF16 and the mask
-// bits.  Nodes: second = m (rows of P1).  Edges (EDGE): second = h[i] + h[j], the sum
-// of the edge's end rows of P1 = h, formed while staging.
-template <bool EDGE>
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_FWD)
-upd_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ P1, const int2* __restrict__ ends, int N, int E,
-               const bf16* __restrict__ Wpk, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask,
-               int* err)
+// Node stage of a layer: m = sum over a node's slots of relu(Wm [h[src] | e] + bm) (FP32, slot
+// order) rounded to BF16, then hout = h + relu(Wu [h | m] + bu).  7 steps a tile (6
+// slots, the update), each staged while the step before is computed: two operand
+// buffers, a barrier a step.  in_tab [6][N]: (source node, edge) of every slot, -1 where
+// empty.  m non-NULL (training): m and the mask bits mm, mu are kept.
+constexpr int TC_SMEM_NODE_FWD = 4 * OP64 + 4 * W64, TC_CTAS_NODE_FWD = 2;
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_NODE_FWD)
+node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* __restrict__ h, const bf16* __restrict__ e,
+                const bf16* __restrict__ Wm, const float* __restrict__ bm, const bf16* __restrict__ Wu, const float* __restrict__ bu,
+                bf16* __restrict__ hout, bf16* __restrict__ m, uint2* __restrict__ mm, uint2* __restrict__ mu, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char* As = tc_smem;                         // [16 row groups][16 k-chunks][8 rows][16 B]
-    unsigned char* Ws = tc_smem + TC_A_FWD;
+    unsigned char* const Ws = tc_smem + 4 * OP64;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
-    __shared__ const uint4* endp[2][2][TC_ROWS];         // EDGE: the two end rows of this and the next tile's edges
-    __shared__ float bias_sm[HD];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid < HD) bias_sm[tid] = bias[tid];
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, Wpk, HD * KIN * 2);
+    __shared__ float bias[2][HD];
+    __shared__ unsigned char used[2][TC_ROWS];              // slot not empty (per operand buffer)
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
+    if (tid < HD) bias[0][tid] = bm[tid];
+    else if (tid < 2 * HD) bias[1][tid - HD] = bu[tid - HD];
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, Wm, 2 * W64, Wu, 2 * W64);
     const uint32_t tmem = tmem_sh;
-    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);
-    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
-    uint32_t phase = 0;
-    auto lookup = [&](int t, int buf) {
-        if (!EDGE) return;
-        const int row = tid & (TC_ROWS - 1), which = tid >> 7, r = t * TC_ROWS + row;
-        const uint4* p = nullptr;
-        if (r < rows) {
-            const int b = r / E, l = r - b * E;
-            const int2 ij = ends[l];
-            p = reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + (which == 0 ? ij.x : ij.y)) * HD);
+    const int ntiles = (nodes + TC_ROWS - 1) / TC_ROWS;
+    const int q = warp & 3, row = q * 32 + lane, cb = (warp >> 2) * (HD / 2);       // epilogue: accumulator row, first column
+    const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + cb;
+    // what is staged next: tile lt, step ls, the table entries of this thread's rows
+    int lt = blockIdx.x, ls = 0, ln[4], lb[4];
+    int2 ent[4];
+    auto entries = [&]() {
+        if (lt >= ntiles || ls >= SLOTS) return;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (ls == 0) {
+                const int n = lt * TC_ROWS + srow + 32 * j;
+                lb[j] = n < nodes ? n / N : -1;
+                ln[j] = n - lb[j] * N;
+            }
+            ent[j] = lb[j] >= 0 ? in_tab[ls * N + ln[j]] : make_int2(-1, -1);
         }
-        endp[buf][which][row] = p;
     };
-    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
-    int buf = 0;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
-        const int r0 = tile * TC_ROWS;
-        __syncthreads();
-        if (EDGE) {
-            for (int i = tid; i < 8 * TC_ROWS; i += TC_THREADS) {        // first half: chunk kc of row, consecutive rows of P0
-                const int kc = (i >> 3) & 7, row = ((i >> 6) << 3) | (i & 7), r = r0 + row;
-                cp_async16(As + (((row >> 3) * 16 + kc) * 8 + (row & 7)) * 16, P0 + (size_t)(r < rows ? r : 0) * HD + kc * 8, r < rows);
-            }
+    auto stage = [&](int buf) {
+        if (lt >= ntiles) return;
+        unsigned char* A = tc_smem + buf * 2 * OP64;
 #pragma unroll
-            for (int j = 0; j < 8 * TC_ROWS / TC_THREADS; ++j) {         // second half: the sum of the end rows
-                const int i = tid + j * TC_THREADS, kc = (i >> 3) & 7, row = ((i >> 6) << 3) | (i & 7);
-                const uint4 *p = endp[buf][0][row], *q = endp[buf][1][row];
-                *reinterpret_cast<uint4*>(As + (((row >> 3) * 16 + 8 + kc) * 8 + (row & 7)) * 16) =
-                    p ? add_bf16x8(p[kc], q[kc]) : make_uint4(0u, 0u, 0u, 0u);
-            }
-        } else {
-            for (int i = tid; i < 16 * TC_ROWS; i += TC_THREADS) {
-                const int kc = (i >> 3) & 15, row = ((i >> 7) << 3) | (i & 7), r = r0 + row;
-                cp_async16(As + i * 16, (kc < 8 ? P0 : P1) + (size_t)(r < rows ? r : 0) * HD + (kc & 7) * 8, r < rows);
+        for (int j = 0; j < 4; ++j) {
+            const int r = srow + 32 * j;
+            if (ls < SLOTS) {
+                const bool v = ent[j].x >= 0;
+                cp_async16_l1(op_at(A, q8, r), h + (v ? (size_t)lb[j] * N + ent[j].x : 0) * HD + q8 * 8, v);
+                cp_async16(op_at(A, 8 + q8, r), e + (v ? (size_t)lb[j] * E + ent[j].y : 0) * HD + q8 * 8, v);
+                if (q8 == 0) used[buf][r] = v;
+            } else {
+                const int n = lt * TC_ROWS + r;
+                cp_async16(op_at(A, q8, r), h + (size_t)(n < nodes ? n : 0) * HD + q8 * 8, n < nodes);
             }
         }
-        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) {
+        if (++ls > SLOTS) { ls = 0; lt += gridDim.x; }
+        entries();
+    };
+    entries();
+    if (!failed) stage(0);
+    uint32_t phase = 0;
+    int buf = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
+        const int r0 = tile * TC_ROWS;
+        float acc[HD / 2];
 #pragma unroll
-            for (int ks = 0; ks < KIN / 16; ++ks)
-                tc_mma(tmem, tc_desc(smem_u32(As) + ks * 256, 128, 16 * 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 16 * 128),
-                       IDESC, ks > 0 ? 1u : 0u);
+        for (int i = 0; i < HD / 2; ++i) acc[i] = 0.f;
+        for (int s = 0; s < SLOTS; ++s, buf ^= 1) {
+            if ((failed = tc_ready(!ok))) break;
+            unsigned char* const A = tc_smem + buf * 2 * OP64;
+            if (tid == 0) {
+                mma_forward(tmem, A, Ws);
+                tc_commit(&bar_mma);
+            }
+            stage(buf ^ 1);
+            ok = mbar_wait(&bar_mma, phase);
+            phase ^= 1u;
+            tc_fence_after();
+            const bool v = used[buf][row];
+            uint32_t bits = 0u;
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                float z[16];
+                tmem_ld16(tl + 16 * hh, z);
+                tmem_ld_wait();
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    z[i] += bias[0][cb + 16 * hh + i];
+                    bits |= positive_bf16(z[i]) << (16 * hh + i);
+                    acc[16 * hh + i] += v ? fmaxf(z[i], 0.f) : 0.f;
+                }
+            }
+            if (m && r0 + row < nodes) reinterpret_cast<uint32_t*>(mm + (size_t)s * nodes + r0 + row)[warp >> 2] = bits;
+        }
+        if (failed) break;
+        // m: into the update's operand, and (training) to memory through the last slot's consumed operand
+        uint32_t w[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) w[i] = pack_bf2(acc[2 * i], acc[2 * i + 1]);
+        unsigned char* const A = tc_smem + buf * 2 * OP64;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint4*>(op_at(A, 8 + (cb >> 3) + c, row)) = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+        if (m)
+            store_bf16x32(tc_smem + (buf ^ 1) * 2 * OP64 + warp * 2048, w, m + (size_t)(r0 + q * 32) * HD + cb, nodes - r0 - q * 32, lane);
+        if ((failed = tc_ready(!ok))) break;
+        if (tid == 0) {
+            mma_forward(tmem, A, Ws + 2 * W64);
             tc_commit(&bar_mma);
         }
-        const bool ok = mbar_wait(&bar_mma, phase);
+        stage(buf ^ 1);
+        ok = mbar_wait(&bar_mma, phase);
         phase ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
         tc_fence_after();
-        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row0 = r0 + q * 32, row = q * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-        unsigned char* stage = As + warp * 4096;
-        uint32_t yw[HD / 4], bits = 0u;
+        uint32_t bits = 0u;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
             const int c0 = cb + 16 * hh;
             float z[16];
-            tmem_ld16(tl + c0, z);
+            tmem_ld16(tl + 16 * hh, z);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                z[i] += bias[1][c0 + i];
+                bits |= positive_bf16(z[i]) << (16 * hh + i);
+            }
+#pragma unroll
+            for (int kc = 0; kc < 2; ++kc) {                // the residual input is staged: chunks c0 / 8 and c0 / 8 + 1
+                const uint4 b4 = *reinterpret_cast<const uint4*>(op_at(A, (c0 >> 3) + kc, row));
+                const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 bb = unpack_bf2(bw[i]);
+                    w[8 * hh + 4 * kc + i] = pack_bf2(bb.x + fmaxf(z[8 * kc + 2 * i], 0.f), bb.y + fmaxf(z[8 * kc + 2 * i + 1], 0.f));
+                }
+            }
+        }
+        if (m && r0 + row < nodes) reinterpret_cast<uint32_t*>(mu + r0 + row)[warp >> 2] = bits;
+        // through the consumed half of m; the next step's barrier comes before this buffer is staged again
+        store_bf16x32(A + OP64 + warp * 2048, w, hout + (size_t)(r0 + q * 32) * HD + cb, nodes - r0 - q * 32, lane);
+        buf ^= 1;
+    }
+    failed = __syncthreads_or(failed || !ok);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc_teardown(tmem, 64, failed, err);
+}
+
+// Edge update: Y = P0 + relu([P0 | h[i] + h[j]] W^T + bias) as BF16 and the mask bits;
+// the sum of the edge's end rows is formed while staging.
+constexpr int TC_SMEM_EDGE_FWD = 2 * OP64 + 2 * W64, TC_CTAS_EDGE_FWD = 4;
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_EDGE_FWD)
+edge_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ h, const int2* __restrict__ ends, int N, int E,
+                const bf16* __restrict__ W, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask, int* err)
+{
+    extern __shared__ __align__(128) unsigned char tc_smem[];
+    unsigned char *const As = tc_smem, *const Ws = tc_smem + 2 * OP64;
+    __shared__ __align__(8) uint64_t bar_w, bar_mma;
+    __shared__ uint32_t tmem_sh;
+    __shared__ int2 endn[2][TC_ROWS];                       // the two end nodes of this and the next tile's edges, -1: no row
+    __shared__ float bias_sm[HD];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
+    if (tid < HD) bias_sm[tid] = bias[tid];
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 64, Ws, W, 2 * W64, nullptr, 0);
+    const uint32_t tmem = tmem_sh;
+    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
+    const int q = warp & 3, row = q * 32 + lane, cb = (warp >> 2) * (HD / 2);
+    const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + cb;
+    uint32_t phase = 0;
+    auto lookup = [&](int t, int buf) {
+        if (t >= ntiles || tid >= TC_ROWS) return;
+        const int r = t * TC_ROWS + tid;
+        int2 ij = make_int2(-1, -1);
+        if (r < rows) {
+            const int b = r / E;
+            ij = ends[r - b * E];
+            ij.x += b * N;
+            ij.y += b * N;
+        }
+        endn[buf][tid] = ij;
+    };
+    lookup(blockIdx.x, 0);
+    __syncthreads();
+    int buf = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
+        const int r0 = tile * TC_ROWS;
+        uint4 a[4], b[4];                                   // every load before the first use
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int r = srow + 32 * j;
+            const int2 ij = endn[buf][r];
+            const bool v = ij.x >= 0;
+            cp_async16(op_at(As, q8, r), P0 + (size_t)(v ? r0 + r : 0) * HD + q8 * 8, v);
+            a[j] = b[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (v) {
+                a[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij.x * HD + q8 * 8);
+                b[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij.y * HD + q8 * 8);
+            }
+        }
+        lookup(tile + gridDim.x, buf ^ 1);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(op_at(As, 8 + q8, srow + 32 * j)) = add_bf16x8(a[j], b[j]);
+        tc_ready(false);
+        if (tid == 0) {
+            mma_forward(tmem, As, Ws);
+            tc_commit(&bar_mma);
+        }
+        const bool ok = mbar_wait(&bar_mma, phase);
+        phase ^= 1u;
+        tc_fence_after();
+        uint32_t yw[16], bits = 0u;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+            const int c0 = cb + 16 * hh;
+            float z[16];
+            tmem_ld16(tl + 16 * hh, z);
             tmem_ld_wait();
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 z[i] += bias_sm[c0 + i];
                 bits |= positive_bf16(z[i]) << (16 * hh + i);
             }
-            // the residual input is half 0 of this row, already staged: k-chunks c0/8 and c0/8 + 1
 #pragma unroll
-            for (int kc = 0; kc < 2; ++kc) {
-                const uint4 b4 = *reinterpret_cast<const uint4*>(As + (((row >> 3) * 16 + (c0 >> 3) + kc) * 128) + (row & 7) * 16);
+            for (int kc = 0; kc < 2; ++kc) {                // the residual input is staged: chunks c0 / 8 and c0 / 8 + 1
+                const uint4 b4 = *reinterpret_cast<const uint4*>(op_at(As, (c0 >> 3) + kc, row));
                 const uint32_t bw[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
@@ -566,393 +614,414 @@ upd_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ P
             }
         }
         if (mask && r0 + row < rows) reinterpret_cast<uint32_t*>(mask + r0 + row)[warp >> 2] = bits;
-        __syncthreads();                                   // every residual read before any slice is overwritten
-        store_bf16x32(stage, yw, Yout + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+        store_bf16x32(As + OP64 + warp * 2048, yw, Yout + (size_t)(r0 + q * 32) * HD + cb, rows - r0 - q * 32, lane);
+        failed = __syncthreads_or(!ok);                     // the operand is consumed
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     tc_teardown(tmem, 64, failed, err);
 }
 
-// ---- backward: input gradient dX = dZ W and weight gradient dW += dZ^T X of a tile
-// Shared memory: X [16 input groups][16 row groups][8 rows][16 B] (32 KB, the weight
-// gradient's A operand), dZ [16 row groups][8 k-chunks][8 rows][16 B] (16 KB), W^T
-// (one or both 8 KB halves of 64 inputs).  Tensor memory: columns 0..63 dW^T
-// accumulated over the CTA's tiles, 64..127 the current half of dX.  db: a thread
-// stages one 8-column chunk of every eighth row group and adds it up on the way.
-constexpr int BW_X = TC_ROWS * KIN * 2, BW_Z = TC_ROWS * HD * 2, BW_W = HD * HD * 2;
-constexpr int TC_SMEM_UPD_BWD = BW_X + BW_Z + 2 * BW_W, TC_SMEM_EDGE_BWD = BW_X + BW_Z + BW_W;
-constexpr int TC_CTAS_UPD_BWD = 3, TC_CTAS_EDGE_BWD = 3;
-
-__device__ __forceinline__ void bwd_mma_wgrad(uint32_t tmem, const unsigned char* Xs, const unsigned char* Zs, bool first)
+// ---- backward
+// Adds the BF16 values of a staged dZ chunk to this thread's column sums.
+__device__ __forceinline__ void add_db(float* db, uint32_t a, uint32_t b)
 {
-    constexpr uint32_t IDESC = tc_idesc_bf16(KIN, HD) | (1u << 15) | (1u << 16);   // M = 128 inputs, N = 64, both MN-major
-#pragma unroll
-    for (int ks = 0; ks < TC_ROWS / 16; ++ks)
-        tc_mma(tmem, tc_desc(smem_u32(Xs) + ks * 256, 128, 16 * 128), tc_desc(smem_u32(Zs) + ks * 2048, 1024, 128), IDESC,
-               first && ks == 0 ? 0u : 1u);
+    const float2 x = unpack_bf2(a), y = unpack_bf2(b);
+    db[0] += x.x;
+    db[1] += x.y;
+    db[2] += y.x;
+    db[3] += y.y;
 }
 
-__device__ __forceinline__ void bwd_mma_input(uint32_t tmem, const unsigned char* Zs, const unsigned char* Wh)
+// A CTA's partial of a bias gradient: a thread's 8 column sums are those of chunk q8
+// (f32 false) or of the 4 columns from 4 q8 and from 32 + 4 q8 (true); the 32 threads of a
+// column in thread order, through 8 KB of shared memory.
+__device__ __forceinline__ void db_partial(float* P, const float (&db)[8], bool f32, float* sm)
 {
-    constexpr uint32_t IDESC = tc_idesc_bf16(TC_ROWS, HD);                         // one half: 64 inputs
+    const int tid = threadIdx.x, q8 = tid & 7, slot = tid >> 3;
+    __syncthreads();
 #pragma unroll
-    for (int ks = 0; ks < HD / 16; ++ks)
-        tc_mma(tmem + HD, tc_desc(smem_u32(Zs) + ks * 256, 128, 8 * 128), tc_desc(smem_u32(Wh) + ks * 256, 128, 8 * 128), IDESC,
-               ks > 0 ? 1u : 0u);
-}
-
-// Adds the 8 BF16 values of a staged dZ chunk to this thread's column sums.
-__device__ __forceinline__ void add_db(float (&db)[8], uint4 z)
-{
-    const uint32_t w[4] = {z.x, z.y, z.z, z.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 v = unpack_bf2(w[i]);
-        db[2 * i] += v.x;
-        db[2 * i + 1] += v.y;
-    }
-}
-
-// The CTA's partials: dW [64][128] from tensor memory (lane = input), db [64] from the
-// threads' column sums (thread: chunk kc of 8 columns; the 32 threads of a chunk in
-// thread order), through `sm` (8 KB of shared memory).
-__device__ __forceinline__ void bwd_partials(uint32_t tmem, float* P, const float (&db)[8], int kc, float* sm)
-{
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (warp < 4) {
-        const int in = warp * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll
-        for (int c0 = 0; c0 < HD; c0 += 16) {
-            float d[16];
-            tmem_ld16(tl + c0, d);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) P[(c0 + i) * KIN + in] = d[i];
-        }
-    }
-    __syncthreads();                                        // the last tile's staging slices are read
-    // threads of chunk kc: 8 per warp in the 4 warps with warp & 1 == kc >> 2
-    const int slot = (warp >> 1) * 8 + (lane & 7);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) sm[(kc * 8 + i) * 32 + slot] = db[i];
+    for (int i = 0; i < 8; ++i) sm[(f32 ? (i >> 2) * 32 + q8 * 4 + (i & 3) : q8 * 8 + i) * 32 + (slot ^ (q8 << 2))] = db[i];
     __syncthreads();
     if (tid < HD) {
         float s = 0.f;
-        for (int j = 0; j < 32; ++j) s += sm[tid * 32 + j];
+        const int x = (f32 ? (tid & 31) >> 2 : tid >> 3) << 2;
+        for (int j = 0; j < 32; ++j) s += sm[tid * 32 + (j ^ x)];
         P[HD * KIN + tid] = s;
     }
 }
 
-// Node and edge updates.  EDGE: dZ = de & mask, de += dX[:, :64] in place, ds = dX[:, 64:]
-// (FP32); X = [e | h_i + h_j].  Nodes: dh += sum over the node's edges of ds (inc order; inc NULL: none),
-// dZ = dh & mask, dh += dX[:, :64], dm = dX[:, 64:] rounded to BF16 (the one form that
-// the messages' dZ = dm & mask takes it in); X = [h | m].
-template <bool EDGE>
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_UPD_BWD)
-upd_bwd_kernel(int rows, int N, int E, const uint2* __restrict__ mask, float* g, const bf16* __restrict__ P0,
-               const bf16* __restrict__ P1, const int2* __restrict__ ends, const int* __restrict__ inc, float* ds,
-               bf16* __restrict__ dm, const bf16* __restrict__ WTpk, float* __restrict__ part, int* err)
+// A CTA's partial of dW [64][128] from tensor memory (lane = input).
+__device__ __forceinline__ void dw_partial(uint32_t tcol, float* P, int warp, int lane)
+{
+    const int q = warp & 3, in = q * 32 + lane, cb = (warp >> 2) * (HD / 2);
+    const uint32_t tl = tcol + ((uint32_t)(q * 32) << 16) + cb;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        float d[16];
+        tmem_ld16(tl + 16 * hh, d);
+        tmem_ld_wait();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) P[(cb + 16 * hh + i) * KIN + in] = d[i];
+    }
+}
+
+constexpr int TC_CTAS_BWD = 2;
+
+// Nodes.  PRE, messages of a layer: dh[n] += sum over the messages that n sends of
+// (dm[target] & mask) Wm[:, :64], slot by slot (out_tab [6][N]: target node * 8 + its slot,
+// -1 where empty), and dh[n] += sum over n's edges of ds (inc [6][N], NULL: none).
+// POST, node update of the layer below: dZ = dh & mu, dh += dX[:, :64], dmo = dX[:, 64:]
+// rounded to BF16 (the one form that the messages' dZ = dm & mask takes it in), weight
+// gradient with X = [h | m].  A slot's rows are loaded while the slot before is
+// computed; two operand buffers.
+constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64;
+template <bool PRE, bool POST>
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
+node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
+                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* __restrict__ ds, float* dh,
+                const uint2* __restrict__ mu, const bf16* __restrict__ h, const bf16* __restrict__ m, const bf16* __restrict__ WuT,
+                bf16* __restrict__ dmo, float* __restrict__ part, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char *Xs = tc_smem, *Zs = tc_smem + BW_X, *Ws = Zs + BW_Z;
+    unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 2 * OP64, *const Ws = tc_smem + 4 * OP64;     // Ws: Wm^T (h half), Wu^T
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk, 2 * BW_W);
-    const uint32_t tmem = tmem_sh;
-    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
-    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;     // a warp stages 8 rows x 4 chunks at a time
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 256, Ws, WmT, PRE ? W64 : 0, WuT, POST ? 2 * W64 : 0);
+    const uint32_t tmem = tmem_sh, tdw = tmem + KIN;        // dX: columns 0..127, dW^T: 128..191
+    const int ntiles = (nodes + TC_ROWS - 1) / TC_ROWS;
     float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
-        const int r0 = tile * TC_ROWS;
+        int nb[4], nl[4];                                   // graph (-1: no row) and node in the graph of this thread's rows
+        float4 ga[4], gb[4];                                // dh: columns 4 q8 .. and 32 + 4 q8 ..
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {                       // X
-            const int u = warp + 8 * j, rg = u >> 2, kc = (u & 3) * 4 + q4, row = rg * 8 + r8, r = r0 + row;
-            unsigned char* dst = Xs + (kc * 16 + rg) * 128 + r8 * 16;
-            const bool v = r < rows;
-            if (!EDGE || (u & 2) == 0) {
-                cp_async16(dst, (kc < 8 ? P0 : P1) + (size_t)(v ? r : 0) * HD + (kc & 7) * 8, v);
-            } else {
-                uint4 s = make_uint4(0u, 0u, 0u, 0u);
-                if (v) {
-                    const int b = r / E;
-                    const int2 ij = ends[r - b * E];
-                    s = add_bf16x8(*reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + ij.x) * HD + (kc & 7) * 8),
-                                   *reinterpret_cast<const uint4*>(P1 + ((size_t)b * N + ij.y) * HD + (kc & 7) * 8));
-                }
-                *reinterpret_cast<uint4*>(dst) = s;
+        for (int j = 0; j < 4; ++j) {
+            const int n = tile * TC_ROWS + srow + 32 * j;
+            const bool v = n < nodes;
+            nb[j] = v ? n / N : -1;
+            nl[j] = n - nb[j] * N;
+            if (POST) {
+                cp_async16(op_at(Xs, q8, srow + 32 * j), h + (size_t)(v ? n : 0) * HD + q8 * 8, v);
+                cp_async16(op_at(Xs, 8 + q8, srow + 32 * j), m + (size_t)(v ? n : 0) * HD + q8 * 8, v);
+            }
+            ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (v) {
+                ga[j] = reinterpret_cast<const float4*>(dh + (size_t)n * HD)[q8];
+                gb[j] = reinterpret_cast<const float4*>(dh + (size_t)n * HD)[8 + q8];
             }
         }
+        bool ok = true;
+        if (PRE) {
+            uint4 z[4];
+            uint32_t mk[4];
+            auto load = [&](int s) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {                       // dZ: chunk kz of row groups (warp >> 1) + 4 j
-            const int rg = (warp >> 1) + 4 * j, row = rg * 8 + r8, r = r0 + row;
-            uint4 z = make_uint4(0u, 0u, 0u, 0u);
-            if (r < rows) {
-                float4* gp = reinterpret_cast<float4*>(g + (size_t)r * HD + kz * 8);
-                float4 a = gp[0], b = gp[1];
-                if (!EDGE && inc) {
-                    const int bi = r / N;
-                    const int* il = inc + (r - bi * N) * NODE_ROWS;
-                    float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
-#pragma unroll
-                    for (int s = 0; s < NODE_ROWS; ++s) {
-                        const int ed = il[s];
-                        if (ed < 0) continue;
-                        const float4* dp = reinterpret_cast<const float4*>(ds + ((size_t)bi * E + ed) * HD + kz * 8);
-                        const float4 x = dp[0], y = dp[1];
-                        s0.x += x.x; s0.y += x.y; s0.z += x.z; s0.w += x.w;
-                        s1.x += y.x; s1.y += y.y; s1.z += y.z; s1.w += y.w;
+                for (int j = 0; j < 4; ++j) {
+                    const int t = nb[j] >= 0 ? out_tab[s * N + nl[j]] : -1;
+                    z[j] = make_uint4(0u, 0u, 0u, 0u);
+                    mk[j] = 0u;
+                    if (t >= 0) {
+                        const size_t n = (size_t)nb[j] * N + (t >> 3);
+                        z[j] = *reinterpret_cast<const uint4*>(dm + n * HD + q8 * 8);
+                        mk[j] = mask_byte(mm, (size_t)(t & 7) * nodes + n, q8);
                     }
-                    a.x += s0.x; a.y += s0.y; a.z += s0.z; a.w += s0.w;
-                    b.x += s1.x; b.y += s1.y; b.z += s1.z; b.w += s1.w;
-                    gp[0] = a;                              // the epilogue adds dX to it
-                    gp[1] = b;
                 }
-                z = mask_bf16x8(make_uint4(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w), pack_bf2(b.x, b.y), pack_bf2(b.z, b.w)),
-                                mask_byte(mask, r, kz));
-            }
-            add_db(db, z);
-            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
-        }
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        const int q = warp & 3, row0 = r0 + q * 32, cb = (warp >> 2) * (HD / 2);
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
-        unsigned char* stage = Xs + warp * 4096;
+            };
+            load(0);
+            for (int s = 0; s < SLOTS; ++s) {
+                unsigned char* const Z = Zs + (s & 1) * OP64;     // its MMA before last is done: the wait below
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
+                for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(op_at(Z, q8, srow + 32 * j)) = mask_bf16x8(z[j], mk[j]);
+                // (the copies of X are not waited for here)
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                tc_fence_before();
+                __syncthreads();
+                tc_fence_after();
+                if (tid == 0) {
+                    mma_input<HD>(tmem, Z, Ws, s > 0);
+                    tc_commit(&bar_mma);
+                }
+                if (s + 1 < SLOTS) load(s + 1);
+                if (inc) {
+                    float4 x[4], y[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int ed = nb[j] >= 0 ? inc[s * N + nl[j]] : -1;
+                        x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (ed >= 0) {
+                            const float4* dp = reinterpret_cast<const float4*>(ds + ((size_t)nb[j] * E + ed) * HD);
+                            x[j] = dp[q8];
+                            y[j] = dp[8 + q8];
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        ga[j] = add4(ga[j], x[j]);
+                        gb[j] = add4(gb[j], y[j]);
+                    }
+                }
+                ok = mbar_wait(&bar_mma, phase) && ok;
+                phase ^= 1u;
+            }
+            if ((failed = __syncthreads_or(!ok))) break;
+            tc_fence_after();
+            tmem_to_tile(Zs, tmem, warp, lane);
+            tc_fence_before();
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                ga[j] = add4(ga[j], *tile_f32(Zs, srow + 32 * j, q8));
+                gb[j] = add4(gb[j], *tile_f32(Zs, srow + 32 * j, 8 + q8));
+            }
+            __syncthreads();
+        }
+        if (POST) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int n = tile * TC_ROWS + srow + 32 * j;
+                const uint2 mk = nb[j] >= 0 ? mu[n] : make_uint2(0u, 0u);
+                const uint2 a = mask_f32x4(ga[j], mk.x >> (4 * q8)), b = mask_f32x4(gb[j], mk.y >> (4 * q8));
+                add_db(db, a.x, a.y);
+                add_db(db + 4, b.x, b.y);
+                *reinterpret_cast<uint2*>(op_at(Zs, q8 >> 1, srow + 32 * j) + (q8 & 1) * 8) = a;
+                *reinterpret_cast<uint2*>(op_at(Zs, 4 + (q8 >> 1), srow + 32 * j) + (q8 & 1) * 8) = b;
+            }
+            tc_ready(false);
             if (tid == 0) {
-                bwd_mma_input(tmem, Zs, Ws + half * BW_W);
-                if (half == 0) bwd_mma_wgrad(tmem, Xs, Zs, first);
+                mma_input<KIN>(tmem, Zs, Ws + (PRE ? W64 : 0), false);
+                mma_wgrad(tdw, Xs, Zs, !first);
                 tc_commit(&bar_mma);
             }
-            const bool ok = mbar_wait(&bar_mma, phase);
+            first = false;
+            ok = mbar_wait(&bar_mma, phase);
             phase ^= 1u;
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                break;
-            }
+            if ((failed = __syncthreads_or(!ok))) break;
             tc_fence_after();
-            uint32_t w[16];
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                float d[16];
-                tmem_ld16(tl + 16 * hh, d);
-                tmem_ld_wait();
-                if (half == 0 || EDGE) {
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        stage_f32(stage, lane, 4 * hh + c, make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]));
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) w[8 * hh + i] = pack_bf2(d[2 * i], d[2 * i + 1]);
-                }
-            }
-            if (half == 0) flush_add_f32x32(stage, g + (size_t)row0 * HD + cb, HD, rows - row0, lane);
-            else if (EDGE) flush_f32x32(stage, ds + (size_t)row0 * HD + cb, HD, rows - row0, lane);
-            else store_bf16x32(stage, w, dm + (size_t)row0 * HD + cb, HD, rows - row0, lane);
+            tmem_to_tile(Xs, tmem, warp, lane);
+            tmem_to_tile(Zs, tmem + HD, warp, lane);
             tc_fence_before();
-            __syncthreads();                                // dX read, the slices free: the next half or tile
+            __syncthreads();
             tc_fence_after();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int r = srow + 32 * j, n = tile * TC_ROWS + r;
+                ga[j] = add4(ga[j], *tile_f32(Xs, r, q8));
+                gb[j] = add4(gb[j], *tile_f32(Xs, r, 8 + q8));
+                const float4 a = *tile_f32(Zs, r, q8), b = *tile_f32(Zs, r, 8 + q8);
+                if (nb[j] < 0) continue;
+                reinterpret_cast<uint2*>(dmo + (size_t)n * HD)[q8] = make_uint2(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w));
+                reinterpret_cast<uint2*>(dmo + (size_t)n * HD)[8 + q8] = make_uint2(pack_bf2(b.x, b.y), pack_bf2(b.z, b.w));
+            }
         }
-        first = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int n = tile * TC_ROWS + srow + 32 * j;
+            if (nb[j] < 0) continue;
+            reinterpret_cast<float4*>(dh + (size_t)n * HD)[q8] = ga[j];
+            reinterpret_cast<float4*>(dh + (size_t)n * HD)[8 + q8] = gb[j];
+        }
+        __syncthreads();                                    // the tiles are read: the next staging
     }
-    if (!failed) bwd_partials(tmem, part + (size_t)blockIdx.x * WPART, db, kz, reinterpret_cast<float*>(Xs));
-    tc_teardown(tmem, 128, failed, err);
+    if (POST && !failed) {
+        dw_partial(tdw, part + (size_t)blockIdx.x * WPART, warp, lane);
+        db_partial(part + (size_t)blockIdx.x * WPART, db, true, reinterpret_cast<float*>(Xs));
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc_teardown(tmem, 256, failed, err);
 }
 
-// Messages, edge half: rows 2e and 2e + 1 are the two directions of edge e; dZ = dm[tgt]
-// & mask, de[e] += dX[2e][64:] + dX[2e + 1][64:] (set: =), weight gradient with X = [h[src] | e].
-// msg_tab [2E]: (source node, mask row = target node * 6 + slot).
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_EDGE_BWD)
-msg_bwd_edge_kernel(int rows, int N, int E, const int2* __restrict__ msg_tab, const uint2* __restrict__ mask,
-                    const bf16* __restrict__ dm, const bf16* __restrict__ h, const bf16* __restrict__ e,
-                    const bf16* __restrict__ WTpk, float* de, int set, float* __restrict__ part, int* err)
+// Edges.  Messages of a layer, edge half, both directions d of an edge (msg_tab [E]: source
+// node and target node * 8 + its slot of either): dZ_d = dm[target] & mask,
+// de += sum_d dX_d[:, 64:] (set: =), weight gradient with X_d = [h[src_d] | e].
+// POST, edge update of the layer below: dZ = de & me, de += dX[:, :64], ds = dX[:, 64:] (FP32),
+// weight gradient with X = [eb | h_i + h_j], whose end rows are the messages' source rows.
+// Operands R0 | R1 | R2: h[src_0], e, h[src_1], then (POST) eb in R1 and the sum in R2.
+// The two directions' weight gradients differ in the order of their halves ([R0 | R1] and
+// [R1 | R2]) and are kept apart in tensor memory.
+constexpr int TC_SMEM_EDGE_BWD = 5 * OP64 + 3 * W64;
+template <bool POST>
+__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
+edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
+                const bf16* __restrict__ h, const bf16* __restrict__ e, const bf16* __restrict__ WmT, float* de, int set,
+                const uint2* __restrict__ me, const bf16* __restrict__ eb, const bf16* __restrict__ WeT, float* __restrict__ ds,
+                float* __restrict__ partm, float* __restrict__ parte, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char *Xs = tc_smem, *Zs = tc_smem + BW_X, *Ws = Zs + BW_Z;
+    unsigned char *const R0 = tc_smem, *const R1 = R0 + OP64, *const R2 = R1 + OP64, *const Zs = R2 + OP64, *const Ws = Zs + 2 * OP64;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
-    __shared__ int4 rowt[2][TC_ROWS];                       // this and the next tile: source row, edge row, target row, mask row
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk + HD * HD, BW_W);
-    const uint32_t tmem = tmem_sh;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
+    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 256, Ws, WmT, W64, WeT, POST ? 2 * W64 : 0);
+    const uint32_t tmem = tmem_sh;                          // dX, then dWm^T of direction 0 and 1, dWe^T: 64 columns each
     const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
-    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;
-    float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const size_t nodes = (size_t)(rows / E) * N;
+    float dbm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dbe[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
-    auto lookup = [&](int t, int buf) {
-        if (tid >= TC_ROWS) return;
-        const int r = t * TC_ROWS + tid;
-        int4 v = make_int4(-1, 0, 0, 0);
-        if (r < rows) {
-            const int b = r / (2 * E), l = r - b * 2 * E;
-            const int2 s = msg_tab[l];
-            v = make_int4(b * N + s.x, b * E + (l >> 1), b * N + s.y / NODE_ROWS, b * N * NODE_ROWS + s.y);
-        }
-        rowt[buf][tid] = v;
-    };
-    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
-    int buf = 0;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
         const int r0 = tile * TC_ROWS;
-        __syncthreads();
+        int4 ent[4];
+        int bN[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int u = warp + 8 * j, rg = u >> 2, kc = (u & 3) * 4 + q4;
-            const int4 t = rowt[buf][rg * 8 + r8];
-            const bf16* p = kc < 8 ? h + (size_t)(t.x < 0 ? 0 : t.x) * HD : e + (size_t)t.y * HD;
-            cp_async16(Xs + (kc * 16 + rg) * 128 + r8 * 16, p + (kc & 7) * 8, t.x >= 0);
+        for (int j = 0; j < 4; ++j) {
+            const int r = r0 + srow + 32 * j, b = r / E;
+            bN[j] = b * N;
+            ent[j] = r < rows ? msg_tab[r - b * E] : make_int4(-1, 0, 0, 0);
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int rg = (warp >> 1) + 4 * j;
-            const int4 t = rowt[buf][rg * 8 + r8];
-            uint4 z = make_uint4(0u, 0u, 0u, 0u);
-            if (t.x >= 0)
-                z = mask_bf16x8(*reinterpret_cast<const uint4*>(dm + (size_t)t.z * HD + kz * 8), mask_byte(mask, t.w, kz));
-            add_db(db, z);
-            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
+            const int row = srow + 32 * j;
+            const bool v = ent[j].x >= 0;
+            cp_async16_l1(op_at(R0, q8, row), h + (v ? (size_t)bN[j] + ent[j].x : 0) * HD + q8 * 8, v);
+            cp_async16(op_at(R1, q8, row), e + (size_t)(v ? r0 + row : 0) * HD + q8 * 8, v);
+            cp_async16_l1(op_at(R2, q8, row), h + (v ? (size_t)bN[j] + ent[j].z : 0) * HD + q8 * 8, v);
         }
-        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        uint4 z0[4], z1[4];                                 // every load before the first use
+        uint32_t m0[4], m1[4];
+        float4 ga[4], gb[4];                                // de: columns 4 q8 .. and 32 + 4 q8 ..
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            z0[j] = z1[j] = make_uint4(0u, 0u, 0u, 0u);
+            m0[j] = m1[j] = 0u;
+            ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ent[j].x >= 0) {
+                const size_t r = r0 + srow + 32 * j, n0 = (size_t)bN[j] + (ent[j].y >> 3), n1 = (size_t)bN[j] + (ent[j].w >> 3);
+                z0[j] = *reinterpret_cast<const uint4*>(dm + n0 * HD + q8 * 8);
+                z1[j] = *reinterpret_cast<const uint4*>(dm + n1 * HD + q8 * 8);
+                m0[j] = mask_byte(mm, (ent[j].y & 7) * nodes + n0, q8);
+                m1[j] = mask_byte(mm, (ent[j].w & 7) * nodes + n1, q8);
+                if (!set) {
+                    ga[j] = reinterpret_cast<const float4*>(de + r * HD)[q8];
+                    gb[j] = reinterpret_cast<const float4*>(de + r * HD)[8 + q8];
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            z0[j] = mask_bf16x8(z0[j], m0[j]);
+            z1[j] = mask_bf16x8(z1[j], m1[j]);
+            add_db(dbm, z0[j].x, z0[j].y);
+            add_db(dbm + 4, z0[j].z, z0[j].w);
+            add_db(dbm, z1[j].x, z1[j].y);
+            add_db(dbm + 4, z1[j].z, z1[j].w);
+            *reinterpret_cast<uint4*>(op_at(Zs, q8, srow + 32 * j)) = z0[j];
+            *reinterpret_cast<uint4*>(op_at(Zs + OP64, q8, srow + 32 * j)) = z1[j];
+        }
+        tc_ready(false);
+        if (tid == 0) {
+            mma_input<HD>(tmem, Zs, Ws, false);
+            mma_input<HD>(tmem, Zs + OP64, Ws, true);
+            mma_wgrad(tmem + HD, R0, Zs, !first);
+            mma_wgrad(tmem + 2 * HD, R1, Zs + OP64, !first);
+            tc_commit(&bar_mma);
+        }
+        bool ok = mbar_wait(&bar_mma, phase);
+        phase ^= 1u;
+        if ((failed = __syncthreads_or(!ok))) break;
+        tc_fence_after();
+        if (POST) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int row = srow + 32 * j;
+                cp_async16(op_at(R1, q8, row), eb + (size_t)(ent[j].x >= 0 ? r0 + row : 0) * HD + q8 * 8, ent[j].x >= 0);
+                uint4* const s = reinterpret_cast<uint4*>(op_at(R2, q8, row));
+                *s = add_bf16x8(*reinterpret_cast<const uint4*>(op_at(R0, q8, row)), *s);
+            }
+        }
+        tmem_to_tile(Zs, tmem, warp, lane);
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (tid == 0) {
-            bwd_mma_input(tmem, Zs, Ws);
-            bwd_mma_wgrad(tmem, Xs, Zs, first);
-            tc_commit(&bar_mma);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            ga[j] = add4(ga[j], *tile_f32(Zs, srow + 32 * j, q8));
+            gb[j] = add4(gb[j], *tile_f32(Zs, srow + 32 * j, 8 + q8));
+        }
+        if (POST) {
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int row = srow + 32 * j;
+                const uint2 k = ent[j].x >= 0 ? me[r0 + row] : make_uint2(0u, 0u);
+                const uint2 a = mask_f32x4(ga[j], k.x >> (4 * q8)), b = mask_f32x4(gb[j], k.y >> (4 * q8));
+                add_db(dbe, a.x, a.y);
+                add_db(dbe + 4, b.x, b.y);
+                *reinterpret_cast<uint2*>(op_at(Zs, q8 >> 1, row) + (q8 & 1) * 8) = a;
+                *reinterpret_cast<uint2*>(op_at(Zs, 4 + (q8 >> 1), row) + (q8 & 1) * 8) = b;
+            }
+            tc_ready(false);
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                if (tid == 0) {
+                    mma_input<HD>(tmem, Zs, Ws + (1 + half) * W64, false);
+                    if (half == 0) mma_wgrad(tmem + 3 * HD, R1, Zs, !first);
+                    tc_commit(&bar_mma);
+                }
+                ok = mbar_wait(&bar_mma, phase);
+                phase ^= 1u;
+                if ((failed = __syncthreads_or(!ok))) break;      // also: the other half's tile is read
+                tc_fence_after();
+                tmem_to_tile(R0, tmem, warp, lane);
+                tc_fence_before();
+                __syncthreads();
+                tc_fence_after();
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int row = srow + 32 * j;
+                    const float4 a = *tile_f32(R0, row, q8), b = *tile_f32(R0, row, 8 + q8);
+                    if (half == 0) {
+                        ga[j] = add4(ga[j], a);
+                        gb[j] = add4(gb[j], b);
+                    } else if (ent[j].x >= 0) {
+                        reinterpret_cast<float4*>(ds + (size_t)(r0 + row) * HD)[q8] = a;
+                        reinterpret_cast<float4*>(ds + (size_t)(r0 + row) * HD)[8 + q8] = b;
+                    }
+                }
+            }
+            if (failed) break;
         }
         first = false;
-        const bool ok = mbar_wait(&bar_mma, phase);
-        phase ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        tc_fence_after();
-        const int q = warp & 3, row0 = r0 + q * 32, cb = (warp >> 2) * (HD / 2);
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
-        unsigned char* stage = Xs + warp * 4096;
 #pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            float d[16];
-            tmem_ld16(tl + 16 * hh, d);
-            tmem_ld_wait();
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                stage_f32(stage, lane, 4 * hh + c, make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]));
-        }
-        // a warp's 32 rows are 16 whole edges (row0 is even)
-        flush_pairs_f32x32(stage, de + (size_t)(row0 / 2) * HD + cb, HD, (rows - row0) / 2, lane, set != 0);
-        tc_fence_before();
-    }
-    __syncthreads();
-    tc_fence_after();
-    if (!failed) bwd_partials(tmem, part + (size_t)blockIdx.x * WPART, db, kz, reinterpret_cast<float*>(Xs));
-    tc_teardown(tmem, 128, failed, err);
-}
-
-// Messages, node half: the rows of 21 source nodes (out_tab [N][6]: mask row of the
-// message in a slot, -1 where empty); dh[n] += sum over n's slots of dX[:, :64].
-// dZ (16 KB), then the FP32 rows over it (32 KB); W^T half; 12 KB unused, so that 4 CTAs fit and no fifth
-constexpr int TC_SMEM_NODE_BWD = TC_ROWS * HD * 4 + BW_W + 12 * 1024;
-constexpr int TC_CTAS_NODE_BWD = 4;
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_NODE_BWD)
-msg_bwd_node_kernel(int nodes, int N, const int* __restrict__ out_tab, const uint2* __restrict__ mask,
-                    const bf16* __restrict__ dm, const bf16* __restrict__ WTpk, float* dh, int* err)
-{
-    extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char *Zs = tc_smem, *Ws = tc_smem + TC_ROWS * HD * 4;
-    __shared__ __align__(8) uint64_t bar_w, bar_mma;
-    __shared__ uint32_t tmem_sh;
-    __shared__ int rowm[2][TC_ROWS];                        // this and the next tile: mask row (-1: none)
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 128, Ws, WTpk, BW_W);
-    const uint32_t tmem = tmem_sh;
-    const int ntiles = (nodes + TILE_NODES - 1) / TILE_NODES;
-    const int r8 = lane & 7, q4 = lane >> 3, kz = (warp & 1) * 4 + q4;
-    uint32_t phase = 0;
-    auto lookup = [&](int t, int buf) {
-        if (tid >= TC_ROWS) return;
-        const int k = tid / NODE_ROWS, n = t * TILE_NODES + k;
-        int v = -1;
-        if (k < TILE_NODES && n < nodes) {
-            const int b = n / N, s = out_tab[(n - b * N) * NODE_ROWS + tid - k * NODE_ROWS];
-            if (s >= 0) v = b * N * NODE_ROWS + s;
-        }
-        rowm[buf][tid] = v;
-    };
-    if (blockIdx.x < ntiles) lookup(blockIdx.x, 0);
-    int buf = 0;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int rg = (warp >> 1) + 4 * j, t = rowm[buf][rg * 8 + r8];
-            uint4 z = make_uint4(0u, 0u, 0u, 0u);
-            if (t >= 0)
-                z = mask_bf16x8(*reinterpret_cast<const uint4*>(dm + (size_t)(t / NODE_ROWS) * HD + kz * 8), mask_byte(mask, t, kz));
-            *reinterpret_cast<uint4*>(Zs + (rg * 8 + kz) * 128 + r8 * 16) = z;
-        }
-        if (tile + (int)gridDim.x < ntiles) lookup(tile + gridDim.x, buf ^ 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        tc_fence_before();
-        __syncthreads();
-        tc_fence_after();
-        if (tid == 0) {
-            bwd_mma_input(tmem, Zs, Ws);
-            tc_commit(&bar_mma);
-        }
-        const bool ok = mbar_wait(&bar_mma, phase);
-        phase ^= 1u;
-        if (__syncthreads_or(!ok)) {
-            failed = true;
-            break;
-        }
-        tc_fence_after();
-        const int q = warp & 3, cb = (warp >> 2) * (HD / 2), row = q * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + HD + cb;
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            float d[16];
-            tmem_ld16(tl + 16 * hh, d);
-            tmem_ld_wait();
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                *reinterpret_cast<float4*>(Zs + row * 256 + ((((cb + 16 * hh) >> 2) + c) ^ (row & 7)) * 16) =
-                    make_float4(d[4 * c], d[4 * c + 1], d[4 * c + 2], d[4 * c + 3]);
-        }
-        tc_fence_before();
-        __syncthreads();
-        for (int i = tid; i < TILE_NODES * (HD / 2); i += TC_THREADS) {
-            const int k = i >> 5, cp = i & 31, n = tile * TILE_NODES + k;
-            if (n >= nodes) break;
-            float x = 0.f, y = 0.f;
-#pragma unroll
-            for (int s = 0; s < NODE_ROWS; ++s) {
-                const int r = k * NODE_ROWS + s;
-                if (rowm[buf][r] < 0) continue;
-                const float2 v = *reinterpret_cast<const float2*>(Zs + r * 256 + (((cp >> 1) ^ (r & 7)) << 4) + (cp & 1) * 8);
-                x += v.x;
-                y += v.y;
+        for (int j = 0; j < 4; ++j)
+            if (ent[j].x >= 0) {
+                reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[q8] = ga[j];
+                reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[8 + q8] = gb[j];
             }
-            float2* p = reinterpret_cast<float2*>(dh + (size_t)n * HD) + cp;
-            float2 o = *p;
-            o.x += x;
-            o.y += y;
-            *p = o;
+        __syncthreads();                                    // the tiles are read: the next staging
+    }
+    if (!failed) {
+        // dWm^T: direction 1 has its halves (TMEM lanes) exchanged; it goes through shared memory, [column][input]
+        float* const P = partm + (size_t)blockIdx.x * WPART;
+        float* const sm = reinterpret_cast<float*>(tc_smem);
+        const int q = warp & 3, in = q * 32 + lane, cb = (warp >> 2) * (HD / 2);
+        const uint32_t tl = tmem + HD + ((uint32_t)(q * 32) << 16) + cb;
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+            float d[16];
+            tmem_ld16(tl + HD + 16 * hh, d);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sm[(cb + 16 * hh + i) * KIN + (in ^ HD)] = d[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+            float d[16];
+            tmem_ld16(tl + 16 * hh, d);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < 16; ++i) P[(cb + 16 * hh + i) * KIN + in] = d[i] + sm[(cb + 16 * hh + i) * KIN + in];
+        }
+        db_partial(P, dbm, false, sm);
+        if (POST) {
+            dw_partial(tmem + 3 * HD, parte + (size_t)blockIdx.x * WPART, warp, lane);
+            db_partial(parte + (size_t)blockIdx.x * WPART, dbe, true, sm);
         }
     }
-    tc_teardown(tmem, 128, failed, err);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    tc_teardown(tmem, 256, failed, err);
 }
 
 // dW += sum over a map's CTA partials, db likewise, for all maps at once (blockIdx.y):
@@ -1231,7 +1300,8 @@ struct sg_model {
     // graph + activation buffers for the current (L, Bcap)
     int L = 0, N = 0, E = 0, Bcap = 0;
     int *d_u = nullptr, *d_inc = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
-    int2 *d_ends = nullptr, *d_in_tab = nullptr, *d_msg_tab = nullptr;
+    int2 *d_ends = nullptr, *d_in_tab = nullptr;
+    int4* d_msg_tab = nullptr;
     int8_t* d_J = nullptr;
     float *d_t = nullptr, *d_y = nullptr, *d_g = nullptr, *d_z = nullptr;
     float *d_dy = nullptr, *d_sq = nullptr;   // per graph: output gradient, loss term (readout)
@@ -1239,7 +1309,7 @@ struct sg_model {
     std::vector<bf16*> h, e, m;
     std::vector<uint2*> mm, mu, me;   // per layer: sign bits of the message, node and edge pre-activations
     float *dh = nullptr, *de = nullptr, *ds = nullptr;
-    bf16* dm = nullptr;
+    bf16* dm[2] = {nullptr, nullptr};         // messages' gradient of this layer and of the one below
     float* wpart = nullptr;       // weight-gradient partials: [3 layers maps][wcap CTAs][WPART]
     int wcap = 0;
     uint64_t launches = 0;
@@ -1274,11 +1344,12 @@ void free_graph(sg_model* M)
     cudaFree(M->d_u); cudaFree(M->d_inc); cudaFree(M->d_out_tab);
     cudaFree(M->d_ends); cudaFree(M->d_in_tab); cudaFree(M->d_msg_tab);
     M->d_u = M->d_inc = M->d_out_tab = nullptr;
-    M->d_ends = M->d_in_tab = M->d_msg_tab = nullptr;
+    M->d_ends = M->d_in_tab = nullptr;
+    M->d_msg_tab = nullptr;
     cudaFree(M->d_J); M->d_J = nullptr;
     float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_epart, &M->dh, &M->de, &M->ds, &M->wpart};
     for (float** p : fl) { cudaFree(*p); *p = nullptr; }
-    cudaFree(M->dm); M->dm = nullptr;
+    for (bf16*& p : M->dm) { cudaFree(p); p = nullptr; }
     for (auto* v : {&M->h, &M->e, &M->m}) {
         for (bf16* p : *v) cudaFree(p);
         v->clear();
@@ -1290,10 +1361,10 @@ void free_graph(sg_model* M)
     M->L = M->Bcap = 0;
 }
 
-// Persistent CTAs for `rows` rows in tiles of `per` at ctas_per_sm residents.
-int tc_grid(const sg_model* M, int rows, int ctas_per_sm, int per = TC_ROWS)
+// Persistent CTAs for `rows` rows at ctas_per_sm residents.
+int tc_grid(const sg_model* M, int rows, int ctas_per_sm)
 {
-    const int tiles = (rows + per - 1) / per, cap = ctas_per_sm * M->sms;
+    const int tiles = (rows + TC_ROWS - 1) / TC_ROWS, cap = ctas_per_sm * M->sms;
     return tiles < cap ? (tiles > 0 ? tiles : 1) : cap;
 }
 
@@ -1316,23 +1387,25 @@ int prepare(sg_model* M, int L, int B)
     for (int r = 0; r < L; ++r)
         for (int c = 0; c + 1 < L; ++c)
             for (int k = 0; k < 4; ++k) { ei.push_back(idx(r, c, 1, k)); ej.push_back(idx(r, c + 1, 1, k)); }
-    // message row 2e: source ej -> target ei; row 2e+1: source ei -> target ej.  A node's incoming and
-    // outgoing rows and its edges fill its 6 slots in ascending order
+    // messages 2e: source ej -> target ei, 2e + 1: source ei -> target ej.  A node's incoming and outgoing
+    // messages and its edges fill its 6 slots in ascending order; tables are slot-major [6][N]
     std::vector<int> u(N), inc(N * MAXDEG, -1), out_tab(N * MAXDEG, -1);
-    std::vector<int2> ends(E), in_tab(N * MAXDEG, make_int2(-1, -1)), msg_tab(2 * E);
+    std::vector<int2> ends(E), in_tab(N * MAXDEG, make_int2(-1, -1));
+    std::vector<int4> msg_tab(E);
     std::vector<int> cin(N, 0), cout(N, 0), cinc(N, 0);
     for (int i = 0; i < N; ++i) u[i] = (i >> 2) & 1;
     for (int e2 = 0; e2 < E; ++e2) {
         ends[e2] = make_int2(ei[e2], ej[e2]);
+        int at[2];
         for (int d = 0; d < 2; ++d) {
-            const int src = d == 0 ? ej[e2] : ei[e2], tgt = d == 0 ? ei[e2] : ej[e2];
-            const int slot = tgt * MAXDEG + cin[tgt]++;
-            in_tab[slot] = make_int2(src, e2);
-            msg_tab[2 * e2 + d] = make_int2(src, slot);
-            out_tab[src * MAXDEG + cout[src]++] = slot;
+            const int src = d == 0 ? ej[e2] : ei[e2], tgt = d == 0 ? ei[e2] : ej[e2], slot = cin[tgt]++;
+            in_tab[slot * N + tgt] = make_int2(src, e2);
+            at[d] = tgt * 8 + slot;
+            out_tab[cout[src]++ * N + src] = at[d];
         }
-        inc[ei[e2] * MAXDEG + cinc[ei[e2]]++] = e2;
-        inc[ej[e2] * MAXDEG + cinc[ej[e2]]++] = e2;
+        msg_tab[e2] = make_int4(ej[e2], at[0], ei[e2], at[1]);
+        inc[cinc[ei[e2]]++ * N + ei[e2]] = e2;
+        inc[cinc[ej[e2]]++ * N + ej[e2]] = e2;
     }
     auto up = [&](auto** d, const auto& v) -> cudaError_t {
         cudaError_t r = salloc(d, v.size());
@@ -1365,10 +1438,10 @@ int prepare(sg_model* M, int L, int B)
         SK(salloc(&M->mu[l], nN), "cudaMalloc node mask");
         if (l + 1 < M->layers) SK(salloc(&M->me[l], nE), "cudaMalloc edge mask");
     }
-    M->wcap = tc_grid(M, B * 2 * E, TC_CTAS_UPD_BWD > TC_CTAS_EDGE_BWD ? TC_CTAS_UPD_BWD : TC_CTAS_EDGE_BWD);
+    M->wcap = tc_grid(M, B * E, TC_CTAS_BWD);
     SK(salloc(&M->wpart, (size_t)3 * M->layers * M->wcap * WPART), "cudaMalloc wpart");
     SK(salloc(&M->dh, nN * HD), "cudaMalloc dh");
-    SK(salloc(&M->dm, nN * HD), "cudaMalloc dm");
+    for (bf16*& p : M->dm) SK(salloc(&p, nN * HD), "cudaMalloc dm");
     SK(salloc(&M->de, nE * HD), "cudaMalloc de");
     SK(salloc(&M->ds, nE * HD), "cudaMalloc ds");
     M->L = L; M->N = N; M->E = E; M->Bcap = B;
@@ -1396,15 +1469,12 @@ void forward(sg_model* M, int B, bool train)
                                                                              M->theta + M->oJ, M->h[0], M->e[0]);
     M->launches++;
     for (int l = 0; l < M->layers; ++l) {
-        msg_fwd_kernel<<<tc_grid(M, B * N, TC_CTAS_FWD, TILE_NODES), TC_THREADS, TC_SMEM_FWD, st>>>(
-            B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], M->m[l], train ? M->mm[l] : nullptr,
-            M->d_err);
-        upd_fwd_kernel<false><<<tc_grid(M, B * N, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(
-            B * N, M->h[l], M->m[l], nullptr, N, E, wpk_fwd(M, l, 1), M->theta + M->obu[l], M->h[l + 1], train ? M->mu[l] : nullptr,
-            M->d_err);
-        M->launches += 2;
+        node_fwd_kernel<<<tc_grid(M, B * N, TC_CTAS_NODE_FWD), TC_THREADS, TC_SMEM_NODE_FWD, st>>>(
+            B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], wpk_fwd(M, l, 1), M->theta + M->obu[l],
+            M->h[l + 1], train ? M->m[l] : nullptr, M->mm[l], M->mu[l], M->d_err);
+        M->launches++;
         if (l + 1 == M->layers) break;
-        upd_fwd_kernel<true><<<tc_grid(M, B * E, TC_CTAS_FWD), TC_THREADS, TC_SMEM_FWD, st>>>(
+        edge_fwd_kernel<<<tc_grid(M, B * E, TC_CTAS_EDGE_FWD), TC_THREADS, TC_SMEM_EDGE_FWD, st>>>(
             B * E, M->e[l], M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
             train ? M->me[l] : nullptr, M->d_err);
         M->launches++;
@@ -1434,27 +1504,34 @@ int backward_all(sg_model* M, int B)
         maps.n[nmaps] = n;
         return M->wpart + stride * nmaps++;
     };
-    for (int l = M->layers - 1; l >= 0; --l) {
-        const bool last = l + 1 == M->layers;             // its edge update has no gradient
-        if (!last) {
-            const int g = tc_grid(M, B * E, TC_CTAS_UPD_BWD);
-            upd_bwd_kernel<true><<<g, TC_THREADS, TC_SMEM_UPD_BWD, st>>>(B * E, N, E, M->me[l], M->de, M->e[l], M->h[l + 1],
-                                                                         M->d_ends, nullptr, M->ds, nullptr, wpk_bwd(M, l, 2),
-                                                                         map(M->oWe[l], M->obe[l], g), M->d_err);
-            M->launches++;
-        }
-        int g = tc_grid(M, B * N, TC_CTAS_UPD_BWD);
-        upd_bwd_kernel<false><<<g, TC_THREADS, TC_SMEM_UPD_BWD, st>>>(B * N, N, E, M->mu[l], M->dh, M->h[l], M->m[l], nullptr,
-                                                                      last ? nullptr : M->d_inc, M->ds, M->dm, wpk_bwd(M, l, 1),
-                                                                      map(M->oWu[l], M->obu[l], g), M->d_err);
-        g = tc_grid(M, B * 2 * E, TC_CTAS_EDGE_BWD);
-        msg_bwd_edge_kernel<<<g, TC_THREADS, TC_SMEM_EDGE_BWD, st>>>(B * 2 * E, N, E, M->d_msg_tab, M->mm[l], M->dm, M->h[l],
-                                                                     M->e[l], wpk_bwd(M, l, 0), M->de, last ? 1 : 0,
-                                                                     map(M->oWm[l], M->obm[l], g), M->d_err);
-        msg_bwd_node_kernel<<<tc_grid(M, B * N, TC_CTAS_NODE_BWD, TILE_NODES), TC_THREADS, TC_SMEM_NODE_BWD, st>>>(
-            B * N, N, M->d_out_tab, M->mm[l], M->dm, wpk_bwd(M, l, 0), M->dh, M->d_err);
-        M->launches += 3;
+    // layer l's node update; then per layer its messages with the updates of the layer below
+    const int top = M->layers - 1, gn = tc_grid(M, B * N, TC_CTAS_BWD), ge = tc_grid(M, B * E, TC_CTAS_BWD);
+    const size_t nodes = (size_t)B * N;
+    auto node = [&](int l, auto kernel, int smem) {      // messages of layer l (if any), update of layer l - 1 (if any)
+        const bool pre = l <= top, post = l > 0;
+        kernel<<<gn, TC_THREADS, smem, st>>>(
+            (int)nodes, N, E, pre ? M->d_out_tab : nullptr, pre ? M->mm[l] : nullptr, M->dm[l & 1], pre ? wpk_bwd(M, l, 0) : nullptr,
+            pre && post ? M->d_inc : nullptr, M->ds, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
+            post ? M->m[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 1) : nullptr, M->dm[(l & 1) ^ 1],
+            post ? map(M->oWu[l - 1], M->obu[l - 1], gn) : nullptr, M->d_err);
+        M->launches++;
+    };
+    auto edge = [&](int l, auto kernel, int smem) {
+        const bool post = l > 0;
+        float* pm = map(M->oWm[l], M->obm[l], ge);
+        kernel<<<ge, TC_THREADS, smem, st>>>(
+            B * E, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
+            post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, pm,
+            post ? map(M->oWe[l - 1], M->obe[l - 1], ge) : nullptr, M->d_err);
+        M->launches++;
+    };
+    node(top + 1, node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD);
+    for (int l = top; l > 0; --l) {
+        edge(l, edge_bwd_kernel<true>, TC_SMEM_EDGE_BWD);
+        node(l, node_bwd_kernel<true, true>, TC_SMEM_NODE_BWD);
     }
+    edge(0, edge_bwd_kernel<false>, TC_SMEM_EDGE_BWD);
+    node(0, node_bwd_kernel<true, false>, TC_SMEM_NODE_BWD);
     wgrad_reduce_kernel<<<dim3((WPART + 255) / 256, nmaps), 256, 0, st>>>(maps, stride, M->wpart);
     embed_bwd_kernel<<<4 * M->sms, 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->dh, M->de, M->d_epart);
     embed_bwd_reduce<<<(8 * HD + 255) / 256, 256, 0, st>>>(4 * M->sms, M->d_epart, G + M->oX, G + M->oJ);
@@ -1554,13 +1631,13 @@ int sg_create(sg_model** out, int32_t hidden, int32_t layers, void* stream)
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const struct { const void* k; int smem; } tk[] = {
-            {(const void*)msg_fwd_kernel, TC_SMEM_FWD},
-            {(const void*)upd_fwd_kernel<false>, TC_SMEM_FWD},
-            {(const void*)upd_fwd_kernel<true>, TC_SMEM_FWD},
-            {(const void*)upd_bwd_kernel<false>, TC_SMEM_UPD_BWD},
-            {(const void*)upd_bwd_kernel<true>, TC_SMEM_UPD_BWD},
-            {(const void*)msg_bwd_edge_kernel, TC_SMEM_EDGE_BWD},
-            {(const void*)msg_bwd_node_kernel, TC_SMEM_NODE_BWD}};
+            {(const void*)node_fwd_kernel, TC_SMEM_NODE_FWD},
+            {(const void*)edge_fwd_kernel, TC_SMEM_EDGE_FWD},
+            {(const void*)node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD},
+            {(const void*)node_bwd_kernel<true, true>, TC_SMEM_NODE_BWD},
+            {(const void*)node_bwd_kernel<true, false>, TC_SMEM_NODE_BWD},
+            {(const void*)edge_bwd_kernel<true>, TC_SMEM_EDGE_BWD},
+            {(const void*)edge_bwd_kernel<false>, TC_SMEM_EDGE_BWD}};
         for (const auto& t : tk)
             if (e == cudaSuccess) e = cudaFuncSetAttribute(t.k, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem);
         if (e != cudaSuccess) {

@@ -1,5 +1,5 @@
-"""The surrogate's kernels where their tiles have edges: 21 target or source nodes per tile and
-tiles of 128 rows, against batch sizes and lattice sides that leave every remainder, and one to
+"""The surrogate's kernels where their tiles have edges: 128 nodes or 128 edges per tile, across
+graph borders, against batch sizes and lattice sides that leave every remainder, and one to
 eight layers (the last one updates no edges).  Two properties that hold for any tiling:
 
 * a graph's prediction does not depend on the graphs beside it, bit for bit (its rows meet the
