@@ -22,9 +22,9 @@
 // batches.  So per layer 2 forward and 2 backward kernels, each with every linear map of
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
-// messages, pre-activations and masked gradients in memory (97 launches, 22 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.53 ms, of 128 C_4 graphs 1.01 -> 0.44 ms, 64 C_8
-// predictions 0.42 -> 0.20 ms.  (With a kernel per map and message rows of 21 nodes
+// messages, pre-activations and masked gradients in memory (97 launches, 19 now):
+// gradient of 256 C_8 graphs 3.95 -> 1.34 ms, of 128 C_4 graphs 1.01 -> 0.37 ms, 64 C_8
+// predictions 0.42 -> 0.19 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <cmath>
 #include <cstdint>
@@ -632,6 +632,14 @@ __device__ __forceinline__ void add_db(float* db, uint32_t a, uint32_t b)
     db[3] += y.y;
 }
 
+__device__ __forceinline__ void add_f4(float* s, float4 v)
+{
+    s[0] += v.x;
+    s[1] += v.y;
+    s[2] += v.z;
+    s[3] += v.w;
+}
+
 // A CTA's partial of a bias gradient: a thread's 8 column sums are those of chunk q8
 // (f32 false) or of the 4 columns from 4 q8 and from 32 + 4 q8 (true); the 32 threads of a
 // column in thread order, through 8 KB of shared memory.
@@ -673,13 +681,15 @@ constexpr int TC_CTAS_BWD = 2;
 // POST, node update of the layer below: dZ = dh & mu, dh += dX[:, :64], dmo = dX[:, 64:]
 // rounded to BF16 (the one form that the messages' dZ = dm & mask takes it in), weight
 // gradient with X = [h | m].  A slot's rows are loaded while the slot before is
-// computed; two operand buffers.
+// computed; two operand buffers.  Without PRE (the last layer) every node of a graph starts
+// from the readout's gradient dg [graphs][64]; without POST (the first) dh is not kept,
+// only its sums over the nodes of either orientation, part [CTA][2][64].
 constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64;
 template <bool PRE, bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
 node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
-                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* __restrict__ ds, float* dh,
-                const uint2* __restrict__ mu, const bf16* __restrict__ h, const bf16* __restrict__ m, const bf16* __restrict__ WuT,
+                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* __restrict__ ds, const float* __restrict__ dg,
+                float* dh, const uint2* __restrict__ mu, const bf16* __restrict__ h, const bf16* __restrict__ m, const bf16* __restrict__ WuT,
                 bf16* __restrict__ dmo, float* __restrict__ part, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -708,8 +718,9 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
             }
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (v) {
-                ga[j] = reinterpret_cast<const float4*>(dh + (size_t)n * HD)[q8];
-                gb[j] = reinterpret_cast<const float4*>(dh + (size_t)n * HD)[8 + q8];
+                const float4* gp = reinterpret_cast<const float4*>(PRE ? dh + (size_t)n * HD : dg + (size_t)nb[j] * HD);
+                ga[j] = gp[q8];
+                gb[j] = gp[8 + q8];
             }
         }
         bool ok = true;
@@ -819,14 +830,31 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
         for (int j = 0; j < 4; ++j) {
             const int n = tile * TC_ROWS + srow + 32 * j;
             if (nb[j] < 0) continue;
-            reinterpret_cast<float4*>(dh + (size_t)n * HD)[q8] = ga[j];
-            reinterpret_cast<float4*>(dh + (size_t)n * HD)[8 + q8] = gb[j];
+            if (POST) {
+                reinterpret_cast<float4*>(dh + (size_t)n * HD)[q8] = ga[j];
+                reinterpret_cast<float4*>(dh + (size_t)n * HD)[8 + q8] = gb[j];
+            } else {                                        // orientation of n: bit 2, this warp's lowest
+                add_f4(db, ga[j]);
+                add_f4(db + 4, gb[j]);
+            }
         }
         __syncthreads();                                    // the tiles are read: the next staging
     }
     if (POST && !failed) {
         dw_partial(tdw, part + (size_t)blockIdx.x * WPART, warp, lane);
         db_partial(part + (size_t)blockIdx.x * WPART, db, true, reinterpret_cast<float*>(Xs));
+    }
+    if (!POST && !failed) {
+        float* const sm = reinterpret_cast<float*>(Zs);     // [orientation][column][16 threads]
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            sm[((warp & 1) * HD + (i >> 2) * 32 + q8 * 4 + (i & 3)) * 17 + (warp >> 1) * 4 + (lane >> 3)] = db[i];
+        __syncthreads();
+        if (tid < 2 * HD) {
+            float t = 0.f;
+            for (int j = 0; j < 16; ++j) t += sm[tid * 17 + j];
+            part[(size_t)blockIdx.x * 2 * HD + tid] = t;
+        }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     tc_teardown(tmem, 256, failed, err);
@@ -839,14 +867,17 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 // weight gradient with X = [eb | h_i + h_j], whose end rows are the messages' source rows.
 // Operands R0 | R1 | R2: h[src_0], e, h[src_1], then (POST) eb in R1 and the sum in R2.
 // The two directions' weight gradients differ in the order of their halves ([R0 | R1] and
-// [R1 | R2]) and are kept apart in tensor memory.
+// [R1 | R2]) and are kept apart in tensor memory.  Without POST (the first layer) de is not
+// kept, only its sums over the edges of every coupler value (J; -3 .. 3 without 0), epart
+// [CTA][6][64]: the finished tile goes back to shared memory and a thread adds up a
+// column of 32 rows, a row's class being the same for the whole warp.
 constexpr int TC_SMEM_EDGE_BWD = 5 * OP64 + 3 * W64;
 template <bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
 edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
                 const bf16* __restrict__ h, const bf16* __restrict__ e, const bf16* __restrict__ WmT, float* de, int set,
                 const uint2* __restrict__ me, const bf16* __restrict__ eb, const bf16* __restrict__ WeT, float* __restrict__ ds,
-                float* __restrict__ partm, float* __restrict__ parte, int* err)
+                float* __restrict__ partm, float* __restrict__ parte, const int8_t* __restrict__ J, float* __restrict__ epart, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char *const R0 = tc_smem, *const R1 = R0 + OP64, *const R2 = R1 + OP64, *const Zs = R2 + OP64, *const Ws = Zs + 2 * OP64;
@@ -857,11 +888,14 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
     const uint32_t tmem = tmem_sh;                          // dX, then dWm^T of direction 0 and 1, dWe^T: 64 columns each
     const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
     const size_t nodes = (size_t)(rows / E) * N;
+    __shared__ signed char cls[TC_ROWS];                    // coupler values of the tile (without POST)
+    float sj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float dbm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dbe[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
         const int r0 = tile * TC_ROWS;
+        if (!POST && tid < TC_ROWS) cls[tid] = r0 + tid < rows ? J[r0 + tid] : 1;
         int4 ent[4];
         int bN[4];
 #pragma unroll
@@ -983,18 +1017,44 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
             if (failed) break;
         }
         first = false;
+        if (POST) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (ent[j].x >= 0) {
-                reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[q8] = ga[j];
-                reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[8 + q8] = gb[j];
+            for (int j = 0; j < 4; ++j)
+                if (ent[j].x >= 0) {
+                    reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[q8] = ga[j];
+                    reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[8 + q8] = gb[j];
+                }
+        } else {
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {                   // the places that this thread has read
+                *tile_f32(Zs, srow + 32 * j, q8) = ent[j].x >= 0 ? ga[j] : zero;
+                *tile_f32(Zs, srow + 32 * j, 8 + q8) = ent[j].x >= 0 ? gb[j] : zero;
             }
+            __syncthreads();
+            const int c = tid & (HD - 1);
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i) {
+                const int row = (tid >> 6) * 32 + i, k = cls[row];
+                const float v = reinterpret_cast<const float*>(tile_f32(Zs, row, c >> 2))[c & 3];
+#pragma unroll
+                for (int q = 0; q < 6; ++q) sj[q] += k == (q < 3 ? q - 3 : q - 2) ? v : 0.f;
+            }
+        }
         __syncthreads();                                    // the tiles are read: the next staging
+    }
+    if (!POST && !failed) {
+        float* const sm = reinterpret_cast<float*>(Zs);     // [row group][value][column]
+#pragma unroll
+        for (int q = 0; q < 6; ++q) sm[((tid >> 6) * 6 + q) * HD + (tid & (HD - 1))] = sj[q];
+        __syncthreads();
+        for (int i = tid; i < 6 * HD; i += TC_THREADS)
+            epart[(size_t)blockIdx.x * 6 * HD + i] = (sm[i] + sm[6 * HD + i]) + (sm[12 * HD + i] + sm[18 * HD + i]);
     }
     if (!failed) {
         // dWm^T: direction 1 has its halves (TMEM lanes) exchanged; it goes through shared memory, [column][input]
         float* const P = partm + (size_t)blockIdx.x * WPART;
-        float* const sm = reinterpret_cast<float*>(tc_smem);
+        float* const sm = reinterpret_cast<float*>(tc_smem);     // R0, R1: not the sums above
         const int q = warp & 3, in = q * 32 + lane, cb = (warp >> 2) * (HD / 2);
         const uint32_t tl = tmem + HD + ((uint32_t)(q * 32) << 16) + cb;
 #pragma unroll
@@ -1024,26 +1084,95 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
     tc_teardown(tmem, 256, failed, err);
 }
 
-// dW += sum over a map's CTA partials, db likewise, for all maps at once (blockIdx.y):
-// four interleaved sums added in a fixed order.
-struct WMaps {
-    float *dW[24], *db[24];
-    int n[24];                       // partials of the map
+// Every sum over CTAs or graphs that is left of a gradient, in one launch (blockIdx.y): the
+// partials of up to 26 parameter blocks (weight maps with their biases, embeddings; no
+// partials: 0), then the readout's.  16 columns of 16 bytes x 16 threads that each take
+// every 16th partial, added in a fixed order (bit-reproducible).  11 maps of 304 partials
+// (110 MB, 256 C_8 graphs) in 26 us with the readout's sums; one thread per output in order
+// took 35 us, the readout's 18 us and the embeddings' 117 us in launches of their own.
+constexpr int MAXPARTS = 27;
+struct Parts {
+    float* dst[MAXPARTS];
+    const float* src[MAXPARTS];
+    int n[MAXPARTS], count[MAXPARTS];        // partials; floats of one
+    int blocks;
 };
-__global__ void wgrad_reduce_kernel(WMaps maps, size_t stride, const float* __restrict__ part)
+// Readout: dW1[c][k] = sum_b dz_b[c] g_b[k] with dz_b[c] = dy_b w2[c] where z_b[c] > 0, db1[c],
+// dw2[c] (block c < 64); db2 and the loss (block 64).
+struct ReadoutGrad {
+    int B;
+    const float *g, *z, *dy, *sq, *w2;
+    float *loss, *dW1, *db1, *dw2, *db2;
+};
+
+__device__ void readout_grad(const ReadoutGrad& r, float* sm)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
-    if (i >= WPART) return;
-    const float* p = part + k * stride + i;
-    float s[4] = {0.f, 0.f, 0.f, 0.f};
-    int b = 0;
-    for (; b + 4 <= maps.n[k]; b += 4)
+    const int c = blockIdx.x, tid = threadIdx.x, k = tid & (HD - 1), grp = tid >> 6;
+    if (c < HD) {
+        const float w = r.w2[c];
+        float acc = 0.f, a1 = 0.f, a2 = 0.f;
+#pragma unroll 4
+        for (int b = grp; b < r.B; b += 4) {
+            const float z = r.z[b * HD + c], dy = r.dy[b];
+            const float dz = z > 0.f ? dy * w : 0.f;
+            acc += dz * r.g[b * HD + k];
+            a1 += dz;
+            a2 += dy * fmaxf(z, 0.f);
+        }
+        sm[tid] = acc;
+        if (k == 0) {
+            sm[256 + grp] = a1;
+            sm[260 + grp] = a2;
+        }
+        __syncthreads();
+        if (tid < HD) r.dW1[c * HD + k] = (sm[k] + sm[64 + k]) + (sm[128 + k] + sm[192 + k]);
+        if (tid == 0) {
+            r.db1[c] = (sm[256] + sm[257]) + (sm[258] + sm[259]);
+            r.dw2[c] = (sm[260] + sm[261]) + (sm[262] + sm[263]);
+        }
+    } else if (c == HD && tid < 2) {         // in graph order
+        const float* x = tid == 0 ? r.dy : r.sq;
+        float t = 0.f;
+#pragma unroll 8
+        for (int b = 0; b < r.B; ++b) t += x[b];
+        *(tid == 0 ? r.db2 : r.loss) = t;
+    }
+}
+
+constexpr int RED_THREADS = 256, RED_COLS = 16, RED_PER = RED_THREADS / RED_COLS;
+__global__ void __launch_bounds__(RED_THREADS) reduce_kernel(Parts p, ReadoutGrad r)
+{
+    __shared__ float4 sm[RED_PER][RED_COLS + 1];
+    const int k = blockIdx.y;
+    if (k == p.blocks) {
+        readout_grad(r, reinterpret_cast<float*>(sm));
+        return;
+    }
+    const int q = p.count[k] / 4, c = threadIdx.x % RED_COLS, g = threadIdx.x / RED_COLS, i = blockIdx.x * RED_COLS + c, n = p.n[k];
+    if (blockIdx.x * RED_COLS >= q) return;
+    float4 s[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[j] += p[(size_t)(b + j) * WPART];
-    for (int j = 0; b < maps.n[k]; ++b, ++j) s[j] += p[(size_t)b * WPART];
-    const float t = (s[0] + s[1]) + (s[2] + s[3]);
-    if (i < HD * KIN) maps.dW[k][i] += t;
-    else maps.db[k][i - HD * KIN] += t;
+    for (int j = 0; j < 4; ++j) s[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < q) {
+        const float4* src = reinterpret_cast<const float4*>(p.src[k]) + i;
+        int b = g;
+        for (; b + 3 * RED_PER < n; b += 4 * RED_PER) {
+            float4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = src[(size_t)(b + j * RED_PER) * q];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[j] = add4(s[j], v[j]);
+        }
+        for (; b < n; b += RED_PER) s[0] = add4(s[0], src[(size_t)b * q]);
+    }
+    sm[g][c] = add4(add4(s[0], s[1]), add4(s[2], s[3]));
+    __syncthreads();
+    if (g == 0 && i < q) {
+        float4 t = sm[0][c];
+#pragma unroll
+        for (int j = 1; j < RED_PER; ++j) t = add4(t, sm[j][c]);
+        reinterpret_cast<float4*>(p.dst[k])[i] = t;
+    }
 }
 
 // Packs the BF16 matrix W [64 outputs][128 inputs] of every layer map into the
@@ -1094,14 +1223,14 @@ __global__ void embed_kernel(int B, int N, int E, const int* __restrict__ u, con
     }
 }
 
-// readout forward + loss gradient (one block of 256 threads per graph).  The node mean is
+// readout forward + loss gradient dg, the same for every node of a graph (one block of 256 threads per graph).  The node mean is
 // summed node by node (64 threads, a column each) from rows that the block stages 64 at a
 // time, the next 64 on their way meanwhile.
 constexpr int RO_ROWS = 64, RO_THREADS = 256;
 __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* __restrict__ h, const float* __restrict__ W1, const float* __restrict__ b1,
                                const float* __restrict__ w2, const float* __restrict__ b2, float* y, float* gbuf,
                                float* zbuf, const float* __restrict__ target, float inv_B, float* dybuf,
-                               float* sqbuf, float* dh)
+                               float* sqbuf, float* dgbuf, const int* __restrict__ err)
 {
     __shared__ __align__(16) float gs[HD];
     __shared__ float as[HD], red[HD], dz[HD];
@@ -1149,6 +1278,7 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
     }
     const float yb = red[0] + b2[0];
     if (c == 0) y[b] = yb;
+    if (b == 0 && c == 1) reinterpret_cast<int*>(y)[gridDim.x] = *err;      // the status of the kernels before
     if (!target) return;
     const float dy = 2.f * (yb - target[b]) * inv_B;
     if (c == 0) {                                  // this graph's loss term and output gradient (summed in order
@@ -1160,96 +1290,8 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
     if (c < HD) {
         float dg = 0.f;
         for (int o = 0; o < HD; ++o) dg += dz[o] * W1[o * HD + c];
-        dg /= (float)N;
-        gs[c] = dg;
+        dgbuf[b * HD + c] = dg / (float)N;
     }
-    __syncthreads();
-    const float4 d = reinterpret_cast<const float4*>(gs)[tid & (HD / 4 - 1)];
-    float4* out = reinterpret_cast<float4*>(dh + (size_t)b * N * HD);
-    for (int i = tid; i < N * (HD / 4); i += RO_THREADS) out[i] = d;
-}
-
-// Readout parameter gradients and the loss, summed over the B graphs in graph
-// order (bit-reproducible): block c < 64, thread k: dW1[c][k] += sum_b dz_b[c]
-// g_b[k] with dz_b[c] = dy_b w2[c] where z_b[c] > 0, and (thread 0) db1[c],
-// dw2[c]; block 64: db2 and the loss.
-__global__ void readout_grad_kernel(int B, const float* __restrict__ gbuf, const float* __restrict__ zbuf,
-                                    const float* __restrict__ dybuf, const float* __restrict__ sqbuf,
-                                    const float* __restrict__ w2, float* loss, float* dW1, float* db1, float* dw2,
-                                    float* db2)
-{
-    const int c = blockIdx.x, k = threadIdx.x;
-    if (c < HD) {
-        const float w = w2[c];
-        float acc = 0.f, a1 = 0.f, a2 = 0.f;
-        for (int b = 0; b < B; ++b) {
-            const float z = zbuf[b * HD + c], dy = dybuf[b];
-            const float dz = z > 0.f ? dy * w : 0.f;
-            acc += dz * gbuf[b * HD + k];
-            a1 += dz;
-            a2 += dy * fmaxf(z, 0.f);
-        }
-        dW1[c * HD + k] += acc;
-        if (k == 0) {
-            db1[c] += a1;
-            dw2[c] += a2;
-        }
-    } else if (k == 0) {
-        float s2 = 0.f, l = 0.f;
-        for (int b = 0; b < B; ++b) {
-            s2 += dybuf[b];
-            l += sqbuf[b];
-        }
-        db2[0] += s2;
-        *loss += l;
-    }
-}
-
-// Embedding gradients: dX[o] += sum of dh over the nodes of orientation o, dJt[v] += sum of de over
-// the edges of coupler value v.  A thread owns column c of a strided set of rows and keeps its 2 + 6
-// class sums in registers; the block adds its 4 lanes' sums in lane order and writes them as its
-// partial part[block][8][64] (classes: orientations 0, 1, coupler values -3..3 without 0), and
-// embed_bwd_reduce adds the partials in block order (bit-reproducible).  256 threads per block.
-__global__ void embed_bwd_kernel(int B, int N, int E, const int* __restrict__ u, const int8_t* __restrict__ J,
-                                 const float* __restrict__ dh, const float* __restrict__ de, float* __restrict__ part)
-{
-    __shared__ float sp[4][8][HD];
-    const int c = threadIdx.x % HD, lane = threadIdx.x / HD, lanes = blockDim.x / HD;
-    const size_t nN = (size_t)B * N, nE = (size_t)B * E, stride = (size_t)gridDim.x * lanes;
-    const size_t first = blockIdx.x * (size_t)lanes + lane;
-    float ax0 = 0.f, ax1 = 0.f, aj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (size_t row = first; row < nN; row += stride) {
-        const float v = dh[row * HD + c];
-        if (u[row % N]) ax1 += v;
-        else ax0 += v;
-    }
-    for (size_t re = first; re < nE; re += stride) {
-        const int j = J[re];
-        const int k = j < 0 ? j + 3 : j + 2;                 // -3,-2,-1,1,2,3 -> 0..5
-        const float v = de[re * HD + c];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) aj[q] += k == q ? v : 0.f;
-    }
-    sp[lane][0][c] = ax0;
-    sp[lane][1][c] = ax1;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) sp[lane][2 + q][c] = aj[q];
-    __syncthreads();
-    for (int i = threadIdx.x; i < 8 * HD; i += blockDim.x) {
-        float t = 0.f;
-        for (int l = 0; l < lanes; ++l) t += sp[l][i / HD][i % HD];
-        part[(size_t)blockIdx.x * 8 * HD + i] = t;
-    }
-}
-
-__global__ void embed_bwd_reduce(int nblocks, const float* __restrict__ part, float* dX, float* dJt)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= 8 * HD) return;
-    float t = 0.f;
-    for (int b = 0; b < nblocks; ++b) t += part[(size_t)b * 8 * HD + i];
-    if (i < 2 * HD) dX[i] += t;
-    else dJt[i - 2 * HD] += t;
 }
 
 __global__ void adam_kernel(int64_t n, float* theta, const float* __restrict__ g, float* m, float* v, float lr,
@@ -1291,7 +1333,7 @@ struct sg_model {
     bf16* wbf = nullptr;          // BF16 copy of theta
     bf16* wpk = nullptr;          // per layer map: W and W^T in the tcgen05 operand layouts (2 x 8192 BF16 each)
     const bf16** d_wptr = nullptr;// device array: the BF16 matrices of every layer map (pack_weights_kernel input)
-    int* d_err = nullptr;         // set by a tensor-core kernel whose bounded wait ran out
+    int* d_err = nullptr;         // the word after dloss, set by a tensor-core kernel whose bounded wait ran out
     int sms = 0;                  // SMs of the device (persistent grids)
     int64_t step = 0;
     // offsets into theta
@@ -1305,7 +1347,8 @@ struct sg_model {
     int8_t* d_J = nullptr;
     float *d_t = nullptr, *d_y = nullptr, *d_g = nullptr, *d_z = nullptr;
     float *d_dy = nullptr, *d_sq = nullptr;   // per graph: output gradient, loss term (readout)
-    float* d_epart = nullptr;                 // embedding-gradient block partials [4 x SMs][8][64]
+    float* d_dg = nullptr;                    // per graph: readout's gradient of a node [64]
+    float* d_epart = nullptr;                 // embedding-gradient partials: edges [CTAs][6][64], then nodes [CTAs][2][64]
     std::vector<bf16*> h, e, m;
     std::vector<uint2*> mm, mu, me;   // per layer: sign bits of the message, node and edge pre-activations
     float *dh = nullptr, *de = nullptr, *ds = nullptr;
@@ -1347,7 +1390,7 @@ void free_graph(sg_model* M)
     M->d_ends = M->d_in_tab = nullptr;
     M->d_msg_tab = nullptr;
     cudaFree(M->d_J); M->d_J = nullptr;
-    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_epart, &M->dh, &M->de, &M->ds, &M->wpart};
+    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_dg, &M->d_epart, &M->dh, &M->de, &M->ds, &M->wpart};
     for (float** p : fl) { cudaFree(*p); *p = nullptr; }
     for (bf16*& p : M->dm) { cudaFree(p); p = nullptr; }
     for (auto* v : {&M->h, &M->e, &M->m}) {
@@ -1421,12 +1464,12 @@ int prepare(sg_model* M, int L, int B)
     const size_t nN = (size_t)B * N, nE = (size_t)B * E;
     SK(salloc(&M->d_J, nE), "cudaMalloc J");
     SK(salloc(&M->d_t, (size_t)B), "cudaMalloc t");
-    SK(salloc(&M->d_y, (size_t)B), "cudaMalloc y");
+    SK(salloc(&M->d_y, (size_t)B + 1), "cudaMalloc y");
     SK(salloc(&M->d_g, (size_t)B * HD), "cudaMalloc g");
     SK(salloc(&M->d_z, (size_t)B * HD), "cudaMalloc z");
     SK(salloc(&M->d_dy, (size_t)B), "cudaMalloc dy");
     SK(salloc(&M->d_sq, (size_t)B), "cudaMalloc sq");
-    SK(salloc(&M->d_epart, (size_t)4 * M->sms * 8 * HD), "cudaMalloc embedding partials");
+    SK(salloc(&M->d_dg, (size_t)B * HD), "cudaMalloc dg");
     M->h.assign(M->layers + 1, nullptr);
     for (auto* v : {&M->e, &M->m}) v->assign(M->layers, nullptr);
     for (auto* v : {&M->mm, &M->mu, &M->me}) v->assign(M->layers, nullptr);
@@ -1439,6 +1482,7 @@ int prepare(sg_model* M, int L, int B)
         if (l + 1 < M->layers) SK(salloc(&M->me[l], nE), "cudaMalloc edge mask");
     }
     M->wcap = tc_grid(M, B * E, TC_CTAS_BWD);
+    SK(salloc(&M->d_epart, (size_t)M->wcap * 8 * HD), "cudaMalloc embedding partials");
     SK(salloc(&M->wpart, (size_t)3 * M->layers * M->wcap * WPART), "cudaMalloc wpart");
     SK(salloc(&M->dh, nN * HD), "cudaMalloc dh");
     for (bf16*& p : M->dm) SK(salloc(&p, nN * HD), "cudaMalloc dm");
@@ -1481,48 +1525,50 @@ void forward(sg_model* M, int B, bool train)
     }
 }
 
-// Gradient of the mean squared error into M->grad (zeroed first); loss into M->dloss.
-int backward_all(sg_model* M, int B)
+// Gradient of the mean squared error into M->grad; loss into M->dloss.
+void backward_all(sg_model* M, int B)
 {
     const int N = M->N, E = M->E;
     cudaStream_t st = M->stream;
     float* G = M->grad;
-    SK(cudaMemsetAsync(G, 0, sizeof(float) * M->nparams, st), "zero grad");
-    SK(cudaMemsetAsync(M->dloss, 0, sizeof(float), st), "zero loss");
     readout_kernel<<<B, RO_THREADS, 0, st>>>(N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1, M->theta + M->ow2,
                                              M->theta + M->ob2, M->d_y, M->d_g, M->d_z, M->d_t, 1.f / (float)B, M->d_dy,
-                                             M->d_sq, M->dh);
-    readout_grad_kernel<<<HD + 1, HD, 0, st>>>(B, M->d_g, M->d_z, M->d_dy, M->d_sq, M->theta + M->ow2, M->dloss,
-                                               G + M->oW1, G + M->ob1, G + M->ow2, G + M->ob2);
-    M->launches += 2;
-    WMaps maps;
+                                             M->d_sq, M->d_dg, M->d_err);
+    M->launches++;
+    Parts parts;
+    parts.blocks = 0;
+    auto sum = [&](int64_t o, const float* src, int n, int count) {
+        parts.dst[parts.blocks] = G + o;
+        parts.src[parts.blocks] = src;
+        parts.n[parts.blocks] = n;
+        parts.count[parts.blocks++] = count;
+    };
     int nmaps = 0;
-    const size_t stride = (size_t)M->wcap * WPART;
-    auto map = [&](int64_t oW, int64_t ob, int n) {      // the next map's partials
-        maps.dW[nmaps] = G + oW;
-        maps.db[nmaps] = G + ob;
-        maps.n[nmaps] = n;
-        return M->wpart + stride * nmaps++;
+    auto map = [&](int64_t oW, int n) {                  // the next map's partials: the matrix, then its bias
+        float* p = M->wpart + (size_t)M->wcap * WPART * nmaps++;
+        sum(oW, p, n, WPART);
+        return p;
     };
     // layer l's node update; then per layer its messages with the updates of the layer below
     const int top = M->layers - 1, gn = tc_grid(M, B * N, TC_CTAS_BWD), ge = tc_grid(M, B * E, TC_CTAS_BWD);
     const size_t nodes = (size_t)B * N;
+    float* const nepart = M->d_epart + (size_t)M->wcap * 6 * HD;
     auto node = [&](int l, auto kernel, int smem) {      // messages of layer l (if any), update of layer l - 1 (if any)
         const bool pre = l <= top, post = l > 0;
         kernel<<<gn, TC_THREADS, smem, st>>>(
             (int)nodes, N, E, pre ? M->d_out_tab : nullptr, pre ? M->mm[l] : nullptr, M->dm[l & 1], pre ? wpk_bwd(M, l, 0) : nullptr,
-            pre && post ? M->d_inc : nullptr, M->ds, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
+            pre && post ? M->d_inc : nullptr, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
             post ? M->m[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 1) : nullptr, M->dm[(l & 1) ^ 1],
-            post ? map(M->oWu[l - 1], M->obu[l - 1], gn) : nullptr, M->d_err);
+            post ? map(M->oWu[l - 1], gn) : nepart, M->d_err);
         M->launches++;
     };
     auto edge = [&](int l, auto kernel, int smem) {
         const bool post = l > 0;
-        float* pm = map(M->oWm[l], M->obm[l], ge);
+        float* pm = map(M->oWm[l], ge);
         kernel<<<ge, TC_THREADS, smem, st>>>(
             B * E, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
             post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, pm,
-            post ? map(M->oWe[l - 1], M->obe[l - 1], ge) : nullptr, M->d_err);
+            post ? map(M->oWe[l - 1], ge) : nullptr, M->d_J, M->d_epart, M->d_err);
         M->launches++;
     };
     node(top + 1, node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD);
@@ -1532,11 +1578,12 @@ int backward_all(sg_model* M, int B)
     }
     edge(0, edge_bwd_kernel<false>, TC_SMEM_EDGE_BWD);
     node(0, node_bwd_kernel<true, false>, TC_SMEM_NODE_BWD);
-    wgrad_reduce_kernel<<<dim3((WPART + 255) / 256, nmaps), 256, 0, st>>>(maps, stride, M->wpart);
-    embed_bwd_kernel<<<4 * M->sms, 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->dh, M->de, M->d_epart);
-    embed_bwd_reduce<<<(8 * HD + 255) / 256, 256, 0, st>>>(4 * M->sms, M->d_epart, G + M->oX, G + M->oJ);
-    M->launches += 3;
-    return PT_OK;
+    sum(M->oX, nepart, gn, 2 * HD);
+    sum(M->oJ, M->d_epart, ge, 6 * HD);
+    sum(M->oWe[top], nullptr, 0, WPART);
+    const ReadoutGrad ro = {B, M->d_g, M->d_z, M->d_dy, M->d_sq, M->theta + M->ow2, M->dloss, G + M->oW1, G + M->ob1, G + M->ow2, G + M->ob2};
+    reduce_kernel<<<dim3((WPART / 4 + RED_COLS - 1) / RED_COLS, parts.blocks + 1), RED_THREADS, 0, st>>>(parts, ro);
+    M->launches++;
 }
 
 // A tensor-core kernel whose bounded mbarrier wait ran out leaves 1 in d_err
@@ -1603,7 +1650,7 @@ int sg_create(sg_model** out, int32_t hidden, int32_t layers, void* stream)
         M->own_stream = true;
     }
     if (salloc(&M->theta, o) != cudaSuccess || salloc(&M->grad, o) != cudaSuccess || salloc(&M->mom1, o) != cudaSuccess ||
-        salloc(&M->mom2, o) != cudaSuccess || salloc(&M->wbf, o) != cudaSuccess || salloc(&M->dloss, 1) != cudaSuccess) {
+        salloc(&M->mom2, o) != cudaSuccess || salloc(&M->wbf, o) != cudaSuccess || salloc(&M->dloss, 2) != cudaSuccess) {
         M->err = "cudaMalloc parameters failed";
         return bail(PT_ERR_OOM);
     }
@@ -1621,12 +1668,13 @@ int sg_create(sg_model** out, int32_t hidden, int32_t layers, void* stream)
         }
         int dev = 0, sms = 0;
         if (salloc(&M->wpk, (size_t)layers * 3 * 2 * HD * KIN) != cudaSuccess ||
-            salloc(&M->d_wptr, ptrs.size()) != cudaSuccess || salloc(&M->d_err, 1) != cudaSuccess) {
+            salloc(&M->d_wptr, ptrs.size()) != cudaSuccess) {
             M->err = "cudaMalloc tensor-core operands failed";
             return bail(PT_ERR_OOM);
         }
         cudaError_t e = cudaMemcpy(M->d_wptr, ptrs.data(), sizeof(bf16*) * ptrs.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(M->wpk, 0, sizeof(bf16) * (size_t)layers * 3 * 2 * HD * KIN);
+        M->d_err = reinterpret_cast<int*>(M->dloss + 1);
         if (e == cudaSuccess) e = cudaMemset(M->d_err, 0, sizeof(int));
         if (e == cudaSuccess) e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1656,7 +1704,7 @@ void sg_destroy(sg_model* M)
     if (M->stream) cudaStreamSynchronize(M->stream);
     free_graph(M);
     cudaFree(M->theta); cudaFree(M->grad); cudaFree(M->mom1); cudaFree(M->mom2); cudaFree(M->wbf); cudaFree(M->dloss);
-    cudaFree(M->wpk); cudaFree(M->d_wptr); cudaFree(M->d_err);
+    cudaFree(M->wpk); cudaFree(M->d_wptr);
     if (M->own_stream && M->stream) cudaStreamDestroy(M->stream);
     delete M;
 }
@@ -1693,13 +1741,15 @@ int sg_forward(sg_model* M, int32_t L, int32_t B, const int8_t* J, float* y)
     forward(M, B, false);
     readout_kernel<<<B, RO_THREADS, 0, M->stream>>>(M->N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1,
                                             M->theta + M->ow2, M->theta + M->ob2, M->d_y, M->d_g, M->d_z, nullptr,
-                                            0.f, nullptr, nullptr, nullptr);
+                                            0.f, nullptr, nullptr, nullptr, M->d_err);
     M->launches++;
     SK(cudaGetLastError(), "forward kernels");
-    SK(cudaMemcpyAsync(y, M->d_y, sizeof(float) * B, cudaMemcpyDeviceToHost, M->stream), "download y");
-    int terr = 0;
-    SK(cudaMemcpyAsync(&terr, M->d_err, sizeof(int), cudaMemcpyDeviceToHost, M->stream), "download status");
+    float out[4096 + 1];                             // the predictions and the status word (load_batch: B <= 4096)
+    SK(cudaMemcpyAsync(out, M->d_y, sizeof(float) * ((size_t)B + 1), cudaMemcpyDeviceToHost, M->stream), "download y");
     SK(cudaStreamSynchronize(M->stream), "sync forward");
+    std::memcpy(y, out, sizeof(float) * B);
+    int terr = 0;
+    std::memcpy(&terr, out + B, sizeof terr);
     return tc_status(M, terr);
 }
 
@@ -1709,16 +1759,14 @@ int sg_grad(sg_model* M, int32_t L, int32_t B, const int8_t* J, const float* t, 
     int rc = load_batch(M, L, B, J, t);
     if (rc) return rc;
     forward(M, B, true);
-    if ((rc = backward_all(M, B))) return rc;
+    backward_all(M, B);
     SK(cudaGetLastError(), "gradient kernels");
     if (grad) SK(cudaMemcpyAsync(grad, M->grad, sizeof(float) * M->nparams, cudaMemcpyDeviceToHost, M->stream), "download grad");
-    float lv = 0.f;
-    int terr = 0;
-    SK(cudaMemcpyAsync(&lv, M->dloss, sizeof(float), cudaMemcpyDeviceToHost, M->stream), "download loss");
-    SK(cudaMemcpyAsync(&terr, M->d_err, sizeof(int), cudaMemcpyDeviceToHost, M->stream), "download status");
+    struct { float loss; int status; } res = {0.f, 0};
+    SK(cudaMemcpyAsync(&res, M->dloss, sizeof res, cudaMemcpyDeviceToHost, M->stream), "download loss and status");
     SK(cudaStreamSynchronize(M->stream), "sync grad");
-    if (loss) *loss = lv;
-    return tc_status(M, terr);
+    if (loss) *loss = res.loss;
+    return tc_status(M, res.status);
 }
 
 int sg_adam(sg_model* M, float lr)
