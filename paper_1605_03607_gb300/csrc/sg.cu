@@ -23,8 +23,8 @@
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
 // messages, pre-activations and masked gradients in memory (97 launches, 19 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.34 ms, of 128 C_4 graphs 1.01 -> 0.37 ms, 64 C_8
-// predictions 0.42 -> 0.19 ms.  (With a kernel per map and message rows of 21 nodes
+// gradient of 256 C_8 graphs 3.95 -> 1.31 ms, of 128 C_4 graphs 1.01 -> 0.32 ms, 64 C_8
+// predictions 0.42 -> 0.17 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <cmath>
 #include <cstdint>
@@ -266,6 +266,17 @@ __device__ __forceinline__ bool tc_setup(uint32_t* tmem_sh, uint64_t* bar_w, uin
     return !__syncthreads_or(!ok);
 }
 
+// Launches of a pass are programmatically dependent: a kernel may start while the one before
+// still runs, sets up (weights, topology tables: not written by any kernel of a pass) and
+// waits here for it to end before it touches what it computed (pointers to that are not
+// __restrict__: such loads may move across the wait).  Lets the next kernel start.
+// 128 C_4 graphs: gradient 358 -> 319 us.
+__device__ __forceinline__ void pass_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // The staged operands are complete: this thread's copies have landed and its stores are
 // visible to the tensor core; tensor-memory reads before it are ordered before the MMAs
 // after it.  True (for every thread) if any thread's last wait failed.
@@ -282,30 +293,29 @@ __device__ __forceinline__ bool tc_ready(bool failed)
 // Z = A W^T: A 128 columns, W [8 output groups][16 k-chunks][8 outputs][16 B]
 __device__ __forceinline__ void mma_forward(uint32_t tmem, const unsigned char* As, const unsigned char* Ws)
 {
+    const uint64_t a = tc_desc(smem_u32(As), CH, 128), b = tc_desc(smem_u32(Ws), 128, 16 * 128);     // + bytes / 16: a later start
 #pragma unroll
     for (int ks = 0; ks < KIN / 16; ++ks)
-        tc_mma(tmem, tc_desc(smem_u32(As) + ks * 2 * CH, CH, 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 16 * 128),
-               tc_idesc_bf16(TC_ROWS, HD), ks > 0 ? 1u : 0u);
+        tc_mma(tmem, a + ks * 2 * CH / 16, b + ks * 16, tc_idesc_bf16(TC_ROWS, HD), ks > 0 ? 1u : 0u);
 }
 
 // dX (+)= dZ W over nin (64 or 128) inputs: W^T [nin / 8 input groups][8 k-chunks][8][16 B]
 template <int NIN>
 __device__ __forceinline__ void mma_input(uint32_t tmem, const unsigned char* Zs, const unsigned char* Ws, bool add)
 {
+    const uint64_t a = tc_desc(smem_u32(Zs), CH, 128), b = tc_desc(smem_u32(Ws), 128, 8 * 128);
 #pragma unroll
     for (int ks = 0; ks < HD / 16; ++ks)
-        tc_mma(tmem, tc_desc(smem_u32(Zs) + ks * 2 * CH, CH, 128), tc_desc(smem_u32(Ws) + ks * 256, 128, 8 * 128),
-               tc_idesc_bf16(TC_ROWS, NIN), add || ks > 0 ? 1u : 0u);
+        tc_mma(tmem, a + ks * 2 * CH / 16, b + ks * 16, tc_idesc_bf16(TC_ROWS, NIN), add || ks > 0 ? 1u : 0u);
 }
 
 // dW^T (+)= X^T dZ: X 128 columns (M), dZ 64 (N), K = 128 rows; both MN-major
 __device__ __forceinline__ void mma_wgrad(uint32_t tmem, const unsigned char* Xs, const unsigned char* Zs, bool add)
 {
     constexpr uint32_t IDESC = tc_idesc_bf16(KIN, HD) | (1u << 15) | (1u << 16);
+    const uint64_t a = tc_desc(smem_u32(Xs), 128, CH), b = tc_desc(smem_u32(Zs), 128, CH);
 #pragma unroll
-    for (int ks = 0; ks < TC_ROWS / 16; ++ks)
-        tc_mma(tmem, tc_desc(smem_u32(Xs) + ks * 256, 128, CH), tc_desc(smem_u32(Zs) + ks * 256, 128, CH), IDESC,
-               add || ks > 0 ? 1u : 0u);
+    for (int ks = 0; ks < TC_ROWS / 16; ++ks) tc_mma(tmem, a + ks * 16, b + ks * 16, IDESC, add || ks > 0 ? 1u : 0u);
 }
 
 __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t ncols, bool failed, int* err)
@@ -384,18 +394,19 @@ __device__ __forceinline__ uint4 add_bf16x8(uint4 a, uint4 b)
 // slots, the update), each staged while the step before is computed: two operand
 // buffers, a barrier a step.  in_tab [6][N]: (source node, edge) of every slot, -1 where
 // empty.  m non-NULL (training): m and the mask bits mm, mu are kept.
-constexpr int TC_SMEM_NODE_FWD = 4 * OP64 + 4 * W64, TC_CTAS_NODE_FWD = 2;
+constexpr int TC_SMEM_NODE_FWD = 4 * OP64 + 4 * W64 + 2 * SLOTS * TC_ROWS * 8, TC_CTAS_NODE_FWD = 2;
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_NODE_FWD)
-node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* __restrict__ h, const bf16* __restrict__ e,
+node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* h, const bf16* e,
                 const bf16* __restrict__ Wm, const float* __restrict__ bm, const bf16* __restrict__ Wu, const float* __restrict__ bu,
                 bf16* __restrict__ hout, bf16* __restrict__ m, uint2* __restrict__ mm, uint2* __restrict__ mu, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char* const Ws = tc_smem + 4 * OP64;
+    // rows of h and e (-1: none) of this and the next tile's slots [2][6][128]
+    int2* const tab = reinterpret_cast<int2*>(Ws + 4 * W64);
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
     __shared__ float bias[2][HD];
-    __shared__ unsigned char used[2][TC_ROWS];              // slot not empty (per operand buffer)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
     if (tid < HD) bias[0][tid] = bm[tid];
     else if (tid < 2 * HD) bias[1][tid - HD] = bu[tid - HD];
@@ -404,21 +415,17 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
     const int ntiles = (nodes + TC_ROWS - 1) / TC_ROWS;
     const int q = warp & 3, row = q * 32 + lane, cb = (warp >> 2) * (HD / 2);       // epilogue: accumulator row, first column
     const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16) + cb;
-    // what is staged next: tile lt, step ls, the table entries of this thread's rows
-    int lt = blockIdx.x, ls = 0, ln[4], lb[4];
-    int2 ent[4];
-    auto entries = [&]() {
-        if (lt >= ntiles || ls >= SLOTS) return;
+    auto lookup = [&](int t, int which) {
+        if (t >= ntiles) return;
+        const int n = t * TC_ROWS + (tid & (TC_ROWS - 1)), b = n / N, l = n - b * N;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (ls == 0) {
-                const int n = lt * TC_ROWS + srow + 32 * j;
-                lb[j] = n < nodes ? n / N : -1;
-                ln[j] = n - lb[j] * N;
-            }
-            ent[j] = lb[j] >= 0 ? in_tab[ls * N + ln[j]] : make_int2(-1, -1);
+        for (int s = tid >> 7; s < SLOTS; s += 2) {
+            int2 v = n < nodes ? in_tab[s * N + l] : make_int2(-1, -1);
+            if (v.x >= 0) v = make_int2(b * N + v.x, b * E + v.y);
+            tab[(which * SLOTS + s) * TC_ROWS + (tid & (TC_ROWS - 1))] = v;
         }
     };
+    int lt = blockIdx.x, ls = 0, lw = 0;                    // what is staged next: tile, step, its table
     auto stage = [&](int buf) {
         if (lt >= ntiles) return;
         unsigned char* A = tc_smem + buf * 2 * OP64;
@@ -426,24 +433,24 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
         for (int j = 0; j < 4; ++j) {
             const int r = srow + 32 * j;
             if (ls < SLOTS) {
-                const bool v = ent[j].x >= 0;
-                cp_async16_l1(op_at(A, q8, r), h + (v ? (size_t)lb[j] * N + ent[j].x : 0) * HD + q8 * 8, v);
-                cp_async16(op_at(A, 8 + q8, r), e + (v ? (size_t)lb[j] * E + ent[j].y : 0) * HD + q8 * 8, v);
-                if (q8 == 0) used[buf][r] = v;
+                const int2 v = tab[(lw * SLOTS + ls) * TC_ROWS + r];
+                cp_async16_l1(op_at(A, q8, r), h + (size_t)max(v.x, 0) * HD + q8 * 8, v.x >= 0);
+                cp_async16(op_at(A, 8 + q8, r), e + (size_t)max(v.y, 0) * HD + q8 * 8, v.x >= 0);
             } else {
                 const int n = lt * TC_ROWS + r;
                 cp_async16(op_at(A, q8, r), h + (size_t)(n < nodes ? n : 0) * HD + q8 * 8, n < nodes);
             }
         }
-        if (++ls > SLOTS) { ls = 0; lt += gridDim.x; }
-        entries();
+        if (++ls > SLOTS) { ls = 0; lt += gridDim.x; lw ^= 1; }
     };
-    entries();
+    lookup(blockIdx.x, 0);
+    __syncthreads();
+    pass_begin();
     if (!failed) stage(0);
     uint32_t phase = 0;
-    int buf = 0;
+    int buf = 0, which = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
         const int r0 = tile * TC_ROWS;
         float acc[HD / 2];
 #pragma unroll
@@ -456,10 +463,11 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
                 tc_commit(&bar_mma);
             }
             stage(buf ^ 1);
+            if (s == 1) lookup(tile + gridDim.x, which ^ 1);      // the other table's last row was staged a barrier ago
             ok = mbar_wait(&bar_mma, phase);
             phase ^= 1u;
             tc_fence_after();
-            const bool v = used[buf][row];
+            const bool v = tab[(which * SLOTS + s) * TC_ROWS + row].x >= 0;
             uint32_t bits = 0u;
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
@@ -532,7 +540,7 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
 // the sum of the edge's end rows is formed while staging.
 constexpr int TC_SMEM_EDGE_FWD = 2 * OP64 + 2 * W64, TC_CTAS_EDGE_FWD = 4;
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_EDGE_FWD)
-edge_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ h, const int2* __restrict__ ends, int N, int E,
+edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict__ ends, int N, int E,
                 const bf16* __restrict__ W, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -563,6 +571,7 @@ edge_fwd_kernel(int rows, const bf16* __restrict__ P0, const bf16* __restrict__ 
     };
     lookup(blockIdx.x, 0);
     __syncthreads();
+    pass_begin();
     int buf = 0;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
         const int r0 = tile * TC_ROWS;
@@ -684,16 +693,18 @@ constexpr int TC_CTAS_BWD = 2;
 // computed; two operand buffers.  Without PRE (the last layer) every node of a graph starts
 // from the readout's gradient dg [graphs][64]; without POST (the first) dh is not kept,
 // only its sums over the nodes of either orientation, part [CTA][2][64].
-constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64;
+constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64 + 4 * SLOTS * TC_ROWS * 4;
 template <bool PRE, bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
-node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
-                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* __restrict__ ds, const float* __restrict__ dg,
-                float* dh, const uint2* __restrict__ mu, const bf16* __restrict__ h, const bf16* __restrict__ m, const bf16* __restrict__ WuT,
+node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* mm, const bf16* dm,
+                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* ds, const float* dg,
+                float* dh, const uint2* mu, const bf16* h, const bf16* m, const bf16* __restrict__ WuT,
                 bf16* __restrict__ dmo, float* __restrict__ part, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 2 * OP64, *const Ws = tc_smem + 4 * OP64;     // Ws: Wm^T (h half), Wu^T
+    // of this and the next tile's slots [2][6][128], -1: none: target row * 8 + its slot, row of ds
+    int *const otab = reinterpret_cast<int*>(Ws + 3 * W64), *const itab = otab + 2 * SLOTS * TC_ROWS;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
@@ -703,22 +714,34 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
     float db[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
-        int nb[4], nl[4];                                   // graph (-1: no row) and node in the graph of this thread's rows
+    auto lookup = [&](int t, int which) {
+        if (!PRE || t >= ntiles) return;
+        const int r = tid & (TC_ROWS - 1), n = t * TC_ROWS + r, b = n / N, l = n - b * N;
+#pragma unroll
+        for (int s = tid >> 7; s < SLOTS; s += 2) {
+            const int o = n < nodes ? out_tab[s * N + l] : -1, i = n < nodes && inc ? inc[s * N + l] : -1;
+            otab[(which * SLOTS + s) * TC_ROWS + r] = o < 0 ? -1 : b * N * 8 + o;
+            itab[(which * SLOTS + s) * TC_ROWS + r] = i < 0 ? -1 : b * E + i;
+        }
+    };
+    lookup(blockIdx.x, 0);
+    __syncthreads();
+    pass_begin();
+    int which = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
         float4 ga[4], gb[4];                                // dh: columns 4 q8 .. and 32 + 4 q8 ..
+        lookup(tile + gridDim.x, which ^ 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = tile * TC_ROWS + srow + 32 * j;
             const bool v = n < nodes;
-            nb[j] = v ? n / N : -1;
-            nl[j] = n - nb[j] * N;
             if (POST) {
                 cp_async16(op_at(Xs, q8, srow + 32 * j), h + (size_t)(v ? n : 0) * HD + q8 * 8, v);
                 cp_async16(op_at(Xs, 8 + q8, srow + 32 * j), m + (size_t)(v ? n : 0) * HD + q8 * 8, v);
             }
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (v) {
-                const float4* gp = reinterpret_cast<const float4*>(PRE ? dh + (size_t)n * HD : dg + (size_t)nb[j] * HD);
+                const float4* gp = reinterpret_cast<const float4*>(PRE ? dh + (size_t)n * HD : dg + (size_t)(n / N) * HD);
                 ga[j] = gp[q8];
                 gb[j] = gp[8 + q8];
             }
@@ -730,11 +753,11 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
             auto load = [&](int s) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int t = nb[j] >= 0 ? out_tab[s * N + nl[j]] : -1;
+                    const int t = otab[(which * SLOTS + s) * TC_ROWS + srow + 32 * j];
                     z[j] = make_uint4(0u, 0u, 0u, 0u);
                     mk[j] = 0u;
                     if (t >= 0) {
-                        const size_t n = (size_t)nb[j] * N + (t >> 3);
+                        const size_t n = t >> 3;
                         z[j] = *reinterpret_cast<const uint4*>(dm + n * HD + q8 * 8);
                         mk[j] = mask_byte(mm, (size_t)(t & 7) * nodes + n, q8);
                     }
@@ -759,10 +782,10 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                     float4 x[4], y[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int ed = nb[j] >= 0 ? inc[s * N + nl[j]] : -1;
+                        const int ed = itab[(which * SLOTS + s) * TC_ROWS + srow + 32 * j];
                         x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (ed >= 0) {
-                            const float4* dp = reinterpret_cast<const float4*>(ds + ((size_t)nb[j] * E + ed) * HD);
+                            const float4* dp = reinterpret_cast<const float4*>(ds + (size_t)ed * HD);
                             x[j] = dp[q8];
                             y[j] = dp[8 + q8];
                         }
@@ -792,7 +815,7 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int n = tile * TC_ROWS + srow + 32 * j;
-                const uint2 mk = nb[j] >= 0 ? mu[n] : make_uint2(0u, 0u);
+                const uint2 mk = n < nodes ? mu[n] : make_uint2(0u, 0u);
                 const uint2 a = mask_f32x4(ga[j], mk.x >> (4 * q8)), b = mask_f32x4(gb[j], mk.y >> (4 * q8));
                 add_db(db, a.x, a.y);
                 add_db(db + 4, b.x, b.y);
@@ -821,7 +844,7 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                 ga[j] = add4(ga[j], *tile_f32(Xs, r, q8));
                 gb[j] = add4(gb[j], *tile_f32(Xs, r, 8 + q8));
                 const float4 a = *tile_f32(Zs, r, q8), b = *tile_f32(Zs, r, 8 + q8);
-                if (nb[j] < 0) continue;
+                if (n >= nodes) continue;
                 reinterpret_cast<uint2*>(dmo + (size_t)n * HD)[q8] = make_uint2(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w));
                 reinterpret_cast<uint2*>(dmo + (size_t)n * HD)[8 + q8] = make_uint2(pack_bf2(b.x, b.y), pack_bf2(b.z, b.w));
             }
@@ -829,7 +852,7 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = tile * TC_ROWS + srow + 32 * j;
-            if (nb[j] < 0) continue;
+            if (n >= nodes) continue;
             if (POST) {
                 reinterpret_cast<float4*>(dh + (size_t)n * HD)[q8] = ga[j];
                 reinterpret_cast<float4*>(dh + (size_t)n * HD)[8 + q8] = gb[j];
@@ -874,9 +897,9 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 constexpr int TC_SMEM_EDGE_BWD = 5 * OP64 + 3 * W64;
 template <bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
-edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const uint2* __restrict__ mm, const bf16* __restrict__ dm,
-                const bf16* __restrict__ h, const bf16* __restrict__ e, const bf16* __restrict__ WmT, float* de, int set,
-                const uint2* __restrict__ me, const bf16* __restrict__ eb, const bf16* __restrict__ WeT, float* __restrict__ ds,
+edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const uint2* mm, const bf16* dm,
+                const bf16* h, const bf16* e, const bf16* __restrict__ WmT, float* de, int set,
+                const uint2* me, const bf16* eb, const bf16* __restrict__ WeT, float* __restrict__ ds,
                 float* __restrict__ partm, float* __restrict__ parte, const int8_t* __restrict__ J, float* __restrict__ epart, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -888,29 +911,37 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
     const uint32_t tmem = tmem_sh;                          // dX, then dWm^T of direction 0 and 1, dWe^T: 64 columns each
     const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
     const size_t nodes = (size_t)(rows / E) * N;
+    __shared__ int4 tab[2][TC_ROWS];                        // this and the next tile: source row, target row * 8 + slot, twice; -1: no row
     __shared__ signed char cls[TC_ROWS];                    // coupler values of the tile (without POST)
     float sj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float dbm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dbe[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
     bool first = true;
-    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x) {
+    auto lookup = [&](int t, int which) {
+        if (t >= ntiles || tid >= TC_ROWS) return;
+        const int r = t * TC_ROWS + tid, b = r / E;
+        int4 v = r < rows ? msg_tab[r - b * E] : make_int4(-1, 0, 0, 0);
+        if (v.x >= 0) v = make_int4(b * N + v.x, b * N * 8 + v.y, b * N + v.z, b * N * 8 + v.w);
+        tab[which][tid] = v;
+    };
+    lookup(blockIdx.x, 0);
+    __syncthreads();
+    pass_begin();
+    int which = 0;
+    for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
         const int r0 = tile * TC_ROWS;
         if (!POST && tid < TC_ROWS) cls[tid] = r0 + tid < rows ? J[r0 + tid] : 1;
         int4 ent[4];
-        int bN[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int r = r0 + srow + 32 * j, b = r / E;
-            bN[j] = b * N;
-            ent[j] = r < rows ? msg_tab[r - b * E] : make_int4(-1, 0, 0, 0);
-        }
+        for (int j = 0; j < 4; ++j) ent[j] = tab[which][srow + 32 * j];
+        lookup(tile + gridDim.x, which ^ 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int row = srow + 32 * j;
             const bool v = ent[j].x >= 0;
-            cp_async16_l1(op_at(R0, q8, row), h + (v ? (size_t)bN[j] + ent[j].x : 0) * HD + q8 * 8, v);
+            cp_async16_l1(op_at(R0, q8, row), h + (size_t)(v ? ent[j].x : 0) * HD + q8 * 8, v);
             cp_async16(op_at(R1, q8, row), e + (size_t)(v ? r0 + row : 0) * HD + q8 * 8, v);
-            cp_async16_l1(op_at(R2, q8, row), h + (v ? (size_t)bN[j] + ent[j].z : 0) * HD + q8 * 8, v);
+            cp_async16_l1(op_at(R2, q8, row), h + (size_t)(v ? ent[j].z : 0) * HD + q8 * 8, v);
         }
         uint4 z0[4], z1[4];                                 // every load before the first use
         uint32_t m0[4], m1[4];
@@ -921,7 +952,7 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
             m0[j] = m1[j] = 0u;
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (ent[j].x >= 0) {
-                const size_t r = r0 + srow + 32 * j, n0 = (size_t)bN[j] + (ent[j].y >> 3), n1 = (size_t)bN[j] + (ent[j].w >> 3);
+                const size_t r = r0 + srow + 32 * j, n0 = ent[j].y >> 3, n1 = ent[j].w >> 3;
                 z0[j] = *reinterpret_cast<const uint4*>(dm + n0 * HD + q8 * 8);
                 z1[j] = *reinterpret_cast<const uint4*>(dm + n1 * HD + q8 * 8);
                 m0[j] = mask_byte(mm, (ent[j].y & 7) * nodes + n0, q8);
@@ -1144,6 +1175,7 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_kernel(Parts p, ReadoutGra
 {
     __shared__ float4 sm[RED_PER][RED_COLS + 1];
     const int k = blockIdx.y;
+    pass_begin();
     if (k == p.blocks) {
         readout_grad(r, reinterpret_cast<float*>(sm));
         return;
@@ -1204,6 +1236,7 @@ __global__ void pack_weights_kernel(int nmat, const bf16* const* __restrict__ Ws
 __global__ void embed_kernel(int B, int N, int E, const int* __restrict__ u, const int8_t* __restrict__ J,
                              const float* __restrict__ Xemb, const float* __restrict__ Jemb, bf16* h, bf16* e)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t nN = (size_t)B * N, total = (nN + (size_t)B * E) * (HD / 8);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
         const size_t row = i / (HD / 8);
@@ -1227,7 +1260,7 @@ __global__ void embed_kernel(int B, int N, int E, const int* __restrict__ u, con
 // summed node by node (64 threads, a column each) from rows that the block stages 64 at a
 // time, the next 64 on their way meanwhile.
 constexpr int RO_ROWS = 64, RO_THREADS = 256;
-__global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* __restrict__ h, const float* __restrict__ W1, const float* __restrict__ b1,
+__global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* h, const float* __restrict__ W1, const float* __restrict__ b1,
                                const float* __restrict__ w2, const float* __restrict__ b2, float* y, float* gbuf,
                                float* zbuf, const float* __restrict__ target, float inv_B, float* dybuf,
                                float* sqbuf, float* dgbuf, const int* __restrict__ err)
@@ -1236,6 +1269,7 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
     __shared__ float as[HD], red[HD], dz[HD];
     __shared__ __align__(16) bf16 rows[RO_ROWS][HD];
     const int b = blockIdx.x, tid = threadIdx.x, c = tid;
+    pass_begin();
     const uint4* src = reinterpret_cast<const uint4*>(h + (size_t)b * N * HD);
     constexpr int PER = RO_ROWS * HD / 8 / RO_THREADS;      // 16-byte pieces per thread
     uint4 v[PER];
@@ -1504,6 +1538,24 @@ void pack_weights(sg_model* M)
 const bf16* wpk_fwd(const sg_model* M, int l, int which) { return M->wpk + ((size_t)(l * 3 + which) * 2) * HD * KIN; }
 const bf16* wpk_bwd(const sg_model* M, int l, int which) { return wpk_fwd(M, l, which) + HD * KIN; }
 
+// One launch of a pass (see pass_begin); errors are left for cudaGetLastError.
+template <class... Params, class... Args>
+void launch(sg_model* M, void (*kernel)(Params...), dim3 grid, int threads, int smem, Args... args)
+{
+    cudaLaunchAttribute a = {};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = M->stream;
+    c.attrs = &a;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, args...);
+    M->launches++;
+}
+
 // The last layer updates no edges: nothing after it reads them.
 void forward(sg_model* M, int B, bool train)
 {
@@ -1513,28 +1565,29 @@ void forward(sg_model* M, int B, bool train)
                                                                              M->theta + M->oJ, M->h[0], M->e[0]);
     M->launches++;
     for (int l = 0; l < M->layers; ++l) {
-        node_fwd_kernel<<<tc_grid(M, B * N, TC_CTAS_NODE_FWD), TC_THREADS, TC_SMEM_NODE_FWD, st>>>(
+        launch(M, node_fwd_kernel, tc_grid(M, B * N, TC_CTAS_NODE_FWD), TC_THREADS, TC_SMEM_NODE_FWD,
             B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], wpk_fwd(M, l, 1), M->theta + M->obu[l],
             M->h[l + 1], train ? M->m[l] : nullptr, M->mm[l], M->mu[l], M->d_err);
-        M->launches++;
         if (l + 1 == M->layers) break;
-        edge_fwd_kernel<<<tc_grid(M, B * E, TC_CTAS_EDGE_FWD), TC_THREADS, TC_SMEM_EDGE_FWD, st>>>(
+        launch(M, edge_fwd_kernel, tc_grid(M, B * E, TC_CTAS_EDGE_FWD), TC_THREADS, TC_SMEM_EDGE_FWD,
             B * E, M->e[l], M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
             train ? M->me[l] : nullptr, M->d_err);
-        M->launches++;
     }
+}
+
+// Predictions; train: also the loss terms and the gradient of every graph's nodes.
+void readout(sg_model* M, int B, bool train)
+{
+    launch(M, readout_kernel, B, RO_THREADS, 0, M->N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1, M->theta + M->ow2,
+           M->theta + M->ob2, M->d_y, M->d_g, M->d_z, train ? M->d_t : nullptr, 1.f / (float)B, M->d_dy, M->d_sq, M->d_dg, M->d_err);
 }
 
 // Gradient of the mean squared error into M->grad; loss into M->dloss.
 void backward_all(sg_model* M, int B)
 {
     const int N = M->N, E = M->E;
-    cudaStream_t st = M->stream;
     float* G = M->grad;
-    readout_kernel<<<B, RO_THREADS, 0, st>>>(N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1, M->theta + M->ow2,
-                                             M->theta + M->ob2, M->d_y, M->d_g, M->d_z, M->d_t, 1.f / (float)B, M->d_dy,
-                                             M->d_sq, M->d_dg, M->d_err);
-    M->launches++;
+    readout(M, B, true);
     Parts parts;
     parts.blocks = 0;
     auto sum = [&](int64_t o, const float* src, int n, int count) {
@@ -1555,21 +1608,19 @@ void backward_all(sg_model* M, int B)
     float* const nepart = M->d_epart + (size_t)M->wcap * 6 * HD;
     auto node = [&](int l, auto kernel, int smem) {      // messages of layer l (if any), update of layer l - 1 (if any)
         const bool pre = l <= top, post = l > 0;
-        kernel<<<gn, TC_THREADS, smem, st>>>(
+        launch(M, kernel, gn, TC_THREADS, smem,
             (int)nodes, N, E, pre ? M->d_out_tab : nullptr, pre ? M->mm[l] : nullptr, M->dm[l & 1], pre ? wpk_bwd(M, l, 0) : nullptr,
             pre && post ? M->d_inc : nullptr, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
             post ? M->m[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 1) : nullptr, M->dm[(l & 1) ^ 1],
             post ? map(M->oWu[l - 1], gn) : nepart, M->d_err);
-        M->launches++;
     };
     auto edge = [&](int l, auto kernel, int smem) {
         const bool post = l > 0;
         float* pm = map(M->oWm[l], ge);
-        kernel<<<ge, TC_THREADS, smem, st>>>(
+        launch(M, kernel, ge, TC_THREADS, smem,
             B * E, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
             post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, pm,
             post ? map(M->oWe[l - 1], ge) : nullptr, M->d_J, M->d_epart, M->d_err);
-        M->launches++;
     };
     node(top + 1, node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD);
     for (int l = top; l > 0; --l) {
@@ -1582,8 +1633,7 @@ void backward_all(sg_model* M, int B)
     sum(M->oJ, M->d_epart, ge, 6 * HD);
     sum(M->oWe[top], nullptr, 0, WPART);
     const ReadoutGrad ro = {B, M->d_g, M->d_z, M->d_dy, M->d_sq, M->theta + M->ow2, M->dloss, G + M->oW1, G + M->ob1, G + M->ow2, G + M->ob2};
-    reduce_kernel<<<dim3((WPART / 4 + RED_COLS - 1) / RED_COLS, parts.blocks + 1), RED_THREADS, 0, st>>>(parts, ro);
-    M->launches++;
+    launch(M, reduce_kernel, dim3((WPART / 4 + RED_COLS - 1) / RED_COLS, parts.blocks + 1), RED_THREADS, 0, parts, ro);
 }
 
 // A tensor-core kernel whose bounded mbarrier wait ran out leaves 1 in d_err
@@ -1739,10 +1789,7 @@ int sg_forward(sg_model* M, int32_t L, int32_t B, const int8_t* J, float* y)
     int rc = load_batch(M, L, B, J, nullptr);
     if (rc) return rc;
     forward(M, B, false);
-    readout_kernel<<<B, RO_THREADS, 0, M->stream>>>(M->N, M->h[M->layers], M->theta + M->oW1, M->theta + M->ob1,
-                                            M->theta + M->ow2, M->theta + M->ob2, M->d_y, M->d_g, M->d_z, nullptr,
-                                            0.f, nullptr, nullptr, nullptr, M->d_err);
-    M->launches++;
+    readout(M, B, false);
     SK(cudaGetLastError(), "forward kernels");
     float out[4096 + 1];                             // the predictions and the status word (load_batch: B <= 4096)
     SK(cudaMemcpyAsync(out, M->d_y, sizeof(float) * ((size_t)B + 1), cudaMemcpyDeviceToHost, M->stream), "download y");
