@@ -351,7 +351,11 @@ constexpr int SLOTS = MAXDEG;
 
 // z's sign bit of the backward's mask: positive after rounding to BF16 (2^-133 is
 // the smallest BF16 number; 2^-134 and below round to zero).
-__device__ __forceinline__ uint32_t positive_bf16(float z) { return z > 0x1p-134f ? 1u : 0u; }
+// Appends it to `bits` from below.
+__device__ __forceinline__ uint32_t push_positive(uint32_t bits, float z)
+{
+    return __funnelshift_l(__float_as_uint(0x1p-134f - z), bits, 1);       // the sign bit of a NaN result is 0
+}
 
 // 8 BF16 values (one 16-byte chunk) with the columns whose mask bit is 0 cleared.
 __device__ __forceinline__ uint4 mask_bf16x8(uint4 v, uint32_t bits)
@@ -468,20 +472,21 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
             phase ^= 1u;
             tc_fence_after();
             const bool v = tab[(which * SLOTS + s) * TC_ROWS + row].x >= 0;
-            uint32_t bits = 0u;
+            float z[2][16];
+            tmem_ld16(tl, z[0]);
+            tmem_ld16(tl + 16, z[1]);
+            tmem_ld_wait();
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                float z[16];
-                tmem_ld16(tl + 16 * hh, z);
-                tmem_ld_wait();
+            for (int i = 0; i < 32; ++i) z[i >> 4][i & 15] += bias[0][cb + i];
+            if (m) {
+                uint32_t bits = 0u;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    z[i] += bias[0][cb + 16 * hh + i];
-                    bits |= positive_bf16(z[i]) << (16 * hh + i);
-                    acc[16 * hh + i] += v ? fmaxf(z[i], 0.f) : 0.f;
-                }
+                for (int i = 31; i >= 0; --i) bits = push_positive(bits, z[i >> 4][i & 15]);
+                if (r0 + row < nodes) reinterpret_cast<uint32_t*>(mm + (size_t)s * nodes + r0 + row)[warp >> 2] = bits;
             }
-            if (m && r0 + row < nodes) reinterpret_cast<uint32_t*>(mm + (size_t)s * nodes + r0 + row)[warp >> 2] = bits;
+            if (v)
+#pragma unroll
+                for (int i = 0; i < 32; ++i) acc[i] += fmaxf(z[i >> 4][i & 15], 0.f);
         }
         if (failed) break;
         // m: into the update's operand, and (training) to memory through the last slot's consumed operand
@@ -511,10 +516,11 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
             tmem_ld16(tl + 16 * hh, z);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                z[i] += bias[1][c0 + i];
-                bits |= positive_bf16(z[i]) << (16 * hh + i);
-            }
+            for (int i = 0; i < 16; ++i) z[i] += bias[1][c0 + i];
+            uint32_t part = 0u;
+#pragma unroll
+            for (int i = 15; i >= 0; --i) part = push_positive(part, z[i]);
+            bits |= part << (16 * hh);
 #pragma unroll
             for (int kc = 0; kc < 2; ++kc) {                // the residual input is staged: chunks c0 / 8 and c0 / 8 + 1
                 const uint4 b4 = *reinterpret_cast<const uint4*>(op_at(A, (c0 >> 3) + kc, row));
@@ -607,10 +613,11 @@ edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict_
             tmem_ld16(tl + 16 * hh, z);
             tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                z[i] += bias_sm[c0 + i];
-                bits |= positive_bf16(z[i]) << (16 * hh + i);
-            }
+            for (int i = 0; i < 16; ++i) z[i] += bias_sm[c0 + i];
+            uint32_t part = 0u;
+#pragma unroll
+            for (int i = 15; i >= 0; --i) part = push_positive(part, z[i]);
+            bits |= part << (16 * hh);
 #pragma unroll
             for (int kc = 0; kc < 2; ++kc) {                // the residual input is staged: chunks c0 / 8 and c0 / 8 + 1
                 const uint4 b4 = *reinterpret_cast<const uint4*>(op_at(As, (c0 >> 3) + kc, row));
