@@ -693,24 +693,27 @@ constexpr int TC_CTAS_BWD = 2;
 
 // Nodes.  PRE, messages of a layer: dh[n] += sum over the messages that n sends of
 // (dm[target] & mask) Wm[:, :64], slot by slot (out_tab [6][N]: target node * 8 + its slot,
-// -1 where empty), and dh[n] += sum over n's edges of ds (inc [6][N], NULL: none).
+// -1 where empty).
+// Both: dh[n] += the sums of the edge updates' gradients over n's edges, dc[n] for those in
+// its cell, ds of the up to two between cells (inter [2][N]: their number in the graph, -1
+// where empty).
 // POST, node update of the layer below: dZ = dh & mu, dh += dX[:, :64], dmo = dX[:, 64:]
 // rounded to BF16 (the one form that the messages' dZ = dm & mask takes it in), weight
 // gradient with X = [h | m].  A slot's rows are loaded while the slot before is
 // computed; two operand buffers.  Without PRE (the last layer) every node of a graph starts
 // from the readout's gradient dg [graphs][64]; without POST (the first) dh is not kept,
 // only its sums over the nodes of either orientation, part [CTA][2][64].
-constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64 + 4 * SLOTS * TC_ROWS * 4;
+constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64 + 2 * (SLOTS + 2) * TC_ROWS * 4;
 template <bool PRE, bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
 node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* mm, const bf16* dm,
-                const bf16* __restrict__ WmT, const int* __restrict__ inc, const float* ds, const float* dg,
+                const bf16* __restrict__ WmT, const int* __restrict__ inter, const float* dc, const float* ds, const float* dg,
                 float* dh, const uint2* mu, const bf16* h, const bf16* m, const bf16* __restrict__ WuT,
                 bf16* __restrict__ dmo, float* __restrict__ part, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 2 * OP64, *const Ws = tc_smem + 4 * OP64;     // Ws: Wm^T (h half), Wu^T
-    // of this and the next tile's slots [2][6][128], -1: none: target row * 8 + its slot, row of ds
+    // of this and the next tile, -1: none: target row * 8 + its slot [2][6][128], rows of ds [2][2][128]
     int *const otab = reinterpret_cast<int*>(Ws + 3 * W64), *const itab = otab + 2 * SLOTS * TC_ROWS;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
@@ -726,9 +729,12 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
         const int r = tid & (TC_ROWS - 1), n = t * TC_ROWS + r, b = n / N, l = n - b * N;
 #pragma unroll
         for (int s = tid >> 7; s < SLOTS; s += 2) {
-            const int o = n < nodes ? out_tab[s * N + l] : -1, i = n < nodes && inc ? inc[s * N + l] : -1;
+            const int o = n < nodes ? out_tab[s * N + l] : -1;
             otab[(which * SLOTS + s) * TC_ROWS + r] = o < 0 ? -1 : b * N * 8 + o;
-            itab[(which * SLOTS + s) * TC_ROWS + r] = i < 0 ? -1 : b * E + i;
+        }
+        if (POST) {
+            const int s = tid >> 7, i = n < nodes ? inter[s * N + l] : -1;
+            itab[(which * 2 + s) * TC_ROWS + r] = i < 0 ? -1 : b * (E - 2 * N) + i;
         }
     };
     lookup(blockIdx.x, 0);
@@ -771,6 +777,23 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                 }
             };
             load(0);
+            if (POST) {
+                float4 x[4], y[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int n = tile * TC_ROWS + srow + 32 * j;
+                    x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (n < nodes) {
+                        x[j] = reinterpret_cast<const float4*>(dc + (size_t)n * HD)[q8];
+                        y[j] = reinterpret_cast<const float4*>(dc + (size_t)n * HD)[8 + q8];
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    ga[j] = add4(ga[j], x[j]);
+                    gb[j] = add4(gb[j], y[j]);
+                }
+            }
             for (int s = 0; s < SLOTS; ++s) {
                 unsigned char* const Z = Zs + (s & 1) * OP64;     // its MMA before last is done: the wait below
 #pragma unroll
@@ -785,11 +808,11 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                     tc_commit(&bar_mma);
                 }
                 if (s + 1 < SLOTS) load(s + 1);
-                if (inc) {
+                if (POST && s < 2) {
                     float4 x[4], y[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int ed = itab[(which * SLOTS + s) * TC_ROWS + srow + 32 * j];
+                        const int ed = itab[(which * 2 + s) * TC_ROWS + srow + 32 * j];
                         x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (ed >= 0) {
                             const float4* dp = reinterpret_cast<const float4*>(ds + (size_t)ed * HD);
@@ -893,20 +916,25 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 // Edges.  Messages of a layer, edge half, both directions d of an edge (msg_tab [E]: source
 // node and target node * 8 + its slot of either): dZ_d = dm[target] & mask,
 // de += sum_d dX_d[:, 64:] (set: =), weight gradient with X_d = [h[src_d] | e].
-// POST, edge update of the layer below: dZ = de & me, de += dX[:, :64], ds = dX[:, 64:] (FP32),
-// weight gradient with X = [eb | h_i + h_j], whose end rows are the messages' source rows.
+// POST, edge update of the layer below: dZ = de & me, de += dX[:, :64], weight gradient with
+// X = [eb | h_i + h_j], whose end rows are the messages' source rows.  dX[:, 64:] (FP32) goes to
+// the edge's two nodes: a tile is 8 cells (16 edges each) or 128 edges between cells;
+// the former sums it for its 64 nodes (dc), the latter keeps its rows (ds), so that
+// node_bwd_kernel reads 3 rows a node instead of 6.
 // Operands R0 | R1 | R2: h[src_0], e, h[src_1], then (POST) eb in R1 and the sum in R2.
 // The two directions' weight gradients differ in the order of their halves ([R0 | R1] and
 // [R1 | R2]) and are kept apart in tensor memory.  Without POST (the first layer) de is not
 // kept, only its sums over the edges of every coupler value (J; -3 .. 3 without 0), epart
 // [CTA][6][64]: the finished tile goes back to shared memory and a thread adds up a
 // column of 32 rows, a row's class being the same for the whole warp.
+__host__ __device__ inline int edge_tiles_in(int graphs, int N) { return (graphs * (N / 8) + 7) / 8; }
+__host__ __device__ inline int edge_tiles_between(int graphs, int N, int E) { return (graphs * (E - 2 * N) + TC_ROWS - 1) / TC_ROWS; }
 constexpr int TC_SMEM_EDGE_BWD = 5 * OP64 + 3 * W64;
 template <bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
-edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const uint2* mm, const bf16* dm,
+edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, const uint2* mm, const bf16* dm,
                 const bf16* h, const bf16* e, const bf16* __restrict__ WmT, float* de, int set,
-                const uint2* me, const bf16* eb, const bf16* __restrict__ WeT, float* __restrict__ ds,
+                const uint2* me, const bf16* eb, const bf16* __restrict__ WeT, float* __restrict__ ds, float* __restrict__ dc,
                 float* __restrict__ partm, float* __restrict__ parte, const int8_t* __restrict__ J, float* __restrict__ epart, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
@@ -916,9 +944,10 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
     bool failed = !tc_setup(&tmem_sh, &bar_w, &bar_mma, 256, Ws, WmT, W64, WeT, POST ? 2 * W64 : 0);
     const uint32_t tmem = tmem_sh;                          // dX, then dWm^T of direction 0 and 1, dWe^T: 64 columns each
-    const int ntiles = (rows + TC_ROWS - 1) / TC_ROWS;
-    const size_t nodes = (size_t)(rows / E) * N;
-    __shared__ int4 tab[2][TC_ROWS];                        // this and the next tile: source row, target row * 8 + slot, twice; -1: no row
+    const int nin = edge_tiles_in(graphs, N), ntiles = nin + edge_tiles_between(graphs, N, E), nodes = graphs * N;
+    // this and the next tile: source row, target row * 8 + slot, twice; edge row, -1: none
+    __shared__ int4 tab[2][TC_ROWS];
+    __shared__ int erow[2][TC_ROWS];
     __shared__ signed char cls[TC_ROWS];                    // coupler values of the tile (without POST)
     float sj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float dbm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dbe[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -926,29 +955,40 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
     bool first = true;
     auto lookup = [&](int t, int which) {
         if (t >= ntiles || tid >= TC_ROWS) return;
-        const int r = t * TC_ROWS + tid, b = r / E;
-        int4 v = r < rows ? msg_tab[r - b * E] : make_int4(-1, 0, 0, 0);
-        if (v.x >= 0) v = make_int4(b * N + v.x, b * N * 8 + v.y, b * N + v.z, b * N * 8 + v.w);
+        const bool in = t < nin;
+        const int per = in ? N / 8 : E - 2 * N, g = in ? t * 8 + (tid >> 4) : (t - nin) * TC_ROWS + tid;     // cells, edges between them
+        int4 v = make_int4(0, 0, 0, 0);
+        int r = -1;
+        if (g < graphs * per) {
+            const int b = g / per, l = in ? (g - b * per) * 16 + (tid & 15) : 2 * N + g - b * per;
+            v = msg_tab[l];
+            v = make_int4(b * N + v.x, b * N * 8 + v.y, b * N + v.z, b * N * 8 + v.w);
+            r = b * E + l;
+        }
         tab[which][tid] = v;
+        erow[which][tid] = r;
     };
     lookup(blockIdx.x, 0);
     __syncthreads();
     pass_begin();
     int which = 0;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
-        const int r0 = tile * TC_ROWS;
-        if (!POST && tid < TC_ROWS) cls[tid] = r0 + tid < rows ? J[r0 + tid] : 1;
+        if (!POST && tid < TC_ROWS) cls[tid] = erow[which][tid] >= 0 ? J[erow[which][tid]] : 1;
         int4 ent[4];
+        int er[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ent[j] = tab[which][srow + 32 * j];
+        for (int j = 0; j < 4; ++j) {
+            ent[j] = tab[which][srow + 32 * j];
+            er[j] = erow[which][srow + 32 * j];
+        }
         lookup(tile + gridDim.x, which ^ 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int row = srow + 32 * j;
-            const bool v = ent[j].x >= 0;
-            cp_async16_l1(op_at(R0, q8, row), h + (size_t)(v ? ent[j].x : 0) * HD + q8 * 8, v);
-            cp_async16(op_at(R1, q8, row), e + (size_t)(v ? r0 + row : 0) * HD + q8 * 8, v);
-            cp_async16_l1(op_at(R2, q8, row), h + (size_t)(v ? ent[j].z : 0) * HD + q8 * 8, v);
+            const bool v = er[j] >= 0;
+            cp_async16_l1(op_at(R0, q8, row), h + (size_t)ent[j].x * HD + q8 * 8, v);
+            cp_async16(op_at(R1, q8, row), e + (size_t)max(er[j], 0) * HD + q8 * 8, v);
+            cp_async16_l1(op_at(R2, q8, row), h + (size_t)ent[j].z * HD + q8 * 8, v);
         }
         uint4 z0[4], z1[4];                                 // every load before the first use
         uint32_t m0[4], m1[4];
@@ -958,12 +998,12 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
             z0[j] = z1[j] = make_uint4(0u, 0u, 0u, 0u);
             m0[j] = m1[j] = 0u;
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (ent[j].x >= 0) {
-                const size_t r = r0 + srow + 32 * j, n0 = ent[j].y >> 3, n1 = ent[j].w >> 3;
+            if (er[j] >= 0) {
+                const size_t r = er[j], n0 = ent[j].y >> 3, n1 = ent[j].w >> 3;
                 z0[j] = *reinterpret_cast<const uint4*>(dm + n0 * HD + q8 * 8);
                 z1[j] = *reinterpret_cast<const uint4*>(dm + n1 * HD + q8 * 8);
-                m0[j] = mask_byte(mm, (ent[j].y & 7) * nodes + n0, q8);
-                m1[j] = mask_byte(mm, (ent[j].w & 7) * nodes + n1, q8);
+                m0[j] = mask_byte(mm, (size_t)(ent[j].y & 7) * nodes + n0, q8);
+                m1[j] = mask_byte(mm, (size_t)(ent[j].w & 7) * nodes + n1, q8);
                 if (!set) {
                     ga[j] = reinterpret_cast<const float4*>(de + r * HD)[q8];
                     gb[j] = reinterpret_cast<const float4*>(de + r * HD)[8 + q8];
@@ -997,7 +1037,7 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int row = srow + 32 * j;
-                cp_async16(op_at(R1, q8, row), eb + (size_t)(ent[j].x >= 0 ? r0 + row : 0) * HD + q8 * 8, ent[j].x >= 0);
+                cp_async16(op_at(R1, q8, row), eb + (size_t)max(er[j], 0) * HD + q8 * 8, er[j] >= 0);
                 uint4* const s = reinterpret_cast<uint4*>(op_at(R2, q8, row));
                 *s = add_bf16x8(*reinterpret_cast<const uint4*>(op_at(R0, q8, row)), *s);
             }
@@ -1016,7 +1056,7 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int row = srow + 32 * j;
-                const uint2 k = ent[j].x >= 0 ? me[r0 + row] : make_uint2(0u, 0u);
+                const uint2 k = er[j] >= 0 ? me[er[j]] : make_uint2(0u, 0u);
                 const uint2 a = mask_f32x4(ga[j], k.x >> (4 * q8)), b = mask_f32x4(gb[j], k.y >> (4 * q8));
                 add_db(dbe, a.x, a.y);
                 add_db(dbe + 4, b.x, b.y);
@@ -1039,16 +1079,31 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
                 tc_fence_before();
                 __syncthreads();
                 tc_fence_after();
+                if (half == 0) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int row = srow + 32 * j;
-                    const float4 a = *tile_f32(R0, row, q8), b = *tile_f32(R0, row, 8 + q8);
-                    if (half == 0) {
-                        ga[j] = add4(ga[j], a);
-                        gb[j] = add4(gb[j], b);
-                    } else if (ent[j].x >= 0) {
-                        reinterpret_cast<float4*>(ds + (size_t)(r0 + row) * HD)[q8] = a;
-                        reinterpret_cast<float4*>(ds + (size_t)(r0 + row) * HD)[8 + q8] = b;
+                    for (int j = 0; j < 4; ++j) {
+                        ga[j] = add4(ga[j], *tile_f32(R0, srow + 32 * j, q8));
+                        gb[j] = add4(gb[j], *tile_f32(R0, srow + 32 * j, 8 + q8));
+                    }
+                } else if (tile < nin) {                    // node 8 c + 4 u + k of the tile: edges 16 c + 4 k + k' (u = 0), 16 c + 4 k' + k
+                    const int c = tid & 15;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int nd = (tid >> 4) + 16 * i, step = nd & 4 ? 4 : 1, first_row = (nd >> 3) * 16 + (nd & 3) * (nd & 4 ? 1 : 4);
+                        float4 x = *tile_f32(R0, first_row, c);
+#pragma unroll
+                        for (int k = 1; k < 4; ++k) x = add4(x, *tile_f32(R0, first_row + k * step, c));
+                        if (tile * 64 + nd < nodes) reinterpret_cast<float4*>(dc + (size_t)(tile * 64 + nd) * HD)[c] = x;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int row = srow + 32 * j;
+                        const float4 a = *tile_f32(R0, row, q8), b = *tile_f32(R0, row, 8 + q8);
+                        if (er[j] < 0) continue;
+                        float4* const dp = reinterpret_cast<float4*>(ds + ((size_t)(tile - nin) * TC_ROWS + row) * HD);
+                        dp[q8] = a;
+                        dp[8 + q8] = b;
                     }
                 }
             }
@@ -1058,16 +1113,16 @@ edge_bwd_kernel(int rows, int N, int E, const int4* __restrict__ msg_tab, const 
         if (POST) {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (ent[j].x >= 0) {
-                    reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[q8] = ga[j];
-                    reinterpret_cast<float4*>(de + (size_t)(r0 + srow + 32 * j) * HD)[8 + q8] = gb[j];
+                if (er[j] >= 0) {
+                    reinterpret_cast<float4*>(de + (size_t)er[j] * HD)[q8] = ga[j];
+                    reinterpret_cast<float4*>(de + (size_t)er[j] * HD)[8 + q8] = gb[j];
                 }
         } else {
             const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {                   // the places that this thread has read
-                *tile_f32(Zs, srow + 32 * j, q8) = ent[j].x >= 0 ? ga[j] : zero;
-                *tile_f32(Zs, srow + 32 * j, 8 + q8) = ent[j].x >= 0 ? gb[j] : zero;
+                *tile_f32(Zs, srow + 32 * j, q8) = er[j] >= 0 ? ga[j] : zero;
+                *tile_f32(Zs, srow + 32 * j, 8 + q8) = er[j] >= 0 ? gb[j] : zero;
             }
             __syncthreads();
             const int c = tid & (HD - 1);
@@ -1382,7 +1437,7 @@ struct sg_model {
     std::vector<int64_t> oWm, obm, oWu, obu, oWe, obe;
     // graph + activation buffers for the current (L, Bcap)
     int L = 0, N = 0, E = 0, Bcap = 0;
-    int *d_u = nullptr, *d_inc = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
+    int *d_u = nullptr, *d_inter = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
     int2 *d_ends = nullptr, *d_in_tab = nullptr;
     int4* d_msg_tab = nullptr;
     int8_t* d_J = nullptr;
@@ -1392,7 +1447,7 @@ struct sg_model {
     float* d_epart = nullptr;                 // embedding-gradient partials: edges [CTAs][6][64], then nodes [CTAs][2][64]
     std::vector<bf16*> h, e, m;
     std::vector<uint2*> mm, mu, me;   // per layer: sign bits of the message, node and edge pre-activations
-    float *dh = nullptr, *de = nullptr, *ds = nullptr;
+    float *dh = nullptr, *de = nullptr, *ds = nullptr, *dc = nullptr;
     bf16* dm[2] = {nullptr, nullptr};         // messages' gradient of this layer and of the one below
     float* wpart = nullptr;       // weight-gradient partials: [3 layers maps][wcap CTAs][WPART]
     int wcap = 0;
@@ -1425,13 +1480,13 @@ cudaError_t salloc(T** p, size_t n)
 
 void free_graph(sg_model* M)
 {
-    cudaFree(M->d_u); cudaFree(M->d_inc); cudaFree(M->d_out_tab);
+    cudaFree(M->d_u); cudaFree(M->d_inter); cudaFree(M->d_out_tab);
     cudaFree(M->d_ends); cudaFree(M->d_in_tab); cudaFree(M->d_msg_tab);
-    M->d_u = M->d_inc = M->d_out_tab = nullptr;
+    M->d_u = M->d_inter = M->d_out_tab = nullptr;
     M->d_ends = M->d_in_tab = nullptr;
     M->d_msg_tab = nullptr;
     cudaFree(M->d_J); M->d_J = nullptr;
-    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_dg, &M->d_epart, &M->dh, &M->de, &M->ds, &M->wpart};
+    float** fl[] = {&M->d_t, &M->d_y, &M->d_g, &M->d_z, &M->d_dy, &M->d_sq, &M->d_dg, &M->d_epart, &M->dh, &M->de, &M->ds, &M->dc, &M->wpart};
     for (float** p : fl) { cudaFree(*p); *p = nullptr; }
     for (bf16*& p : M->dm) { cudaFree(p); p = nullptr; }
     for (auto* v : {&M->h, &M->e, &M->m}) {
@@ -1450,6 +1505,11 @@ int tc_grid(const sg_model* M, int rows, int ctas_per_sm)
 {
     const int tiles = (rows + TC_ROWS - 1) / TC_ROWS, cap = ctas_per_sm * M->sms;
     return tiles < cap ? (tiles > 0 ? tiles : 1) : cap;
+}
+
+int edge_grid(const sg_model* M, int B, int N, int E)
+{
+    return tc_grid(M, (edge_tiles_in(B, N) + edge_tiles_between(B, N, E)) * TC_ROWS, TC_CTAS_BWD);
 }
 
 // Builds the Chimera C_L topology in the coupler order of pt.h and sizes the
@@ -1472,8 +1532,9 @@ int prepare(sg_model* M, int L, int B)
         for (int c = 0; c + 1 < L; ++c)
             for (int k = 0; k < 4; ++k) { ei.push_back(idx(r, c, 1, k)); ej.push_back(idx(r, c + 1, 1, k)); }
     // messages 2e: source ej -> target ei, 2e + 1: source ei -> target ej.  A node's incoming and outgoing
-    // messages and its edges fill its 6 slots in ascending order; tables are slot-major [6][N]
-    std::vector<int> u(N), inc(N * MAXDEG, -1), out_tab(N * MAXDEG, -1);
+    // messages fill its 6 slots in ascending order, its edges between cells (numbers 16 L^2 and up) 2;
+    // tables are slot-major [6][N], [2][N]
+    std::vector<int> u(N), inter(2 * N, -1), out_tab(N * MAXDEG, -1);
     std::vector<int2> ends(E), in_tab(N * MAXDEG, make_int2(-1, -1));
     std::vector<int4> msg_tab(E);
     std::vector<int> cin(N, 0), cout(N, 0), cinc(N, 0);
@@ -1488,8 +1549,9 @@ int prepare(sg_model* M, int L, int B)
             out_tab[cout[src]++ * N + src] = at[d];
         }
         msg_tab[e2] = make_int4(ej[e2], at[0], ei[e2], at[1]);
-        inc[cinc[ei[e2]]++ * N + ei[e2]] = e2;
-        inc[cinc[ej[e2]]++ * N + ej[e2]] = e2;
+        if (e2 < 2 * N) continue;
+        inter[cinc[ei[e2]]++ * N + ei[e2]] = e2 - 2 * N;
+        inter[cinc[ej[e2]]++ * N + ej[e2]] = e2 - 2 * N;
     }
     auto up = [&](auto** d, const auto& v) -> cudaError_t {
         cudaError_t r = salloc(d, v.size());
@@ -1497,7 +1559,7 @@ int prepare(sg_model* M, int L, int B)
         return cudaMemcpy(*d, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
     };
     SK(up(&M->d_u, u), "upload topology");
-    SK(up(&M->d_inc, inc), "upload topology");
+    SK(up(&M->d_inter, inter), "upload topology");
     SK(up(&M->d_out_tab, out_tab), "upload topology");
     SK(up(&M->d_ends, ends), "upload topology");
     SK(up(&M->d_in_tab, in_tab), "upload topology");
@@ -1522,13 +1584,14 @@ int prepare(sg_model* M, int L, int B)
         SK(salloc(&M->mu[l], nN), "cudaMalloc node mask");
         if (l + 1 < M->layers) SK(salloc(&M->me[l], nE), "cudaMalloc edge mask");
     }
-    M->wcap = tc_grid(M, B * E, TC_CTAS_BWD);
+    M->wcap = edge_grid(M, B, N, E);
     SK(salloc(&M->d_epart, (size_t)M->wcap * 8 * HD), "cudaMalloc embedding partials");
     SK(salloc(&M->wpart, (size_t)3 * M->layers * M->wcap * WPART), "cudaMalloc wpart");
     SK(salloc(&M->dh, nN * HD), "cudaMalloc dh");
     for (bf16*& p : M->dm) SK(salloc(&p, nN * HD), "cudaMalloc dm");
     SK(salloc(&M->de, nE * HD), "cudaMalloc de");
-    SK(salloc(&M->ds, nE * HD), "cudaMalloc ds");
+    SK(salloc(&M->ds, (size_t)B * (E - 2 * N) * HD), "cudaMalloc ds");
+    SK(salloc(&M->dc, nN * HD), "cudaMalloc dc");
     M->L = L; M->N = N; M->E = E; M->Bcap = B;
     return PT_OK;
 }
@@ -1610,14 +1673,14 @@ void backward_all(sg_model* M, int B)
         return p;
     };
     // layer l's node update; then per layer its messages with the updates of the layer below
-    const int top = M->layers - 1, gn = tc_grid(M, B * N, TC_CTAS_BWD), ge = tc_grid(M, B * E, TC_CTAS_BWD);
+    const int top = M->layers - 1, gn = tc_grid(M, B * N, TC_CTAS_BWD), ge = edge_grid(M, B, N, E);
     const size_t nodes = (size_t)B * N;
     float* const nepart = M->d_epart + (size_t)M->wcap * 6 * HD;
     auto node = [&](int l, auto kernel, int smem) {      // messages of layer l (if any), update of layer l - 1 (if any)
         const bool pre = l <= top, post = l > 0;
         launch(M, kernel, gn, TC_THREADS, smem,
             (int)nodes, N, E, pre ? M->d_out_tab : nullptr, pre ? M->mm[l] : nullptr, M->dm[l & 1], pre ? wpk_bwd(M, l, 0) : nullptr,
-            pre && post ? M->d_inc : nullptr, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
+            pre && post ? M->d_inter : nullptr, M->dc, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
             post ? M->m[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 1) : nullptr, M->dm[(l & 1) ^ 1],
             post ? map(M->oWu[l - 1], gn) : nepart, M->d_err);
     };
@@ -1625,8 +1688,8 @@ void backward_all(sg_model* M, int B)
         const bool post = l > 0;
         float* pm = map(M->oWm[l], ge);
         launch(M, kernel, ge, TC_THREADS, smem,
-            B * E, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
-            post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, pm,
+            B, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
+            post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, M->dc, pm,
             post ? map(M->oWe[l - 1], ge) : nullptr, M->d_J, M->d_epart, M->d_err);
     };
     node(top + 1, node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD);
