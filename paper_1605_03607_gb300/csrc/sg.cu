@@ -23,9 +23,10 @@
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
 // messages, pre-activations and masked gradients in memory (97 launches, 19 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.31 ms, of 128 C_4 graphs 1.01 -> 0.32 ms, 64 C_8
-// predictions 0.42 -> 0.17 ms.  (With a kernel per map and message rows of 21 nodes
+// gradient of 256 C_8 graphs 3.95 -> 1.24 ms, of 128 C_4 graphs 1.01 -> 0.30 ms, 64 C_8
+// predictions 0.42 -> 0.16 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -543,9 +544,12 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
 }
 
 // Edge update: Y = P0 + relu([P0 | h[i] + h[j]] W^T + bias) as BF16 and the mask bits;
-// the sum of the edge's end rows is formed while staging.
-constexpr int TC_SMEM_EDGE_FWD = 2 * OP64 + 2 * W64, TC_CTAS_EDGE_FWD = 4;
-__global__ void __launch_bounds__(TC_THREADS, TC_CTAS_EDGE_FWD)
+// the sum of the edge's end rows is formed while staging.  3 CTAs an SM up to 12 tiles an
+// SM, 4 above: the fewer have more L1 for the gathered rows (64 C_8 predictions 166 ->
+// 157 us), the more hide more latency (256: 434 -> 414 us).
+constexpr int TC_SMEM_EDGE_FWD = 2 * OP64 + 2 * W64, EDGE_FWD_FEW = 12;
+template <int CTAS>
+__global__ void __launch_bounds__(TC_THREADS, CTAS)
 edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict__ ends, int N, int E,
                 const bf16* __restrict__ W, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask, int* err)
 {
@@ -582,17 +586,22 @@ edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict_
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, buf ^= 1) {
         const int r0 = tile * TC_ROWS;
         uint4 a[4], b[4];                                   // every load before the first use
+        int2 ij[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ij[j] = endn[buf][srow + 32 * j];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            a[j] = b[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (ij[j].x >= 0) {
+                a[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij[j].x * HD + q8 * 8);
+                b[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij[j].y * HD + q8 * 8);
+            }
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int r = srow + 32 * j;
-            const int2 ij = endn[buf][r];
-            const bool v = ij.x >= 0;
+            const bool v = ij[j].x >= 0;
             cp_async16(op_at(As, q8, r), P0 + (size_t)(v ? r0 + r : 0) * HD + q8 * 8, v);
-            a[j] = b[j] = make_uint4(0u, 0u, 0u, 0u);
-            if (v) {
-                a[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij.x * HD + q8 * 8);
-                b[j] = *reinterpret_cast<const uint4*>(h + (size_t)ij.y * HD + q8 * 8);
-            }
         }
         lookup(tile + gridDim.x, buf ^ 1);
 #pragma unroll
@@ -1608,6 +1617,8 @@ void pack_weights(sg_model* M)
 const bf16* wpk_fwd(const sg_model* M, int l, int which) { return M->wpk + ((size_t)(l * 3 + which) * 2) * HD * KIN; }
 const bf16* wpk_bwd(const sg_model* M, int l, int which) { return wpk_fwd(M, l, which) + HD * KIN; }
 
+// More than half of an SM's shared memory (see launch): gradient of 32 C_8 graphs 325 -> 292 us.
+constexpr int TC_SMEM_ALONE = 116 * 1024;
 // One launch of a pass (see pass_begin); errors are left for cudaGetLastError.
 template <class... Params, class... Args>
 void launch(sg_model* M, void (*kernel)(Params...), dim3 grid, int threads, int smem, Args... args)
@@ -1618,7 +1629,9 @@ void launch(sg_model* M, void (*kernel)(Params...), dim3 grid, int threads, int 
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = dim3(threads);
-    c.dynamicSmemBytes = smem;
+    // CTAs that may start while the kernel before drains go where there is room first: a grid of at most one
+    // CTA per SM would share SMs and leave others idle, so it takes more than half of an SM's shared memory
+    c.dynamicSmemBytes = smem > 0 && 2 * (int)grid.x > M->sms && (int)grid.x <= M->sms ? std::max(smem, TC_SMEM_ALONE) : smem;
     c.stream = M->stream;
     c.attrs = &a;
     c.numAttrs = 1;
@@ -1639,7 +1652,8 @@ void forward(sg_model* M, int B, bool train)
             B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], wpk_fwd(M, l, 1), M->theta + M->obu[l],
             M->h[l + 1], train ? M->m[l] : nullptr, M->mm[l], M->mu[l], M->d_err);
         if (l + 1 == M->layers) break;
-        launch(M, edge_fwd_kernel, tc_grid(M, B * E, TC_CTAS_EDGE_FWD), TC_THREADS, TC_SMEM_EDGE_FWD,
+        const bool few = (B * E + TC_ROWS - 1) / TC_ROWS <= EDGE_FWD_FEW * M->sms;
+        launch(M, few ? edge_fwd_kernel<3> : edge_fwd_kernel<4>, tc_grid(M, B * E, few ? 3 : 4), TC_THREADS, TC_SMEM_EDGE_FWD,
             B * E, M->e[l], M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
             train ? M->me[l] : nullptr, M->d_err);
     }
@@ -1800,14 +1814,15 @@ int sg_create(sg_model** out, int32_t hidden, int32_t layers, void* stream)
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const struct { const void* k; int smem; } tk[] = {
             {(const void*)node_fwd_kernel, TC_SMEM_NODE_FWD},
-            {(const void*)edge_fwd_kernel, TC_SMEM_EDGE_FWD},
+            {(const void*)edge_fwd_kernel<3>, TC_SMEM_EDGE_FWD},
+            {(const void*)edge_fwd_kernel<4>, TC_SMEM_EDGE_FWD},
             {(const void*)node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD},
             {(const void*)node_bwd_kernel<true, true>, TC_SMEM_NODE_BWD},
             {(const void*)node_bwd_kernel<true, false>, TC_SMEM_NODE_BWD},
             {(const void*)edge_bwd_kernel<true>, TC_SMEM_EDGE_BWD},
             {(const void*)edge_bwd_kernel<false>, TC_SMEM_EDGE_BWD}};
         for (const auto& t : tk)
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(t.k, cudaFuncAttributeMaxDynamicSharedMemorySize, t.smem);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(t.k, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(t.smem, TC_SMEM_ALONE));
         if (e != cudaSuccess) {
             M->err = std::string("tensor-core set-up: ") + cudaGetErrorString(e);
             return bail(PT_ERR_CUDA);
