@@ -22,9 +22,9 @@
 // batches.  So per layer 2 forward and 2 backward kernels, each with every linear map of
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
-// messages, pre-activations and masked gradients in memory (97 launches, 19 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.24 ms, of 128 C_4 graphs 1.01 -> 0.30 ms, 64 C_8
-// predictions 0.42 -> 0.16 ms.  (With a kernel per map and message rows of 21 nodes
+// messages, pre-activations and masked gradients in memory (97 launches, 18 now):
+// gradient of 256 C_8 graphs 3.95 -> 1.20 ms, of 128 C_4 graphs 1.01 -> 0.29 ms, 64 C_8
+// predictions 0.42 -> 0.15 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <algorithm>
 #include <cmath>
@@ -163,6 +163,12 @@ __device__ __forceinline__ void cp_async16_l1(void* dst, const void* src, bool v
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0)
                  : "memory");
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid, bool l1)
+{
+    if (l1) cp_async16_l1(dst, src, valid);
+    else cp_async16(dst, src, valid);
 }
 
 __device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accum)
@@ -346,9 +352,16 @@ __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t ncols, bool 
 //     tensor memory;
 //   * a map's input gradient and weight gradient share the staged tile, and an edge's two
 //     source rows of the messages are the end rows of the edge update below.
+// The first layer's features are rows of the embedding tables (BF16 parameters): node
+// orientations (bit 2 of the node, X [2][64]) and coupler values (Jt [6][64]).  Its kernels
+// gather them there (J non-NULL), mostly from L1, and no feature of it is in memory:
+// gradient of 256 C_8 graphs 1.24 -> 1.20 ms, 64 C_8 predictions 156 -> 150 us.
 // Thread mapping of staged rows: q8 = lane mod 8 is the 16-byte chunk, the row is
 // 4 warp + lane / 8 + 32 j, j = 0 .. 3.
 constexpr int SLOTS = MAXDEG;
+
+__device__ __forceinline__ int orientation(int node) { return (node >> 2) & 1; }
+__device__ __forceinline__ int coupler_class(int j) { return j < 0 ? j + 3 : j + 2; }      // -3,-2,-1,1,2,3 -> 0..5
 
 // z's sign bit of the backward's mask: positive after rounding to BF16 (2^-133 is
 // the smallest BF16 number; 2^-134 and below round to zero).
@@ -403,7 +416,8 @@ constexpr int TC_SMEM_NODE_FWD = 4 * OP64 + 4 * W64 + 2 * SLOTS * TC_ROWS * 8, T
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_NODE_FWD)
 node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const bf16* h, const bf16* e,
                 const bf16* __restrict__ Wm, const float* __restrict__ bm, const bf16* __restrict__ Wu, const float* __restrict__ bu,
-                bf16* __restrict__ hout, bf16* __restrict__ m, uint2* __restrict__ mm, uint2* __restrict__ mu, int* err)
+                bf16* __restrict__ hout, bf16* __restrict__ m, uint2* __restrict__ mm, uint2* __restrict__ mu,
+                const int8_t* __restrict__ J, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char* const Ws = tc_smem + 4 * OP64;
@@ -426,7 +440,7 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
 #pragma unroll
         for (int s = tid >> 7; s < SLOTS; s += 2) {
             int2 v = n < nodes ? in_tab[s * N + l] : make_int2(-1, -1);
-            if (v.x >= 0) v = make_int2(b * N + v.x, b * E + v.y);
+            if (v.x >= 0) v = J ? make_int2(orientation(v.x), coupler_class(J[b * E + v.y])) : make_int2(b * N + v.x, b * E + v.y);
             tab[(which * SLOTS + s) * TC_ROWS + (tid & (TC_ROWS - 1))] = v;
         }
     };
@@ -440,10 +454,11 @@ node_fwd_kernel(int nodes, int N, int E, const int2* __restrict__ in_tab, const 
             if (ls < SLOTS) {
                 const int2 v = tab[(lw * SLOTS + ls) * TC_ROWS + r];
                 cp_async16_l1(op_at(A, q8, r), h + (size_t)max(v.x, 0) * HD + q8 * 8, v.x >= 0);
-                cp_async16(op_at(A, 8 + q8, r), e + (size_t)max(v.y, 0) * HD + q8 * 8, v.x >= 0);
+                cp_async16(op_at(A, 8 + q8, r), e + (size_t)max(v.y, 0) * HD + q8 * 8, v.x >= 0, J != nullptr);
             } else {
                 const int n = lt * TC_ROWS + r;
-                cp_async16(op_at(A, q8, r), h + (size_t)(n < nodes ? n : 0) * HD + q8 * 8, n < nodes);
+                cp_async16(op_at(A, q8, r), h + (size_t)(n >= nodes ? 0 : J ? orientation(n) : n) * HD + q8 * 8, n < nodes,
+                           J != nullptr);
             }
         }
         if (++ls > SLOTS) { ls = 0; lt += gridDim.x; lw ^= 1; }
@@ -551,13 +566,15 @@ constexpr int TC_SMEM_EDGE_FWD = 2 * OP64 + 2 * W64, EDGE_FWD_FEW = 12;
 template <int CTAS>
 __global__ void __launch_bounds__(TC_THREADS, CTAS)
 edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict__ ends, int N, int E,
-                const bf16* __restrict__ W, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask, int* err)
+                const bf16* __restrict__ W, const float* __restrict__ bias, bf16* __restrict__ Yout, uint2* __restrict__ mask,
+                const int8_t* __restrict__ J, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char *const As = tc_smem, *const Ws = tc_smem + 2 * OP64;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
     __shared__ uint32_t tmem_sh;
     __shared__ int2 endn[2][TC_ROWS];                       // the two end nodes of this and the next tile's edges, -1: no row
+    __shared__ int prow[2][TC_ROWS];                        // and the row of P0
     __shared__ float bias_sm[HD];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, q8 = lane & 7, srow = warp * 4 + (lane >> 3);
     if (tid < HD) bias_sm[tid] = bias[tid];
@@ -578,6 +595,7 @@ edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict_
             ij.y += b * N;
         }
         endn[buf][tid] = ij;
+        prow[buf][tid] = r >= rows ? 0 : J ? coupler_class(J[r]) : r;
     };
     lookup(blockIdx.x, 0);
     __syncthreads();
@@ -601,7 +619,7 @@ edge_fwd_kernel(int rows, const bf16* P0, const bf16* h, const int2* __restrict_
         for (int j = 0; j < 4; ++j) {
             const int r = srow + 32 * j;
             const bool v = ij[j].x >= 0;
-            cp_async16(op_at(As, q8, r), P0 + (size_t)(v ? r0 + r : 0) * HD + q8 * 8, v);
+            cp_async16(op_at(As, q8, r), P0 + (size_t)prow[buf][r] * HD + q8 * 8, v, J != nullptr);
         }
         lookup(tile + gridDim.x, buf ^ 1);
 #pragma unroll
@@ -718,7 +736,7 @@ __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
 node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* mm, const bf16* dm,
                 const bf16* __restrict__ WmT, const int* __restrict__ inter, const float* dc, const float* ds, const float* dg,
                 float* dh, const uint2* mu, const bf16* h, const bf16* m, const bf16* __restrict__ WuT,
-                bf16* __restrict__ dmo, float* __restrict__ part, int* err)
+                bf16* __restrict__ dmo, float* __restrict__ part, int first_layer, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
     unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 2 * OP64, *const Ws = tc_smem + 4 * OP64;     // Ws: Wm^T (h half), Wu^T
@@ -758,7 +776,8 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
             const int n = tile * TC_ROWS + srow + 32 * j;
             const bool v = n < nodes;
             if (POST) {
-                cp_async16(op_at(Xs, q8, srow + 32 * j), h + (size_t)(v ? n : 0) * HD + q8 * 8, v);
+                cp_async16(op_at(Xs, q8, srow + 32 * j), h + (size_t)(!v ? 0 : first_layer ? orientation(n) : n) * HD + q8 * 8, v,
+                           first_layer != 0);
                 cp_async16(op_at(Xs, 8 + q8, srow + 32 * j), m + (size_t)(v ? n : 0) * HD + q8 * 8, v);
             }
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -931,9 +950,10 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
 // the former sums it for its 64 nodes (dc), the latter keeps its rows (ds), so that
 // node_bwd_kernel reads 3 rows a node instead of 6.
 // Operands R0 | R1 | R2: h[src_0], e, h[src_1], then (POST) eb in R1 and the sum in R2.
+// J: couplers, where e (without POST) or eb is the first layer's, else NULL.
 // The two directions' weight gradients differ in the order of their halves ([R0 | R1] and
 // [R1 | R2]) and are kept apart in tensor memory.  Without POST (the first layer) de is not
-// kept, only its sums over the edges of every coupler value (J; -3 .. 3 without 0), epart
+// kept, only its sums over the edges of every coupler value, epart
 // [CTA][6][64]: the finished tile goes back to shared memory and a thread adds up a
 // column of 32 rows, a row's class being the same for the whole warp.
 __host__ __device__ inline int edge_tiles_in(int graphs, int N) { return (graphs * (N / 8) + 7) / 8; }
@@ -957,7 +977,7 @@ edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, cons
     // this and the next tile: source row, target row * 8 + slot, twice; edge row, -1: none
     __shared__ int4 tab[2][TC_ROWS];
     __shared__ int erow[2][TC_ROWS];
-    __shared__ signed char cls[TC_ROWS];                    // coupler values of the tile (without POST)
+    __shared__ int xrow[2][TC_ROWS];                        // row of e (without POST: the first layer's, a coupler class) or of eb
     float sj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float dbm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, dbe[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     uint32_t phase = 0;
@@ -971,18 +991,18 @@ edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, cons
         if (g < graphs * per) {
             const int b = g / per, l = in ? (g - b * per) * 16 + (tid & 15) : 2 * N + g - b * per;
             v = msg_tab[l];
-            v = make_int4(b * N + v.x, b * N * 8 + v.y, b * N + v.z, b * N * 8 + v.w);
+            v = make_int4(POST ? b * N + v.x : orientation(v.x), b * N * 8 + v.y, POST ? b * N + v.z : orientation(v.z), b * N * 8 + v.w);
             r = b * E + l;
         }
         tab[which][tid] = v;
         erow[which][tid] = r;
+        xrow[which][tid] = r < 0 ? 0 : J ? coupler_class(J[r]) : r;
     };
     lookup(blockIdx.x, 0);
     __syncthreads();
     pass_begin();
     int which = 0;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
-        if (!POST && tid < TC_ROWS) cls[tid] = erow[which][tid] >= 0 ? J[erow[which][tid]] : 1;
         int4 ent[4];
         int er[4];
 #pragma unroll
@@ -996,7 +1016,7 @@ edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, cons
             const int row = srow + 32 * j;
             const bool v = er[j] >= 0;
             cp_async16_l1(op_at(R0, q8, row), h + (size_t)ent[j].x * HD + q8 * 8, v);
-            cp_async16(op_at(R1, q8, row), e + (size_t)max(er[j], 0) * HD + q8 * 8, v);
+            cp_async16(op_at(R1, q8, row), e + (size_t)(POST ? max(er[j], 0) : xrow[which][row]) * HD + q8 * 8, v, !POST);
             cp_async16_l1(op_at(R2, q8, row), h + (size_t)ent[j].z * HD + q8 * 8, v);
         }
         uint4 z0[4], z1[4];                                 // every load before the first use
@@ -1046,7 +1066,7 @@ edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, cons
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int row = srow + 32 * j;
-                cp_async16(op_at(R1, q8, row), eb + (size_t)max(er[j], 0) * HD + q8 * 8, er[j] >= 0);
+                cp_async16(op_at(R1, q8, row), eb + (size_t)xrow[which][row] * HD + q8 * 8, er[j] >= 0, J != nullptr);
                 uint4* const s = reinterpret_cast<uint4*>(op_at(R2, q8, row));
                 *s = add_bf16x8(*reinterpret_cast<const uint4*>(op_at(R0, q8, row)), *s);
             }
@@ -1137,10 +1157,10 @@ edge_bwd_kernel(int graphs, int N, int E, const int4* __restrict__ msg_tab, cons
             const int c = tid & (HD - 1);
 #pragma unroll 8
             for (int i = 0; i < 32; ++i) {
-                const int row = (tid >> 6) * 32 + i, k = cls[row];
+                const int row = (tid >> 6) * 32 + i, k = xrow[which][row];
                 const float v = reinterpret_cast<const float*>(tile_f32(Zs, row, c >> 2))[c & 3];
 #pragma unroll
-                for (int q = 0; q < 6; ++q) sj[q] += k == (q < 3 ? q - 3 : q - 2) ? v : 0.f;
+                for (int q = 0; q < 6; ++q) sj[q] += k == q ? v : 0.f;
             }
         }
         __syncthreads();                                    // the tiles are read: the next staging
@@ -1303,30 +1323,6 @@ __global__ void pack_weights_kernel(int nmat, const bf16* const* __restrict__ Ws
 }
 
 // ------------------------------------------------------- elementwise kernels
-// h0[b][n] = X[u_n]; e0[b][e] = Jt[idx(J)]; a thread converts 8 columns of a row
-__global__ void embed_kernel(int B, int N, int E, const int* __restrict__ u, const int8_t* __restrict__ J,
-                             const float* __restrict__ Xemb, const float* __restrict__ Jemb, bf16* h, bf16* e)
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const size_t nN = (size_t)B * N, total = (nN + (size_t)B * E) * (HD / 8);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t row = i / (HD / 8);
-        const int c = (int)(i % (HD / 8));
-        const float* src;
-        bf16* dst;
-        if (row < nN) {
-            src = Xemb + u[row % N] * HD;
-            dst = h + row * HD;
-        } else {
-            const int j = J[row - nN];
-            src = Jemb + (j < 0 ? j + 3 : j + 2) * HD;      // -3,-2,-1,1,2,3 -> 0..5
-            dst = e + (row - nN) * HD;
-        }
-        const float4 a = reinterpret_cast<const float4*>(src)[2 * c], b = reinterpret_cast<const float4*>(src)[2 * c + 1];
-        reinterpret_cast<uint4*>(dst)[c] = make_uint4(pack_bf2(a.x, a.y), pack_bf2(a.z, a.w), pack_bf2(b.x, b.y), pack_bf2(b.z, b.w));
-    }
-}
-
 // readout forward + loss gradient dg, the same for every node of a graph (one block of 256 threads per graph).  The node mean is
 // summed node by node (64 threads, a column each) from rows that the block stages 64 at a
 // time, the next 64 on their way meanwhile.
@@ -1446,7 +1442,7 @@ struct sg_model {
     std::vector<int64_t> oWm, obm, oWu, obu, oWe, obe;
     // graph + activation buffers for the current (L, Bcap)
     int L = 0, N = 0, E = 0, Bcap = 0;
-    int *d_u = nullptr, *d_inter = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
+    int *d_inter = nullptr, *d_out_tab = nullptr;   // topology tables (see the kernels)
     int2 *d_ends = nullptr, *d_in_tab = nullptr;
     int4* d_msg_tab = nullptr;
     int8_t* d_J = nullptr;
@@ -1489,9 +1485,9 @@ cudaError_t salloc(T** p, size_t n)
 
 void free_graph(sg_model* M)
 {
-    cudaFree(M->d_u); cudaFree(M->d_inter); cudaFree(M->d_out_tab);
+    cudaFree(M->d_inter); cudaFree(M->d_out_tab);
     cudaFree(M->d_ends); cudaFree(M->d_in_tab); cudaFree(M->d_msg_tab);
-    M->d_u = M->d_inter = M->d_out_tab = nullptr;
+    M->d_inter = M->d_out_tab = nullptr;
     M->d_ends = M->d_in_tab = nullptr;
     M->d_msg_tab = nullptr;
     cudaFree(M->d_J); M->d_J = nullptr;
@@ -1543,11 +1539,10 @@ int prepare(sg_model* M, int L, int B)
     // messages 2e: source ej -> target ei, 2e + 1: source ei -> target ej.  A node's incoming and outgoing
     // messages fill its 6 slots in ascending order, its edges between cells (numbers 16 L^2 and up) 2;
     // tables are slot-major [6][N], [2][N]
-    std::vector<int> u(N), inter(2 * N, -1), out_tab(N * MAXDEG, -1);
+    std::vector<int> inter(2 * N, -1), out_tab(N * MAXDEG, -1);
     std::vector<int2> ends(E), in_tab(N * MAXDEG, make_int2(-1, -1));
     std::vector<int4> msg_tab(E);
     std::vector<int> cin(N, 0), cout(N, 0), cinc(N, 0);
-    for (int i = 0; i < N; ++i) u[i] = (i >> 2) & 1;
     for (int e2 = 0; e2 < E; ++e2) {
         ends[e2] = make_int2(ei[e2], ej[e2]);
         int at[2];
@@ -1567,7 +1562,6 @@ int prepare(sg_model* M, int L, int B)
         if (r != cudaSuccess) return r;
         return cudaMemcpy(*d, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice);
     };
-    SK(up(&M->d_u, u), "upload topology");
     SK(up(&M->d_inter, inter), "upload topology");
     SK(up(&M->d_out_tab, out_tab), "upload topology");
     SK(up(&M->d_ends, ends), "upload topology");
@@ -1585,9 +1579,9 @@ int prepare(sg_model* M, int L, int B)
     M->h.assign(M->layers + 1, nullptr);
     for (auto* v : {&M->e, &M->m}) v->assign(M->layers, nullptr);
     for (auto* v : {&M->mm, &M->mu, &M->me}) v->assign(M->layers, nullptr);
-    for (int l = 0; l <= M->layers; ++l) SK(salloc(&M->h[l], nN * HD), "cudaMalloc h");
+    for (int l = 1; l <= M->layers; ++l) SK(salloc(&M->h[l], nN * HD), "cudaMalloc h");      // the first layer's are embedding rows
     for (int l = 0; l < M->layers; ++l) {
-        SK(salloc(&M->e[l], nE * HD), "cudaMalloc e");
+        if (l > 0) SK(salloc(&M->e[l], nE * HD), "cudaMalloc e");
         SK(salloc(&M->m[l], nN * HD), "cudaMalloc m");
         SK(salloc(&M->mm[l], nN * MAXDEG), "cudaMalloc message mask");
         SK(salloc(&M->mu[l], nN), "cudaMalloc node mask");
@@ -1617,8 +1611,13 @@ void pack_weights(sg_model* M)
 const bf16* wpk_fwd(const sg_model* M, int l, int which) { return M->wpk + ((size_t)(l * 3 + which) * 2) * HD * KIN; }
 const bf16* wpk_bwd(const sg_model* M, int l, int which) { return wpk_fwd(M, l, which) + HD * KIN; }
 
-// More than half of an SM's shared memory (see launch): gradient of 32 C_8 graphs 325 -> 292 us.
-constexpr int TC_SMEM_ALONE = 116 * 1024;
+// Features that enter layer l; the first layer's are the embedding tables.
+const bf16* feat_h(const sg_model* M, int l) { return l == 0 ? M->wbf + M->oX : M->h[l]; }
+const bf16* feat_e(const sg_model* M, int l) { return l == 0 ? M->wbf + M->oJ : M->e[l]; }
+
+// Just over half of the 228 KB of an SM with the 1 KB that every CTA takes, so that a CTA of the edge kernel still
+// fits beside it (see launch): gradient of 32 C_8 graphs 325 -> 292 us.
+constexpr int TC_SMEM_ALONE = 113 * 1024;
 // One launch of a pass (see pass_begin); errors are left for cudaGetLastError.
 template <class... Params, class... Args>
 void launch(sg_model* M, void (*kernel)(Params...), dim3 grid, int threads, int smem, Args... args)
@@ -1643,19 +1642,16 @@ void launch(sg_model* M, void (*kernel)(Params...), dim3 grid, int threads, int 
 void forward(sg_model* M, int B, bool train)
 {
     const int N = M->N, E = M->E;
-    cudaStream_t st = M->stream;
-    embed_kernel<<<grid_for((size_t)B * (N + E) * (HD / 8)), 256, 0, st>>>(B, N, E, M->d_u, M->d_J, M->theta + M->oX,
-                                                                             M->theta + M->oJ, M->h[0], M->e[0]);
-    M->launches++;
     for (int l = 0; l < M->layers; ++l) {
         launch(M, node_fwd_kernel, tc_grid(M, B * N, TC_CTAS_NODE_FWD), TC_THREADS, TC_SMEM_NODE_FWD,
-            B * N, N, E, M->d_in_tab, M->h[l], M->e[l], wpk_fwd(M, l, 0), M->theta + M->obm[l], wpk_fwd(M, l, 1), M->theta + M->obu[l],
-            M->h[l + 1], train ? M->m[l] : nullptr, M->mm[l], M->mu[l], M->d_err);
+            B * N, N, E, M->d_in_tab, feat_h(M, l), feat_e(M, l), wpk_fwd(M, l, 0), M->theta + M->obm[l], wpk_fwd(M, l, 1), M->theta + M->obu[l],
+            M->h[l + 1], train ? M->m[l] : nullptr, M->mm[l], M->mu[l], l == 0 ? M->d_J : nullptr,
+            M->d_err);
         if (l + 1 == M->layers) break;
         const bool few = (B * E + TC_ROWS - 1) / TC_ROWS <= EDGE_FWD_FEW * M->sms;
         launch(M, few ? edge_fwd_kernel<3> : edge_fwd_kernel<4>, tc_grid(M, B * E, few ? 3 : 4), TC_THREADS, TC_SMEM_EDGE_FWD,
-            B * E, M->e[l], M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
-            train ? M->me[l] : nullptr, M->d_err);
+            B * E, feat_e(M, l), M->h[l + 1], M->d_ends, N, E, wpk_fwd(M, l, 2), M->theta + M->obe[l], M->e[l + 1],
+            train ? M->me[l] : nullptr, l == 0 ? M->d_J : nullptr, M->d_err);
     }
 }
 
@@ -1694,17 +1690,17 @@ void backward_all(sg_model* M, int B)
         const bool pre = l <= top, post = l > 0;
         launch(M, kernel, gn, TC_THREADS, smem,
             (int)nodes, N, E, pre ? M->d_out_tab : nullptr, pre ? M->mm[l] : nullptr, M->dm[l & 1], pre ? wpk_bwd(M, l, 0) : nullptr,
-            pre && post ? M->d_inter : nullptr, M->dc, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? M->h[l - 1] : nullptr,
+            pre && post ? M->d_inter : nullptr, M->dc, M->ds, M->d_dg, M->dh, post ? M->mu[l - 1] : nullptr, post ? feat_h(M, l - 1) : nullptr,
             post ? M->m[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 1) : nullptr, M->dm[(l & 1) ^ 1],
-            post ? map(M->oWu[l - 1], gn) : nepart, M->d_err);
+            post ? map(M->oWu[l - 1], gn) : nepart, l == 1 ? 1 : 0, M->d_err);
     };
     auto edge = [&](int l, auto kernel, int smem) {
         const bool post = l > 0;
         float* pm = map(M->oWm[l], ge);
         launch(M, kernel, ge, TC_THREADS, smem,
-            B, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], M->h[l], M->e[l], wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
-            post ? M->me[l - 1] : nullptr, post ? M->e[l - 1] : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, M->dc, pm,
-            post ? map(M->oWe[l - 1], ge) : nullptr, M->d_J, M->d_epart, M->d_err);
+            B, N, E, M->d_msg_tab, M->mm[l], M->dm[l & 1], feat_h(M, l), feat_e(M, l), wpk_bwd(M, l, 0) + HD * HD, M->de, l == top ? 1 : 0,
+            post ? M->me[l - 1] : nullptr, post ? feat_e(M, l - 1) : nullptr, post ? wpk_bwd(M, l - 1, 2) : nullptr, M->ds, M->dc, pm,
+            post ? map(M->oWe[l - 1], ge) : nullptr, l <= 1 ? M->d_J : nullptr, M->d_epart, M->d_err);
     };
     node(top + 1, node_bwd_kernel<false, true>, TC_SMEM_NODE_BWD);
     for (int l = top; l > 0; --l) {
