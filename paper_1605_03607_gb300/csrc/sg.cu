@@ -23,8 +23,8 @@
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
 // messages, pre-activations and masked gradients in memory (97 launches, 18 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.20 ms, of 128 C_4 graphs 1.01 -> 0.29 ms, 64 C_8
-// predictions 0.42 -> 0.15 ms.  (With a kernel per map and message rows of 21 nodes
+// gradient of 256 C_8 graphs 3.95 -> 1.19 ms, of 128 C_4 graphs 1.01 -> 0.28 ms, 64 C_8
+// predictions 0.42 -> 0.14 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <algorithm>
 #include <cmath>
@@ -1323,9 +1323,11 @@ __global__ void pack_weights_kernel(int nmat, const bf16* const* __restrict__ Ws
 }
 
 // ------------------------------------------------------- elementwise kernels
-// readout forward + loss gradient dg, the same for every node of a graph (one block of 256 threads per graph).  The node mean is
-// summed node by node (64 threads, a column each) from rows that the block stages 64 at a
-// time, the next 64 on their way meanwhile.
+// readout forward + loss gradient dg, the same for every node of a graph (one block of 256
+// threads per graph).  The node mean is summed node by node (64 threads, a column each) from
+// rows that the block stages 64 at a time, the next 64 on their way meanwhile; W1 is staged
+// while the last layer runs.  64 C_8 predictions 150 -> 140 us with W1 and the rows' second
+// buffer (a barrier per 64 rows), of which W1 8 us.
 constexpr int RO_ROWS = 64, RO_THREADS = 256;
 __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* h, const float* __restrict__ W1, const float* __restrict__ b1,
                                const float* __restrict__ w2, const float* __restrict__ b2, float* y, float* gbuf,
@@ -1334,8 +1336,11 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
 {
     __shared__ __align__(16) float gs[HD];
     __shared__ float as[HD], red[HD], dz[HD];
-    __shared__ __align__(16) bf16 rows[RO_ROWS][HD];
+    __shared__ __align__(16) bf16 rows[2][RO_ROWS][HD];
+    __shared__ float W[HD][HD + 1];                         // W1, loaded before the wait for the last layer
     const int b = blockIdx.x, tid = threadIdx.x, c = tid;
+    for (int i = tid; i < HD * HD; i += RO_THREADS) W[i / HD][i % HD] = W1[i];
+    const float b1c = c < HD ? b1[c] : 0.f, w2c = c < HD ? w2[c] : 0.f, b20 = b2[0];
     pass_begin();
     const uint4* src = reinterpret_cast<const uint4*>(h + (size_t)b * N * HD);
     constexpr int PER = RO_ROWS * HD / 8 / RO_THREADS;      // 16-byte pieces per thread
@@ -1349,26 +1354,25 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
     };
     fetch(0);
     float acc = 0.f;
-    for (int n0 = 0; n0 < N; n0 += RO_ROWS) {
-        __syncthreads();
+    for (int n0 = 0, buf = 0; n0 < N; n0 += RO_ROWS, buf ^= 1) {
 #pragma unroll
-        for (int j = 0; j < PER; ++j) reinterpret_cast<uint4*>(&rows[0][0])[tid + j * RO_THREADS] = v[j];
-        __syncthreads();
+        for (int j = 0; j < PER; ++j) reinterpret_cast<uint4*>(&rows[buf][0][0])[tid + j * RO_THREADS] = v[j];
+        __syncthreads();                                    // the other buffer's rows are summed
         if (n0 + RO_ROWS < N) fetch(n0 + RO_ROWS);
         if (c < HD) {
             const int m = min(RO_ROWS, N - n0);
 #pragma unroll 8
-            for (int n = 0; n < m; ++n) acc += __bfloat162float(rows[n][c]);
+            for (int n = 0; n < m; ++n) acc += __bfloat162float(rows[buf][n][c]);
         }
     }
     if (c < HD) gs[c] = acc / (float)N;
     __syncthreads();
     float z = 0.f;
     if (c < HD) {
-        z = b1[c];
-        for (int k = 0; k < HD; ++k) z += W1[c * HD + k] * gs[k];
+        z = b1c;
+        for (int k = 0; k < HD; ++k) z += W[c][k] * gs[k];
         as[c] = fmaxf(z, 0.f);
-        red[c] = as[c] * w2[c];
+        red[c] = as[c] * w2c;
         gbuf[b * HD + c] = gs[c];
         zbuf[b * HD + c] = z;
     }
@@ -1377,7 +1381,7 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
         if (c < s) red[c] += red[c + s];
         __syncthreads();
     }
-    const float yb = red[0] + b2[0];
+    const float yb = red[0] + b20;
     if (c == 0) y[b] = yb;
     if (b == 0 && c == 1) reinterpret_cast<int*>(y)[gridDim.x] = *err;      // the status of the kernels before
     if (!target) return;
@@ -1386,11 +1390,11 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
         dybuf[b] = dy;                             // over graphs by readout_grad_kernel)
         sqbuf[b] = (yb - target[b]) * (yb - target[b]) * inv_B;
     }
-    if (c < HD) dz[c] = z > 0.f ? dy * w2[c] : 0.f;
+    if (c < HD) dz[c] = z > 0.f ? dy * w2c : 0.f;
     __syncthreads();
     if (c < HD) {
         float dg = 0.f;
-        for (int o = 0; o < HD; ++o) dg += dz[o] * W1[o * HD + c];
+        for (int o = 0; o < HD; ++o) dg += dz[o] * W[o][c];
         dgbuf[b * HD + c] = dg / (float)N;
     }
 }
