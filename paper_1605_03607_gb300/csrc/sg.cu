@@ -23,7 +23,7 @@
 // its rows and everything around them, no message row in memory, and rows that a tile
 // gathers several times taken from L1.  Measured against one kernel per step with FP32
 // messages, pre-activations and masked gradients in memory (97 launches, 18 now):
-// gradient of 256 C_8 graphs 3.95 -> 1.19 ms, of 128 C_4 graphs 1.01 -> 0.28 ms, 64 C_8
+// gradient of 256 C_8 graphs 3.95 -> 1.16 ms, of 128 C_4 graphs 1.01 -> 0.28 ms, 64 C_8
 // predictions 0.42 -> 0.14 ms.  (With a kernel per map and message rows of 21 nodes
 // summed through shared memory: 2.24, 0.59 and 0.26 ms.)
 #include <algorithm>
@@ -726,11 +726,12 @@ constexpr int TC_CTAS_BWD = 2;
 // where empty).
 // POST, node update of the layer below: dZ = dh & mu, dh += dX[:, :64], dmo = dX[:, 64:]
 // rounded to BF16 (the one form that the messages' dZ = dm & mask takes it in), weight
-// gradient with X = [h | m].  A slot's rows are loaded while the slot before is
-// computed; two operand buffers.  Without PRE (the last layer) every node of a graph starts
+// gradient with X = [h | m].  Slots go in two groups of three operand buffers: a step's
+// fence, barrier and load latency cost more than its MMAs (256 C_8 graphs, a launch: 74
+// us, slot by slot 82).  Without PRE (the last layer) every node of a graph starts
 // from the readout's gradient dg [graphs][64]; without POST (the first) dh is not kept,
 // only its sums over the nodes of either orientation, part [CTA][2][64].
-constexpr int TC_SMEM_NODE_BWD = 4 * OP64 + 3 * W64 + 2 * (SLOTS + 2) * TC_ROWS * 4;
+constexpr int TC_SMEM_NODE_BWD = 5 * OP64 + 3 * W64 + 2 * (SLOTS + 2) * TC_ROWS * 4;
 template <bool PRE, bool POST>
 __global__ void __launch_bounds__(TC_THREADS, TC_CTAS_BWD)
 node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const uint2* mm, const bf16* dm,
@@ -739,7 +740,7 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                 bf16* __restrict__ dmo, float* __restrict__ part, int first_layer, int* err)
 {
     extern __shared__ __align__(128) unsigned char tc_smem[];
-    unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 2 * OP64, *const Ws = tc_smem + 4 * OP64;     // Ws: Wm^T (h half), Wu^T
+    unsigned char *const Zs = tc_smem, *const Xs = tc_smem + 3 * OP64, *const Ws = tc_smem + 5 * OP64;     // Ws: Wm^T (h half), Wu^T
     // of this and the next tile, -1: none: target row * 8 + its slot [2][6][128], rows of ds [2][2][128]
     int *const otab = reinterpret_cast<int*>(Ws + 3 * W64), *const itab = otab + 2 * SLOTS * TC_ROWS;
     __shared__ __align__(8) uint64_t bar_w, bar_mma;
@@ -770,7 +771,6 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
     int which = 0;
     for (int tile = blockIdx.x; !failed && tile < ntiles; tile += gridDim.x, which ^= 1) {
         float4 ga[4], gb[4];                                // dh: columns 4 q8 .. and 32 + 4 q8 ..
-        lookup(tile + gridDim.x, which ^ 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = tile * TC_ROWS + srow + 32 * j;
@@ -781,39 +781,69 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                 cp_async16(op_at(Xs, 8 + q8, srow + 32 * j), m + (size_t)(v ? n : 0) * HD + q8 * 8, v);
             }
             ga[j] = gb[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (v) {
-                const float4* gp = reinterpret_cast<const float4*>(PRE ? dh + (size_t)n * HD : dg + (size_t)(n / N) * HD);
-                ga[j] = gp[q8];
-                gb[j] = gp[8 + q8];
+            if (!PRE && v) {
+                ga[j] = reinterpret_cast<const float4*>(dg + (size_t)(n / N) * HD)[q8];
+                gb[j] = reinterpret_cast<const float4*>(dg + (size_t)(n / N) * HD)[8 + q8];
             }
         }
         bool ok = true;
         if (PRE) {
-            uint4 z[4];
-            uint32_t mk[4];
-            auto load = [&](int s) {
+            constexpr int GRP = SLOTS / 2;
+            uint4 z[GRP][4];
+            uint32_t mk[GRP][4];
+            auto load = [&](int s0) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int t = otab[(which * SLOTS + s) * TC_ROWS + srow + 32 * j];
-                    z[j] = make_uint4(0u, 0u, 0u, 0u);
-                    mk[j] = 0u;
-                    if (t >= 0) {
-                        const size_t n = t >> 3;
-                        z[j] = *reinterpret_cast<const uint4*>(dm + n * HD + q8 * 8);
-                        mk[j] = mask_byte(mm, (size_t)(t & 7) * nodes + n, q8);
+                for (int i = 0; i < GRP; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int t = otab[(which * SLOTS + s0 + i) * TC_ROWS + srow + 32 * j];
+                        z[i][j] = make_uint4(0u, 0u, 0u, 0u);
+                        mk[i][j] = 0u;
+                        if (t >= 0) {
+                            const size_t n = t >> 3;
+                            z[i][j] = *reinterpret_cast<const uint4*>(dm + n * HD + q8 * 8);
+                            mk[i][j] = mask_byte(mm, (size_t)(t & 7) * nodes + n, q8);
+                        }
                     }
-                }
             };
             load(0);
-            if (POST) {
+#pragma unroll
+            for (int grp = 0; grp < 2; ++grp) {
+                if (grp > 0) {                              // the first group's MMAs are done
+                    ok = mbar_wait(&bar_mma, phase);
+                    phase ^= 1u;
+                }
+#pragma unroll
+                for (int i = 0; i < GRP; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<uint4*>(op_at(Zs + i * OP64, q8, srow + 32 * j)) = mask_bf16x8(z[i][j], mk[i][j]);
+                // (the copies of X are not waited for here)
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                tc_fence_before();
+                __syncthreads();
+                tc_fence_after();
+                if (tid == 0) {
+#pragma unroll
+                    for (int i = 0; i < GRP; ++i) mma_input<HD>(tmem, Zs + i * OP64, Ws, grp + i > 0);
+                    tc_commit(&bar_mma);
+                }
+                if (grp == 0) load(GRP);
+            }
+            lookup(tile + gridDim.x, which ^ 1);
+            // the node's FP32 rows: ds twice, dc, dh
+#pragma unroll
+            for (int s = POST ? 0 : 3; s < 4; ++s) {
                 float4 x[4], y[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int n = tile * TC_ROWS + srow + 32 * j;
+                    const int r = s < 2 ? itab[(which * 2 + s) * TC_ROWS + srow + 32 * j] : n < nodes ? n : -1;
+                    const float4* rp = reinterpret_cast<const float4*>((s < 2 ? ds : s == 2 ? dc : dh) + (size_t)max(r, 0) * HD);
                     x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (n < nodes) {
-                        x[j] = reinterpret_cast<const float4*>(dc + (size_t)n * HD)[q8];
-                        y[j] = reinterpret_cast<const float4*>(dc + (size_t)n * HD)[8 + q8];
+                    if (r >= 0) {
+                        x[j] = rp[q8];
+                        y[j] = rp[8 + q8];
                     }
                 }
 #pragma unroll
@@ -822,41 +852,8 @@ node_bwd_kernel(int nodes, int N, int E, const int* __restrict__ out_tab, const 
                     gb[j] = add4(gb[j], y[j]);
                 }
             }
-            for (int s = 0; s < SLOTS; ++s) {
-                unsigned char* const Z = Zs + (s & 1) * OP64;     // its MMA before last is done: the wait below
-#pragma unroll
-                for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4*>(op_at(Z, q8, srow + 32 * j)) = mask_bf16x8(z[j], mk[j]);
-                // (the copies of X are not waited for here)
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                tc_fence_before();
-                __syncthreads();
-                tc_fence_after();
-                if (tid == 0) {
-                    mma_input<HD>(tmem, Z, Ws, s > 0);
-                    tc_commit(&bar_mma);
-                }
-                if (s + 1 < SLOTS) load(s + 1);
-                if (POST && s < 2) {
-                    float4 x[4], y[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int ed = itab[(which * 2 + s) * TC_ROWS + srow + 32 * j];
-                        x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (ed >= 0) {
-                            const float4* dp = reinterpret_cast<const float4*>(ds + (size_t)ed * HD);
-                            x[j] = dp[q8];
-                            y[j] = dp[8 + q8];
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        ga[j] = add4(ga[j], x[j]);
-                        gb[j] = add4(gb[j], y[j]);
-                    }
-                }
-                ok = mbar_wait(&bar_mma, phase) && ok;
-                phase ^= 1u;
-            }
+            ok = mbar_wait(&bar_mma, phase) && ok;
+            phase ^= 1u;
             if ((failed = __syncthreads_or(!ok))) break;
             tc_fence_after();
             tmem_to_tile(Zs, tmem, warp, lane);
