@@ -174,7 +174,7 @@ __host__ __device__ inline LaneLayout lane_layout(int L, int NT, int kt, int gr,
     o.spins = 32 * L2;
     o.col_bytes = 64 * (L2 + 2 * L);
     o.runs = o.spins + o.ncols * o.col_bytes;
-    o.run_bytes = (int32_t)(item_layout(0, NT, 0, walk).bytes + 64 * ((NT + 6) / 8 + 1));   // + exchange scratch
+    o.run_bytes = (int32_t)(item_layout(0, NT, 0, walk).bytes + (NT > 32 ? 64 * ((NT + 6) / 8 + 1) : 128));   // + exchange scratch
     o.group_bytes = o.runs + gr * o.run_bytes;
     o.bytes = o.groups + ngroups * o.group_bytes;
     return o;
