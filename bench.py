@@ -11,7 +11,7 @@ candidate is kept early).
 
 Reported: spin-flip attempts/s (value, device time), PT-TTS evaluations/s and
 RAO steps/s, the end-to-end number through the same C-ABI call, the roofline
-of the dominant kernel (pt_sweep_kernel, integer-issue bound), the CPU oracle
+of the dominant kernel (the sweep kernel, integer-issue bound), the CPU oracle
 on a bounded sample, and SM clocks sampled during the timed region.
 
 --impl reference times the CPU oracle (plain C, one thread) on a bounded
@@ -374,7 +374,7 @@ def run_gpu(args):
                      "traffic": PROFILED_TRAFFIC.get((h.mapping(), *h.schedule()[:2], R * spec)),
                      "traffic_source": "profiled constant (one ncu capture of this schedule), not measured "
                                        "in this run",
-                     "kernel": "pt_sweep_kernel",
+                     "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule",
                      "ops_per_attempt": OPS_PER_ATTEMPT,
                      "avg_launch_ms": sweep_ms / max(sweep_launches, 1), "launches": sweep_launches,
                      "peak_source": f"{sms} SMs x {INT_LANES_PER_SM_CLK} lanes x "
@@ -452,7 +452,7 @@ def measure_batched(args, steps, warmup):
         "instances_solved_within_S": n_solved,
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                      "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops,
-                     "kernel": "pt_sweep_kernel (persistent)", "ops_per_attempt": OPS_PER_ATTEMPT,
+                     "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule (persistent)", "ops_per_attempt": OPS_PER_ATTEMPT,
                      "avg_launch_ms": kern_ms / max(steps, 1), "peak_source": peak_kind},
         "schedule": {str(k): v for k, v in sched.items()}, "info": b.info(), "clocks": clocks,
         "timing": "value over the host wall clock of reset + run + TTS per step; kernel_attempts_per_s "
@@ -644,7 +644,7 @@ def run_lao(args):
         "overlaps_final": ov,
         "schedule": list(h.schedule()), "team": h.mapping(),
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
-                     "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops, "kernel": "pt_sweep_kernel",
+                     "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops, "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule",
                      "ops_per_attempt": OPS_PER_ATTEMPT, "peak_source": kind},
         "clocks": clocks, "data": "synthetic"}))
     h.close()

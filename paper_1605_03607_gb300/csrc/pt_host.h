@@ -230,6 +230,7 @@ inline int lane_threads(int NT, const LaneShape& s) { return 32 * s.W * lane_col
 // one more than the others), exchange and barriers 910, which the groups of the SM overlap;
 // no group is faster than alone.  Fitted to 900 measured (shape, size) pairs from C_2 to
 // C_16: the lowest estimate's time is 0.5 % above the best shape's on average, 3 % at most.
+// (Fitted before the exchange became 200 to 300 clocks shorter.)
 inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);      // what the warps of a column share out

@@ -20,8 +20,8 @@
 // sub-partition for two cycles (4 on its pipe); 82 instructions and 16 wide
 // multiplies a word leave 115 clocks at the 85 % issue rate that this mix reaches,
 // against 110 instructions and 199 clocks before.  Measured, C_8 x 32 slots,
-// 1024 runs: 14.4 us per sweep (1.17e12 attempts/s; slot-major 4/32/1: 20.7 us,
-// 8.1e11); one C_8 instance of 64 runs: 3.1 us per sweep (cell-major default: 11.7).
+// 1024 runs: 13.4 us per sweep (1.25e12 attempts/s; slot-major 4/32/1: 20.7 us,
+// 8.1e11); one C_8 instance of 64 runs: 2.8 us per sweep (cell-major default: 11.7).
 // Measured and left: 1 or 2 cells a step instead of 4 (1 % slower), keys as immediates
 // (recomputed per round, 7 more uniform instructions a word), accept flags by LOP3
 // instead of adds (1 % slower), by selects (2 % slower).
