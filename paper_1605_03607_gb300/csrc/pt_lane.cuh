@@ -234,17 +234,21 @@ __device__ __forceinline__ int lane_exchange(int32_t* Es, uint8_t* perm, uint8_t
     constexpr int H = TWO ? 2 : 1;
     const int np = NT - 1, npad = (np + 7) & ~7;
     int m = INT_MAX;
-    uint32_t rej[H], count[H];          // (the swap counters are loaded early: nothing waits for them after the chain)
+    // up to 32 slots: a lane's energy, configuration and swap counter are loaded before the chain and exchanged by
+    // shuffles after it, while every other warp of the group waits
+    int held = 0, own = 0;
+    if (!TWO) held = lane < NT ? perm[lane] : 0;
+    uint32_t rej[H], count[H];
 #pragma unroll
     for (int h = 0; h < H; ++h) count[h] = !TWO && lane < np ? xacc[lane] : 0u;
     if (!TWO) {
         // lane p: the energy carried on from a rejection of pair p, lane 31 the one carried into pair 0; where it is
         // rejected next; then the set of rejections that lane 31 reaches, doubling the number of hops
         int* const crit = reinterpret_cast<int*>(xp);
-        const int own = lane < NT ? Es[lane] : INT_MAX;
+        own = lane < NT ? Es[lane] : INT_MAX;
         const int e = Es[lane < np ? lane + 1 : 0];                      // lane 31: Es[0]
         crit[lane] = lane < np ? e - 2 * cc[lane] : INT_MIN;
-        m = own;
+        m = __reduce_min_sync(FULL, own);
         __syncwarp();
         uint32_t hit[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
@@ -317,11 +321,15 @@ __device__ __forceinline__ int lane_exchange(int32_t* Es, uint8_t* perm, uint8_t
         if ((acc[h] >> lane) & 1u) src[h] = s + 1;
         e_new[h] = b_new[h] = 0;
         if (s < NT) {
-            e_new[h] = Es[src[h]];
-            b_new[h] = perm[src[h]];
+            e_new[h] = TWO ? Es[src[h]] : 0;
+            b_new[h] = TWO ? perm[src[h]] : 0;
         }
     }
-    m = __reduce_min_sync(FULL, m);
+    if (TWO) m = __reduce_min_sync(FULL, m);
+    else {
+        e_new[0] = __shfl_sync(FULL, own, src[0]);
+        b_new[0] = __shfl_sync(FULL, held, src[0]);
+    }
 #pragma unroll
     for (int h = 0; h < H; ++h) {
         const int s = lane + 32 * h;
@@ -502,9 +510,9 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
                 if (W > 1) gsync();
                 if (busy) lane_phase<LT, 1>(lut0 + L2 * 192, s1, s0, pre + L2, w, W, L, lc, dk, pc);
                 const int n = (int)(pc >> 7), sk = (int)(dk >> 7) - 127 * n;   // accepted flips, sum of their k
-                if (valid) {
-                    if (sk) atomicAdd(reinterpret_cast<int32_t*>(rb + rl.E) + t, 2 * sk);
-                    if (n) atomicAdd(reinterpret_cast<uint32_t*>(rb + rl.macc) + t, (uint32_t)n);
+                if (valid) {                // also zeros: a branch each cost C_4 sweeps 4 %
+                    atomicAdd(reinterpret_cast<int32_t*>(rb + rl.E) + t, 2 * sk);
+                    atomicAdd(reinterpret_cast<uint32_t*>(rb + rl.macc) + t, (uint32_t)n);
                 }
             }
             gsync();
