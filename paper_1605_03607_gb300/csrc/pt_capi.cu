@@ -202,19 +202,6 @@ bool doubling_ok(int32_t S0, int32_t Smax, int32_t pass_mult)
     return x == Smax;
 }
 
-// Default schedule: about 256 threads per run, a multiple of 32.
-void default_schedule(int L, int NT, int R, int& sp, int& ipc, int kt)
-{
-    const int L2 = L * L;
-    sp = std::max(1, 256 / L2);
-    if (sp > NT) sp = NT;
-    while ((sp * L2) % 32 != 0) ++sp;
-    const int tpi = sp * L2;
-    ipc = std::max(1, 512 / tpi);
-    if (ipc > R) ipc = R;
-    while (ipc > 1 && bundle_smem_bytes(L, NT, ipc, 0, false, kt) > 110 * 1024) --ipc;
-}
-
 int check_schedule(pt_handle* h, int L, int NT, int sp, int ipc, int team)
 {
     const int L2 = L * L;
@@ -301,6 +288,34 @@ int planned_shape(pt_handle* h, const Group& g, int n_inst, int R, LaneShape& s)
     return PT_OK;
 }
 
+// Bundles of the first R runs of the listed instances in the planned shape, and their launch but for its list.
+int planned_launch(pt_handle* h, const Group& g, const std::vector<int>& insts, int R, std::vector<Bundle>& bundles, Launch& l)
+{
+    LaneShape s;
+    if (int rc = planned_shape(h, g, (int)insts.size(), R, s)) return rc;
+    if (s.cell_sp) {
+        bundles.clear();
+        for (int i : insts)
+            for (int r = 0; r < R; r += s.cell_ipc) {
+                Bundle b;
+                b.inst = i; b.run0 = r; b.nitems = std::min(s.cell_ipc, R - r); b.sp = s.cell_sp; b.team = 0;
+                bundles.push_back(b);
+            }
+        l.team = 0;
+        l.threads = s.cell_sp * g.L * g.L * s.cell_ipc;
+        l.smem = (int)bundle_smem_bytes(g.L, g.NT, s.cell_ipc, 0, g.walk, h->kt);
+    } else {
+        lane_bundles(s, insts, R, bundles);
+        l.team = -s.gr;
+        l.threads = lane_threads(g.NT, s);
+        l.smem = (int)lane_smem(g.L, g.NT, h->kt, s, g.walk);
+    }
+    int cap = 0;
+    CK(sweep_smem_capacity(&cap), "shared memory capacity");
+    CK(set_sweep_smem_limit(cap, l.team, g.walk, g.L), "cudaFuncSetAttribute");
+    return PT_OK;
+}
+
 // The new bundle list replaces the group's only when every step succeeded, so
 // a failure leaves the previous schedule in place and launchable.
 int group_schedule(pt_handle* h, Group& g)
@@ -310,14 +325,9 @@ int group_schedule(pt_handle* h, Group& g)
     CK(sweep_smem_capacity(&cap), "shared memory capacity");
     Launch l;
     if (h->planned) {
-        LaneShape shape;
-        if (int rc = planned_shape(h, g, g.n_inst, g.R, shape)) return rc;
         std::vector<int> insts(g.n_inst);
         for (int i = 0; i < g.n_inst; ++i) insts[i] = i;
-        lane_bundles(shape, insts, g.R, bundles);
-        l.team = -shape.gr;
-        l.threads = lane_threads(g.NT, shape);
-        l.smem = (int)lane_smem(g.L, g.NT, h->kt, shape, g.walk);
+        if (int rc = planned_launch(h, g, insts, g.R, bundles, l)) return rc;
     } else {
         for (int i = 0; i < g.n_inst; ++i)
             for (int r = 0; r < g.R; r += h->ipc) {
@@ -360,12 +370,7 @@ int subset_launch(pt_handle* h, Group& g, const std::vector<int>& insts, int R, 
     l = g.all;
     std::vector<Bundle> sub;
     if (h->planned) {
-        LaneShape shape;
-        if (int rc = planned_shape(h, g, (int)insts.size(), R, shape)) return rc;
-        lane_bundles(shape, insts, R, sub);
-        l.team = -shape.gr;
-        l.threads = lane_threads(g.NT, shape);
-        l.smem = (int)lane_smem(g.L, g.NT, h->kt, shape, g.walk);
+        if (int rc = planned_launch(h, g, insts, R, sub, l)) return rc;
     } else {
         std::vector<char> in((size_t)g.desc.size(), 0);
         for (int i : insts) in[(size_t)i] = 1;

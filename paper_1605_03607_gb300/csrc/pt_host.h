@@ -219,6 +219,7 @@ inline std::string build_tables(int NT, int kt, const double* betas, Tables& tb)
 struct LaneShape {
     int W = 1, gr = 1, G = 1;          // warps per column, runs per group, groups per CTA
     bool span = false;                 // a CTA may hold runs of two instances (with the same tables)
+    int cell_sp = 0, cell_ipc = 0;     // not 0: the cell-major mapping instead, its threads per cell and runs per CTA
 };
 
 inline int lane_columns(int NT, int gr) { return (gr * NT + 31) / 32; }
@@ -241,12 +242,38 @@ inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
     return std::max(together, 0.25 * words * (117.0 + 130.0 / w1) + x);
 }
 
+// Default schedule: about 256 threads per run, a multiple of 32.
+inline void default_schedule(int L, int NT, int R, int& sp, int& ipc, int kt)
+{
+    const int L2 = L * L;
+    sp = std::max(1, 256 / L2);
+    if (sp > NT) sp = NT;
+    while ((sp * L2) % 32 != 0) ++sp;
+    const int tpi = sp * L2;
+    ipc = std::max(1, 512 / tpi);
+    if (ipc > R) ipc = R;
+    while (ipc > 1 && bundle_smem_bytes(L, NT, ipc, 0, false, kt) > 110 * 1024) --ipc;
+}
+
+// Estimated SM clocks per sweep of a cell-major CTA with the SM to itself, its threads per cell and
+// runs as above: 300 a warp, and for every further slot of a thread 800 + 75 a warp; the exchange is
+// taken at half its 2100 (sweeps without one cost nothing there).  Fitted to one run and two runs a
+// CTA on C_8, C_12 and C_16 with 1 to 8 slots.
+inline double cell_clocks(int L, int NT, int sp, int ipc)
+{
+    const double w = sp * L * L * ipc / 32.0;
+    return 2700.0 + 300.0 * w + (NT > 1 ? 1000.0 : 0.0) + ((NT + sp - 1) / sp - 1) * (800.0 + 75.0 * w);
+}
+
 // The shape with the lowest estimate for n_inst instances of R runs on `sms` SMs: all CTAs
 // of a launch run at once if they fit, else in waves.  One run per CTA spreads best over
 // the SMs; more runs share the field tables (384 L^2 bytes an instance), which decides at
 // large L.  Runs that do not divide into whole CTAs fill them up with the next instance's
 // (span): 16 C_8 instances of 64 runs (32 temperatures) are 147 CTAs of 7, one for each SM,
 // where CTAs of one instance came in two waves: 2048 sweeps 29.9 -> 28.1 ms.
+// With up to 10 slots most lanes are empty, and on large lattices a lane per cell is the
+// faster mapping while its CTAs come to at most two an SM (C_16: 1.5 times with 4 slots and
+// one run, even at 8; C_12: 1.2 times with 4; below C_8 with more than 2 slots never).
 inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, int sms, int cap)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
@@ -274,6 +301,16 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
                     if (t < best_t * 0.999) { best_t = t; best = s; }
                 }
             }
+    if (NT <= 10) {
+        int sp, ipc;
+        default_schedule(L, NT, R, sp, ipc, kt);
+        const int64_t ctas = n_inst * (int64_t)((R + ipc - 1) / ipc);
+        if (sp * L * L * ipc <= MAX_THREADS && bundle_smem_bytes(L, NT, ipc, 0, walk, kt) <= cap && ctas <= 2 * sms &&
+            (NT == 1 || cell_clocks(L, NT, sp, ipc) * (ctas > sms ? 1.5 : 1.0) < best_t)) {
+            best.cell_sp = sp;
+            best.cell_ipc = ipc;
+        }
+    }
     return best;
 }
 

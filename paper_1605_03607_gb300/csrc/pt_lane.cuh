@@ -21,7 +21,7 @@
 // multiplies a word leave 115 clocks at the 85 % issue rate that this mix reaches,
 // against 110 instructions and 199 clocks before.  Measured, C_8 x 32 slots,
 // 1024 runs: 13.4 us per sweep (1.25e12 attempts/s; slot-major 4/32/1: 20.7 us,
-// 8.1e11); one C_8 instance of 64 runs: 2.8 us per sweep (cell-major default: 11.7).
+// 8.1e11); one C_8 instance of 64 runs: 2.7 us per sweep (cell-major default: 11.7).
 // Measured and left: 1 or 2 cells a step instead of 4 (1 % slower), keys as immediates
 // (recomputed per round, 7 more uniform instructions a word), accept flags by LOP3
 // instead of adds (1 % slower), by selects (2 % slower).
@@ -521,7 +521,7 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
                 int32_t* Es = reinterpret_cast<int32_t*>(xb + rl.E);
                 int32_t* misc = reinterpret_cast<int32_t*>(xb + rl.misc);
                 int m;
-                const int record = misc[0];         // loaded before the chain: C_4 sweeps 6 % faster, with the counters 7 %
+                const int record = misc[0];         // loaded before the chain: C_4 sweeps 6 % faster
                 if (do_x) {
                     uint32_t* xacc = reinterpret_cast<uint32_t*>(xb + rl.xacc);
                     const int32_t* cc = reinterpret_cast<const int32_t*>(xb + rl.ccrit) + (s & 1u) * NT;

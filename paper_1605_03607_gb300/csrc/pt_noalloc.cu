@@ -137,6 +137,7 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
         int cap = 0;
         cudaError_t e2 = sweep_smem_capacity(&cap);
         for (int l = 1; l <= MAX_L && e2 == cudaSuccess; ++l) e2 = set_sweep_smem_limit(cap, -1, false, l);
+        if (e2 == cudaSuccess) e2 = set_sweep_smem_limit(cap, 0, false, 1);
         if (e2 == cudaSuccess) e2 = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (e2 != cudaSuccess) return noalloc_cuda_fail("setting the sweep kernel's shared-memory limit", e2, nullptr, false);
         g_smem_cap[dev] = cap;
@@ -155,14 +156,16 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
     // the shape a handle of this size plans for itself
     const int L2 = L * L;
     const LaneShape shape = lane_plan(L, n_temps, kt, n_runs, 1, false, g_sms[dev], g_smem_cap[dev]);
-    const int ipc = shape.gr * shape.G, block = lane_threads(n_temps, shape);
-    const int smem = (int)bundle_smem_bytes(L, n_temps, ipc, -shape.gr, false, kt);
+    const bool cell = shape.cell_sp > 0;                  // then a run per CTA
+    const int ipc = cell ? 1 : shape.gr * shape.G, block = cell ? shape.cell_sp * L2 : lane_threads(n_temps, shape);
+    const int team = cell ? 0 : -shape.gr;
+    const int smem = (int)bundle_smem_bytes(L, n_temps, ipc, team, false, kt);
     int n_bundles = 0;
     for (int r = 0; r < n_runs; ++r) {
         h_items[r] = make_int2(0, r);
         if (r % ipc != 0) continue;
         Bundle& b = h_bundles[n_bundles++];
-        b.inst = 0; b.run0 = r; b.nitems = n_runs - r < ipc ? n_runs - r : ipc; b.sp = shape.W; b.team = -shape.gr;
+        b.inst = 0; b.run0 = r; b.nitems = n_runs - r < ipc ? n_runs - r : ipc; b.sp = cell ? shape.cell_sp : shape.W; b.team = team;
     }
     if (smem > g_smem_cap[dev])
         return noalloc_fail(PT_ERR_ARG, "one run needs more shared memory than a CTA can have");
@@ -236,7 +239,7 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
     for (int64_t done = 0; done < total;) {
         const int chunk = (int)(total - done < 4096 ? total - done : 4096);
         if ((ce = launch_sweeps(dd, db, n_bundles, n_bundles, block, smem, (uint32_t)done, chunk, exchange_every, 0,
-                                nullptr, st, -shape.gr, false, L)) != cudaSuccess)
+                                nullptr, st, team, false, L)) != cudaSuccess)
             return noalloc_cuda_fail("sweep kernel", ce, st, true);
         done += chunk;
     }

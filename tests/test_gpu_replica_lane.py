@@ -60,6 +60,32 @@ def test_planned_mapping_bit_exact(P, L, NT, R, n, x):
     assert np.array_equal(st["E"], ref.full_energies())
 
 
+@pytest.mark.parametrize("L,NT,R,walk", [(16, 4, 3, False), (16, 8, 1, True), (12, 5, 2, False), (8, 2, 1, False), (6, 1, 4, False),
+                                         (12, 2, 200, False)])
+def test_planned_few_temperatures(P, L, NT, R, walk):
+    """Few replicas on a large lattice: a plan may take a lane per cell, with the same bytes, also for a single
+    exchange, for candidates of fewer runs (a doubling budget) and in the evaluation without allocation."""
+    J = W.random_couplers(L, 3, NT)
+    betas = W.beta_ladder(NT, 0.1, 3.0) if NT > 1 else np.array([1.0])
+    ref = oracle.PTState(L, J, betas, R, 3, NT)
+    with P.PTHandle(L, J, betas, R, 3, NT) as h:
+        if walk:
+            h.set_walk_stats(True)
+        h.sweep(5, 1)
+        h.exchange()
+        h.sweep(4, 2)
+        ref.sweeps(5, 1)
+        ref.exchange()
+        ref.sweeps(4, 2)
+        st = h.state()
+        for k in ("spins", "E", "best", "first", "macc") + (("xacc",) if NT > 1 else ()):
+            assert np.array_equal(st[k], getattr(ref, k)), k
+        out = h.tts_eval_many(np.stack([J, J]), [1, 2], 2, max_sweeps=4)
+    for i in range(2):
+        assert (out["tts"][i], out["n_hit"][i], out["target"][i]) == tuple(
+            oracle.tts_eval_doubling(L, J, betas, R, 3, i + 1, 2, 4, 1)[:3])
+
+
 @pytest.mark.parametrize("L,NT,R,k", [(4, 24, 64, 16), (6, 20, 24, 3)])
 def test_planned_groups_of_candidates(P, L, NT, R, k):
     """Several groups per CTA and several CTAs per instance, every candidate with its own couplers."""
