@@ -520,6 +520,21 @@ int pt_batch_create(pt_batch** out, int32_t n_inst, const pt_instance_desc* d, i
             if (b->L[i] == g.L) g.work += (int64_t)n_runs * b->NT[i] * b->N[i];
         default_shape_sched(g.L, g.ntmax, n_runs, false, g.s, b->kt);
         g.s.planned = true;
+        if (g.ntmax <= 10) {                   // few lanes in use: cell-major where lane_plan would take it
+            std::vector<int> nts;
+            for (int i = 0; i < n_inst; ++i)
+                if (b->L[i] == g.L) nts.push_back(b->NT[i]);
+            const int64_t ctas = (int64_t)nts.size() * ((n_runs + g.s.ipc - 1) / g.s.ipc);
+            int W = 1, ct = 1, cap = 0, dev = 0, sms = 0;
+            double clocks = 0.0;
+            BKC(sweep_smem_capacity(&cap), "shared memory capacity");
+            BKC(cudaGetDevice(&dev), "cudaGetDevice");
+            BKC(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "device attribute");
+            if (ctas <= sms && g.s.sp * g.L * g.L * g.s.ipc <= MAX_THREADS &&
+                lane_plan_batch(g.L, nts, b->kt, n_runs, sms, cap, &W, &ct, &clocks) &&
+                cell_clocks(g.L, g.ntmax, g.s.sp, g.s.ipc) < clocks)
+                g.s.planned = false;
+        }
         b->groups.push_back(g);
     }
     std::stable_sort(b->groups.begin(), b->groups.end(),

@@ -274,7 +274,8 @@ inline double cell_clocks(int L, int NT, int sp, int ipc)
 // With up to 10 slots most lanes are empty, and on large lattices a lane per cell is the
 // faster mapping while its CTAs come to at most two an SM (C_16: 1.5 times with 4 slots and
 // one run, even at 8; C_12: 1.2 times with 4; below C_8 with more than 2 slots never).
-inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, int sms, int cap)
+// cell_runs: at most so many runs in a cell-major CTA.
+inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, int sms, int cap, int cell_runs = 1 << 20)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
     LaneShape best;
@@ -304,6 +305,7 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
     if (NT <= 10) {
         int sp, ipc;
         default_schedule(L, NT, R, sp, ipc, kt);
+        ipc = std::min(ipc, cell_runs);
         const int64_t ctas = n_inst * (int64_t)((R + ipc - 1) / ipc);
         if (sp * L * L * ipc <= MAX_THREADS && bundle_smem_bytes(L, NT, ipc, 0, walk, kt) <= cap && ctas <= 2 * sms &&
             (NT == 1 || cell_clocks(L, NT, sp, ipc) * (ctas > sms ? 1.5 : 1.0) < best_t)) {
@@ -365,7 +367,8 @@ inline bool lane_fill(int L, int NT, int kt, int R, int W, int Ct, int cap, Lane
     return fewest > 0;
 }
 
-inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, int sms, int cap, int* W, int* Ct)
+inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, int sms, int cap, int* W, int* Ct,
+                            double* clocks = nullptr)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
     double best = 1e300;
@@ -396,6 +399,7 @@ inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, i
             t = 0.5 * (t + std::max(t, longest * (double)((ctas + (int64_t)k * sms - 1) / ((int64_t)k * sms))));
             if (t < best * 0.999) { best = t; *W = w; *Ct = ct; }
         }
+    if (clocks) *clocks = best;
     return best < 1e300;
 }
 

@@ -155,7 +155,7 @@ extern "C" int pt_tts_eval_noalloc(int32_t L, const int8_t* J, int32_t n_edges, 
 
     // the shape a handle of this size plans for itself
     const int L2 = L * L;
-    const LaneShape shape = lane_plan(L, n_temps, kt, n_runs, 1, false, g_sms[dev], g_smem_cap[dev]);
+    const LaneShape shape = lane_plan(L, n_temps, kt, n_runs, 1, false, g_sms[dev], g_smem_cap[dev], 1);
     const bool cell = shape.cell_sp > 0;                  // then a run per CTA
     const int ipc = cell ? 1 : shape.gr * shape.G, block = cell ? shape.cell_sp * L2 : lane_threads(n_temps, shape);
     const int team = cell ? 0 : -shape.gr;

@@ -159,3 +159,21 @@ def test_planned_batch_of_uneven_instances(P):
             ref.sweeps(12, 2)
             for k in ("spins", "E", "best", "first", "macc") + (("xacc",) if len(x["betas"]) > 1 else ()):
                 assert np.array_equal(st[k], getattr(ref, k)), (i, k)
+
+
+@pytest.mark.parametrize("n", [2, 40])
+def test_planned_batch_of_few_temperatures(P, n):
+    """Batches whose groups have up to 10 temperatures: cell-major groups for few CTAs on a large lattice."""
+    R, seed = 2, 78
+    inst = [dict(L=L, J=W.random_couplers(L, seed, i), betas=W.beta_ladder(NT, 0.1, 3.0), uid=i)
+            for i, (L, NT) in enumerate([(16, 4), (12, 5), (4, 8)] * n)][:n + 1]
+    with P.PTBatch(inst, R, seed) as b:
+        b.run(6, 1)
+        b.run(5, 2)
+        for i, x in enumerate(inst):
+            st = b.state(i)
+            ref = oracle.PTState(x["L"], x["J"], x["betas"], R, seed, i)
+            ref.sweeps(6, 1)
+            ref.sweeps(5, 2)
+            for k in ("spins", "E", "best", "first", "macc", "xacc"):
+                assert np.array_equal(st[k], getattr(ref, k)), (i, k)
