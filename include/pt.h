@@ -404,7 +404,7 @@ int pt_restore(pt_handle *h, const void *buf, size_t len);
 
 /* Launch schedule (results are identical for every valid choice).  A new handle
  * plans its launches itself, from the sizes and the device (replica-lane mapping:
- * a lane per replica); pt_set_schedule and pt_set_mapping replace the plan by the
+ * a lane per replica; with few temperatures on a large lattice cell-major); pt_set_schedule and pt_set_mapping replace the plan by the
  * given mapping, and pt_get_schedule / pt_get_mapping return the values they start
  * from:
  * slot_parallel = temperature slots one CTA processes concurrently per run
@@ -549,7 +549,7 @@ int pt_batch_get_state(pt_batch *b, int32_t inst, int8_t *spins, int32_t *E, int
                        int32_t *first, uint64_t *macc, uint64_t *xacc);
 
 /* Schedule of the instances of size chimera_L (a new batch plans each size itself,
- * with the replica-lane mapping; a set schedule or mapping replaces that plan):
+ * with the replica-lane mapping (few temperatures: cell-major); a set schedule or mapping replaces that plan):
  * slot_parallel slots
  * (cell-major: slot_parallel * L^2 threads per run) or teams (slot-major:
  * slot_parallel * team threads per run, at the size's largest temperature

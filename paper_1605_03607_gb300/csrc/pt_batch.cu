@@ -34,7 +34,8 @@ namespace {
 // of L^2 threads (cell-major, team 0) or slot_parallel teams of `team` lanes
 // (slot-major, at the size's largest temperature count).  block 0: the CTA
 // size is the bundle's thread count rounded up to a warp.  planned: until a
-// schedule is set, the replica-lane mapping (lane_plan_batch) instead.
+// schedule is set, the replica-lane mapping (lane_plan_batch) instead, but for few
+// temperatures where cell-major is faster.
 struct ShapeSched {
     int sp = 0, ipc = 0, team = 0, block = 0;
     bool planned = false;

@@ -91,7 +91,7 @@ struct pt_handle {
     size_t stage_bytes = 0;
     int sp = 0, ipc = 0, spl = 4096;
     int team = 0;              // 0: cell-major mapping; > 0: slot-major with teams of this size
-    bool planned = true;       // until a schedule is set: the replica-lane mapping, shaped by lane_plan
+    bool planned = true;       // until a schedule is set: mapping and shape by lane_plan
     struct Plan { int kt, n_inst, R; bool walk; LaneShape s; };
     std::vector<Plan> plans;   // shapes made so far (at most MAX_PLANS)
     uint64_t launches = 0;
