@@ -405,8 +405,8 @@ int pt_restore(pt_handle *h, const void *buf, size_t len);
 /* Launch schedule (results are identical for every valid choice).  A new handle
  * plans its launches itself, from the sizes and the device (replica-lane mapping:
  * a lane per replica; with few temperatures on a large lattice cell-major);
- * pt_set_schedule and pt_set_mapping replace the plan by the given mapping, and pt_get_schedule / pt_get_mapping return the values they start
- * from:
+ * pt_set_schedule and pt_set_mapping replace the plan by the given mapping, and
+ * pt_get_schedule / pt_get_mapping return the values they start from:
  * slot_parallel = temperature slots one CTA processes concurrently per run
  * (threads per run = slot_parallel * L^2, a multiple of 32, <= 1024),
  * runs_per_cta = runs sharing one CTA, sweeps_per_launch = sweeps per kernel
