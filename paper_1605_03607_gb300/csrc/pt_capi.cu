@@ -54,13 +54,14 @@ struct Group {
     InstDesc* d_desc = nullptr;
     int2* d_items = nullptr;
     Bundle* d_bundles = nullptr;
-    Bundle* d_sub = nullptr;         // the list of the last subset_launch
+    Bundle* d_sub = nullptr;         // the list of the last subset_launch: room for a bundle per run
     int32_t* d_tts = nullptr;        // [n_inst][3]
     int32_t* d_targets = nullptr;    // [n_inst] per-instance TTS targets (LAO)
     int* d_queue = nullptr;
     std::vector<InstDesc> desc;
     std::vector<Bundle> bundles;
     Launch all;                      // every run of every instance
+    bool planned = true;             // what `bundles` was made from: the plan, or a set schedule
     uint64_t sweep = 0;
     // temperature random walk (main group only, when tracked)
     bool walk = false;
@@ -344,8 +345,7 @@ int group_schedule(pt_handle* h, Group& g)
     Bundle* d = nullptr;
     Bundle* dsub = nullptr;
     CK(dalloc(&d, bundles.size()), "cudaMalloc bundles");
-    // room for any subset: of the list, or (planned) with a shape of its own, a run per CTA at most
-    cudaError_t e = dalloc(&dsub, h->planned ? (size_t)g.n_inst * g.R : bundles.size());
+    cudaError_t e = dalloc(&dsub, (size_t)g.n_inst * g.R);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d, bundles.data(), sizeof(Bundle) * bundles.size(), cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) {
@@ -361,15 +361,17 @@ int group_schedule(pt_handle* h, Group& g)
     l.d = d;
     l.n = (int)g.bundles.size();
     g.all = l;
+    g.planned = h->planned;
     return PT_OK;
 }
 
-// The launch over the first R runs of the listed instances, in the group's list of subsets.
+// The launch over the first R runs of the listed instances, in the group's list of subsets: from what the
+// group's own list was made from, which after a failed change of schedule need not be the handle's mapping.
 int subset_launch(pt_handle* h, Group& g, const std::vector<int>& insts, int R, Launch& l)
 {
     l = g.all;
     std::vector<Bundle> sub;
-    if (h->planned) {
+    if (g.planned) {
         if (int rc = planned_launch(h, g, insts, R, sub, l)) return rc;
     } else {
         std::vector<char> in((size_t)g.desc.size(), 0);
@@ -1946,6 +1948,15 @@ int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
             for (int ipc : {1, 2, 4})
                 if (nt >= 1 && nt * team >= 32 && nt * team * ipc <= MAX_THREADS_SM) cands.push_back({false, team, nt, ipc});
     }
+    // a failure gives the candidate batch back, which the last trial left in its schedule: the next one is
+    // made in the handle's own
+    auto give_up = [&](int code) {
+        h->timing = old_timing;
+        h->planned = old_planned;
+        h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
+        free_group(h->cand);
+        return code;
+    };
     h->timing = true;
     double best_ms = 1e300;
     Cand best = cands[0];
@@ -1963,18 +1974,13 @@ int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
             e = cudaEventElapsedTime(&t, h->ev[2 * i], h->ev[2 * i + 1]);
             ms += t;
         }
-        if (rc || e != cudaSuccess) {
-            h->timing = old_timing;
-            h->planned = old_planned;
-            h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
-            return rc ? rc : cuda_fail(h, e, "sync autotune");
-        }
+        if (rc || e != cudaSuccess) return give_up(rc ? rc : cuda_fail(h, e, "sync autotune"));
         if (ms < best_ms) { best_ms = ms; best = c; }
     }
     h->timing = old_timing;
     h->planned = old_planned;
     h->team = old_team; h->sp = old_sp; h->ipc = old_ipc;
-    if ((rc = apply_schedule(h, best.planned, best.team, best.sp, best.ipc))) return rc;
+    if ((rc = apply_schedule(h, best.planned, best.team, best.sp, best.ipc))) return give_up(rc);
     CK(cudaStreamSynchronize(h->stream), "sync autotune");
     return PT_OK;
 }

@@ -1,0 +1,83 @@
+"""The handle runtime's launch lists and copies on error paths, on the CPU (tests/host_runtime.py)."""
+import numpy as np
+import pytest
+
+import host_runtime
+import workloads as W
+
+
+@pytest.fixture(scope="module")
+def host_lib(tmp_path_factory):
+    lib = host_runtime.build(tmp_path_factory.mktemp("host_runtime"))
+    if lib is None:
+        pytest.skip("no host compiler or CUDA headers")
+    return lib
+
+
+@pytest.fixture
+def rt(host_lib, monkeypatch):
+    from paper_1605_03607_gb300 import _lib
+    monkeypatch.setattr(_lib, "_lib", host_lib)
+    host_lib.host_fail_launches(0, 0)
+    host_lib.host_fail_allocs(0, 0)
+    host_lib.host_fastest(0, -1)
+    before = host_lib.host_overruns()
+    yield host_lib
+    host_lib.host_fail_launches(0, 0)
+    host_lib.host_fail_allocs(0, 0)
+    assert host_lib.host_overruns() == before
+
+
+def handle(L, NT, R):
+    import paper_1605_03607_gb300 as P
+    return P.PTHandle(L, W.random_couplers(L, 3, 0), W.beta_ladder(NT, 0.1, 3.0), R, 3, 0)
+
+
+def evaluate(rt, h, k):
+    """Candidates, and the handle's own runs under a doubling budget: every run in the launches once."""
+    J = np.stack([h.couplers()] * k)
+    h.tts_eval_many(J, np.arange(k), 4)
+    assert rt.host_last_launch_ok(k, h.R)
+    h.tts_eval_many(J[:1], np.arange(1), 4, max_sweeps=8)
+    assert rt.host_last_launch_ok(1, h.R)
+    h.tts_eval_doubling(1, 4, 8)
+    assert rt.host_last_launch_ok(1, h.R)
+
+
+@pytest.mark.parametrize("L,NT,R,k", [(16, 48, 32, 4), (8, 32, 64, 1), (7, 30, 100, 3), (4, 6, 40, 2)])
+@pytest.mark.parametrize("what", ["launches", "allocs"])
+def test_failed_autotune_leaves_launchable_lists(rt, L, NT, R, k, what):
+    """A tuning run that fails at its n-th launch, or from its n-th allocation on, for every n."""
+    import paper_1605_03607_gb300 as P
+    with handle(L, NT, R) as h:
+        rt.host_fail_launches(0, 0)
+        rt.host_fail_allocs(0, 0)
+        h.autotune(k, 2)
+        total = getattr(rt, "host_" + what)()
+    assert total > 3
+    for n in range(1, total + 1):
+        with handle(L, NT, R) as h:
+            getattr(rt, "host_fail_" + what)(n, total + 1000)
+            with pytest.raises(P.PTError):
+                h.autotune(k, 2)
+            getattr(rt, "host_fail_" + what)(0, 0)
+            evaluate(rt, h, k)
+
+
+@pytest.mark.parametrize("L,NT,R,k", [(16, 48, 32, 4), (8, 32, 64, 2)])
+def test_failed_mapping_change_leaves_launchable_lists(rt, L, NT, R, k):
+    """A change of mapping that runs out of memory, with the way back failing too or not."""
+    import paper_1605_03607_gb300 as P
+    for n in range(1, 9):
+        for last in (n, 1000):
+            with handle(L, NT, R) as h:
+                evaluate(rt, h, k)
+                rt.host_fail_allocs(n, last)
+                try:
+                    h.set_mapping(4, NT, 2 if L == 8 else 1)
+                    failed = False
+                except P.PTError:
+                    failed = True
+                rt.host_fail_allocs(0, 0)
+                assert failed == (n <= 4)        # two groups, two lists each
+                evaluate(rt, h, k)
