@@ -1329,7 +1329,7 @@ constexpr int RO_ROWS = 64, RO_THREADS = 256;
 __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* h, const float* __restrict__ W1, const float* __restrict__ b1,
                                const float* __restrict__ w2, const float* __restrict__ b2, float* y, float* gbuf,
                                float* zbuf, const float* __restrict__ target, float inv_B, float* dybuf,
-                               float* sqbuf, float* dgbuf, const int* __restrict__ err)
+                               float* sqbuf, float* dgbuf, const volatile int* err)
 {
     __shared__ __align__(16) float gs[HD];
     __shared__ float as[HD], red[HD], dz[HD];
