@@ -1814,10 +1814,11 @@ int pt_set_schedule(pt_handle* h, int32_t sp, int32_t ipc, int32_t spl)
     if (!h) return PT_ERR_ARG;
     const int nsp = sp > 0 ? sp : h->sp, nipc = ipc > 0 ? ipc : h->ipc;
     if (spl < 0) return fail(h, PT_ERR_ARG, "sweeps_per_launch must be >= 0");
-    int rc = check_schedule(h, h->L, h->NT, nsp, nipc, h->team);
-    if (rc) return rc;
-    const bool keep = h->planned && sp <= 0 && ipc <= 0;       // only the launch length changes
-    if (!keep && (rc = apply_schedule(h, false, h->team, nsp, nipc))) return rc;
+    if (!(h->planned && sp <= 0 && ipc <= 0)) {        // else only the launch length changes, and the plan stays
+        int rc = check_schedule(h, h->L, h->NT, nsp, nipc, h->team);
+        if (!rc) rc = apply_schedule(h, false, h->team, nsp, nipc);
+        if (rc) return rc;
+    }
     if (spl > 0) h->spl = spl;
     CK(cudaStreamSynchronize(h->stream), "sync schedule");
     return PT_OK;

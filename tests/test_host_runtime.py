@@ -81,3 +81,18 @@ def test_failed_mapping_change_leaves_launchable_lists(rt, L, NT, R, k):
                 rt.host_fail_allocs(0, 0)
                 assert failed == (n <= 4)        # two groups, two lists each
                 evaluate(rt, h, k)
+
+
+@pytest.mark.parametrize("L", [4, 7, 11, 14, 15])
+def test_launch_length_of_a_planned_handle(rt, L):
+    """A new launch length keeps the plan, also where the set mappings' default does not fit a CTA."""
+    with handle(L, 20, 6) as h:
+        rt.host_fail_launches(0, 0)
+        h.sweep(20, 1)
+        assert rt.host_launches() == 1
+        block = rt.host_last_block()
+        h.set_schedule(0, 0, 7)
+        assert h.schedule()[2] == 7
+        rt.host_fail_launches(0, 0)
+        h.sweep(20, 1)
+        assert rt.host_launches() == 3 and rt.host_last_team() < 0 and rt.host_last_block() == block
