@@ -1962,7 +1962,8 @@ int pt_autotune(pt_handle* h, int32_t n_inst, int32_t trial_sweeps)
     double best_ms = 1e300;
     Cand best = cands[0];
     for (const Cand& c : cands) {
-        if (!c.planned && (c.ipc > h->R || bundle_smem_bytes(h->L, h->NT, c.ipc, c.team, false, h->kt) > cap)) continue;
+        // what is kept has to fit the main runs too, with their walk counters where these are tracked
+        if (!c.planned && (c.ipc > h->R || bundle_smem_bytes(h->L, h->NT, c.ipc, c.team, h->main.walk, h->kt) > cap)) continue;
         h->planned = c.planned;
         h->team = c.team;
         h->sp = c.sp;

@@ -96,3 +96,15 @@ def test_launch_length_of_a_planned_handle(rt, L):
         rt.host_fail_launches(0, 0)
         h.sweep(20, 1)
         assert rt.host_launches() == 3 and rt.host_last_team() < 0 and rt.host_last_block() == block
+
+
+@pytest.mark.parametrize("L,NT,team,block", [(16, 55, 0, 1024), (11, 51, 2, 408)])
+def test_autotune_keeps_a_schedule_that_the_walk_counters_fit(rt, L, NT, team, block):
+    """The fastest trial fits a CTA without the main runs' walk counters and not with them."""
+    with handle(L, NT, 4) as h:
+        h.set_walk_stats(True)
+        rt.host_fastest(team, block)
+        h.autotune(2, 2)
+        h.sweep(3, 1)
+        assert rt.host_last_launch_ok(1, 4)
+        evaluate(rt, h, 2)
