@@ -1086,37 +1086,37 @@ int pt_get_state(pt_handle* h, int8_t* spins, int32_t* E, uint8_t* perm, int32_t
     if (!h) return PT_ERR_ARG;
     Group& g = h->main;
     const size_t reps = (size_t)h->R * h->NT, N = h->N;
-    // one copy of the records, or of the whole state, into the pinned staging where it fits (a copy of
-    // each array into pageable memory costs about 8 us); larger spins go straight to the caller's side
-    const bool whole = spins && g.block_bytes <= h->stage_bytes;
-    const size_t from = whole ? 0 : g.rec_off, bytes = g.block_bytes - from;
-    std::vector<uint8_t> rec;
+    std::vector<uint8_t> pm;                  // the slot map, which the spins need
+    if (spins && !perm) pm.resize(reps);
+    uint8_t* const slots = perm ? perm : pm.data();
+    const struct { void* to; const void* from; size_t bytes; } arrays[] = {
+        {E, g.E, 4 * reps}, {slots, g.perm, reps}, {best, g.best, 4 * (size_t)h->R}, {first, g.first, 4 * (size_t)h->R},
+        {macc, g.macc, 8 * reps}, {h->NT > 1 ? xacc : nullptr, g.xacc, 8 * (size_t)h->R * (h->NT - 1)}};
+    // Records that fit the pinned staging come in one copy, with the spins where these fit too (a copy of each
+    // array into pageable memory costs about 8 us); larger ones array by array, those asked for, to their places
+    const size_t rec_bytes = g.block_bytes - g.rec_off;
+    const bool staged = rec_bytes <= h->stage_bytes, whole = spins && g.block_bytes <= h->stage_bytes;
+    const size_t off = whole ? 0 : g.rec_off;
     std::vector<int8_t> sp;
-    uint8_t* host = h->stage;
-    if (bytes > h->stage_bytes) {
-        rec.resize(bytes);
-        host = rec.data();
-    }
-    CK(cudaMemcpyAsync(host, g.block + from, bytes, cudaMemcpyDeviceToHost, h->stream), "download state");
+    if (staged)
+        CK(cudaMemcpyAsync(h->stage, g.block + off, g.block_bytes - off, cudaMemcpyDeviceToHost, h->stream), "download state");
+    else
+        for (const auto& a : arrays)
+            if (a.to) CK(cudaMemcpyAsync(a.to, a.from, a.bytes, cudaMemcpyDeviceToHost, h->stream), "download state");
     if (spins && !whole) {
         sp.resize(reps * N);
         CK(cudaMemcpyAsync(sp.data(), g.spins, reps * N, cudaMemcpyDeviceToHost, h->stream), "download spins");
     }
     CK(cudaStreamSynchronize(h->stream), "sync get_state");
-    auto at = [&](const void* d) { return host + (static_cast<const uint8_t*>(d) - g.block) - from; };
-    const uint8_t* pm = at(g.perm);
-    if (E) std::memcpy(E, at(g.E), 4 * reps);
-    if (best) std::memcpy(best, at(g.best), 4 * (size_t)h->R);
-    if (first) std::memcpy(first, at(g.first), 4 * (size_t)h->R);
-    if (macc) std::memcpy(macc, at(g.macc), 8 * reps);
-    if (xacc && h->NT > 1) std::memcpy(xacc, at(g.xacc), 8 * (size_t)h->R * (h->NT - 1));
-    if (perm) std::memcpy(perm, pm, reps);
-    if (spins) {                              // slot order: slot t holds buffer perm[t]
-        const int8_t* src = whole ? reinterpret_cast<const int8_t*>(at(g.spins)) : sp.data();
+    if (staged)
+        for (const auto& a : arrays)
+            if (a.to) std::memcpy(a.to, h->stage + (static_cast<const uint8_t*>(a.from) - g.block) - off, a.bytes);
+    if (spins) {                              // slot order: slot t holds buffer slots[t]
+        const int8_t* src = whole ? reinterpret_cast<const int8_t*>(h->stage) : sp.data();
         for (int r = 0; r < h->R; ++r)
             for (int t = 0; t < h->NT; ++t)
                 std::memcpy(spins + ((size_t)r * h->NT + t) * N,
-                            src + ((size_t)r * h->NT + pm[(size_t)r * h->NT + t]) * N, N);
+                            src + ((size_t)r * h->NT + slots[(size_t)r * h->NT + t]) * N, N);
     }
     if (sweep) *sweep = g.sweep;
     return PT_OK;

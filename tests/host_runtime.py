@@ -3,8 +3,8 @@ few lines, for tests of its bookkeeping and error paths without a GPU.
 
 Device memory is host memory.  Every copy is checked against the allocations it touches, every sweep
 launch against what its bundles need (threads, shared memory, the launch's mapping), and the n-th
-allocation or launch from now on can be made to fail.  Kernels compute nothing: a TTS reduction
-returns zeros, so every evaluation counts as decided.
+allocation or launch from now on can be made to fail.  Kernels compute nothing: set_spins leaves
+records by their index, a TTS reduction zeros, so every evaluation counts as decided.
 """
 import ctypes as C
 import os
@@ -111,7 +111,23 @@ namespace ptg {
 cudaError_t sweep_smem_capacity(int* b) { *b = 232448 - 16; return cudaSuccess; }
 cudaError_t set_sweep_smem_limit(int, int, bool, int) { return cudaSuccess; }
 cudaError_t launch_init(const InstDesc*, const int2*, int, bool, cudaStream_t) { return cudaSuccess; }
-cudaError_t launch_energy(const InstDesc*, const int2*, int, int32_t, cudaStream_t) { return cudaSuccess; }
+// a state that can be told apart: records by their index, slots in reverse order
+cudaError_t launch_energy(const InstDesc* insts, const int2* items, int nitems, int32_t, cudaStream_t)
+{
+    for (int i = 0; i < nitems; ++i) {
+        const InstDesc& d = insts[items[i].x];
+        const int r = items[i].y, np = d.NT > 1 ? d.NT - 1 : 1;
+        for (int t = 0, x = r * d.NT; t < d.NT; ++t, ++x) {
+            d.E[x] = 7 * x + 3;
+            d.perm[x] = (uint8_t)(d.NT - 1 - t);
+            d.macc[x] = 11 * x;
+        }
+        for (int t = 0; t < np; ++t) d.xacc[r * np + t] = 13 * (r * np + t);
+        d.best[r] = -r;
+        d.first[r] = r + 1;
+    }
+    return cudaSuccess;
+}
 cudaError_t launch_hamming(const InstDesc*, int, const int32_t*, const int32_t*, int32_t*, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_tts(const InstDesc*, int n, int32_t, int32_t, int32_t* out, cudaStream_t, const int32_t*)
 {

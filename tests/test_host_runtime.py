@@ -108,3 +108,27 @@ def test_autotune_keeps_a_schedule_that_the_walk_counters_fit(rt, L, NT, team, b
         h.sweep(3, 1)
         assert rt.host_last_launch_ok(1, 4)
         evaluate(rt, h, 2)
+
+
+@pytest.mark.parametrize("L,NT,R", [(2, 64, 1024), (4, 30, 700), (4, 16, 8), (8, 32, 64), (2, 1, 3)])
+def test_state_downloads_what_is_asked_for(rt, L, NT, R):
+    """Records too large for the staging: only the arrays asked for are copied, each once."""
+    from paper_1605_03607_gb300._lib import _ptr
+    N, x, r = 8 * L * L, np.arange(R * NT), np.arange(R)
+    with handle(L, NT, R) as h:
+        s = np.where(np.random.default_rng(1).random((R, NT, N)) < 0.5, -1, 1).astype(np.int8)
+        h.set_spins(s)
+        want = dict(spins=s[:, ::-1].copy(), E=(7 * x + 3).astype(np.int32),
+                    perm=np.tile(np.arange(NT)[::-1], R).astype(np.uint8), best=(-r).astype(np.int32),
+                    first=(r + 1).astype(np.int32), macc=(11 * x).astype(np.uint64),
+                    xacc=(13 * np.arange(R * (NT - 1))).astype(np.uint64))
+        large = sum(a.nbytes for k, a in want.items() if k != "spins") > 256 * 1024
+        for names in (tuple(want), ("E",), ("spins",), ("spins", "perm"), ("best", "xacc")):
+            out = {k: np.full(want[k].shape, 99, want[k].dtype) for k in names}
+            rt.host_downloaded()
+            assert rt.pt_get_state(h.h, *(_ptr(out.get(k)) for k in want), None) == 0
+            got = rt.host_downloaded()
+            if large:
+                assert got == sum(want[k].nbytes for k in set(names) | ({"perm"} if "spins" in names else set())), names
+            for k in names:
+                assert np.array_equal(out[k], want[k]), k
