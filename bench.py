@@ -48,6 +48,12 @@ UNIT = "spin-flip attempts/s"
 #   flip, energy and accept-count updates                     =  3
 #   spin loads (4 words per 4 spins) and store (1 per 4)      =  1.25
 OPS_PER_ATTEMPT = 31.25
+# What the roofline's fraction counts, where a kernel executes fewer operations than the method has.
+COUNTS = ("the method's operations, not executed instructions: the replica-lane kernel takes local fields from "
+          "tables and shares Philox terms between replicas, so its fraction includes work saved")
+# Widening multiplies that no such sharing removes: 16 per Philox call of a warp's 128 attempts, 4 clocks each on
+# a sub-partition.
+MULTIPLY_CLOCKS_PER_WORD = 64
 # Integer issue peak per SM and clock: 4 sub-partitions x 32 lanes.
 INT_LANES_PER_SM_CLK = 128
 # DRAM bytes (read + write) of one sweep-kernel launch, taken from one ncu
@@ -58,6 +64,11 @@ INT_LANES_PER_SM_CLK = 128
 # depend on the sweeps per launch.  Any other schedule reports null, and so
 # does every schedule while the kernel has changed since the last capture.
 PROFILED_TRAFFIC = {(4, 32, 1, 1024): 17554176}
+
+
+def kernel_of(shape):
+    """Sweep kernel of a launch shape (PTHandle.launch_shape, PTBatch.launch_shape)."""
+    return "pt_lane_kernel" if shape["mapping"] == "replica-lane" else "pt_sweep_kernel"
 
 
 def load_peaks():
@@ -79,6 +90,12 @@ def measured_int_issue(P, stream, peak_ops, iters=1 << 18, reps=3):
         out[kind] = {"Tops_s": ops / 1e12, "of_derived_peak": ops / peak_ops if peak_ops else None,
                      "ms_per_launch": ms}
     return out
+
+
+def multiply_floor(attempts, ms, sms, peaks):
+    """Attempts/s against the rate of the widening multiplies alone, which bounds every mapping."""
+    top = sms * 4 * float(peaks.get("sm_max_mhz", 2070.0)) * 1e6 * 128 / MULTIPLY_CLOCKS_PER_WORD
+    return {"attempts_per_s": top, "frac": attempts / (ms / 1e3) / top if ms > 0 else None}
 
 
 class ClockSampler:
@@ -335,6 +352,7 @@ def run_gpu(args):
     if rank != 0:
         h.close()
         return 0
+    shape = h.launch_shape(spec)                 # of the speculative batches
     issue = measured_int_issue(P, stream.cuda_stream, peak_ops)
     cpu = None
     if ws == 1 and not args.no_cpu:
@@ -356,7 +374,7 @@ def run_gpu(args):
                                "beta geometric [0.1,4], 64 PT runs, S=2^16, target from 4x pass, "
                                "exchange every sweep",
                    "step": f"engineer_run: {spec} RAO steps, candidates evaluated in batches of {spec}",
-                   "speculation": spec, "schedule": list(h.schedule()), "team": h.mapping(),
+                   "speculation": spec, "launch": shape, "sweeps_per_launch": h.schedule()[2],
                    "l2": "flushed between steps",
                    "parallelism": f"{ws} independent instance(s), one per GPU"},
         "pt_tts_evals_per_s": tot_evals / t_dev,
@@ -371,11 +389,12 @@ def run_gpu(args):
         "gpu_launches": int(launches),
         "roofline": {"bound": "alu", "achieved": achieved_ops / 1e12, "peak": peak_ops / 1e12,
                      "unit": "Tops/s (int32 issue)", "frac": achieved_ops / peak_ops if peak_ops else None,
-                     "traffic": PROFILED_TRAFFIC.get((h.mapping(), *h.schedule()[:2], R * spec)),
+                     "traffic": PROFILED_TRAFFIC.get((shape["team"], shape["slot_parallel"], shape["runs_per_cta"],
+                                                      R * spec)),
                      "traffic_source": "profiled constant (one ncu capture of this schedule), not measured "
                                        "in this run",
-                     "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule",
-                     "ops_per_attempt": OPS_PER_ATTEMPT,
+                     "kernel": kernel_of(shape), "ops_per_attempt": OPS_PER_ATTEMPT, "counts": COUNTS,
+                     "multiply_floor": multiply_floor(attempts, sweep_ms, sms, peaks),
                      "avg_launch_ms": sweep_ms / max(sweep_launches, 1), "launches": sweep_launches,
                      "peak_source": f"{sms} SMs x {INT_LANES_PER_SM_CLK} lanes x "
                                     f"{peaks.get('sm_max_mhz', 2070.0)} MHz ({peak_kind} max clock)",
@@ -441,7 +460,7 @@ def measure_batched(args, steps, warmup):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     peak_ops = sms * INT_LANES_PER_SM_CLK * float(peaks.get("sm_max_mhz", 2070.0)) * 1e6
     achieved = attempts * steps * OPS_PER_ATTEMPT / (kern_ms / 1e3)
-    sched = {L: b.schedule(L) + (b.mapping(L),) for L in (4, 8, 12, 16)}
+    shapes = {L: b.launch_shape(L) for L in (4, 8, 12, 16)}
     out = {
         "workload": "batched_256: 256 instances, 64 each of C_4/C_8/C_12/C_16, 24..48 temps (beta [0.1,4]), "
                     "32 runs each, 2^14 sweeps, one persistent graph-captured launch per size group",
@@ -452,9 +471,11 @@ def measure_batched(args, steps, warmup):
         "instances_solved_within_S": n_solved,
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
                      "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops,
-                     "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule (persistent)", "ops_per_attempt": OPS_PER_ATTEMPT,
+                     "kernel": " + ".join(sorted({kernel_of(x) for x in shapes.values()})) + " (persistent)",
+                     "ops_per_attempt": OPS_PER_ATTEMPT, "counts": COUNTS,
+                     "multiply_floor": multiply_floor(attempts * steps, kern_ms, sms, peaks),
                      "avg_launch_ms": kern_ms / max(steps, 1), "peak_source": peak_kind},
-        "schedule": {str(k): v for k, v in sched.items()}, "info": b.info(), "clocks": clocks,
+        "launch": {str(k): v for k, v in shapes.items()}, "info": b.info(), "clocks": clocks,
         "timing": "value over the host wall clock of reset + run + TTS per step; kernel_attempts_per_s "
                   "and the roofline over the graph replay's CUDA-event time"}
     b.close()
@@ -517,7 +538,7 @@ def run_mixing(args):
         "metric": "spin-flip attempts/s (walk tracked)", "value": rates[True], "unit": UNIT,
         "untracked_attempts_per_s": rates[False], "tracking_cost": 1.0 - rates[True] / rates[False],
         "chains": R, "emcs": args.mixing_emcs, "sweeps": n_sweeps, "exchange_passes": passes,
-        "schedule": list(h.schedule()), "team": h.mapping(),
+        "launch": h.launch_shape(), "sweeps_per_launch": h.schedule()[2],
         "walk": {"min_hot_fraction": float(frac.min()), "median_hot_fraction": float(np.median(frac)),
                  "criterion_hot_half": bool(frac.min() >= 0.2),
                  "round_trips_per_copy_mean": mean_trips, "round_trips_min": int(trips.min()),
@@ -626,6 +647,7 @@ def run_lao(args):
     peak_ops = sms * INT_LANES_PER_SM_CLK * float(peaks.get("sm_max_mhz", 2070.0)) * 1e6
     achieved = attempts * OPS_PER_ATTEMPT / (sweep_ms / 1e3)
     st = h.lao_state()
+    shape = h.launch_shape(spec)
     # ground / first-excited overlaps of the engineered instance (Sec. III.B): one
     # fresh PT pass of the handle's runs, then per run its coldest replica at
     # each of the two levels
@@ -642,10 +664,11 @@ def run_lao(args):
         "accepted_warmup": accepted_warmup, "tts_initial": tts0, "tts_after_warmup": tts_warm,
         "tts_final": st["tts"], "unsolved_cap": S + 1, "E_gs_initial": e_gs0, "E_gs_final": st["E_gs"],
         "overlaps_final": ov,
-        "schedule": list(h.schedule()), "team": h.mapping(),
+        "launch": shape, "sweeps_per_launch": h.schedule()[2],
         "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12,
-                     "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops, "kernel": "pt_lane_kernel, or pt_sweep_kernel under a set schedule",
-                     "ops_per_attempt": OPS_PER_ATTEMPT, "peak_source": kind},
+                     "unit": "Tops/s (int32 issue)", "frac": achieved / peak_ops, "kernel": kernel_of(shape),
+                     "ops_per_attempt": OPS_PER_ATTEMPT, "counts": COUNTS,
+                     "multiply_floor": multiply_floor(attempts, sweep_ms, sms, peaks), "peak_source": kind},
         "clocks": clocks, "data": "synthetic"}))
     h.close()
     return 0
@@ -801,8 +824,8 @@ def run_profile_case(args):
     ms, n = h.sweep_timing_total()
     att = args.profile_sweeps * spl * h.R * h.NT * h.N
     print(json.dumps({"profile_case": True, "L": L, "n_temps": h.NT, "launches": n, "ms": ms,
-                      "attempts_per_s": att / (ms / 1e3), "runs": h.R, "schedule": list(h.schedule()),
-                      "team": h.mapping()}))
+                      "attempts_per_s": att / (ms / 1e3), "runs": h.R, "launch": h.launch_shape(),
+                      "sweeps_per_launch": spl}))
     h.close()
     return 0
 

@@ -416,6 +416,19 @@ int pt_set_schedule(pt_handle *h, int32_t slot_parallel, int32_t runs_per_cta,
 int pt_get_schedule(const pt_handle *h, int32_t *slot_parallel, int32_t *runs_per_cta,
                     int32_t *sweeps_per_launch);
 
+/* What a sweep launch runs, planned or set: of this handle's runs (n_inst 0), or of a batch
+ * of n_inst (1..256) candidates with n_runs runs each (engineer_run, pt_tts_eval_many).
+ *   team           0 cell-major, > 0 slot-major (lanes of a team), < 0 replica-lane (-team runs
+ *                  in a group)
+ *   slot_parallel  slots a CTA processes concurrently per run, teams, or warps per column of 32
+ *                  replicas
+ *   runs_per_cta   most runs of a CTA
+ *   ctas, threads  CTAs of the launch and threads of one
+ *   shared_ctas    CTAs that hold runs of two candidates
+ * Any output may be NULL. */
+int pt_get_launch(pt_handle *h, int32_t n_inst, int32_t *team, int32_t *slot_parallel, int32_t *runs_per_cta,
+                  int32_t *ctas, int32_t *threads, int32_t *shared_ctas);
+
 /* Thread mapping of the sweep kernel.  team == 0: cell-major (a thread owns
  * one Chimera cell and every slot_parallel-th temperature slot).  team > 0
  * (a power of two <= 32): slot-major, slot_parallel teams of `team` lanes per
@@ -575,6 +588,11 @@ int pt_batch_get_schedule(const pt_batch *b, int32_t chimera_L, int32_t *block,
 int pt_batch_set_mapping(pt_batch *b, int32_t chimera_L, int32_t team, int32_t slot_parallel,
                          int32_t runs_per_cta);
 int pt_batch_get_mapping(const pt_batch *b, int32_t chimera_L, int32_t *team);
+
+/* What the launch of size chimera_L runs, planned or set, in the terms of pt_get_launch: team and
+ * slot_parallel of the size's longest bundle, most runs of a bundle, persistent CTAs, their threads. */
+int pt_batch_get_launch(const pt_batch *b, int32_t chimera_L, int32_t *team, int32_t *slot_parallel,
+                        int32_t *runs_per_cta, int32_t *ctas, int32_t *threads);
 
 /* Autotuner: size by size, times the planned shape and every feasible cell-major (slot_parallel,
  * runs_per_cta) and slot-major (team, slot_parallel, runs_per_cta) on all

@@ -100,6 +100,7 @@ SIGNATURES = [
     ("pt_autotune", C.c_int, [_VP, C.c_int32, C.c_int32]),
     ("pt_set_mapping", C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32]),
     ("pt_get_mapping", C.c_int, [_VP, _I32P]),
+    ("pt_get_launch", C.c_int, [_VP, C.c_int32] + [_I32P] * 6),
     ("pt_set_walk_stats", C.c_int, [_VP, C.c_int32]),
     ("pt_get_walk_stats", C.c_int, [_VP, _VP, _VP, C.POINTER(C.c_uint64)]),
     ("pt_launch_count", C.c_uint64, [_VP]),
@@ -125,6 +126,7 @@ SIGNATURES = [
     ("pt_batch_get_schedule", C.c_int, [_VP, C.c_int32, _I32P, _I32P, _I32P]),
     ("pt_batch_set_mapping", C.c_int, [_VP, C.c_int32, C.c_int32, C.c_int32, C.c_int32]),
     ("pt_batch_get_mapping", C.c_int, [_VP, C.c_int32, _I32P]),
+    ("pt_batch_get_launch", C.c_int, [_VP, C.c_int32] + [_I32P] * 5),
     ("pt_batch_autotune", C.c_int, [_VP, C.c_int32, _I32P]),
     ("pt_batch_info", C.c_int, [_VP, C.POINTER(C.c_double), _I32P, _I32P, _I32P, C.POINTER(C.c_uint64)]),
     ("sg_last_error", C.c_char_p, [_VP]),
@@ -206,6 +208,11 @@ def _check(rc, h=None):
     if rc != PT_OK:
         msg = load().pt_last_error(h)
         raise PTError(rc, msg.decode() if msg else "")
+
+
+def _shape(values, names):
+    d = dict(zip(names, (x.value for x in values)))
+    return dict(mapping="replica-lane" if d["team"] < 0 else "slot-major" if d["team"] else "cell-major", **d)
 
 
 class PTHandle:
@@ -462,6 +469,13 @@ class PTHandle:
         _check(load().pt_get_mapping(self.h, C.byref(t)), self.h)
         return t.value
 
+    def launch_shape(self, n_inst=0):
+        """What a sweep launch of this handle's runs (n_inst 0) or of n_inst candidates runs, planned or set: dict of
+        mapping, team, slot_parallel, runs_per_cta, ctas, threads, shared_ctas (pt_get_launch)."""
+        v = [C.c_int32() for _ in range(6)]
+        _check(load().pt_get_launch(self.h, int(n_inst), *(C.byref(x) for x in v)), self.h)
+        return _shape(v, ("team", "slot_parallel", "runs_per_cta", "ctas", "threads", "shared_ctas"))
+
     def set_walk_stats(self, on=True):
         _check(load().pt_set_walk_stats(self.h, 1 if on else 0), self.h)
 
@@ -620,6 +634,12 @@ class PTBatch:
         t = C.c_int32()
         _check_batch(load().pt_batch_get_mapping(self.b, int(L), C.byref(t)), self.b)
         return t.value
+
+    def launch_shape(self, L):
+        """What the launch of size L runs, planned or set (pt_batch_get_launch)."""
+        v = [C.c_int32() for _ in range(5)]
+        _check_batch(load().pt_batch_get_launch(self.b, int(L), *(C.byref(x) for x in v)), self.b)
+        return _shape(v, ("team", "slot_parallel", "runs_per_cta", "ctas", "threads"))
 
     def autotune(self, trial_sweeps=32):
         blk = C.c_int32()

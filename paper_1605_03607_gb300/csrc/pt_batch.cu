@@ -752,6 +752,23 @@ int pt_batch_get_mapping(const pt_batch* b, int32_t chimera_L, int32_t* team)
     return PT_OK;
 }
 
+int pt_batch_get_launch(const pt_batch* b, int32_t chimera_L, int32_t* team, int32_t* sp, int32_t* ipc, int32_t* ctas,
+                        int32_t* threads)
+{
+    if (!b) return PT_ERR_ARG;
+    const int k = group_of(b, chimera_L);
+    if (k < 0) return PT_ERR_ARG;
+    const SizeGroup& g = b->groups[k];
+    int most = 0;
+    for (const Bundle& x : g.bundles) most = std::max(most, x.nitems);
+    if (team) *team = g.bundles[0].team;
+    if (sp) *sp = g.bundles[0].sp;
+    if (ipc) *ipc = most;
+    if (ctas) *ctas = g.grid;
+    if (threads) *threads = g.block;
+    return PT_OK;
+}
+
 // Times candidate schedules and keeps the fastest, size by size: the planned
 // replica-lane shape, every cell-major (slot_parallel, runs_per_cta) and slot-major (team,
 // slot_parallel, runs_per_cta) that fits runs all instances of that size

@@ -317,6 +317,26 @@ int planned_launch(pt_handle* h, const Group& g, const std::vector<int>& insts, 
     return PT_OK;
 }
 
+// Bundles of every run of every instance of g in the handle's mapping, and their launch but for its list.
+int group_bundles(pt_handle* h, const Group& g, std::vector<Bundle>& bundles, Launch& l)
+{
+    if (h->planned) {
+        std::vector<int> insts(g.n_inst);
+        for (int i = 0; i < g.n_inst; ++i) insts[i] = i;
+        return planned_launch(h, g, insts, g.R, bundles, l);
+    }
+    for (int i = 0; i < g.n_inst; ++i)
+        for (int r = 0; r < g.R; r += h->ipc) {
+            Bundle b;
+            b.inst = i; b.run0 = r; b.nitems = std::min(h->ipc, g.R - r); b.sp = h->sp; b.team = h->team;
+            bundles.push_back(b);
+        }
+    l.team = h->team;
+    l.threads = (h->team > 0 ? h->sp * h->team : h->sp * g.L * g.L) * h->ipc;
+    l.smem = (int)bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, g.walk, h->kt);
+    return PT_OK;
+}
+
 // The new bundle list replaces the group's only when every step succeeded, so
 // a failure leaves the previous schedule in place and launchable.
 int group_schedule(pt_handle* h, Group& g)
@@ -325,21 +345,7 @@ int group_schedule(pt_handle* h, Group& g)
     int cap = 0;
     CK(sweep_smem_capacity(&cap), "shared memory capacity");
     Launch l;
-    if (h->planned) {
-        std::vector<int> insts(g.n_inst);
-        for (int i = 0; i < g.n_inst; ++i) insts[i] = i;
-        if (int rc = planned_launch(h, g, insts, g.R, bundles, l)) return rc;
-    } else {
-        for (int i = 0; i < g.n_inst; ++i)
-            for (int r = 0; r < g.R; r += h->ipc) {
-                Bundle b;
-                b.inst = i; b.run0 = r; b.nitems = std::min(h->ipc, g.R - r); b.sp = h->sp; b.team = h->team;
-                bundles.push_back(b);
-            }
-        l.team = h->team;
-        l.threads = (h->team > 0 ? h->sp * h->team : h->sp * g.L * g.L) * h->ipc;
-        l.smem = (int)bundle_smem_bytes(g.L, g.NT, h->ipc, h->team, g.walk, h->kt);
-    }
+    if (int rc = group_bundles(h, g, bundles, l)) return rc;
     if (l.smem > cap) return fail(h, PT_ERR_ARG, "bundle needs more shared memory than a CTA can have");
     CK(set_sweep_smem_limit(cap, l.team, g.walk, g.L), "cudaFuncSetAttribute");
     Bundle* d = nullptr;
@@ -1993,6 +1999,34 @@ int pt_get_schedule(const pt_handle* h, int32_t* sp, int32_t* ipc, int32_t* spl)
     if (sp) *sp = h->sp;
     if (ipc) *ipc = h->ipc;
     if (spl) *spl = h->spl;
+    return PT_OK;
+}
+
+int pt_get_launch(pt_handle* h, int32_t n_inst, int32_t* team, int32_t* sp, int32_t* ipc, int32_t* ctas, int32_t* threads,
+                  int32_t* shared_ctas)
+{
+    if (!h) return PT_ERR_ARG;
+    if (n_inst < 0 || n_inst > 256) return fail(h, PT_ERR_ARG, "n_inst must be in [0, 256]");
+    std::vector<Bundle> list;
+    Launch l = h->main.all;
+    if (n_inst == 0) {
+        list = h->main.bundles;
+    } else {
+        Group g;                              // candidates: no walk
+        g.L = h->L; g.NT = h->NT; g.R = h->R; g.n_inst = n_inst;
+        if (int rc = group_bundles(h, g, list, l)) return rc;
+    }
+    int most = 0, shared = 0;
+    for (const Bundle& b : list) {
+        most = std::max(most, b.nitems + b.nitems2);
+        shared += b.nitems2 > 0;
+    }
+    if (team) *team = l.team;
+    if (sp) *sp = list[0].sp;
+    if (ipc) *ipc = most;
+    if (ctas) *ctas = (int32_t)list.size();
+    if (threads) *threads = l.threads;
+    if (shared_ctas) *shared_ctas = shared;
     return PT_OK;
 }
 

@@ -24,7 +24,7 @@ namespace {
 std::map<char*, size_t> device;
 long overruns = 0, down = 0, launches = 0, allocs = 0;
 long fail_launch = 0, launch_last = 0, fail_alloc = 0, alloc_last = 0;     // failing range, counted from 1
-int fast_team = 0, fast_block = -1, last_team = 0, last_block = 0;
+int fast_team = 0, fast_block = -1, last_team = 0, last_block = 0, last_ctas = 0;
 std::vector<int> seen;                        // runs covered by the last launch: instance * 4096 + run
 bool bad_launch = false;
 bool inside(const void* p, size_t n)
@@ -93,6 +93,7 @@ long host_overruns() { return overruns; }
 long host_downloaded() { const long n = down; down = 0; return n; }
 int host_last_team() { return last_team; }
 int host_last_block() { return last_block; }
+int host_last_ctas() { return last_ctas; }
 // 1 if the last sweep launch covered runs 0 .. runs - 1 of n instances once each and its bundles fitted it
 int host_last_launch_ok(int n, int runs)
 {
@@ -135,7 +136,7 @@ cudaError_t launch_tts(const InstDesc*, int n, int32_t, int32_t, int32_t* out, c
     std::memset(out, 0, 12 * (size_t)n);
     return cudaSuccess;
 }
-cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nb, int, int block, int smem, uint32_t, int, int,
+cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nb, int grid, int block, int smem, uint32_t, int, int,
                           int, int*, cudaStream_t, int team, bool walk, int)
 {
     if (fails(launches, fail_launch, launch_last)) return cudaErrorLaunchOutOfResources;
@@ -143,6 +144,7 @@ cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nb, 
     bad_launch = smem > 232448 - 16 || block > 1024;
     last_team = team;
     last_block = block;
+    last_ctas = grid;
     if (!inside(bundles, sizeof(Bundle) * (size_t)nb)) { ++overruns; bad_launch = true; return cudaSuccess; }
     for (int i = 0; i < nb; ++i) {
         const Bundle& b = bundles[i];

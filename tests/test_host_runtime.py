@@ -132,3 +132,59 @@ def test_state_downloads_what_is_asked_for(rt, L, NT, R):
                 assert got == sum(want[k].nbytes for k in set(names) | ({"perm"} if "spins" in names else set())), names
             for k in names:
                 assert np.array_equal(out[k], want[k]), k
+
+
+SHAPES = [
+    # L, NT, R, candidates, mapping of the handle's runs, CTAs of two candidates
+    (8, 32, 64, 16, "replica-lane", True),
+    (4, 16, 8, 4, "replica-lane", False),
+    (2, 17, 25, 24, "replica-lane", True),
+    (3, 7, 100, 24, "replica-lane", True),
+    (6, 17, 25, 24, "replica-lane", True),
+    (8, 7, 256, 16, "replica-lane", True),
+    (16, 4, 3, 1, "cell-major", False),
+    (16, 8, 1, 2, "cell-major", False),
+    (12, 5, 2, 2, "cell-major", False),
+    (12, 2, 200, 2, "cell-major", False),
+    (14, 40, 3, 2, "replica-lane", False),
+]
+
+
+@pytest.mark.parametrize("L,NT,R,k,mapping,shared", SHAPES)
+def test_launch_shape_is_what_is_launched(rt, L, NT, R, k, mapping, shared):
+    with handle(L, NT, R) as h:
+        s = h.launch_shape()
+        h.sweep(3, 1)
+        assert s["mapping"] == mapping and rt.host_last_launch_ok(1, R)
+        assert (rt.host_last_team(), rt.host_last_block(), rt.host_last_ctas()) == (s["team"], s["threads"], s["ctas"])
+        s = h.launch_shape(k)
+        h.tts_eval_many(np.stack([h.couplers()] * k), np.arange(k), 4)
+        assert rt.host_last_launch_ok(k, R) and (s["shared_ctas"] > 0) == shared
+        assert (rt.host_last_team(), rt.host_last_block(), rt.host_last_ctas()) == (s["team"], s["threads"], s["ctas"])
+        if L in (4, 8, 12, 16):
+            for m in ((0, 1 if L == 16 else 2, 1), (4, max(NT, 8), 1)):
+                h.set_mapping(*m)
+                s = h.launch_shape(k)
+                assert s["mapping"] == ("slot-major" if m[0] else "cell-major")
+                assert (s["team"], s["slot_parallel"], s["runs_per_cta"], s["ctas"]) == (*m, k * R)
+
+
+def test_planned_lists_cover_every_run_once(rt):
+    """Sizes over the whole range, with the walk tracked or not, short and long threshold tables: the runs' and the
+    candidates' launches hold every run once, in CTAs that fit."""
+    rng = np.random.default_rng(7)
+    for _ in range(150):
+        L, NT, k = int(rng.integers(1, 17)), int(rng.integers(1, 65)), int(rng.integers(1, 17))
+        R = min(int(np.exp(rng.uniform(0, np.log(1025)))), 1024, max(1, 20_000_000 // (8 * L * L * NT * k)))
+        with handle(L, NT, R) as h:
+            if rng.random() < 0.3:
+                h.set_walk_stats(True)
+            h.sweep(1, 1)
+            assert rt.host_last_launch_ok(1, R), (L, NT, R)
+            J = np.stack([h.couplers()] * k)
+            if rng.random() < 0.3 and L < 15:
+                J[0, :4] = 28
+            h.tts_eval_many(J, np.arange(k), 4)
+            assert rt.host_last_launch_ok(k, R), (L, NT, R, k)
+            h.sweep(1, 1)
+            assert rt.host_last_launch_ok(1, R), (L, NT, R)
