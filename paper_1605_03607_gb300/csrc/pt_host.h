@@ -229,9 +229,10 @@ inline int lane_threads(int NT, const LaneShape& s) { return 32 * s.W * lane_col
 // cell and colour of a column) takes 117 + 130 / w clocks of a sub-partition that runs w
 // warps (a CTA's warps go round the four of them: a count that is no multiple of four loads
 // one more than the others), exchange and barriers 910, which the groups of the SM overlap;
-// no group is faster than alone.  Fitted to 900 measured (shape, size) pairs from C_2 to
-// C_16: the lowest estimate's time is 0.5 % above the best shape's on average, 3 % at most.
-// (Fitted before the exchange became 200 to 300 clocks shorter.)
+// no group is faster than alone.  Fitted to 900 (shape, size) pairs from C_2 to C_16, measured on
+// an earlier kernel whose exchange took 200 to 300 clocks longer: there the lowest estimate's
+// shape was 0.5 % slower than the best one on average, 3 % at most.  On the kernel as it is that
+// has not been measured; 750 and 600 in place of 910 changed no plan for the better.
 inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);      // what the warps of a column share out
@@ -240,6 +241,16 @@ inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
     const double w1 = 0.25 * c * s.W, x = 910.0;
     const double together = 0.25 * words * n * (117.0 + 130.0 / (w1 * n)) + x / std::pow(n, 0.7);
     return std::max(together, 0.25 * words * (117.0 + 130.0 / w1) + x);
+}
+
+// CTAs that the estimate counts on an SM, which its constants were fitted with.  The device holds fewer of
+// the small ones: 1024 threads (64 registers each, from 58 in the kernel for odd sides) and 4 CTAs of any
+// size (16 named barriers each, 64 an SM).  That count with the same constants is no better a rule: of 4000
+// random sizes 126 take another shape, 1.07 times faster on average but from 0.87 (C_4 x 58 slots, 195
+// runs, 14 candidates) to 1.43 (C_1 x 39, 133, 16), and a batch of C_2 to C_8 0.68.  It needs a fit of its own.
+inline int lane_counted(int threads, int64_t smem)
+{
+    return std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
 }
 
 // Default schedule: about 256 threads per run, a multiple of 32.
@@ -295,7 +306,7 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
                     s.span = span != 0;
                     const int threads = lane_threads(NT, s);
                     if (threads > LANE_THREADS || (W > units && W > 1)) break;
-                    const int fit = std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
+                    const int fit = lane_counted(threads, smem);
                     const int64_t ctas = span ? (n_inst * per + G - 1) / G : n_inst * ((per + G - 1) / G), wave = (int64_t)fit * sms;
                     const int rest = (int)((ctas % wave + sms - 1) / sms);
                     const double t = (double)(ctas / wave) * lane_clocks(L, NT, s, fit) + (rest ? lane_clocks(L, NT, s, rest) : 0.0);
@@ -386,7 +397,7 @@ inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, i
                 ctas += (R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G);
             }
             if (!ok) continue;
-            const int fit = std::max(1, (int)std::min<int64_t>(std::min(32, 1152 / threads), (228 * 1024) / (smem + 1024)));
+            const int fit = lane_counted(threads, smem);
             const int k = (int)std::min<int64_t>(fit, (ctas + sms - 1) / sms);      // CTAs an SM holds at a time
             double t = 0.0, longest = 0.0;
             for (size_t i = 0; i < NTs.size(); ++i) {

@@ -17,11 +17,12 @@
 //   * 2 x 2 cells a step: half of the neighbours are loaded once for two cells, and
 //     loop and address instructions are shared.
 // Bound: warp instruction issue.  A wide multiply holds the dispatch of its
-// sub-partition for two cycles (4 on its pipe); 82 instructions and 16 wide
-// multiplies a word leave 115 clocks at the 85 % issue rate that this mix reaches,
-// against 110 instructions and 199 clocks before.  Measured, C_8 x 32 slots,
-// 1024 runs: 13.4 us per sweep (1.25e12 attempts/s; slot-major 4/32/1: 20.7 us,
-// 8.1e11); one C_8 instance of 64 runs: 2.7 us per sweep (cell-major default: 11.7).
+// sub-partition for two cycles (4 on its pipe).  Measured, C_8 x 32 slots, 1024 runs
+// as 16 candidates, exchange every sweep: 84.5 instructions a word with everything
+// around it, 16 of them wide multiplies, so 100.5 dispatch cycles of the 123 clocks
+// that a word takes on the 147 SMs in use (slot-major 4/32/1: 118 instructions, 199
+// clocks); 13.4 us per sweep, 1.25e12 attempts/s (20.7 us, 8.1e11); one C_8 instance
+// of 64 runs: 2.7 us per sweep (cell-major default: 11.7).
 // Measured and left: 1 or 2 cells a step instead of 4 (1 % slower), keys as immediates
 // (recomputed per round, 7 more uniform instructions a word), accept flags by LOP3
 // instead of adds (1 % slower), by selects (2 % slower).

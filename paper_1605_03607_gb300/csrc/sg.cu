@@ -1384,7 +1384,7 @@ __global__ void __launch_bounds__(RO_THREADS) readout_kernel(int N, const bf16* 
     if (!target) return;
     const float dy = 2.f * (yb - target[b]) * inv_B;
     if (c == 0) {                                  // this graph's loss term and output gradient (summed in order
-        dybuf[b] = dy;                             // over graphs by readout_grad_kernel)
+        dybuf[b] = dy;                             // over graphs by readout_grad)
         sqbuf[b] = (yb - target[b]) * (yb - target[b]) * inv_B;
     }
     if (c < HD) dz[c] = z > 0.f ? dy * w2c : 0.f;
