@@ -88,8 +88,9 @@ struct pt_handle {
     float* d_xhint = nullptr;
     int16_t* d_nbr = nullptr;
     Group main, cand;
-    uint8_t* stage = nullptr;  // pinned staging of state downloads
+    uint8_t* stage = nullptr;  // pinned staging of state downloads, one at a time (threads may read one handle)
     size_t stage_bytes = 0;
+    std::mutex stage_mu;
     int sp = 0, ipc = 0, spl = 4096;
     int team = 0;              // 0: cell-major mapping; > 0: slot-major with teams of this size
     bool planned = true;       // until a schedule is set: mapping and shape by lane_plan
@@ -1104,11 +1105,14 @@ int pt_get_state(pt_handle* h, int8_t* spins, int32_t* E, uint8_t* perm, int32_t
     const bool staged = rec_bytes <= h->stage_bytes, whole = spins && g.block_bytes <= h->stage_bytes;
     const size_t off = whole ? 0 : g.rec_off;
     std::vector<int8_t> sp;
-    if (staged)
+    std::unique_lock<std::mutex> lock(h->stage_mu, std::defer_lock);
+    if (staged) {
+        lock.lock();
         CK(cudaMemcpyAsync(h->stage, g.block + off, g.block_bytes - off, cudaMemcpyDeviceToHost, h->stream), "download state");
-    else
+    } else {
         for (const auto& a : arrays)
             if (a.to) CK(cudaMemcpyAsync(a.to, a.from, a.bytes, cudaMemcpyDeviceToHost, h->stream), "download state");
+    }
     if (spins && !whole) {
         sp.resize(reps * N);
         CK(cudaMemcpyAsync(sp.data(), g.spins, reps * N, cudaMemcpyDeviceToHost, h->stream), "download spins");

@@ -15,6 +15,8 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1605_03607_gb300", "csrc")
 
 RUNTIME = r"""
+#include <unistd.h>
+#include <atomic>
 #include <cstring>
 #include <map>
 #include <vector>
@@ -22,11 +24,13 @@ RUNTIME = r"""
 
 namespace {
 std::map<char*, size_t> device;
-long overruns = 0, down = 0, launches = 0, allocs = 0;
+std::atomic<long> overruns{0}, down{0};
+long launches = 0, allocs = 0;
 long fail_launch = 0, launch_last = 0, fail_alloc = 0, alloc_last = 0;     // failing range, counted from 1
 int fast_team = 0, fast_block = -1, last_team = 0, last_block = 0, last_ctas = 0;
 std::vector<int> seen;                        // runs covered by the last launch: instance * 4096 + run
 bool bad_launch = false;
+int wait_us = 0;                              // length of a stream synchronisation
 bool inside(const void* p, size_t n)
 {
     auto it = device.upper_bound((char*)p);
@@ -74,7 +78,7 @@ cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t)
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)1; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { if (wait_us) usleep(wait_us); return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int) { return cudaSuccess; }
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
@@ -90,7 +94,8 @@ void host_fastest(int team, int block) { fast_team = team; fast_block = block; }
 long host_launches() { return launches; }
 long host_allocs() { return allocs; }
 long host_overruns() { return overruns; }
-long host_downloaded() { const long n = down; down = 0; return n; }
+long host_downloaded() { return down.exchange(0); }
+void host_wait(int us) { wait_us = us; }
 int host_last_team() { return last_team; }
 int host_last_block() { return last_block; }
 int host_last_ctas() { return last_ctas; }

@@ -1,4 +1,6 @@
 """The handle runtime's launch lists and copies on error paths, on the CPU (tests/host_runtime.py)."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -132,6 +134,39 @@ def test_state_downloads_what_is_asked_for(rt, L, NT, R):
                 assert got == sum(want[k].nbytes for k in set(names) | ({"perm"} if "spins" in names else set())), names
             for k in names:
                 assert np.array_equal(out[k], want[k]), k
+
+
+def test_state_read_by_two_threads(rt):
+    """Two threads that read one handle, one everything and one the energies: neither sees the other's copy."""
+    from paper_1605_03607_gb300._lib import _ptr
+    L, NT, R = 4, 16, 8
+    with handle(L, NT, R) as h:
+        s = np.where(np.random.default_rng(2).random((R, NT, 8 * L * L)) < 0.5, -1, 1).astype(np.int8)
+        h.set_spins(s)
+        want = h.state()
+        wrong = []
+        rt.host_wait(300)
+
+        def everything():
+            for _ in range(60):
+                st = h.state()
+                if any(not np.array_equal(st[k], want[k]) for k in want):
+                    wrong.append("state")
+
+        def energies():
+            for _ in range(60):
+                E = np.zeros((R, NT), np.int32)
+                rt.pt_get_state(h.h, None, _ptr(E), None, None, None, None, None, None)
+                if not np.array_equal(E, want["E"]):
+                    wrong.append("E")
+
+        threads = [threading.Thread(target=f) for f in (everything, energies)]
+        for x in threads:
+            x.start()
+        for x in threads:
+            x.join()
+        rt.host_wait(0)
+        assert not wrong
 
 
 SHAPES = [
