@@ -349,6 +349,7 @@ int group_schedule(pt_handle* h, Group& g)
     if (int rc = group_bundles(h, g, bundles, l)) return rc;
     if (l.smem > cap) return fail(h, PT_ERR_ARG, "bundle needs more shared memory than a CTA can have");
     CK(set_sweep_smem_limit(cap, l.team, g.walk, g.L), "cudaFuncSetAttribute");
+    CK(set_sweep_smem_limit(cap, l.team, g.walk, g.L, 1), "cudaFuncSetAttribute");
     Bundle* d = nullptr;
     Bundle* dsub = nullptr;
     CK(dalloc(&d, bundles.size()), "cudaMalloc bundles");

@@ -866,7 +866,7 @@ namespace {
 
 // Bundles of the replica-lane mapping, one after the other (queue: pulled from
 // the launch's work counter).
-template <int LT>
+template <int LT, bool SWEEP>
 __global__ void __launch_bounds__(LANE_THREADS, 1)
 pt_lane_kernel(const InstDesc* __restrict__ insts, const Bundle* __restrict__ bundles, int nbundles, uint32_t sweep0,
                int nsweeps, int xevery, int mode, int* __restrict__ queue)
@@ -880,7 +880,7 @@ pt_lane_kernel(const InstDesc* __restrict__ insts, const Bundle* __restrict__ bu
         b = s_next;
     }
     while (b < nbundles) {
-        process_bundle_lane<LT>(insts, bundles[b], sweep0, nsweeps, xevery, mode, smem);
+        process_bundle_lane<LT, SWEEP>(insts, bundles[b], sweep0, nsweeps, xevery, smem);
         if (!queue) break;
         if (threadIdx.x == 0) s_next = atomicAdd(queue, 1);
         __syncthreads();
@@ -1099,19 +1099,21 @@ unsigned debug_take() { return 0u; }
 #endif
 
 namespace {
-// The sweep kernel of a mapping (by the sign of `team`) for lattice side L.
-const void* sweep_kernel(int team, bool walk, int L)
+// The sweep kernel of a mapping (by the sign of `team`) for lattice side L; mode 1: the kernel of an exchange alone.
+const void* sweep_kernel(int team, bool walk, int L, int mode)
 {
     if (team < 0) {
+        if (mode == 1) return (const void*)pt_lane_kernel<0, false>;
         switch (L) {
-        case 4: return (const void*)pt_lane_kernel<4>;
-        case 6: return (const void*)pt_lane_kernel<6>;
-        case 8: return (const void*)pt_lane_kernel<8>;
-        case 10: return (const void*)pt_lane_kernel<10>;
-        case 12: return (const void*)pt_lane_kernel<12>;
-        case 14: return (const void*)pt_lane_kernel<14>;
-        case 16: return (const void*)pt_lane_kernel<16>;
-        default: return (const void*)pt_lane_kernel<0>;
+        case 2: return (const void*)pt_lane_kernel<2, true>;
+        case 4: return (const void*)pt_lane_kernel<4, true>;
+        case 6: return (const void*)pt_lane_kernel<6, true>;
+        case 8: return (const void*)pt_lane_kernel<8, true>;
+        case 10: return (const void*)pt_lane_kernel<10, true>;
+        case 12: return (const void*)pt_lane_kernel<12, true>;
+        case 14: return (const void*)pt_lane_kernel<14, true>;
+        case 16: return (const void*)pt_lane_kernel<16, true>;
+        default: return (const void*)pt_lane_kernel<0, true>;
         }
     }
     if (team == 0) return walk ? (const void*)pt_sweep_kernel<false, true> : (const void*)pt_sweep_kernel<false, false>;
@@ -1138,12 +1140,12 @@ cudaError_t sweep_smem_capacity(int* bytes)
 
 cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, int team, bool walk, int L)
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_kernel(team, walk, L), block, smem_bytes);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sweep_kernel(team, walk, L, 0), block, smem_bytes);
 }
 
-cudaError_t set_sweep_smem_limit(int bytes, int team, bool walk, int L)
+cudaError_t set_sweep_smem_limit(int bytes, int team, bool walk, int L, int mode)
 {
-    return cudaFuncSetAttribute(sweep_kernel(team, walk, L), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return cudaFuncSetAttribute(sweep_kernel(team, walk, L, mode), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 cudaError_t launch_init(const InstDesc* insts, const int2* items, int nitems, bool draw,
@@ -1168,7 +1170,7 @@ cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nbun
 {
     if (nbundles <= 0) return cudaSuccess;
     void* args[] = {&insts, &bundles, &nbundles, &sweep0, &nsweeps, &xevery, &mode, &queue};
-    cudaLaunchKernel(sweep_kernel(team, walk, L), dim3(grid), dim3(block), args, smem_bytes, st);
+    cudaLaunchKernel(sweep_kernel(team, walk, L, mode), dim3(grid), dim3(block), args, smem_bytes, st);
     return DBG(cudaGetLastError(), st, "sweep kernel");
 }
 

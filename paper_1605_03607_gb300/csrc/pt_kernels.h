@@ -8,9 +8,9 @@ namespace ptg {
 
 // Largest dynamic shared memory a sweep-kernel CTA may request on the current
 // device, and the limit set for the kernel that launch_sweeps picks for
-// (team, walk, L).
+// (team, walk, L, mode).
 cudaError_t sweep_smem_capacity(int* bytes);
-cudaError_t set_sweep_smem_limit(int bytes, int team = 0, bool walk = false, int L = 0);
+cudaError_t set_sweep_smem_limit(int bytes, int team = 0, bool walk = false, int L = 0, int mode = 0);
 // Resident sweep-kernel CTAs per SM for a block size and dynamic shared memory.
 cudaError_t sweep_occupancy(int block, int smem_bytes, int* blocks_per_sm, int team = 0, bool walk = false,
                             int L = 0);
@@ -22,7 +22,7 @@ cudaError_t launch_energy(const InstDesc* insts, const int2* items, int nitems, 
 // team: the mapping of every bundle by its sign (Bundle::team).  walk: the instances carry
 // walk arrays (InstDesc::whot, wtrips, wstate) and the launch updates them.
 // L: the lattice side of every instance in the launch (0 if unknown or mixed);
-// the replica-lane kernel (even L >= 4) and both slot-major kernels (walk tracked
+// the replica-lane kernel (even L) and both slot-major kernels (walk tracked
 // or not; L = 4, 8, 12, 16) have instantiations with the side as a compile-time
 // constant.
 cudaError_t launch_sweeps(const InstDesc* insts, const Bundle* bundles, int nbundles, int grid,

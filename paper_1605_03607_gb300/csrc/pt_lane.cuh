@@ -39,27 +39,36 @@ __device__ __forceinline__ uint4 lane_pre(uint32_t s, int col, int q, int L, uin
     return make_uint4(p.x0b, p.z2x, p.z3, 0u);
 }
 
-// One entry of the field tables: `which` 0 the cell's opposite group (with the
-// bias of 128 per byte), 1 / 2 the minus / plus neighbour, for the mask `nib` of
-// that group's negative spins.  jw holds the negated couplers (InstDesc), so the
-// three entries of an update add up to 128 - h_i in byte i.
-__device__ __forceinline__ uint32_t lane_field(const uint32_t* jw, int which, int nib)
+// The 16 entries of one field table: `which` 0 the cell's opposite group (with the bias of 128 per byte),
+// 1 / 2 the minus / plus neighbour; entry `nib` for the mask of that group's negative spins.  v: the
+// group's 4 words of negated couplers (InstDesc::jw), those inside the cell for which = 0, those between
+// cells otherwise, so the three entries of an update add up to 128 - h_i in byte i.  A spin's sign moves
+// an entry by twice its couplers, whatever the others are: 15 additions (modulo 2^32, as the sum of the
+// three) instead of 16 sums.
+__device__ __forceinline__ void lane_table(uint4* out, const uint4 v, int which)
 {
-    uint32_t w = 0u, sg = 0u;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sg |= ((nib >> k) & 1 ? 0xFFu : 0x01u) << (8 * k);
+    uint32_t base = which == 0 ? 0x80808080u : 0u, d[4] = {0u, 0u, 0u, 0u};
+    const uint32_t jw[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        int v;
         if (which == 0) {
-            v = 128 + __dp4a((int)jw[k], (int)sg, 0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t j = (uint32_t)(int)(int8_t)(jw[k] >> (8 * i)) << (8 * k);
+                base += j;
+                d[i] -= 2u * j;
+            }
         } else {
-            const int j = (int)(int8_t)(jw[4 + k] >> (16 * (k & 1) + 8 * (which - 1)));
-            v = (nib >> k) & 1 ? -j : j;
+            const uint32_t j = (uint32_t)(int)(int8_t)(jw[k] >> (16 * (k & 1) + 8 * (which - 1))) << (8 * k);
+            base += j;
+            d[k] -= 2u * j;
         }
-        w += (uint32_t)v << (8 * k);
     }
-    return w;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        const uint32_t e = base + (n & 1 ? d[2] : 0u) + (n & 2 ? d[3] : 0u);
+        out[n] = make_uint4(e, e + d[0], e + d[1], e + d[0] + d[1]);
+    }
 }
 
 // 0xFF in every byte of x whose sign bit is set, 0 in the others.
@@ -68,6 +77,73 @@ __device__ __forceinline__ uint32_t byte_signs(uint32_t x)
     uint32_t m;
     asm("prmt.b32 %0, %1, 0, 0xBA98;" : "=r"(m) : "r"(x));
     return m;
+}
+
+// The field tables of an instance.
+__device__ __forceinline__ void make_tables(uint4* lut, const uint4* jw, int L2)
+{
+    for (int i = threadIdx.x; i < 6 * L2; i += blockDim.x) {
+        const int cq = i / 3, which = i - cq * 3, c = cq >= L2, q = cq - c * L2;
+        lane_table(lut + 4 * i, __ldg(jw + 4 * q + 2 * c + (which > 0)), which);
+    }
+}
+
+// The thresholds, a column per slot (the columns beyond them are not used).
+__device__ __forceinline__ void make_thresholds(uint32_t* out, const uint32_t* thr, int NT, int kt)
+{
+    for (int i = threadIdx.x; i < NT * kt; i += blockDim.x) {
+        const int k = i / NT, t = i - k * NT;
+        out[((t >> 5) * kt + k) * 32 + (t & 31)] = __ldg(thr + t * kt + k);
+    }
+}
+
+// The same as functions of their own, for the kernels whose sweeps are faster without them in their midst (the
+// compiler orders the sweep loop by what surrounds it).  Sweeps inline / apart: tables, C_4 1.27 / 1.32 us, C_16 with
+// 48 slots 16.98 / 16.72; thresholds, C_4 1.27 / 1.32, C_7 2.62 / 2.61, C_13 12.37 / 12.23.
+__device__ __noinline__ void make_tables_apart(uint4* lut, const uint4* jw, int L2) { make_tables(lut, jw, L2); }
+__device__ __noinline__ void make_thresholds_apart(uint32_t* out, const uint32_t* thr, int NT, int kt) { make_thresholds(out, thr, NT, kt); }
+
+// Spins of whole runs (cell by cell, buffer by buffer) between memory, where a cell has two words (orientation
+// 0 and 1), and the columns of consecutive groups: word u has colour (row + column + u) & 1.  All runs at once, where
+// run by run each waits for its own loads: for the small lattices, whose CTAs hold many runs (one sweep of 1000 C_2
+// runs of 16 slots 23.3 -> 19.0 us).  On the others it took more from the sweep loop than it gave (C_16 with 48
+// slots 15.45 -> 15.65 us a sweep).
+__device__ __forceinline__ unsigned char* spin_at(unsigned char* columns, int i, int L, int per, int group_bytes, int col_bytes, int& odd)
+{
+    const int L2 = L * L, rb = i / L2, q = i - rb * L2, g = rb / per, p = rb - g * per, y = q / L;
+    odd = (y + q - y * L) & 1;
+    return columns + g * group_bytes + (p >> 5) * col_bytes + (q + L) * 32 + (p & 31);
+}
+
+__device__ __noinline__ void load_spins(unsigned char* columns, const uint2* words, int cells, int L, int per, int group_bytes, int col_bytes)
+{
+    constexpr int AHEAD = 4;                    // loads in flight
+    for (int i0 = threadIdx.x; i0 < cells; i0 += AHEAD * blockDim.x) {
+        uint2 v[AHEAD];
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j)
+            if (i0 + j * (int)blockDim.x < cells) v[j] = words[i0 + j * (int)blockDim.x];
+#pragma unroll
+        for (int j = 0; j < AHEAD; ++j) {
+            const int i = i0 + j * (int)blockDim.x;
+            if (i >= cells) break;
+            int odd;
+            unsigned char* const at = spin_at(columns, i, L, per, group_bytes, col_bytes, odd);
+            at[odd ? col_bytes / 2 : 0] = (unsigned char)(((v[j].x & 0x80808080u) * 0x00204081u) >> 26);
+            at[odd ? 0 : col_bytes / 2] = (unsigned char)(((v[j].y & 0x80808080u) * 0x00204081u) >> 26);
+        }
+    }
+}
+
+__device__ __noinline__ void store_spins(unsigned char* columns, uint2* words, int cells, int L, int per, int group_bytes, int col_bytes)
+{
+    for (int i = threadIdx.x; i < cells; i += blockDim.x) {
+        int odd;
+        const unsigned char* const at = spin_at(columns, i, L, per, group_bytes, col_bytes, odd);
+        const uint32_t a = at[0], b = at[col_bytes / 2];                   // colours 0 and 1
+        words[i] = make_uint2(byte_signs((odd ? b : a) * 0x04081020u) | 0x01010101u,
+                              byte_signs((odd ? a : b) * 0x04081020u) | 0x01010101u);   // 0xFF or 1
+    }
 }
 
 struct LaneConst {
@@ -360,9 +436,12 @@ __device__ __forceinline__ void walk_update_warp(const uint8_t* perm, uint32_t* 
     __syncwarp();
 }
 
-template <int LT>
+// SWEEP: nsweeps sweeps with their exchanges, from counter sweep0 + 1 on; else one exchange with counter sweep0, which
+// needs neither field and threshold tables nor spins (C_12, 24 slots, 16 runs: a call 39.5 -> 14.5 us, and the sweeps
+// without its branches 2 to 3 % faster on C_4 and C_8).
+template <int LT, bool SWEEP>
 __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bundle bd, uint32_t sweep0, int nsweeps,
-                                    int xevery, int mode, unsigned char* smem)
+                                    int xevery, unsigned char* smem)
 {
     const InstDesc& in0 = insts[bd.inst];
 #ifdef PT_DEBUG
@@ -398,14 +477,14 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
     int32_t* xoff_sm = reinterpret_cast<int32_t*>(smem + lay.xtab);
     uint4* pre = reinterpret_cast<uint4*>(gb);
     auto gsync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(gw * 32) : "memory"); };
-    const int n_iter = (mode == 0) ? nsweeps : 1;
-    const uint32_t s_first = (mode == 0) ? sweep0 + 1u : sweep0;
+    const int n_iter = SWEEP ? nsweeps : 1;
+    const uint32_t s_first = SWEEP ? sweep0 + 1u : sweep0;
     const uint32_t* const xthr = in0.xthr;
     // sweeps to the next exchange, counted down from sweep s_first on (0: exchange after that sweep)
-    const bool xon = NT > 1 && (mode == 1 || xevery > 0);
-    const uint32_t xper = mode == 1 || xevery < 1 ? 1u : (uint32_t)xevery;
+    const bool xon = NT > 1 && (!SWEEP || xevery > 0);
+    const uint32_t xper = !SWEEP || xevery < 1 ? 1u : (uint32_t)xevery;
     uint32_t xwait = (xper - s_first % xper) % xper;
-    if (mode == 1) xwait = 0u;
+    if (!SWEEP) xwait = 0u;
 
     // run r of the bundle: its instance, its run there, and its place in shared memory
     auto inst_of = [&](int r) -> const InstDesc& { return r < bd.nitems ? in0 : insts[bd.inst2]; };
@@ -413,31 +492,39 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
     auto slot_of = [&](int r) { return r < bd.nitems ? r : ng1 * gr + r - bd.nitems; };      // group * gr + place
 
     // ---- tables, then this bundle's runs
-    {
-        uint32_t* lut = reinterpret_cast<uint32_t*>(smem + lay.lut);
-        for (int s = 0; s < (bd.nitems2 > 0 ? 2 : 1); ++s, lut += 96 * L2) {
-            const uint32_t* jw = insts[s == 0 ? bd.inst : bd.inst2].jw;
-            for (int i = tid; i < 2 * L2 * 48; i += blockDim.x) {
-                const int cq = i / 48, e = i - cq * 48, c = cq / L2, q = cq - c * L2;
-                lut[i] = lane_field(jw + (q * 2 + c) * 8, e >> 4, e & 15);
+    for (int p = tid; p < NT; p += blockDim.x) {
+        xoff_sm[p] = in0.xoff[p];
+        reinterpret_cast<float*>(xoff_sm + NT)[p] = p < NT - 1 ? in0.xhint[p] : 0.0f;
+    }
+    constexpr bool FLAT = LT == 2;              // staging over all groups and runs at once
+    if (SWEEP) {
+        uint4* lut = reinterpret_cast<uint4*>(smem + lay.lut);
+        for (int s = 0; s < (bd.nitems2 > 0 ? 2 : 1); ++s, lut += 24 * L2) {
+            const uint4* jw = reinterpret_cast<const uint4*>(insts[s == 0 ? bd.inst : bd.inst2].jw);
+            if (LT > 4) make_tables_apart(lut, jw, L2);
+            else make_tables(lut, jw, L2);
+        }
+        uint32_t* const thr = reinterpret_cast<uint32_t*>(smem + lay.thr);
+        if (LT != 4) make_thresholds_apart(thr, in0.thr, NT, kt);
+        else make_thresholds(thr, in0.thr, NT, kt);
+        if (FLAT) {
+            const int nz = lay.ncols * lay.col_bytes / 16;
+            for (int i = tid; i < ngroups * nz; i += blockDim.x)
+                reinterpret_cast<uint4*>(group_base(i / nz) + lay.spins)[i % nz] = make_uint4(0u, 0u, 0u, 0u);
+            for (int i = tid; i < ngroups * 2 * L2; i += blockDim.x) {
+                const int g = i / (2 * L2), q = i - g * 2 * L2;
+                const InstDesc& ig = g < ng1 ? in0 : insts[bd.inst2];
+                reinterpret_cast<uint4*>(group_base(g))[q] = lane_pre(s_first, q >= L2, q >= L2 ? q - L2 : q, L, ig.seed, ig.uid);
             }
-        }
-        uint32_t* thr = reinterpret_cast<uint32_t*>(smem + lay.thr);
-        for (int i = tid; i < (NT + 31) / 32 * 32 * kt; i += blockDim.x) {
-            const int b = i / (32 * kt), k = (i >> 5) - b * kt, t = b * 32 + (i & 31);
-            thr[i] = t < NT ? in0.thr[t * kt + k] : 0u;
-        }
-        for (int p = tid; p < NT; p += blockDim.x) {
-            xoff_sm[p] = in0.xoff[p];
-            reinterpret_cast<float*>(xoff_sm + NT)[p] = p < NT - 1 ? in0.xhint[p] : 0.0f;
-        }
-        for (int g = 0; g < ngroups; ++g) {
-            uint32_t* sp = reinterpret_cast<uint32_t*>(group_base(g) + lay.spins);
-            for (int i = tid; i < lay.ncols * lay.col_bytes / 4; i += blockDim.x) sp[i] = 0u;
-            uint4* pg = reinterpret_cast<uint4*>(group_base(g));
-            const InstDesc& ig = g < ng1 ? in0 : insts[bd.inst2];
-            for (int i = tid; i < 2 * L2; i += blockDim.x)
-                pg[i] = lane_pre(s_first, i >= L2, i >= L2 ? i - L2 : i, L, ig.seed, ig.uid);
+        } else {
+            for (int g = 0; g < ngroups; ++g) {
+                uint32_t* sp = reinterpret_cast<uint32_t*>(group_base(g) + lay.spins);
+                for (int i = tid; i < lay.ncols * lay.col_bytes / 4; i += blockDim.x) sp[i] = 0u;
+                uint4* pg = reinterpret_cast<uint4*>(group_base(g));
+                const InstDesc& ig = g < ng1 ? in0 : insts[bd.inst2];
+                for (int i = tid; i < 2 * L2; i += blockDim.x)
+                    pg[i] = lane_pre(s_first, i >= L2, i >= L2 ? i - L2 : i, L, ig.seed, ig.uid);
+            }
         }
     }
     for (int i = tid; i < nruns * NT; i += blockDim.x) {
@@ -469,7 +556,14 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
         const int p = (at % gr) * NT + b;
         return group_base(at / gr) + lay.spins + (p >> 5) * lay.col_bytes + cl * (lay.col_bytes / 2) + (q + L) * 32 + (p & 31);
     };
-    for (int r = 0; r < nruns; ++r) {
+    if (SWEEP && FLAT) {
+        load_spins(group_base(0) + lay.spins, reinterpret_cast<uint2*>(in0.spins + (size_t)bd.run0 * NT * N), bd.nitems * NT * L2, L,
+           gr * NT, lay.group_bytes, lay.col_bytes);
+        if (bd.nitems2 > 0)
+            load_spins(group_base(ng1) + lay.spins, reinterpret_cast<uint2*>(insts[bd.inst2].spins), bd.nitems2 * NT * L2, L,
+               gr * NT, lay.group_bytes, lay.col_bytes);
+    }
+    for (int r = 0; r < (SWEEP && !FLAT ? nruns : 0); ++r) {
         const uint32_t* gsp = spin_words(r);
         const int at = slot_of(r);
         for (int i = tid; i < NT * NW; i += blockDim.x)
@@ -499,7 +593,7 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
             const uint32_t s = s_first + (uint32_t)it;
             const bool do_x = xon && xwait == 0u;
             xwait = xwait == 0u ? xper - 1u : xwait - 1u;          // from here on: of sweep s + 1
-            if (mode == 0) {
+            if (SWEEP) {
                 uint32_t dk = 0u, pc = 0u;
                 const int t = PT_IDX((int)(rb + rl.inv)[buf], NT, 2u);
                 const PhiloxPre ps = philox_pre(s, 0u, k0, k1);
@@ -535,7 +629,7 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
                 } else {
                     m = slot_min_warp(Es, NT, lane);
                 }
-                if (lane == 0 && mode == 0 && m < record) {
+                if (SWEEP && lane == 0 && m < record) {
                     misc[0] = m;
                     misc[1] = (int32_t)s;
                 }
@@ -555,7 +649,14 @@ __device__ void process_bundle_lane(const InstDesc* __restrict__ insts, const Bu
 
     // ---- write the state back
     __syncthreads();
-    for (int r = 0; r < nruns; ++r) {
+    if (SWEEP && FLAT) {
+        store_spins(group_base(0) + lay.spins, reinterpret_cast<uint2*>(in0.spins + (size_t)bd.run0 * NT * N), bd.nitems * NT * L2, L,
+           gr * NT, lay.group_bytes, lay.col_bytes);
+        if (bd.nitems2 > 0)
+            store_spins(group_base(ng1) + lay.spins, reinterpret_cast<uint2*>(insts[bd.inst2].spins), bd.nitems2 * NT * L2, L,
+               gr * NT, lay.group_bytes, lay.col_bytes);
+    }
+    for (int r = 0; r < (SWEEP && !FLAT ? nruns : 0); ++r) {
         uint32_t* gsp = spin_words(r);
         const int at = slot_of(r);
         for (int i = tid; i < NT * NW; i += blockDim.x)

@@ -115,7 +115,7 @@ int host_last_launch_ok(int n, int runs)
 
 namespace ptg {
 cudaError_t sweep_smem_capacity(int* b) { *b = 232448 - 16; return cudaSuccess; }
-cudaError_t set_sweep_smem_limit(int, int, bool, int) { return cudaSuccess; }
+cudaError_t set_sweep_smem_limit(int, int, bool, int, int) { return cudaSuccess; }
 cudaError_t launch_init(const InstDesc*, const int2*, int, bool, cudaStream_t) { return cudaSuccess; }
 // a state that can be told apart: records by their index, slots in reverse order
 cudaError_t launch_energy(const InstDesc* insts, const int2* items, int nitems, int32_t, cudaStream_t)

@@ -98,6 +98,41 @@ def test_planned_mapping_of_a_size(P, L, NT, R, mapping):
         assert h.launch_shape()["mapping"] == mapping
 
 
+@pytest.mark.parametrize("L,NT,R", [(2, 1, 9), (2, 13, 1000), (2, 33, 5), (2, 64, 130), (1, 5, 600), (3, 32, 70)])
+@pytest.mark.parametrize("spl", [1, 4])
+def test_short_launches_of_small_lattices(P, L, NT, R, spl):
+    """Every launch stages and writes back the state, many runs a CTA."""
+    J, betas = W.random_couplers(L, 4, NT), W.beta_ladder(NT, 0.1, 3.0) if NT > 1 else np.array([1.0])
+    ref = oracle.PTState(L, J, betas, R, 4, NT)
+    ref.sweeps(9, 1)
+    with P.PTHandle(L, J, betas, R, 4, NT) as h:
+        h.set_schedule(0, 0, spl)
+        h.sweep(9, 1)
+        st = h.state()
+    for k in ("spins", "E", "best", "first", "macc") + (("xacc",) if NT > 1 else ()):
+        assert np.array_equal(st[k], getattr(ref, k)), k
+
+
+@pytest.mark.parametrize("L,NT,R", [(4, 2, 3), (8, 32, 70), (7, 33, 5), (12, 24, 16), (16, 64, 2), (2, 40, 300)])
+def test_exchanges_alone(P, L, NT, R):
+    """Exchange passes of their own, one after another and between sweeps, with the walk tracked."""
+    J, betas = W.random_couplers(L, 6, NT), W.beta_ladder(NT, 0.1, 3.0)
+    ref = oracle.PTState(L, J, betas, R, 6, NT, walk=True)
+    with P.PTHandle(L, J, betas, R, 6, NT) as h:
+        h.set_walk_stats(True)
+        for n in (0, 2, 1):
+            h.sweep(n, 0)
+            ref.sweeps(n, 0)
+            for _ in range(3):
+                h.exchange()
+                ref.exchange()
+        hot, trips, passes = h.walk_stats()
+        st = h.state()
+        same_state(st, ref)
+        assert np.array_equal(st["E"], ref.full_energies())
+    assert passes == ref.n_passes and np.array_equal(hot, ref.hot) and np.array_equal(trips, ref.trips)
+
+
 @pytest.mark.parametrize("L,NT,R,k", [(2, 17, 25, 24), (3, 7, 100, 24), (6, 17, 25, 24), (8, 7, 256, 16)])
 def test_candidates_share_ctas(P, L, NT, R, k):
     """Candidates whose run counts do not divide into whole CTAs: some CTA holds runs of two."""
