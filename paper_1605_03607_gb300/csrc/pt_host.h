@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <cstdlib>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "pt_internal.h"
@@ -233,12 +234,17 @@ inline int lane_threads(int NT, const LaneShape& s) { return 32 * s.W * lane_col
 // an earlier kernel whose exchange took 200 to 300 clocks longer: there the lowest estimate's
 // shape was 0.5 % slower than the best one on average, 3 % at most.  On the kernel as it is that
 // has not been measured; 750 and 600 in place of 910 changed no plan for the better.
-inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
+inline double lane_words(int L, int NT, const LaneShape& s)            // of a group, with its shares' imbalance
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);      // what the warps of a column share out
     const int c = lane_columns(NT, s.gr), per = (units + s.W - 1) / s.W, nw = s.G * c * s.W;
-    const double words = 2.0 * L * L * c * per * s.W / units * ((nw + 3) / 4 * 4) / nw, n = (double)k * s.G;
-    const double w1 = 0.25 * c * s.W, x = 910.0;
+    return 2.0 * L * L * c * per * s.W / units * ((nw + 3) / 4 * 4) / nw;
+}
+
+inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
+{
+    const double words = lane_words(L, NT, s), n = (double)k * s.G;
+    const double w1 = 0.25 * lane_columns(NT, s.gr) * s.W, x = 910.0;
     const double together = 0.25 * words * n * (117.0 + 130.0 / (w1 * n)) + x / std::pow(n, 0.7);
     return std::max(together, 0.25 * words * (117.0 + 130.0 / w1) + x);
 }
@@ -296,6 +302,11 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
             for (int span = 0; span < 2; ++span) {
                 const int64_t per = (R + gr - 1) / gr;                  // groups of an instance
                 if (span && (n_inst == 1 || per % G == 0)) continue;    // (G - 1) * gr < R: at most two instances a CTA
+                const int64_t ctas = span ? (n_inst * per + G - 1) / G : n_inst * ((per + G - 1) / G);
+                // groups of the SM with most CTAs: where their words alone, evenly shared, take longer than the best shape
+                // so far, no warp count helps.  Most shapes end here (C_8 x 4 slots x 100 runs: a plan 18 -> 3 us)
+                const double most = (double)((ctas + sms - 1) / sms) * G;
+                if (0.25 * 117.0 * (2.0 * L * L * lane_columns(NT, gr)) * most > best_t) continue;
                 const int64_t smem = lane_layout(L, NT, kt, gr, G, walk, span ? 2 : 1).bytes;
                 if (smem > cap) continue;
                 for (int W : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
@@ -306,10 +317,12 @@ inline LaneShape lane_plan(int L, int NT, int kt, int R, int n_inst, bool walk, 
                     s.span = span != 0;
                     const int threads = lane_threads(NT, s);
                     if (threads > LANE_THREADS || (W > units && W > 1)) break;
+                    if (0.25 * 117.0 * lane_words(L, NT, s) * most > best_t) continue;
                     const int fit = lane_counted(threads, smem);
-                    const int64_t ctas = span ? (n_inst * per + G - 1) / G : n_inst * ((per + G - 1) / G), wave = (int64_t)fit * sms;
+                    const int64_t wave = (int64_t)fit * sms;
                     const int rest = (int)((ctas % wave + sms - 1) / sms);
-                    const double t = (double)(ctas / wave) * lane_clocks(L, NT, s, fit) + (rest ? lane_clocks(L, NT, s, rest) : 0.0);
+                    const double t = (ctas >= wave ? (double)(ctas / wave) * lane_clocks(L, NT, s, fit) : 0.0) +
+                                     (rest ? lane_clocks(L, NT, s, rest) : 0.0);
                     if (t < best_t * 0.999) { best_t = t; best = s; }
                 }
             }
@@ -382,6 +395,14 @@ inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, i
                             double* clocks = nullptr)
 {
     const int units = (L & 1) ? L * L / 2 + 1 : (L / 2) * (L / 2);
+    std::vector<std::pair<int, int>> kinds;            // temperature counts and their instances: a kind is looked at once
+    {
+        std::vector<int> count(MAX_TEMPS + 1, 0);
+        for (int nt : NTs) ++count[(size_t)nt];
+        for (int nt = 1; nt <= MAX_TEMPS; ++nt)
+            if (count[(size_t)nt]) kinds.push_back({nt, count[(size_t)nt]});
+    }
+    std::vector<LaneShape> s(kinds.size());
     double best = 1e300;
     for (int ct = 1; ct <= 32; ++ct)
         for (int w : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32}) {
@@ -389,20 +410,19 @@ inline bool lane_plan_batch(int L, const std::vector<int>& NTs, int kt, int R, i
             if (threads > LANE_THREADS || (w > units && w > 1)) break;
             int64_t smem = 0, ctas = 0;
             bool ok = true;
-            std::vector<LaneShape> s(NTs.size());
-            for (size_t i = 0; ok && i < NTs.size(); ++i) {
-                ok = lane_fill(L, NTs[i], kt, R, w, ct, cap, &s[i]);
+            for (size_t i = 0; ok && i < kinds.size(); ++i) {
+                ok = lane_fill(L, kinds[i].first, kt, R, w, ct, cap, &s[i]);
                 if (!ok) break;
-                smem = std::max<int64_t>(smem, lane_layout(L, NTs[i], kt, s[i].gr, s[i].G, false).bytes);
-                ctas += (R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G);
+                smem = std::max<int64_t>(smem, lane_layout(L, kinds[i].first, kt, s[i].gr, s[i].G, false).bytes);
+                ctas += (int64_t)kinds[i].second * ((R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G));
             }
             if (!ok) continue;
             const int fit = lane_counted(threads, smem);
             const int k = (int)std::min<int64_t>(fit, (ctas + sms - 1) / sms);      // CTAs an SM holds at a time
             double t = 0.0, longest = 0.0;
-            for (size_t i = 0; i < NTs.size(); ++i) {
-                const double one = lane_clocks(L, NTs[i], s[i], k);
-                t += one / k * ((R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G));
+            for (size_t i = 0; i < kinds.size(); ++i) {
+                const double one = lane_clocks(L, kinds[i].first, s[i], k);
+                t += one / k * kinds[i].second * ((R + s[i].gr * s[i].G - 1) / (s[i].gr * s[i].G));
                 longest = std::max(longest, one);
             }
             t = std::max(t / sms, longest);
