@@ -250,7 +250,7 @@ inline double lane_clocks(int L, int NT, const LaneShape& s, int k)
 }
 
 // CTAs that the estimate counts on an SM, which its constants were fitted with.  The device holds fewer of
-// the small ones: 1024 threads (64 registers each, from 58 in the kernel for odd sides) and 4 CTAs of any
+// the small ones: 1024 threads (59 to 62 registers each, allocated as 64) and 4 CTAs of any
 // size (16 named barriers each, 64 an SM).  That count with the same constants is no better a rule: of 4000
 // random sizes 126 take another shape, 1.07 times faster on average but from 0.87 (C_4 x 58 slots, 195
 // runs, 14 candidates) to 1.43 (C_1 x 39, 133, 16), and a batch of C_2 to C_8 0.68.  It needs a fit of its own.

@@ -18,10 +18,10 @@
 //     loop and address instructions are shared.
 // Bound: warp instruction issue.  A wide multiply holds the dispatch of its
 // sub-partition for two cycles (4 on its pipe).  Measured, C_8 x 32 slots, 1024 runs
-// as 16 candidates, exchange every sweep: 84.5 instructions a word with everything
-// around it, 16 of them wide multiplies, so 100.5 dispatch cycles of the 123 clocks
+// as 16 candidates, exchange every sweep: 83.3 instructions a word with everything
+// around it, 16 of them wide multiplies, so 99.3 dispatch cycles of the 122 clocks
 // that a word takes on the 147 SMs in use (slot-major 4/32/1: 118 instructions, 199
-// clocks); 13.4 us per sweep, 1.25e12 attempts/s (20.7 us, 8.1e11); one C_8 instance
+// clocks); 13.2 us per sweep, 1.27e12 attempts/s (20.7 us, 8.1e11); one C_8 instance
 // of 64 runs: 2.7 us per sweep (cell-major default: 11.7).
 // Measured and left: 1 or 2 cells a step instead of 4 (1 % slower), keys as immediates
 // (recomputed per round, 7 more uniform instructions a word), accept flags by LOP3
